@@ -19,7 +19,7 @@ struct WsHeader {
   int sweeps;               // Jacobi sweeps used
   long long r;              // truncation rank chosen by pylom_pod
   unsigned barrier_count;   // grid barrier: arrivals
-  unsigned spare;
+  unsigned gram_y;          // pylom_pod: 1 when Y was left unfactored (the Gram route)
   unsigned rot[64];         // Jacobi: rotations performed in each sweep
   unsigned char pad0[384 - 24 - 64 * 4];
   unsigned barrier_gen;     // grid barrier: generation (own line)

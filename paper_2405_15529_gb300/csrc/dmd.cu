@@ -33,6 +33,7 @@
 //                   POD's top-down pass and leaf modes kernels.
 #include <float.h>
 
+#include "gram.h"
 #include "kernels.h"
 
 namespace pylom {
@@ -164,6 +165,18 @@ __global__ void dmd_t1_kernel(DmdState d, const double* R, const double* S, cons
     double s = 0.0;
     for (int64_t j = (i > 0 ? i - 1 : 0); j < M1; ++j) s = fma(R[i + (j + 1) * M], d.VT[c + j * M1], s);
     d.T1[i + c * M] = s / S[c];
+  }
+}
+
+// T1 for modes formed from the snapshots themselves, Y2 V S^-1 = Y [0; V S^-1]
+__global__ void dmd_shift_kernel(DmdState d, const double* S, const WsHeader* hdr) {
+  const int64_t r = dmd_rank(hdr);
+  if (read_status(hdr) != 0) return;
+  const int64_t M = d.M, M1 = d.M1;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * r;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % M, c = idx / M;
+    d.T1[idx] = i > 0 ? d.VT[c + (i - 1) * M1] / S[c] : 0.0;
   }
 }
 
@@ -930,7 +943,7 @@ int grid_for(int64_t work, int threads) {
 
 size_t dmd_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max) {
   return sizeof(WsHeader) + tsqr_state_bytes(N, M, P, r_max, true) + svd_state_bytes(M - 1) +
-         dmd_small_bytes(M, r_max);
+         dmd_small_bytes(M, r_max) + gram_bytes(M, r_max);
 }
 
 }  // namespace
@@ -1008,8 +1021,24 @@ extern "C" pylom_status pylom_dmd(const void* X, int64_t N, int64_t M, int64_t l
   if ((e = cudaMemsetAsync(ts.arrive, 0, sizeof(unsigned) * (size_t)P, st)) != cudaSuccess)
     return fail("counter clear");
   // Y = D - mean (over all M snapshots) = Q R
-  if ((e = launch_tsqr_fp64(ts, X, ldx, xtype, nullptr, remove_mean, mean, st)) != cudaSuccess)
+  // With the automatic leaf height R comes from the Gram route (gram.cu) and
+  // the modes from Y itself: phi = Y2 V S^-1 w / mu with r already cut to the
+  // numerical rank, the same eps |Y| / s_r accuracy that B = R V S^-1 w / mu
+  // has on the Householder route.
+  const bool gram = leaf_rows == 0 && !tree_requested();
+  GramState gs;
+  if (gram) {
+    gs.hdr = hdr;
+    gs.N = N;
+    gs.ldy = ts.ldy;
+    gs.Y = ts.Y;
+    gs.f32 = false;
+    gram_carve(gs, p2 + svd_state_bytes(M1) + dmd_small_bytes(M, r_max), M, r_max);
+    if ((e = launch_gram_r(gs, X, ldx, xtype, nullptr, remove_mean, mean, ts.Rs, st, nullptr)) != cudaSuccess)
+      return fail("Gram matrix / Cholesky");
+  } else if ((e = launch_tsqr_fp64(ts, X, ldx, xtype, nullptr, remove_mean, mean, st)) != cudaSuccess) {
     return fail("leaf QR / tree");
+  }
   // SVD of Y1 = Q[:, :M-1] R[:M-1, :M-1]; truncation by energy and r_max
   if ((e = launch_svd_fp64(ss, ts.Rs, M, d.UR, M1, S, d.VT, M1, 60, energy, r_max, st)) != cudaSuccess)
     return fail("small SVD");
@@ -1022,8 +1051,15 @@ extern "C" pylom_status pylom_dmd(const void* X, int64_t N, int64_t M, int64_t l
   dmd_p_kernel<<<grid_for(r_max * r_max, kSmallThreads), kSmallThreads, 0, st>>>(d, hdr);
   dmd_q_kernel<<<(unsigned)r_max, kSmallThreads, 0, st>>>(d, S, hdr);
   dmd_amp_kernel<<<1, kSmallThreads, 0, st>>>(d, hdr, mu, b);
+  if (gram) dmd_shift_kernel<<<grid_for(M * r_max, kSmallThreads), kSmallThreads, 0, st>>>(d, S, hdr);
   dmd_pack_kernel<<<grid_for(M * r_max, kSmallThreads), kSmallThreads, 0, st>>>(d, hdr);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail("small DMD kernels");
+  if (gram) {
+    if ((e = launch_modes_direct(gs, d.Bp, nullptr, nullptr, 0, nullptr, 0, Phi, ldphi, r_out, st, nullptr)) !=
+        cudaSuccess)
+      return fail("modes");
+    return PYLOM_OK;
+  }
   // phi = Q [B; 0]: the POD's top-down pass and leaf modes product, r read on the device
   if ((e = launch_modes_fp64(ts, d.Bp, M, -1, nullptr, 0, Phi, ldphi, r_out, st)) != cudaSuccess)
     return fail("modes");

@@ -1,0 +1,659 @@
+// gram.cu -- R of the weighted, mean-removed snapshot matrix Y from its Gram
+// matrix (pyLOM, arXiv 2405.15529, Eq. svdqr1: Y = Q R, R unique up to row
+// signs, R^T R = Y^T Y).
+//
+// In working precision the Gram matrix would lose the small singular values
+// (its rounding error is eps sigma_1^2).  Here it is exact: every element of
+// Y is a fixed-point integer relative to its column's largest magnitude, cut
+// into 8-bit digits whose products run on the tcgen05 tensor cores without
+// rounding (digits.cuh), and the sums stay integers until the end.  The
+// Cholesky factorisation then runs in double-double arithmetic (106 bits),
+// so R carries the backward error of a Householder QR in binary64 (the
+// square root of 2^-104) at a fraction of its binary64 work, which this part
+// does at 1/60 of its binary32 rate.
+//
+// Measured (4,194,304 x 256, binary64): Householder leaves + tree 554 + 13
+// ms; here Y 8.2, Gram matrix 51.5, Cholesky factor 1.3 ms.  1,048,576 x 128
+// leaves + tree 39 + 3.8 ms.  Binary32 leaves (mixed, 4,194,304 x 256) 57.7 +
+// 8.8 ms; here 6.4, 18.6 and 1.3 ms.
+#include <atomic>
+
+#include "digits.cuh"
+#include "gram.h"
+
+namespace pylom {
+
+// ---------------------------------------------------------------------------
+// Y = sqrt(w) (X - mean)
+// ---------------------------------------------------------------------------
+
+constexpr int kPrThreads = 256;   // 8 warps; lane = row, a warp takes every 8th column
+
+struct PrologueArgs {
+  const void* X;
+  int64_t ldx;
+  const double* w;
+  int remove_mean;
+  double* mean;
+  void* Y;
+  int64_t ldy, N, M;
+  int* colE;
+  WsHeader* hdr;
+};
+
+// sum of one thread's values of a row (CT of them, zeros past M) as a binary64
+__device__ __forceinline__ double part_sum(const double* x, int n) {
+  double s = 0.0;
+  for (int t = 0; t < n; ++t) s += x[t];
+  return s;
+}
+
+template <typename TX, typename TY, int CT>
+__global__ void __launch_bounds__(kPrThreads) gram_prologue_kernel(PrologueArgs a) {
+  __shared__ double ssum[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const TX* X = (const TX*)a.X;
+  TY* Y = (TY*)a.Y;
+  int bad = 0;
+  // column groups of 8 CT columns; one group when M <= 8 CT (the row then
+  // stays in registers between its mean and its centred values)
+  int emax[CT];
+#pragma unroll
+  for (int t = 0; t < CT; ++t) emax[t] = 0;
+  const bool one = a.M <= 8 * CT;
+  const int64_t nblk = (a.ldy + 31) / 32;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    const int64_t n = blk * 32 + lane;
+    const bool in = n < a.N;
+    TX x[CT];
+    double s = 0.0;
+    for (int64_t c0 = 0; c0 < a.M; c0 += 8 * CT) {
+#pragma unroll
+      for (int t = 0; t < CT; ++t) {
+        const int64_t c = c0 + warp + 8 * t;
+        x[t] = (in && c < a.M) ? X[n + c * a.ldx] : (TX)0;
+      }
+      if (a.remove_mean) {
+        if constexpr (sizeof(TX) == 4) {
+          // compensated binary32 sums in chunks of at most 16 (binary64
+          // conversions and additions are slow on this part)
+          constexpr int K = CT < 16 ? CT : 16;
+#pragma unroll
+          for (int t0 = 0; t0 < CT; t0 += K) {
+            float v[K], h, l;
+#pragma unroll
+            for (int t = 0; t < K; ++t) v[t] = x[t0 + t];
+            sum32_compensated(v, h, l);
+            s += (double)h + (double)l;
+          }
+        } else {
+#pragma unroll
+          for (int t = 0; t < CT; ++t) s += (double)x[t];
+        }
+      }
+    }
+    double xbar = 0.0;
+    if (a.remove_mean) {
+      ssum[warp][lane] = s;
+      __syncthreads();
+      double tot = 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) tot += ssum[q][lane];
+      xbar = tot / (double)a.M;
+      __syncthreads();
+    }
+    double sw = 1.0;
+    if (a.w && in) {
+      const double wn = a.w[n];
+      if (!(wn > 0.0) || !isfinite(wn)) bad = 1;
+      sw = sqrt(wn);
+    }
+    if (warp == 0 && in && a.mean) a.mean[n] = xbar;
+    const float xh = (float)xbar, xl = (float)(xbar - (double)xh);
+    const float sh = (float)sw, sl = (float)(sw - (double)sh);
+    for (int64_t c0 = 0; c0 < a.M; c0 += 8 * CT) {
+      if (!one) {
+#pragma unroll
+        for (int t = 0; t < CT; ++t) {
+          const int64_t c = c0 + warp + 8 * t;
+          x[t] = (in && c < a.M) ? X[n + c * a.ldx] : (TX)0;
+          emax[t] = 0;
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < CT; ++t) {
+        const int64_t c = c0 + warp + 8 * t;
+        if (c >= a.M) continue;
+        TY y;
+        if constexpr (sizeof(TX) == 4 && sizeof(TY) == 4) {
+          // x - mean as d + e by TwoSum, times sqrt(w) = sh + sl by two FMAs
+          float d, e;
+          two_sum32(x[t], -xh, d, e);
+          y = __fmaf_rn(d, sh, __fmaf_rn(d, sl, __fmul_rn(__fsub_rn(e, xl), sh)));
+        } else {
+          double v = (double)x[t];
+          if (a.remove_mean) v -= xbar;
+          if (a.w) v *= sw;
+          y = (TY)v;
+        }
+        if (!in) y = (TY)0;
+        const int e = exp_field(y);
+        emax[t] = e > emax[t] ? e : emax[t];
+        if (!isfinite(x[t])) bad = 1;
+        if (n < a.ldy) Y[n + c * a.ldy] = y;
+      }
+      if (!one) {
+#pragma unroll
+        for (int t = 0; t < CT; ++t) {
+          const int64_t c = c0 + warp + 8 * t;
+          const int e = __reduce_max_sync(0xffffffffu, emax[t]);
+          if (lane == 0 && c < a.M && e > __ldcg(a.colE + c)) atomicMax(a.colE + c, e);
+        }
+      }
+    }
+  }
+  if (one) {
+#pragma unroll
+    for (int t = 0; t < CT; ++t) {
+      const int64_t c = warp + 8 * t;
+      const int e = __reduce_max_sync(0xffffffffu, emax[t]);
+      if (lane == 0 && c < a.M) atomicMax(a.colE + c, e);
+    }
+  }
+  if (bad) raise_status(a.hdr, PYLOM_ERR_NONFINITE);
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.hdr->gram_y = 1;
+}
+
+// ---------------------------------------------------------------------------
+// exact Gram matrix
+// ---------------------------------------------------------------------------
+// A unit is an output tile of 128 x 64 columns of Y on or above the
+// diagonal, a range of digit levels (two for binary64: eight accumulators of
+// 64 columns fill the tensor memory) and a range of rows.  16 warps cut rows
+// of Y into digit planes in shared memory (a thread takes 8 rows of one
+// column: 64 contiguous bytes in, one conflict-free 16-byte store per digit
+// out) and one thread issues a stage's MMAs once all warps have written it;
+// every 128 rows the accumulators are added to 64-bit integers in registers
+// (after the next stages have been filled, so the warps work while the last
+// MMAs of the sum run), and at the end those go to the global sums by
+// integer atomics, so the result does not depend on the order.
+
+constexpr int kGrThreads = 512;   // 128 registers a thread: 64 hold the integer sums
+
+struct GramArgs {
+  const void* Y;
+  int64_t ldy, N, M;
+  const int* colE;
+  unsigned long long* G;
+  int nJ, items, splits;
+  WsHeader* hdr;
+};
+
+template <typename TY>
+__device__ __forceinline__ void load8(const TY* p, TY (&y)[8]);
+template <>
+__device__ __forceinline__ void load8<double>(const double* p, double (&y)[8]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double2 v = __ldg((const double2*)p + i);
+    y[2 * i] = v.x;
+    y[2 * i + 1] = v.y;
+  }
+}
+template <>
+__device__ __forceinline__ void load8<float>(const float* p, float (&y)[8]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float4 v = __ldg((const float4*)p + i);
+    y[4 * i] = v.x;
+    y[4 * i + 1] = v.y;
+    y[4 * i + 2] = v.z;
+    y[4 * i + 3] = v.w;
+  }
+}
+
+// digits of 8 rows of one column into a stage plane (zeros outside Y)
+template <typename TY>
+__device__ __forceinline__ void put_column8(const TY* Y, int64_t ldy, int64_t row, int64_t col, int64_t M, int E,
+                                            unsigned char* dst, int plane) {
+  constexpr int S = Dig<TY>::S;
+  uint64_t w[8];
+  if (col < M && row < ldy) {
+    TY y[8];
+    load8(Y + row + col * ldy, y);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = bias_digits(to_fixed(y[i], E));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = bias_digits(0);
+  }
+  store_digits<S>(w, dst, plane);
+}
+
+// one integer sum into the global groups: the low 32 bits to group g, the
+// carry to group g + 1 (so no group can overflow)
+__device__ __forceinline__ void add_group(unsigned long long* G, int64_t MM, int64_t at, int g, int64_t v) {
+  if (v == 0) return;
+  atomicAdd(G + g * MM + at, (unsigned long long)(v & 0xffffffffll));
+  atomicAdd(G + (g + 1) * MM + at, (unsigned long long)(v >> 32));
+}
+
+template <typename TY>
+__global__ void __launch_bounds__(kGrThreads, 1) gram_kernel(GramArgs a) {
+  constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST;
+  constexpr int kStage = S * (kPlaneA + kPlaneB);
+  extern __shared__ __align__(1024) unsigned char gsm[];
+  __shared__ __align__(8) uint64_t full[NST], empty[NST], dfull, dempty, fin;
+  __shared__ uint32_t tmem_base;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int item = blockIdx.x % a.items, split = blockIdx.x / a.items;
+  const int half = item % Dig<TY>::HALVES;
+  int I = 0, t = item / Dig<TY>::HALVES;
+  while (t >= a.nJ - 2 * I) {
+    t -= a.nJ - 2 * I;
+    ++I;
+  }
+  const int J = 2 * I + t;
+  const bool diag = (J >> 1) == I;       // B's columns are among A's
+  const int64_t nsum = (a.N + 127) / 128;
+  const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
+  const int64_t nstage = (q1 - q0) * kStagesPerSum;
+  if (tid == 0) {
+    for (int b = 0; b < NST; ++b) {
+      tc05::mbar_init(full + b, kGrThreads / 32);
+      tc05::mbar_init(empty + b, 1);
+    }
+    tc05::mbar_init(&dfull, 1);
+    tc05::mbar_init(&dempty, kGrThreads / 32);
+    tc05::mbar_init(&fin, 1);
+  }
+  if (warp == 0) tc05::tmem_alloc(&tmem_base, 512);
+  tc05::fence_before();
+  __syncthreads();
+  tc05::fence_after();
+  const uint32_t tmem = tmem_base;
+  bool ok = true;
+  const TY* Y = (const TY*)a.Y;
+  const int c8 = lane & 7, kg = lane >> 3;
+  const int ca = warp * 8 + c8;                  // A: 16 warps x 8 columns
+  const int64_t colA = (int64_t)I * 128 + ca;
+  const int EA = colA < a.M ? a.colE[colA] : 1;
+  const uint32_t offA = (uint32_t)((ca >> 3) * kPlaneSbo + kg * 128 + c8 * 16);
+  const bool doB = !diag && warp < 8;            // B: 8 warps x 8 columns
+  const int64_t colB = (int64_t)J * 64 + ca;
+  const int EB = (doB && colB < a.M) ? a.colE[colB] : 1;
+  const int qd = warp & 3, cp = warp >> 2;       // tensor-memory lane quadrant, 16-column part
+  const uint32_t taddr = tmem + ((uint32_t)(qd * 32) << 16) + cp * 16;
+  const int nslots = (sizeof(TY) == 8 && half == 1) ? 7 : 8;
+  int64_t acc0[16], acc1[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
+  auto flush = [&]() {
+    const int64_t gi = (int64_t)I * 128 + qd * 32 + lane;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const int64_t gj = (int64_t)J * 64 + cp * 16 + c;
+      if (gi < a.M && gj < a.M && gi <= gj) {
+        add_group(a.G, a.M * a.M, gi + gj * a.M, half * 2, acc0[c]);
+        add_group(a.G, a.M * a.M, gi + gj * a.M, half * 2 + 1, acc1[c]);
+      }
+      acc0[c] = acc1[c] = 0;
+    }
+  };
+  int64_t issued = 0, drained = 0;
+  for (int64_t j = 0; j <= nstage; ++j) {
+    const int b = (int)(j % NST);
+    if (j < nstage) {
+      if (j >= NST) {
+        ok = __all_sync(0xffffffffu, mbar_wait_fast(empty + b, (uint32_t)((j / NST - 1) & 1)));
+        if (!ok) break;
+      }
+      unsigned char* st = gsm + b * kStage;
+      const int64_t row = (q0 * kStagesPerSum + j) * kStK + kg * 8;
+      put_column8<TY>(Y, a.ldy, row, colA, a.M, EA, st + offA, kPlaneA);
+      if (doB) put_column8<TY>(Y, a.ldy, row, colB, a.M, EB, st + S * kPlaneA + offA, kPlaneB);
+      tc05::fence_smem_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + b);
+    }
+    // the sums of the 128 rows before, once the stages ahead are filled
+    const bool due = (j % kStagesPerSum == NST - 1 && j >= kStagesPerSum && j < nstage) ||
+                     (j == nstage && nstage > 0);
+    if (due) {
+      ok = __all_sync(0xffffffffu, mbar_wait_fast(&dfull, (uint32_t)(drained & 1)));
+      if (!ok) break;
+      tc05::fence_after();
+      drain_slots(taddr, nslots, acc0, acc1);
+      tc05::fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&dempty);
+      ++drained;
+      if ((drained & 8191) == 0) flush();
+    }
+    // MMAs of the stages that are filled; those of a new sum wait until the
+    // last one has been read
+    const bool held = j >= kStagesPerSum && j % kStagesPerSum < NST - 1;
+    if (warp == kGrThreads / 32 - 1 && lane == 0 && j < nstage && !held) {
+      for (; issued <= j && ok; ++issued) {
+        const int ib = (int)(issued % NST);
+        const int64_t sum = issued / kStagesPerSum;
+        const bool first = issued % kStagesPerSum == 0;
+        ok = mbar_wait_fast(full + ib, (uint32_t)((issued / NST) & 1));
+        if (ok && first && sum > 0) ok = mbar_wait_fast(&dempty, (uint32_t)((sum - 1) & 1));
+        if (!ok) break;
+        tc05::fence_after();
+        const uint32_t sa = tc05::smem_u32(gsm) + ib * kStage;
+        const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
+        const uint64_t dB = diag ? tc05::desc(sa + (J & 1) * 8 * kPlaneSbo, 128, kPlaneSbo)
+                                 : tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
+        const int planeB = diag ? kPlaneA : kPlaneB;
+        if (Dig<TY>::HALVES == 2 && half == 1)
+          issue_stage<S, gram_base<TY>(1)>(tmem, dA, dB, planeB, first);
+        else
+          issue_stage<S, gram_base<TY>(0)>(tmem, dA, dB, planeB, first);
+        tc05::commit(empty + ib);
+        if (issued % kStagesPerSum == kStagesPerSum - 1) tc05::commit(&dfull);
+      }
+    }
+    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+    if (!ok) break;
+  }
+  if (ok) flush();
+  if (warp == kGrThreads / 32 - 1 && lane == 0) {
+    // nothing of this block is in flight when it gives its memory back
+    tc05::commit(&fin);
+    if (!mbar_wait_fast(&fin, 0)) ok = false;
+  }
+  if (!ok) raise_status(a.hdr, PYLOM_ERR_TIMEOUT);
+  tc05::fence_before();
+  __syncthreads();
+  if (warp == 0) tc05::tmem_dealloc(tmem, 512);
+}
+
+// ---------------------------------------------------------------------------
+// Cholesky factorisation in double-double arithmetic
+// ---------------------------------------------------------------------------
+
+struct dd { double h, l; };
+
+__device__ __forceinline__ dd dd_two_sum(double a, double b) {
+  const double s = __dadd_rn(a, b), bb = __dsub_rn(s, a);
+  return {s, __dadd_rn(__dsub_rn(a, __dsub_rn(s, bb)), __dsub_rn(b, bb))};
+}
+__device__ __forceinline__ dd dd_quick(double a, double b) {   // |a| >= |b|
+  const double s = __dadd_rn(a, b);
+  return {s, __dsub_rn(b, __dsub_rn(s, a))};
+}
+__device__ __forceinline__ dd dd_mul(dd a, dd b) {
+  const double p = __dmul_rn(a.h, b.h);
+  double e = __fma_rn(a.h, b.h, -p);
+  e = __fma_rn(a.h, b.l, e);
+  e = __fma_rn(a.l, b.h, e);
+  return dd_quick(p, e);
+}
+// s - a b
+__device__ __forceinline__ dd dd_fms(dd s, dd a, dd b) {
+  const double p = __dmul_rn(a.h, b.h);
+  double e = __fma_rn(a.h, b.h, -p);
+  e = __fma_rn(a.h, b.l, e);
+  e = __fma_rn(a.l, b.h, e);
+  const dd t = dd_two_sum(s.h, -p);
+  return dd_quick(t.h, __dadd_rn(t.l, __dsub_rn(s.l, e)));
+}
+__device__ __forceinline__ dd dd_add(dd a, dd b) {
+  const dd t = dd_two_sum(a.h, b.h);
+  return dd_quick(t.h, __dadd_rn(t.l, __dadd_rn(a.l, b.l)));
+}
+// 1 / a: one Newton step in double-double from the binary64 quotient
+__device__ __forceinline__ dd dd_rcp(dd a) {
+  const double x = 1.0 / a.h;
+  double e = __fma_rn(-a.h, x, 1.0);
+  e = __fma_rn(-a.l, x, e);
+  return dd_quick(x, __dmul_rn(x, e));
+}
+
+// integer groups -> double-double, scaled by 2^-64 (squares stay in range)
+__device__ __forceinline__ dd group_sum(const long long* G, int64_t MM, int64_t at, int groups, int lb) {
+  dd s = {0.0, 0.0};
+  for (int g = groups - 1; g >= 0; --g) {
+    const double v = (double)__ldcg(G + g * MM + at);
+    if (v != 0.0) s = dd_add(s, dd{scalbn(v, 32 * g + 8 * lb - 64), 0.0});
+  }
+  return s;
+}
+
+constexpr int kNBC = 16;           // panel height of the factorisation
+constexpr int kChThreads = 256;
+
+struct CholArgs {
+  GramState g;
+  double* R;
+  int groups, lb, bias;
+};
+
+// G = U^T D U (U unit upper triangular), right-looking by row panels of kNBC
+// rows over all blocks of a cooperative launch.  A panel: every block that
+// holds trailing columns factors the 16 x 16 diagonal block itself (a serial
+// chain of 16 pivots, the same in every block) together with its 16-column
+// block of the panel; after a grid barrier the trailing 16 x 16 tiles take
+// A -= U_panel^T (D U)_panel, one thread per entry; a second barrier ends
+// the panel.  R = D^(1/2) U with the columns' scales 2^(E - bias) restored.
+// A pivot at the rounding level of its column (a direction that the other
+// columns span, such as the one that the removed mean leaves) gives a zero
+// row.
+__global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
+  __shared__ dd sP[kNBC][2 * kNBC + 1];   // diagonal block | column block
+  __shared__ dd sU[kNBC][kNBC], sT[kNBC][kNBC];
+  __shared__ dd s_inv;
+  __shared__ double s_root, s_level[kNBC];
+  const GramState& g = c.g;
+  const int tid = threadIdx.x;
+  const int64_t M = g.M, MM = M * M;
+  const int64_t nb = (M + kNBC - 1) / kNBC;
+  const int ty = tid >> 4, tx = tid & 15;
+  // integers -> double-double (upper triangle), zeros below the diagonal of R
+  for (int64_t idx = (int64_t)blockIdx.x * kChThreads + tid; idx < MM; idx += (int64_t)gridDim.x * kChThreads) {
+    const int64_t i = idx % M, j = idx / M;
+    if (i <= j) {
+      const dd v = group_sum(g.G, MM, idx, c.groups, c.lb);
+      g.Lh[idx] = v.h;
+      g.Ll[idx] = v.l;
+    } else {
+      c.R[idx] = 0.0;
+    }
+  }
+  if (!grid_barrier(g.hdr, gridDim.x)) return;
+  for (int64_t p = 0; p < nb; ++p) {
+    const int64_t k = p * kNBC;
+    const int nbk = (int)((M - k) < kNBC ? (M - k) : kNBC);
+    const int64_t units = nb - p - 1 > 0 ? nb - p - 1 : 1;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+      const int64_t c0 = (p + 1 + u) * kNBC;
+      __syncthreads();
+      for (int idx = tid; idx < kNBC * 2 * kNBC; idx += kChThreads) {
+        const int r = idx % kNBC, q = idx / kNBC;
+        const int64_t col = q < kNBC ? k + q : c0 + q - kNBC;
+        dd v = {0.0, 0.0};
+        if (r < nbk && col < M && (q >= kNBC || (q < nbk && r <= q))) {
+          v.h = __ldcg(g.Lh + k + r + col * M);
+          v.l = __ldcg(g.Ll + k + r + col * M);
+        }
+        sP[r][q] = v;
+      }
+      // rounding level of a pivot: its column's own square times 2^-100
+      if (tid < nbk) s_level[tid] = 7.9e-31 * group_sum(g.G, MM, (k + tid) * (M + 1), c.groups, c.lb).h;
+      __syncthreads();
+      for (int j = 0; j < nbk; ++j) {
+        if (tid == 0) {
+          const dd d = sP[j][j];
+          const bool live = d.h > s_level[j];
+          s_inv = live ? dd_rcp(d) : dd{0.0, 0.0};
+          s_root = live ? sqrt(d.h) : 0.0;
+        }
+        __syncthreads();
+        const dd inv = s_inv;
+        const double root = s_root;
+        // rows below take -(u_jr) (t_jq); u = t / d
+        for (int q = tx; q < 2 * kNBC; q += 16) {
+          const int r = ty;
+          if (r > j && r < nbk && (q >= kNBC || q >= r))
+            sP[r][q] = dd_fms(sP[r][q], dd_mul(sP[j][r], inv), sP[j][q]);
+        }
+        // row j of R, of U and of D U for the trailing update
+        if (ty == j && k + j < M) {
+          const int64_t col = c0 + tx;
+          if (col < M) {
+            const dd t = sP[j][kNBC + tx], uu = dd_mul(t, inv);
+            const int64_t at = k + j + col * M;
+            c.R[at] = scalbn(root * uu.h, g.colE[col] - c.bias + 32);
+            g.Lh[at] = uu.h;
+            g.Ll[at] = uu.l;
+            g.Th[j + col * kNBC] = t.h;
+            g.Tl[j + col * kNBC] = t.l;
+          }
+          if (u == 0 && tx >= j && tx < nbk) {
+            const dd uu = tx == j ? dd{1.0, 0.0} : dd_mul(sP[j][tx], inv);
+            c.R[k + j + (k + tx) * M] = scalbn(root * uu.h, g.colE[k + tx] - c.bias + 32);
+          }
+        }
+        __syncthreads();
+      }
+    }
+    if (p + 1 >= nb) break;
+    if (!grid_barrier(g.hdr, gridDim.x)) return;
+    const int64_t nt = nb - p - 1, tiles = nt * (nt + 1) / 2;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+      // tile (bi, bj), bi <= bj, counted column by column
+      int64_t bj = (int64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+      while (bj * (bj + 1) / 2 > t) --bj;
+      while ((bj + 1) * (bj + 2) / 2 <= t) ++bj;
+      const int64_t bi = t - bj * (bj + 1) / 2;
+      const int64_t r0 = (p + 1 + bi) * kNBC, c0 = (p + 1 + bj) * kNBC;
+      __syncthreads();
+      {
+        const int64_t ru = r0 + tx, ct = c0 + tx;
+        dd uu = {0.0, 0.0}, tt = {0.0, 0.0};
+        if (ty < nbk && ru < M) uu = {__ldcg(g.Lh + k + ty + ru * M), __ldcg(g.Ll + k + ty + ru * M)};
+        if (ty < nbk && ct < M) tt = {__ldcg(g.Th + ty + ct * kNBC), __ldcg(g.Tl + ty + ct * kNBC)};
+        sU[ty][tx] = uu;
+        sT[ty][tx] = tt;
+      }
+      __syncthreads();
+      const int64_t r = r0 + tx, cc = c0 + ty;
+      if (r < M && cc < M && r <= cc) {
+        const int64_t at = r + cc * M;
+        dd s = {__ldcg(g.Lh + at), __ldcg(g.Ll + at)};
+#pragma unroll 4
+        for (int q = 0; q < kNBC; ++q) s = dd_fms(s, sU[q][tx], sT[q][ty]);
+        g.Lh[at] = s.h;
+        g.Ll[at] = s.l;
+      }
+    }
+    if (!grid_barrier(g.hdr, gridDim.x)) return;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+
+size_t gram_bytes(int64_t M, int64_t rmax) {
+  const int64_t kt = (rmax + 63) / 64, js = (M + kStK - 1) / kStK;
+  return align256(sizeof(int) * (size_t)M) + align256(sizeof(long long) * (size_t)5 * M * M) +
+         2 * align256(sizeof(double) * (size_t)M * M) + 2 * align256(sizeof(double) * (size_t)kNBC * M) +
+         align256((size_t)kt * js * 8 * kPlaneB) +
+         align256(sizeof(int) * (size_t)kt * 64);
+}
+
+void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax) {
+  const int64_t kt = (rmax + 63) / 64, js = (M + kStK - 1) / kStK;
+  char* p = base;
+  g.M = M;
+  g.rmax = rmax;
+  g.colE = (int*)p;          p += align256(sizeof(int) * (size_t)M);
+  g.G = (long long*)p;       p += align256(sizeof(long long) * (size_t)5 * M * M);
+  g.Lh = (double*)p;         p += align256(sizeof(double) * (size_t)M * M);
+  g.Ll = (double*)p;         p += align256(sizeof(double) * (size_t)M * M);
+  g.Th = (double*)p;         p += align256(sizeof(double) * (size_t)kNBC * M);
+  g.Tl = (double*)p;         p += align256(sizeof(double) * (size_t)kNBC * M);
+  g.Cd = (unsigned char*)p;  p += align256((size_t)kt * js * 8 * kPlaneB);
+  g.Ce = (int*)p;
+}
+
+template <typename TX, typename TY>
+static cudaError_t prologue(const PrologueArgs& a, int sms, cudaStream_t st) {
+  const int64_t nblk = (a.ldy + 31) / 32;
+  const int64_t cap = (int64_t)sms * 4;
+  const unsigned grid = (unsigned)(nblk < cap ? nblk : cap);
+  if (a.M <= 32) gram_prologue_kernel<TX, TY, 4><<<grid, kPrThreads, 0, st>>>(a);
+  else if (a.M <= 64) gram_prologue_kernel<TX, TY, 8><<<grid, kPrThreads, 0, st>>>(a);
+  else if (a.M <= 128) gram_prologue_kernel<TX, TY, 16><<<grid, kPrThreads, 0, st>>>(a);
+  else gram_prologue_kernel<TX, TY, 32><<<grid, kPrThreads, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+// Row splits of a tile list over `sms` blocks: the count whose last wave
+// wastes least, at least 2 sums of 128 rows per unit.
+static int row_splits(int64_t items, int64_t nsum, int sms) {
+  int best = 1;
+  double eff = 0.0;
+  for (int s = 1; s <= sms; ++s) {
+    if (s > 1 && nsum / s < 1) break;
+    const int64_t units = items * s, waves = (units + sms - 1) / sms;
+    if (waves > 4 && s > 1) break;
+    const double e = (double)units / (double)(waves * sms);
+    if (e > eff + 0.02) {
+      eff = e;
+      best = s;
+    }
+  }
+  return best;
+}
+
+template <typename TY>
+static cudaError_t gram_launch(const GramState& g, int sms, cudaStream_t st) {
+  constexpr int S = Dig<TY>::S;
+  constexpr size_t smem = (size_t)Dig<TY>::NST * S * (kPlaneA + kPlaneB);
+  cudaError_t e = ensure_dyn_smem((const void*)gram_kernel<TY>, smem);
+  if (e != cudaSuccess) return e;
+  const int nJ = (int)((g.M + 63) / 64), nI = (int)((g.M + 127) / 128);
+  int tiles = 0;
+  for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;
+  GramArgs a{g.Y, g.ldy, g.N, g.M, g.colE, (unsigned long long*)g.G, nJ, tiles * Dig<TY>::HALVES, 1, g.hdr};
+  a.splits = row_splits(a.items, (g.N + 127) / 128, sms);
+  gram_kernel<TY><<<(unsigned)(a.items * a.splits), kGrThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xtype, const double* w,
+                          int remove_mean, double* mean, double* R, cudaStream_t st, cudaEvent_t mid) {
+  cudaError_t e;
+  int dev = 0, sms = 0, per = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int groups = g.f32 ? 3 : 5;
+  // colE and G are neighbours: one clear
+  const size_t clear = align256(sizeof(int) * (size_t)g.M) + sizeof(long long) * (size_t)groups * g.M * g.M;
+  if ((e = cudaMemsetAsync(g.colE, 0, clear, st)) != cudaSuccess) return e;
+  PrologueArgs pa{X, ldx, w, remove_mean, mean, g.Y, g.ldy, g.N, g.M, g.colE, g.hdr};
+  if (g.f32) e = xtype == PYLOM_F32 ? prologue<float, float>(pa, sms, st) : prologue<double, float>(pa, sms, st);
+  else e = xtype == PYLOM_F32 ? prologue<float, double>(pa, sms, st) : prologue<double, double>(pa, sms, st);
+  if (e != cudaSuccess) return e;
+  e = g.f32 ? gram_launch<float>(g, sms, st) : gram_launch<double>(g, sms, st);
+  if (e != cudaSuccess) return e;
+  if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
+  CholArgs c{g, R, groups, g.f32 ? gram_base<float>(0) : gram_base<double>(0),
+             g.f32 ? fix_bias<float>() : fix_bias<double>()};
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, gram_chol_kernel, kChThreads, 0);
+  if (e != cudaSuccess) return e;
+  if (per < 1) return cudaErrorCooperativeLaunchTooLarge;
+  const int64_t nb = (g.M + kNBC - 1) / kNBC;
+  int64_t grid = nb * (nb - 1) / 2;
+  if (grid < 1) grid = 1;
+  if (grid > sms) grid = sms;
+  void* args[] = {&c};
+  return cudaLaunchCooperativeKernel((const void*)gram_chol_kernel, dim3((unsigned)grid), dim3(kChThreads), args, 0,
+                                     st);
+}
+
+}  // namespace pylom

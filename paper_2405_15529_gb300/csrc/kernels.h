@@ -16,6 +16,8 @@ constexpr int kNB = 16;
 constexpr int64_t kCoopTreeMinM = 384;
 constexpr int64_t kCoopTreeMinP = 64;
 bool use_climb_tree(int64_t M, int64_t P);
+// PYLOM_TREE is set: the caller asks for a particular tree of R factors
+bool tree_requested();
 bool use_pipe_tree(int64_t M, int64_t P);
 
 
@@ -41,7 +43,34 @@ struct TsqrState {
   // = global row row0, Y (and X, w, mean, U) chunks with leading dimension
   // ldy.  In-core: leaf0 = 0, Pl = P, row0 = 0, ldy = N.
   int64_t leaf0, Pl, row0, ldy;
+  // adjoint of a forward whose route only the device knows: if gram_y is
+  // given and *gram_y is 0, the factorisation is the forward's, `shift`
+  // (mixed extra region: `shiftx`) bytes away from these pointers
+  const unsigned* gram_y;
+  int64_t shift, shiftx;
 };
+
+// leading dimension of the working copies (binary64 Y, binary32 Yf): whole
+// 8-row groups, so the digit kernels read them with aligned vector loads
+__host__ __device__ __forceinline__ int64_t y_ld(int64_t N) { return (N + 7) & ~int64_t(7); }
+
+#ifdef __CUDACC__
+// kernels that factor Y: nothing to do when the forward has done it
+__device__ __forceinline__ bool already_factored(const TsqrState& s) { return s.gram_y && *s.gram_y == 0; }
+// kernels that apply the factorisation: take the forward's where it exists
+template <class T>
+__device__ __forceinline__ void shift_ptr(T*& p, int64_t bytes) {
+  p = (T*)((char*)p + bytes);
+}
+__device__ __forceinline__ void select_factors(TsqrState& s) {
+  if (!already_factored(s)) return;
+  shift_ptr(s.Y, s.shift);
+  shift_ptr(s.tau, s.shift);
+  shift_ptr(s.T, s.shift);
+  shift_ptr(s.Rs, s.shift);
+  shift_ptr(s.tau_tree, s.shift);
+}
+#endif
 
 struct SvdState {
   WsHeader* hdr;
@@ -116,6 +145,12 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
                                 const double* dVT, int64_t lddvt, const double* w, int remove_mean,
                                 int physical, int64_t r, void* dX, int64_t lddx, int dxtype,
                                 char* bw_base, char* mixed_extra, cudaStream_t st);
+// Room in the backward's workspace for a factorisation of the forward's Y
+// (forwards with the automatic leaf height may have left Y unfactored), and
+// its state: os (and *extra, mixed path) in the backward's workspace.
+size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed);
+cudaError_t launch_refactor(const TsqrState& fs, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
+                            const double* UR, TsqrState& os, char** extra, double** UR_out, cudaStream_t st);
 // Mixed-precision adjoint support (tsqr_mixed.cu): per leaf C := Q_leaf^T C
 // (FP32, ld N) on tcgen05, top M rows into the binary64 slots Z.
 cudaError_t launch_leaf_qt_mixed(const TsqrState& s, char* extra, float* C, int64_t r, double* Z, cudaStream_t st);

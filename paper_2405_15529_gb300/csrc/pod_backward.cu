@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kLeafThreads) bw_leaf_qt_kernel(TsqrState s, d
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  select_factors(s);
   const double* A = s.Y + r0;
   double* Cl = C + r0;
   for (int64_t pan = 0; pan < s.npan; ++pan) {
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(kLeafThreads) bw_leaf_qt_kernel(TsqrState s, d
     const double* Tg = s.T + (leaf * s.npan + pan) * kSmT;
     for (int idx = tid; idx < kSmT; idx += nthr) sT[idx] = Tg[idx];
     __syncthreads();
-    LeafV V{A, s.N, k, h, nbk};
+    LeafV V{A, s.ldy, k, h, nbk};
     block_reflector<true, false>(V, nbk, k, h, Cl, s.N, (int)r, nullptr, 0, sT, sW, sWp);
     __syncthreads();
   }
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(256) bw_up_pass_kernel(TsqrState s, double* Z,
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int64_t left = (int64_t)blockIdx.x * 2 * step, right = left + step;
   if (right >= s.P) return;
+  select_factors(s);
   const int64_t col = (int64_t)blockIdx.y * nwarps + warp;
   if (col >= r) return;
   const int64_t M = s.M;
@@ -225,6 +227,45 @@ __global__ void __launch_bounds__(256) bw_add_du_c_f32_kernel(const float* C, co
       }
     }
   }
+}
+
+// U_R for the factorisation that the adjoint applies: the forward's own when
+// it factored Y, else its rows with the signs of the Householder R (R is
+// unique up to row signs; the Gram route's has a non-negative diagonal).
+__global__ void bw_signed_ur_kernel(TsqrState s, const double* UR, double* out) {
+  const int64_t M = s.M;
+  const bool same = already_factored(s);
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % M;
+    out[idx] = (!same && s.Rs[i + i * M] < 0.0) ? -UR[idx] : UR[idx];
+  }
+}
+
+size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed) {
+  return align256(sizeof(double) * (size_t)M * M) + tsqr_state_bytes(N, M, P, r_max, !mixed) +
+         (mixed ? mixed_extra_bytes(N, M, P) : 0);
+}
+
+cudaError_t launch_refactor(const TsqrState& fs, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
+                            const double* UR, TsqrState& os, char** extra, double** UR_out, cudaStream_t st) {
+  const size_t ub = align256(sizeof(double) * (size_t)fs.M * fs.M);
+  char* own = base + ub;
+  char* oextra = mixed ? own + tsqr_state_bytes(fs.N, fs.M, fs.P, fs.rmax, false) : nullptr;
+  tsqr_state_carve(os, own, fs.N, fs.M, fs.P, fs.rmax, !mixed);
+  os.hdr = hdr;
+  os.gram_y = &fs.hdr->gram_y;
+  os.shift = (const char*)fs.tau - (const char*)os.tau;
+  os.shiftx = mixed ? fwd_extra - oextra : 0;
+  cudaError_t e = cudaMemsetAsync(os.arrive, 0, sizeof(unsigned) * (size_t)os.P, st);
+  if (e != cudaSuccess) return e;
+  e = mixed ? launch_tsqr_mixed(os, oextra, fwd_extra, y_ld(fs.N), PYLOM_F32, nullptr, 0, nullptr, st)
+            : launch_tsqr_fp64(os, fs.Y, fs.ldy, PYLOM_F64, nullptr, 0, nullptr, st);
+  if (e != cudaSuccess) return e;
+  bw_signed_ur_kernel<<<64, 256, 0, st>>>(os, UR, (double*)base);
+  *UR_out = (double*)base;
+  *extra = oextra;
+  return cudaGetLastError();
 }
 
 struct BwLayout {

@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_qr_kernel(LeafArgs a) {
   double* sW = sout + kSmOut;
   double* sWp = sW + kSmW;
   const TsqrState& s = a.s;
+  if (already_factored(s)) return;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int64_t leaf = s.leaf0 + blockIdx.x;
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(256) down_pass_kernel(TsqrState s, int64_t ste
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int64_t left = (int64_t)blockIdx.x * 2 * step, right = left + step;
   if (right >= s.P) return;
+  select_factors(s);
   const int64_t r = (r_fixed >= 0) ? r_fixed : s.hdr->r;
   const int64_t col = (int64_t)blockIdx.y * nwarps + warp;
   if (col >= r) return;
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(kLeafThreads) modes_kernel(TsqrState s, int64_
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  select_factors(s);
   const int64_t r = (r_fixed >= 0) ? r_fixed : s.hdr->r;
   if (leaf == 0 && tid == 0 && r_out) *r_out = r;
   double* C = U + (r0 - s.row0);
@@ -332,6 +335,8 @@ __global__ void copy_root_kernel(TsqrState s, double* R, int64_t ldr) {
 // PYLOM_TREE ("climb", "coop" or "pipe") overrides the choice.
 static const char* tree_env() { return getenv("PYLOM_TREE"); }
 
+bool tree_requested() { return tree_env() != nullptr; }
+
 bool use_climb_tree(int64_t M, int64_t P) {
   const char* env = tree_env();
   if (P <= 1) return true;
@@ -355,7 +360,7 @@ cudaError_t launch_tree(const TsqrState& s, cudaStream_t st) {
 size_t tsqr_state_bytes(int64_t N, int64_t M, int64_t P, int64_t rmax, bool with_y) {
   const int64_t npan = (M + kNB - 1) / kNB;
   size_t b = 0;
-  if (with_y) b += align256(sizeof(double) * (size_t)N * M);
+  if (with_y) b += align256(sizeof(double) * (size_t)y_ld(N) * M);
   b += align256(sizeof(double) * (size_t)P * M);
   b += align256(sizeof(double) * (size_t)P * npan * kNB * kNB);
   b += align256(sizeof(double) * (size_t)P * M * M);
@@ -375,7 +380,7 @@ void tsqr_state_carve(TsqrState& s, char* base, int64_t N, int64_t M, int64_t P,
   s.rmax = rmax;
   char* p = base;
   s.Y = with_y ? (double*)p : nullptr;
-  if (with_y) p += align256(sizeof(double) * (size_t)N * M);
+  if (with_y) p += align256(sizeof(double) * (size_t)y_ld(N) * M);
   s.tau = (double*)p;      p += align256(sizeof(double) * (size_t)P * M);
   s.T = (double*)p;        p += align256(sizeof(double) * (size_t)P * s.npan * kNB * kNB);
   s.Rs = (double*)p;       p += align256(sizeof(double) * (size_t)P * M * M);
@@ -389,7 +394,9 @@ void tsqr_state_carve(TsqrState& s, char* base, int64_t N, int64_t M, int64_t P,
   s.leaf0 = 0;
   s.Pl = P;
   s.row0 = 0;
-  s.ldy = N;
+  s.ldy = with_y ? y_ld(N) : N;
+  s.gram_y = nullptr;
+  s.shift = s.shiftx = 0;
 }
 
 cudaError_t launch_tsqr_fp64(const TsqrState& s, const void* X, int64_t ldx, int xtype,

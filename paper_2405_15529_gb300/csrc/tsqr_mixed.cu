@@ -73,9 +73,9 @@ constexpr int kMixSmemTotal = kMixSmem > kMergeSmem ? kMixSmem : kMergeSmem;
 // the shared-memory plan keeps them apart
 static_assert(2 * kMixSmemTotal > 228 * 1024, "mixed-leaf CTAs must not share an SM");
 
-// Leading dimension of the FP32 working copy: N rounded up to a multiple of
-// 4, so every column starts on a 16-byte boundary (TMA strides).
-__host__ __device__ __forceinline__ int64_t yf_ld(int64_t N) { return (N + 3) & ~int64_t(3); }
+// Leading dimension of the FP32 working copy: whole 8-row groups, so every
+// column starts on a 16-byte boundary (TMA strides, vector loads).
+__host__ __device__ __forceinline__ int64_t yf_ld(int64_t N) { return y_ld(N); }
 
 struct MixedArgs {
   TsqrState s;
@@ -963,6 +963,7 @@ __global__ void __launch_bounds__(kMxThreads) leaf_qr_mixed_kernel(MixedArgs a, 
   __shared__ __align__(8) uint64_t fullbar[2];
   __shared__ uint32_t tmem_base;
   const TsqrState& s = a.s;
+  if (already_factored(s)) return;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int64_t leaf = blockIdx.x;
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
@@ -1037,6 +1038,10 @@ __global__ void __launch_bounds__(kMxThreads) modes_mixed_kernel(TsqrState s, co
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  if (already_factored(s)) {
+    shift_ptr(Yf, s.shiftx);
+    shift_ptr(T2, s.shiftx);
+  }
   const int64_t npan = (M + kNB2 - 1) / kNB2;
   const int64_t r = (r_fixed >= 0) ? r_fixed : s.hdr->r;
   if (leaf == 0 && tid == 0 && r_out) *r_out = r;
@@ -1093,6 +1098,10 @@ __global__ void __launch_bounds__(kMxThreads) leaf_qt_mixed_kernel(TsqrState s, 
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  if (already_factored(s)) {
+    shift_ptr(Yf, s.shiftx);
+    shift_ptr(T2, s.shiftx);
+  }
   const int64_t npan = (M + kNB2 - 1) / kNB2;
   double* sT = (double*)(msm + kOffT);
   if (tid == 0) tc05::mbar_init(&mbar, 1);
