@@ -81,19 +81,21 @@ struct SvdState {
   int64_t Mb;               // columns padded to a multiple of two blocks
   float* A32;               // M x Mb
   float* V32;               // Mb x Mb
-  double* G;                // Mp x Mp Newton-Schulz scratch
-  double* Tm;               // Mp x Mp Newton-Schulz scratch
-  unsigned* rot32;          // rotations per binary32 sweep
-  double* mmws;             // split-K scratch of the binary64 products
+  double* T[5];             // Mp x Mp scratch of the binary64 products
+  double* A2;               // M x Mp second copy of A
+  int* big;                 // Mp: partner of a column's largest angle
+  unsigned* rot32;          // counters (svd_jacobi32.cu)
 };
 
 // From this size on, binary32 block-Jacobi sweeps precondition the binary64
-// one-sided Jacobi of the small SVD (svd_jacobi32.cu).  At M = 256 they
-// take the SVD from 20.3 to 16.9 ms (11 binary64 sweeps before).
-constexpr int64_t kJac32MinM = 256;
+// one-sided Jacobi of the small SVD (svd_jacobi32.cu): 0.2 ms of launches and
+// rounds whatever M, which is what ten plain sweeps of M = 12 take (M = 5:
+// 0.2 ms, M = 16: 0.4 ms).
+constexpr int64_t kJac32MinM = 12;
 size_t jacobi32_extra_bytes(int64_t M);
 void jacobi32_carve(SvdState& s, char* p);
-cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int64_t ldr, cudaStream_t st);
+cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int64_t ldr, const unsigned** open_pairs,
+                                         cudaStream_t st);
 
 // with_y: include the N x M FP64 working copy (the FP64 path; the mixed
 // path keeps an FP32 copy in its own extra region instead)

@@ -34,7 +34,8 @@ void svd_state_carve(SvdState& s, char* base, int64_t M, bool precond) {
   s.V = (double*)(base + align256(sizeof(double) * (size_t)M * s.Mp));
   s.Mb = 0;
   s.A32 = s.V32 = nullptr;
-  s.G = s.Tm = s.mmws = nullptr;
+  s.A2 = nullptr;
+  for (double*& t : s.T) t = nullptr;
   s.rot32 = nullptr;
   if (precond && M >= kJac32MinM)
     jacobi32_carve(s, (char*)s.V + align256(sizeof(double) * (size_t)s.Mp * s.Mp));
@@ -55,13 +56,19 @@ __global__ void jacobi_init_kernel(SvdState s, const double* R, int64_t ldr) {
 // two columns stay in registers between the dot products and the rotation,
 // so each step reads them from L2 once.
 template <int EL>
-__global__ void __launch_bounds__(kJacThreads) jacobi_kernel(SvdState s, int max_sweeps) {
+__global__ void __launch_bounds__(kJacThreads) jacobi_kernel(SvdState s, int max_sweeps,
+                                                              const unsigned* open_pairs) {
   __shared__ double sred[3 * (kJacThreads / 32)];
   __shared__ double sout[4];
   const int tid = threadIdx.x;
   constexpr int nthr = kJacThreads;
   const int64_t M = s.M, Mp = s.Mp, npairs = Mp / 2;
   const double tol = (double)M * 1.1102230246251565e-16;  // M * 2^-53
+  if (open_pairs && *open_pairs == 0) {
+    // the preconditioning left nothing to rotate: that check is the last sweep
+    if (blockIdx.x == 0 && tid == 0) s.hdr->sweeps = 1;
+    return;
+  }
   int sweep = 0;
   bool converged = false;
   while (sweep < max_sweeps) {
@@ -163,6 +170,58 @@ __global__ void __launch_bounds__(kJacThreads) jacobi_kernel(SvdState s, int max
   }
 }
 
+// Orthonormal completion of the right vectors (rows of VT) for exactly-zero
+// singular values (sorted last): Gram-Schmidt of unit vectors, twice.  All
+// threads of one block; S is the sorted spectrum.
+__device__ void complete_right_vectors(const double* S, int64_t M, double* VT, int64_t ldvt, double* sred, double* sout) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  __syncthreads();
+  int64_t next_e = 0;
+  for (int64_t c = 0; c < M; ++c) {
+    if (!(S[c] == 0.0)) continue;
+    for (; next_e < M; ++next_e) {
+      for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] = (i == next_e) ? 1.0 : 0.0;
+      __syncthreads();
+      for (int pass = 0; pass < 2; ++pass) {
+        for (int64_t q = 0; q < c; ++q) {
+          double v[1] = {0.0};
+          for (int64_t i = tid; i < M; i += nthr) v[0] += VT[q + i * ldvt] * VT[c + i * ldvt];
+          block_sum<1>(v, sred, sout);
+          const double d = sout[0];
+          for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] -= d * VT[q + i * ldvt];
+          __syncthreads();
+        }
+      }
+      double v[1] = {0.0};
+      for (int64_t i = tid; i < M; i += nthr) v[0] += VT[c + i * ldvt] * VT[c + i * ldvt];
+      block_sum<1>(v, sred, sout);
+      const double nn = sqrt(sout[0]);
+      if (nn > 0.5) {
+        for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] /= nn;
+        __syncthreads();
+        ++next_e;
+        break;
+      }
+    }
+  }
+}
+
+// Smallest rank whose share of the energy is at least `energy`, capped at r_max
+// (energy <= 0, or no energy at all: the cap).  One thread.
+__device__ int64_t energy_rank(const double* S, int64_t M, double energy, int64_t r_max) {
+  const int64_t rm = r_max < M ? r_max : M;
+  if (!(energy > 0.0)) return rm;
+  double total = 0.0;
+  for (int64_t i = 0; i < M; ++i) total += S[i] * S[i];
+  if (!(total > 0.0)) return rm;
+  double acc = 0.0;
+  for (int64_t k = 0; k < M; ++k) {
+    acc += S[k] * S[k];
+    if (acc / total >= energy) return (k + 1 < rm) ? k + 1 : rm;
+  }
+  return rm;
+}
+
 // One block.  sigma_j = |a_j|; sort descending (ties by index); left vectors
 // = columns of the rotations J, right vectors = a_j / sigma_j (orthonormal
 // completion where sigma_j == 0); sign so the largest |v| entry is positive
@@ -211,36 +270,7 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
   }
   for (int64_t c = tid; c < M; c += nthr) S[c] = sig[perm[c]];
   __syncthreads();
-  // orthonormal completion of the right vectors for exactly-zero singular
-  // values (sorted last): Gram-Schmidt of unit vectors, twice
-  int64_t next_e = 0;
-  for (int64_t c = 0; c < M; ++c) {
-    if (!(sig[perm[c]] == 0.0)) continue;
-    for (; next_e < M; ++next_e) {
-      for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] = (i == next_e) ? 1.0 : 0.0;
-      __syncthreads();
-      for (int pass = 0; pass < 2; ++pass) {
-        for (int64_t q = 0; q < c; ++q) {
-          double v[1] = {0.0};
-          for (int64_t i = tid; i < M; i += nthr) v[0] += VT[q + i * ldvt] * VT[c + i * ldvt];
-          block_sum<1>(v, sred, sout);
-          const double d = sout[0];
-          for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] -= d * VT[q + i * ldvt];
-          __syncthreads();
-        }
-      }
-      double v[1] = {0.0};
-      for (int64_t i = tid; i < M; i += nthr) v[0] += VT[c + i * ldvt] * VT[c + i * ldvt];
-      block_sum<1>(v, sred, sout);
-      const double nn = sqrt(sout[0]);
-      if (nn > 0.5) {
-        for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] /= nn;
-        __syncthreads();
-        ++next_e;
-        break;
-      }
-    }
-  }
+  complete_right_vectors(S, M, VT, ldvt, sred, sout);
   __syncthreads();
   // sign of each pair from its right vector
   for (int64_t c = warp; c < M; c += nwarps) {
@@ -265,24 +295,101 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
       VT[c + i * ldvt] = -VT[c + i * ldvt];
     }
   }
-  if (tid == 0) {
-    int64_t rm = r_max < M ? r_max : M;
-    int64_t r = rm;
-    if (energy > 0.0) {
-      double total = 0.0;
-      for (int64_t i = 0; i < M; ++i) total += sig[perm[i]] * sig[perm[i]];
-      if (total > 0.0) {
-        double acc = 0.0;
-        for (int64_t k = 0; k < M; ++k) {
-          acc += sig[perm[k]] * sig[perm[k]];
-          if (acc / total >= energy) {
-            r = (k + 1 < rm) ? k + 1 : rm;
-            break;
-          }
-        }
-      }
+  if (tid == 0) s.hdr->r = energy_rank(S, M, energy, r_max);
+}
+
+// The same outputs over the whole chip, when the preconditioning's scratch is
+// there (T[0]: norms, then signs; big: the sorted order).  A single block
+// took 66 us at M = 64, 457 us at M = 256 and 2.8 ms at M = 700.
+__global__ void svd_norms_kernel(SvdState s) {
+  const int lane = threadIdx.x & 31;
+  const int64_t M = s.M, j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (j >= M) return;
+  double a = 0.0, best = -1.0;
+  int kb = 0;
+  for (int64_t i = lane; i < M; i += 32) {
+    const double x = s.A[i + j * M];
+    a += x * x;
+    if (fabs(x) > best) {
+      best = fabs(x);
+      kb = (int)i;
     }
-    s.hdr->r = r;
+  }
+  a = warp_sum(a);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int ok = __shfl_xor_sync(0xffffffffu, kb, o);
+    if (ob > best || (ob == best && ok < kb)) {
+      best = ob;
+      kb = ok;
+    }
+  }
+  if (lane == 0) {
+    s.T[0][j] = sqrt(a);
+    s.T[0][M + j] = s.A[kb + j * M] < 0.0 ? -1.0 : 1.0;
+  }
+}
+
+__global__ void __launch_bounds__(kFinThreads) svd_order_kernel(SvdState s, double* S, double energy, int64_t r_max) {
+  __shared__ double sS[4096];   // M <= 4096 at every entry point
+  const int64_t M = s.M;
+  const double* sig = s.T[0];
+  for (int64_t j = threadIdx.x; j < M; j += blockDim.x) {
+    const double sj = (sig[j] == sig[j]) ? sig[j] : -1.0;   // NaN last
+    int rank = 0;
+    for (int64_t q = 0; q < M; ++q) {
+      const double sq = (sig[q] == sig[q]) ? sig[q] : -1.0;
+      rank += (sq > sj) || (sq == sj && q < j);
+    }
+    s.big[rank] = (int)j;
+    S[rank] = sig[j];
+    sS[rank] = sig[j];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s.hdr->r = energy_rank(sS, M, energy, r_max);
+}
+
+__global__ void svd_output_kernel(SvdState s, double* U, int64_t ldu, double* VT, int64_t ldvt) {
+  const int64_t M = s.M, Mp = s.Mp;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % M, c = idx / M, j = s.big[c];
+    const double sj = s.T[0][j], sg = s.T[0][M + j];
+    U[i + c * ldu] = sg * s.V[i + j * Mp];
+    VT[c + i * ldvt] = (sj > 0.0) ? sg * (s.A[i + j * M] / sj) : 0.0;
+  }
+}
+
+// Rows of V^T of exactly-zero singular values: orthonormal completion (one block).
+__global__ void __launch_bounds__(kFinThreads) svd_complete_kernel(SvdState s, double* U, int64_t ldu, const double* S,
+                                                                   double* VT, int64_t ldvt) {
+  __shared__ double sred[kFinThreads / 32];
+  __shared__ double sout[2];
+  const int64_t M = s.M;
+  if (!(S[M - 1] == 0.0)) return;
+  complete_right_vectors(S, M, VT, ldvt, sred, sout);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int64_t c = warp; c < M; c += blockDim.x >> 5) {
+    if (!(S[c] == 0.0)) continue;
+    double best = -1.0;
+    int64_t kbest = 0;
+    for (int64_t k = lane; k < M; k += 32) {
+      const double a = fabs(VT[c + k * ldvt]);
+      if (a > best) { best = a; kbest = k; }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int64_t ok = __shfl_xor_sync(0xffffffffu, kbest, o);
+      if (ob > best || (ob == best && ok < kbest)) { best = ob; kbest = ok; }
+    }
+    const bool flip = VT[c + kbest * ldvt] < 0.0;
+    __syncwarp();
+    if (flip)
+      for (int64_t k = lane; k < M; k += 32) {
+        VT[c + k * ldvt] = -VT[c + k * ldvt];
+        U[k + c * ldu] = -U[k + c * ldu];
+      }
   }
 }
 
@@ -290,8 +397,10 @@ cudaError_t launch_svd_fp64(const SvdState& s, const double* R, int64_t ldr, dou
                             double* S, double* VT, int64_t ldvt, int max_sweeps, double energy,
                             int64_t r_max, cudaStream_t st) {
   cudaError_t e;
-  if (s.A32) {
-    e = launch_jacobi32_precondition(s, R, ldr, st);
+  // a caller who allows only a few sweeps sees whether those converge
+  const unsigned* open_pairs = nullptr;
+  if (s.A32 && max_sweeps >= 8) {
+    e = launch_jacobi32_precondition(s, R, ldr, &open_pairs, st);
   } else {
     jacobi_init_kernel<<<64, 256, 0, st>>>(s, R, ldr);
     e = cudaGetLastError();
@@ -317,10 +426,18 @@ cudaError_t launch_svd_fp64(const SvdState& s, const double* R, int64_t ldr, dou
   if (grid < 1) grid = 1;
   SvdState sa = s;
   int ms = max_sweeps;
-  void* args[] = {(void*)&sa, (void*)&ms};
+  void* args[] = {(void*)&sa, (void*)&ms, (void*)&open_pairs};
   e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)grid), dim3(kJacThreads),
                                   args, 0, st);
   if (e != cudaSuccess) return e;
+  if (s.A32) {
+    const int gr = s.M <= 64 ? 16 : s.M <= 256 ? 128 : 304;
+    svd_norms_kernel<<<(unsigned)((s.M * 32 + 255) / 256), 256, 0, st>>>(s);
+    svd_order_kernel<<<1, kFinThreads, 0, st>>>(s, S, energy, r_max);
+    svd_output_kernel<<<gr, 256, 0, st>>>(s, U, ldu, VT, ldvt);
+    svd_complete_kernel<<<1, kFinThreads, 0, st>>>(s, U, ldu, S, VT, ldvt);
+    return cudaGetLastError();
+  }
   const size_t fsm = sizeof(double) * 2 * (size_t)s.M + sizeof(int) * (size_t)s.M;
   if (fsm > 48 * 1024 && (e = ensure_dyn_smem((const void*)svd_finalize_kernel, fsm)) != cudaSuccess) return e;
   svd_finalize_kernel<<<1, kFinThreads, fsm, st>>>(s, U, ldu, S, VT, ldvt, energy, r_max);

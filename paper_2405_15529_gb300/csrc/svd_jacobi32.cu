@@ -1,234 +1,622 @@
-// svd_jacobi32.cu -- single-precision preconditioning of the small SVD
-// (Eq. svdqr2 of pyLOM, arXiv 2405.15529) for large M.
+// svd_jacobi32.cu -- preconditioning of the small SVD (Eq. svdqr2 of pyLOM,
+// arXiv 2405.15529) so that the binary64 one-sided Jacobi of svd_jacobi.cu
+// has (nearly) nothing left to rotate.
 //
-// One-sided Jacobi in binary64 costs about 5.5 M^3 FP64 instructions per
-// sweep, and binary64 runs at a small fraction of the binary32 rate on this
-// part, so at M in the thousands the sweeps, not the data, bound the small
-// SVD.  Here the sweeps that do most of the rotating run in binary32:
-//   1. block one-sided Jacobi on A32 = fl32(R^T): the columns are grouped in
-//      blocks of kJB, pairs of blocks (2 kJB columns) are orthogonalised in
-//      shared memory by inner Jacobi sweeps (one warp per column pair), the
-//      accumulated 2 kJB x 2 kJB rotation is applied to V32, and the blocks
-//      follow a round-robin order with one grid barrier per step;
-//   2. V = V32 in binary64, made orthogonal to working precision by two
-//      Newton-Schulz steps V <- V (3 I - V^T V) / 2 (the error squares each
-//      step: about 1e-6, 1e-12, rounding);
-//   3. A = R^T V in binary64.
-// The binary64 one-sided Jacobi of svd_jacobi.cu then starts from (A, V):
-// the columns of A are already orthogonal to about the single-precision
-// tolerance, and its quadratic convergence finishes in a few sweeps.  The
-// result is the binary64 SVD of R (R^T V_final = A_final with orthogonal
-// columns, V_final orthogonal to working precision); only the number of
-// binary64 sweeps changes.
+// A binary64 Jacobi sweep is M - 1 grid barriers and 5.5 M^3 binary64
+// instructions, of which this part issues two per clock and SM; ten or more
+// sweeps made the small SVD the largest part of every POD below a few
+// hundred thousand rows.  Here:
+//   1. binary32 block one-sided Jacobi on A32 = fl32(R^T) (blocks of 16
+//      columns; a step's 32 columns are orthogonalised through their 32 x 32
+//      Gram matrix in shared memory, then the accumulated rotation is
+//      applied), giving V32; V = V32 made orthogonal (one Newton-Schulz
+//      step) and A = R^T V in binary64;
+//   2. the same again on fl32(A): each column now has its own binary32
+//      scale, so columns of small singular value, which fl32(R^T) buried
+//      under the rounding of the large ones, become orthogonal too;
+//   3. two to four binary64 steps of simultaneous rotations: with
+//      G = A^T A, E = V^T V - I and K_ij the Jacobi angle of pair (i, j)
+//      (antisymmetric), Q = I + K + K^2/2 - E/2 and A <- A Q, V <- V Q: all
+//      cosines square (Davies and Modi, "A direct method for completing
+//      eigenproblem solutions on a parallel computer", 1986).  Two columns
+//      whose angle is not small (double singular values) get their exact
+//      rotation instead.
+// Matrix products run on all SMs.  The binary64 sweeps then start from
+// (A, V); when every pair already meets their stopping test they return at
+// once, else they finish the job: the result is the binary64 SVD either way.
+//
+// Bound by the latency of the binary32 rounds (a round of 16 rotations is a
+// chain of three approximate operations and one block barrier, about 300 ns;
+// 7 to 10 sweeps) and, above M = 256, by the binary64 products.  Whole small
+// SVD of a field with a decaying spectrum on a floor, ten binary64 sweeps ->
+// here: M = 32 2.1 -> 0.25 ms, 64 4.2 -> 0.45, 128 9.6 -> 1.0; with the
+// earlier preconditioning (8-column blocks, three binary64 sweeps after it)
+// M = 256 13.3 -> 4.0, 700 114 -> 40 ms; singular values within 1.5e-15
+// S_max (2e-14 before: fewer rotations).
 #include "kernels.h"
 
 namespace pylom {
 
-constexpr int kJB = 8;                 // columns per block; a pair of blocks = 16 columns, one per warp pair
-constexpr int kJ32Threads = 32 * kJB;  // one warp per column pair of a round
-// inner sweeps per block pair and step: one (a block-cyclic sweep); 2 and 3
-// converged in the same number of outer and binary64 sweeps but took longer
-// (M = 256: 12.9 / 15.2 / 16.9 ms; M = 1808: 1.28 / 1.35 / 1.48 s)
-constexpr int kJ32Inner = 1;
-constexpr int kJ32MaxSweeps = 40;
+constexpr int kJB = 16;                // columns per block
+constexpr int kJW = 2 * kJB;           // columns of a step
+constexpr int kJ32Threads = 256;
+constexpr int kJRows = 64;             // rows of the staged tile
+constexpr int kJ32MaxSweeps = 24;
+constexpr int kJClusterMax = 8;        // up to 8 blocks run as one cluster (cheaper barrier)
+// words of s.rot32: rotations of each sweep of the two stages, then
+constexpr int kJScale = 2 * kJ32MaxSweeps;       // largest exponent field of R
+constexpr int kJSteps = 4;                       // binary64 steps of simultaneous rotations
+constexpr int kJOpen = kJScale + 1;              // kJSteps + 1 words: pairs not converged at each check; then: entries of V^T V off
+constexpr int kJWords = kJScale + 8;
 
-__global__ void jacobi32_init_kernel(SvdState s, const double* R, int64_t ldr) {
+__global__ void jacobi32_scale_kernel(SvdState s, const double* R, int64_t ldr) {
+  int e = 0;
+  const int64_t M = s.M;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int f = (__double2hiint(R[idx % M + (idx / M) * ldr]) >> 20) & 0x7ff;
+    e = (f != 0x7ff && f > e) ? f : e;
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0 && e > 0) atomicMax(s.rot32 + kJScale, (unsigned)e);
+}
+
+// A32 = 2^-e src^T or 2^-e src (binary32, zero padding columns), V32 = I
+__global__ void jacobi32_init_kernel(SvdState s, const double* src, int64_t ld, int trans) {
   const int64_t M = s.M, Mb = s.Mb;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int e = 1023 - (int)s.rot32[kJScale];
+  const double sc = __hiloint2double((e < -1021 ? 1 : e > 1023 ? 2046 : e + 1023) << 20, 0);
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * Mb; idx += stride) {
     const int64_t i = idx % M, j = idx / M;
-    s.A32[idx] = (j < M) ? (float)R[j + i * ldr] : 0.f;   // A32 = R^T (zero padding columns)
+    s.A32[idx] = (j < M) ? (float)(sc * (trans ? src[j + i * ld] : src[i + j * ld])) : 0.f;
   }
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mb * Mb; idx += stride)
     s.V32[idx] = (idx % Mb == idx / Mb) ? 1.f : 0.f;
 }
 
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// Jacobi rotation of a pair with squared norms al, be and dot product ga
+// (identity where |ga| is below the level thr2 of its squared cosine): no
+// branches and three approximate operations, since the chain of rounds is
+// latency bound (700 ns a round with IEEE square roots behind a branch).
+// t = sign(d) 2 ga / (|d| + sqrt(d^2 + 4 ga^2)), d = be - al
+__device__ __forceinline__ void rotation(float al, float be, float ga, float thr2, float& c, float& sn) {
+  const float d = be - al, g2 = ga + ga;
+  float r, q;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaf(d, d, g2 * g2)));
+  const float den = fmaxf(fabsf(d) + r, fabsf(g2));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(den));
+  const bool act = ga * ga > thr2 * fabsf(al * be);
+  const float t = act ? copysignf(1.f, d) * g2 * q : 0.f;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(fmaf(t, t, 1.f)));
+  sn = c * t;
 }
 
-// Cooperative launch; dynamic shared memory: 2 kJB columns of M floats plus
-// the 2 kJB x 2 kJB accumulated rotation.
-__global__ void __launch_bounds__(kJ32Threads) jacobi32_block_kernel(SvdState s) {
-  extern __shared__ float jsm[];
-  constexpr int W = 2 * kJB;
-  const int64_t M = s.M, Mb = s.Mb;
-  float* sA = jsm;                // [W][M]
-  float* sJ = sA + W * M;         // [W][W], column-major
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// One binary32 stage.  Blocks follow a round-robin order, a pair of column
+// blocks per thread block and step; steps end with a barrier over all
+// blocks (of the cluster, or of the grid in a cooperative launch).
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kJ32Threads) jacobi32_block_kernel(SvdState s, int stage) {
+  constexpr int LD = kJW + 4;
+  __shared__ __align__(16) float sA[kJRows * LD];
+  __shared__ float sG[2][kJW][kJW + 1];
+  __shared__ __align__(16) float sJ[kJW][LD];
+  __shared__ unsigned char sI[kJW - 1][kJB], sK[kJW - 1][kJB];
   __shared__ unsigned s_rot;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t M = s.M, Mb = s.Mb;
+  const int tid = threadIdx.x;
   const int64_t nblk = Mb / kJB, npairs = nblk / 2;
-  const float tol = 8.f * sqrtf((float)M) * 5.9604645e-8f;   // a few times the rounding level of a dot
+  const float tol = 4.f * sqrtf((float)M) * 5.9604645e-8f;   // the rounding level of a dot product
+  unsigned* rot = s.rot32 + stage * kJ32MaxSweeps;
+  for (int idx = tid; idx < (kJW - 1) * kJB; idx += kJ32Threads) {
+    const int round = idx / kJB, p = idx % kJB;
+    int a, b;
+    if (round < kJB) {                 // across the blocks
+      a = p;
+      b = kJB + (p + round) % kJB;
+    } else {                           // within them: two round-robins of 16 columns
+      const int h = p / 8 * kJB, q = p % 8, r = round - kJB;
+      a = h + ((q == 0) ? 0 : ((q - 1 + r) % (kJB - 1)) + 1);
+      b = h + ((kJB - 2 - q + r) % (kJB - 1)) + 1;
+    }
+    sI[round][p] = (unsigned char)(a < b ? a : b);
+    sK[round][p] = (unsigned char)(a < b ? b : a);
+  }
   for (int sweep = 0; sweep < kJ32MaxSweeps; ++sweep) {
     unsigned local_rot = 0;
-    for (int64_t step = 0; step < nblk - 1; ++step) {
+    const int64_t steps = nblk > 2 ? nblk - 1 : 1;
+    for (int64_t step = 0; step < steps; ++step) {
       for (int64_t pr = blockIdx.x; pr < npairs; pr += gridDim.x) {
         const int64_t p = (pr == 0) ? 0 : ((pr - 1 + step) % (nblk - 1)) + 1;
         const int64_t q = ((nblk - 2 - pr + step) % (nblk - 1)) + 1;
         const int64_t bI = p < q ? p : q, bJ = p < q ? q : p;
-        // the 16 columns: block bI then block bJ
-        for (int64_t idx = tid; idx < (int64_t)W * M; idx += kJ32Threads) {
-          const int l = (int)(idx / M);
-          const int64_t r = idx - (int64_t)l * M;
-          const int64_t col = (l < kJB) ? bI * kJB + l : bJ * kJB + (l - kJB);
-          sA[idx] = s.A32[r + col * M];
-        }
-        for (int idx = tid; idx < W * W; idx += kJ32Threads) sJ[idx] = (idx % W == idx / W) ? 1.f : 0.f;
-        __syncthreads();
-        for (int inner = 0; inner < kJ32Inner; ++inner) {
-          if (tid == 0) s_rot = 0;
-          __syncthreads();
-          // round-robin over the W local columns: W - 1 rounds of kJB disjoint pairs
-          for (int round = 0; round < W - 1; ++round) {
-            const int a = (warp == 0) ? 0 : ((warp - 1 + round) % (W - 1)) + 1;
-            const int b = ((W - 2 - warp + round) % (W - 1)) + 1;
-            const int i = a < b ? a : b, j = a < b ? b : a;
-            float* ai = sA + (int64_t)i * M;
-            float* aj = sA + (int64_t)j * M;
-            float al = 0.f, be = 0.f, ga = 0.f;
-            for (int64_t r = lane; r < M; r += 32) {
-              const float x = ai[r], y = aj[r];
-              al = fmaf(x, x, al);
-              be = fmaf(y, y, be);
-              ga = fmaf(x, y, ga);
-            }
-            al = warp_sum_f(al);
-            be = warp_sum_f(be);
-            ga = warp_sum_f(ga);
-            if (ga != 0.f && fabsf(ga) > tol * sqrtf(al * be)) {
-              const float zeta = (be - al) / (2.f * ga);
-              const float t = ((zeta >= 0.f) ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-              const float c = 1.f / sqrtf(1.f + t * t);
-              const float sn = c * t;
-              for (int64_t r = lane; r < M; r += 32) {
-                const float x = ai[r], y = aj[r];
-                ai[r] = c * x - sn * y;
-                aj[r] = sn * x + c * y;
-              }
-              if (lane < W) {
-                const float x = sJ[lane + i * W], y = sJ[lane + j * W];
-                sJ[lane + i * W] = c * x - sn * y;
-                sJ[lane + j * W] = sn * x + c * y;
-              }
-              if (lane == 0) atomicAdd(&s_rot, 1u);
-            }
-            __syncthreads();
-          }
-          const unsigned rr = s_rot;
-          if (inner == 0) local_rot += rr;
-          __syncthreads();
-          if (rr == 0) break;
-        }
-        // write the columns back; V32[:, cols] <- V32[:, cols] J
-        for (int64_t idx = tid; idx < (int64_t)W * M; idx += kJ32Threads) {
-          const int l = (int)(idx / M);
-          const int64_t r = idx - (int64_t)l * M;
-          const int64_t col = (l < kJB) ? bI * kJB + l : bJ * kJB + (l - kJB);
-          s.A32[r + col * M] = sA[idx];
-        }
-        float* VI = s.V32 + bI * kJB * Mb;
-        float* VJ = s.V32 + bJ * kJB * Mb;
-        for (int64_t r = tid; r < Mb; r += kJ32Threads) {
-          float v[W];
+        auto column = [&](int l) { return (l < kJB ? bI * kJB + l : bJ * kJB + (l - kJB)); };
+        // 32 x 32 Gram matrix: 8 x 8 threads of 4 x 4 entries, 4 row slices
+        const int ti = (tid & 7) * 4, tj = ((tid >> 3) & 7) * 4, sl = tid >> 6;
+        float g[4][4];
 #pragma unroll
-          for (int l = 0; l < kJB; ++l) {
-            v[l] = VI[r + l * Mb];
-            v[kJB + l] = VJ[r + l * Mb];
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) g[a][b] = 0.f;
+        for (int64_t r0 = 0; r0 < M; r0 += kJRows) {
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < kJRows * kJW / kJ32Threads; ++u) {
+            const int idx = tid + u * kJ32Threads;
+            const int r = idx % kJRows, l = idx / kJRows;
+            sA[r * LD + l] = (r0 + r < M) ? __ldcg(s.A32 + r0 + r + column(l) * M) : 0.f;
           }
+          __syncthreads();
+#pragma unroll 4
+          for (int r = sl; r < kJRows; r += 4) {
+            const float4 x = *(const float4*)(sA + r * LD + ti), y = *(const float4*)(sA + r * LD + tj);
+            const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+              for (int b = 0; b < 4; ++b) g[a][b] = fmaf(xa[a], ya[b], g[a][b]);
+          }
+        }
+        __syncthreads();
+        float* part = sA;
+        static_assert(kJW * kJW <= kJRows * LD, "a slice's Gram matrix fits the row tile");
+        for (int h = 3; h >= 1; --h) {
+          // slices 3, 2, 1 hand their sums to slice 0 in a fixed order
+          if (sl == h) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+              for (int b = 0; b < 4; ++b) part[(ti + a) * kJW + tj + b] = g[a][b];
+          }
+          __syncthreads();
+          if (sl == 0) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+              for (int b = 0; b < 4; ++b) g[a][b] += part[(ti + a) * kJW + tj + b];
+          }
+          __syncthreads();
+        }
+        if (tid == 0) s_rot = 0;
+        if (sl == 0) {
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) sG[0][ti + a][tj + b] = g[a][b];
+        }
+        for (int idx = tid; idx < kJW * kJW; idx += kJ32Threads) sJ[idx / kJW][idx % kJW] = idx / kJW == idx % kJW;
+        __syncthreads();
+        // pairs of this step that are not orthogonal yet
+        {
+          unsigned n = 0;
+          for (int idx = tid; idx < kJW * kJW; idx += kJ32Threads) {
+            const int i = idx / kJW, j = idx % kJW;
+            if (i < j && sG[0][i][j] * sG[0][i][j] > tol * tol * (sG[0][i][i] * sG[0][j][j])) ++n;
+          }
+          if (n) atomicAdd(&s_rot, n);
+        }
+        __syncthreads();
+        const unsigned open = s_rot;
+        local_rot += open;
+        if (open == 0) continue;
+        // two-sided rotations on the Gram matrix: the 16 disjoint pairs of a
+        // round at once, a thread per 2 x 2 block, each thread forming the
+        // two rotations of its block itself (one barrier a round, the matrix
+        // double-buffered).  Rounds 0..15 pair the columns of block I with
+        // those of block J; the pairs within the blocks (rounds 16..30)
+        // follow in the first step of a sweep only.
+        const int pb = tid & 15, qb = tid >> 4;
+        const int rounds = step == 0 ? kJW - 1 : kJB;
+        const float thr2 = 0.0625f * tol * tol;
+        int ni = sI[0][pb], nj = sK[0][pb], nk = sI[0][qb], nl = sK[0][qb];
+        for (int round = 0; round < rounds; ++round) {
+          const float(*G0)[kJW + 1] = sG[round & 1];
+          float(*G1)[kJW + 1] = sG[(round & 1) ^ 1];
+          const int i = ni, j = nj, k = nk, l = nl;
+          const int nr = round + 1 < rounds ? round + 1 : 0;
+          ni = sI[nr][pb];
+          nj = sK[nr][pb];
+          nk = sI[nr][qb];
+          nl = sK[nr][qb];
+          float cp, sp, cq, sq;
+          rotation(G0[i][i], G0[j][j], G0[i][j], thr2, cp, sp);
+          rotation(G0[k][k], G0[l][l], G0[k][l], thr2, cq, sq);
+          const float a = G0[i][k], b = G0[i][l], c = G0[j][k], d = G0[j][l];
+          // rows: [c -s; s c] on (i, j), columns the same on (k, l)
+          const float a1 = cp * a - sp * c, c1 = sp * a + cp * c, b1 = cp * b - sp * d, d1 = sp * b + cp * d;
+          G1[i][k] = cq * a1 - sq * b1;
+          G1[i][l] = sq * a1 + cq * b1;
+          G1[j][k] = cq * c1 - sq * d1;
+          G1[j][l] = sq * c1 + cq * d1;
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int r = qb + 16 * u;      // J's columns i, j of pair pb
+            const float x = sJ[r][i], y = sJ[r][j];
+            sJ[r][i] = cp * x - sp * y;
+            sJ[r][j] = sp * x + cp * y;
+          }
+          __syncthreads();
+        }
+        // A32 and V32 columns <- columns J (a thread per row)
+        for (int64_t row = tid; row < M + Mb; row += kJ32Threads) {
+          float* base = row < M ? s.A32 + row : s.V32 + (row - M);
+          const int64_t ld = row < M ? M : Mb;
+          float v[kJW];
+#pragma unroll
+          for (int l = 0; l < kJW; ++l) v[l] = __ldcg(base + column(l) * ld);
 #pragma unroll 1
-          for (int l = 0; l < W; ++l) {   // rolled: keeps the 256 entries of J in shared memory
-            float o = 0.f;
+          for (int l = 0; l < kJW; l += 4) {
+            float o[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int m = 0; m < W; ++m) o = fmaf(v[m], sJ[m + l * W], o);
-            if (l < kJB) VI[r + l * Mb] = o;
-            else VJ[r + (l - kJB) * Mb] = o;
+            for (int m = 0; m < kJW; ++m) {
+              const float4 jv = *(const float4*)&sJ[m][l];
+              o[0] = fmaf(v[m], jv.x, o[0]);
+              o[1] = fmaf(v[m], jv.y, o[1]);
+              o[2] = fmaf(v[m], jv.z, o[2]);
+              o[3] = fmaf(v[m], jv.w, o[3]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) __stcg(base + column(l + u) * ld, o[u]);
           }
         }
-        __syncthreads();
       }
-      if (!grid_barrier(s.hdr, gridDim.x)) return;
+      __syncthreads();
+      if (CLUSTER) cluster_barrier();
+      else if (!grid_barrier(s.hdr, gridDim.x)) return;
     }
-    if (tid == 0 && local_rot) atomicAdd(&s.rot32[sweep], local_rot);
-    if (!grid_barrier(s.hdr, gridDim.x)) return;
-    if (ld_acquire_u32(&s.rot32[sweep]) == 0) break;
+    if (tid == 0 && local_rot) atomicAdd(rot + sweep, local_rot);
+    if (CLUSTER) {
+      __threadfence();
+      __syncthreads();
+      cluster_barrier();
+    } else if (!grid_barrier(s.hdr, gridDim.x)) {
+      return;
+    }
+    if (ld_acquire_u32(rot + sweep) == 0) break;
   }
 }
 
 // V (Mp x Mp, binary64) = the leading Mp x Mp block of V32.
-__global__ void jacobi32_widen_kernel(SvdState s) {
+__global__ void jacobi32_widen_kernel(SvdState s, double* V) {
   const int64_t Mp = s.Mp, Mb = s.Mb;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mp * Mp;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = idx % Mp, j = idx / Mp;
-    s.V[idx] = (double)s.V32[i + j * Mb];
+    V[idx] = (double)s.V32[i + j * Mb];
   }
 }
 
-// V <- (3 V - V G) / 2 with T = V G already formed
-__global__ void newton_schulz_kernel(double* V, const double* T, int64_t n) {
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-       idx += (int64_t)gridDim.x * blockDim.x)
-    V[idx] = 1.5 * V[idx] - 0.5 * T[idx];
+// C = alpha op(A) B + beta D, binary64 on the FP64 tensor pipe, for the
+// small products between the stages (one or two of them in a launch): T x T
+// tiles, the K range split over the four warps of a block and summed in a
+// fixed order.  `skip` (nullable): nothing to do when *skip is 0.
+struct SmallGemm {
+  int ta;
+  int64_t m, n, k;
+  const double* A;
+  int64_t lda;
+  const double* B;
+  int64_t ldb;
+  double alpha, beta;
+  const double* D;   // ld m
+  double* C;         // ld m
+};
+struct SmallGemms {
+  SmallGemm g[2];
+  const unsigned* skip;
+};
+
+template <int T>
+__global__ void __launch_bounds__(128) small_gemm_kernel(SmallGemms gs) {
+  constexpr int U = T / 8;
+  __shared__ double part[4][T][T + 1];
+  if (gs.skip && *gs.skip == 0) return;
+  const SmallGemm& p = gs.g[blockIdx.z];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int64_t i0 = (int64_t)blockIdx.x * T, j0 = (int64_t)blockIdx.y * T;
+  if (i0 >= p.m || j0 >= p.n) return;
+  double acc[U][U][2];
+#pragma unroll
+  for (int a = 0; a < U; ++a)
+#pragma unroll
+    for (int b = 0; b < U; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
+  const int64_t nst = (p.k + 3) / 4;
+#pragma unroll 4
+  for (int64_t st = warp; st < nst; st += 4) {
+    const int64_t kk = st * 4 + t;
+    double av[U], bv[U];
+#pragma unroll
+    for (int a = 0; a < U; ++a) {
+      const int64_t i = i0 + 8 * a + g, j = j0 + 8 * a + g;
+      av[a] = (kk < p.k && i < p.m) ? (p.ta ? __ldg(p.A + kk + i * p.lda) : __ldg(p.A + i + kk * p.lda)) : 0.0;
+      bv[a] = (kk < p.k && j < p.n) ? __ldg(p.B + kk + j * p.ldb) : 0.0;
+    }
+#pragma unroll
+    for (int a = 0; a < U; ++a)
+#pragma unroll
+      for (int b = 0; b < U; ++b) dmma884(acc[a][b][0], acc[a][b][1], av[a], bv[b]);
+  }
+#pragma unroll
+  for (int a = 0; a < U; ++a)
+#pragma unroll
+    for (int b = 0; b < U; ++b) {
+      part[warp][8 * a + g][8 * b + 2 * t] = acc[a][b][0];
+      part[warp][8 * a + g][8 * b + 2 * t + 1] = acc[a][b][1];
+    }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < T * T; idx += 128) {
+    const int r = idx % T, c = idx / T;
+    const int64_t i = i0 + r, j = j0 + c;
+    if (i < p.m && j < p.n) {
+      const double v = (part[0][r][c] + part[1][r][c]) + (part[2][r][c] + part[3][r][c]);
+      p.C[i + j * p.m] = p.alpha * v + (p.D ? p.beta * p.D[i + j * p.m] : 0.0);
+    }
+  }
+}
+
+static cudaError_t small_gemms(const SmallGemms& gs, int count, cudaStream_t st) {
+  int64_t m = gs.g[0].m, n = gs.g[0].n;
+  for (int i = 1; i < count; ++i) {
+    m = gs.g[i].m > m ? gs.g[i].m : m;
+    n = gs.g[i].n > n ? gs.g[i].n : n;
+  }
+  // 8 x 8 tiles while 16 x 16 ones would leave most SMs idle
+  if (m * n * count <= 2 * 144 * 144) {
+    const dim3 grid((unsigned)((m + 7) / 8), (unsigned)((n + 7) / 8), (unsigned)count);
+    small_gemm_kernel<8><<<grid, 128, 0, st>>>(gs);
+  } else {
+    const dim3 grid((unsigned)((m + 15) / 16), (unsigned)((n + 15) / 16), (unsigned)count);
+    small_gemm_kernel<16><<<grid, 128, 0, st>>>(gs);
+  }
+  return cudaGetLastError();
+}
+
+// Jacobi angle of the pair (i, j) of A's columns from G = A^T A as its
+// tangent t: column j gains +t a_i, column i gains -t a_j (antisymmetric).
+__device__ __forceinline__ double pair_tangent(double al, double be, double ga) {
+  if (ga == 0.0) return 0.0;
+  const double zeta = (be - al) / (2.0 * ga);
+  return ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+}
+
+// Whether the pair takes part in a step as a small angle t: pairs that are
+// converged do only where that is harmless (their angle is noise).
+constexpr double kSmallAngle = 0.02;
+__device__ __forceinline__ bool small_angle(bool open, double t, double M) {
+  return open ? fabs(t) <= kSmallAngle : fabs(t) * M <= 1e-3;
+}
+__device__ __forceinline__ bool pair_open(double al, double be, double ga, double tol) {
+  return ga != 0.0 && fabs(ga) > tol * sqrt(al * be);
+}
+
+// Check `c` on G: counts the pairs that the binary64 sweeps would rotate
+// (open[c]), and says for each column what the step does with it: big[j] >= 0
+// is the partner of its largest angle if that is not small, -1: its angles
+// are small and sum to at most `limit`, -2: left alone (a crowd of close
+// singular values, where the angles together would not be a small rotation).
+// With W = V^T V given, entries away from the identity by more than wtol
+// are counted in bad.  A warp per column.
+__global__ void jacobi_check_kernel(SvdState s, const double* G, const double* W, double wtol, unsigned* bad, int c,
+                                    double limit, const unsigned* skip) {
+  if (skip && *skip == 0) return;
+  const int64_t Mp = s.Mp;
+  const int lane = threadIdx.x & 31;
+  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (j >= Mp) return;
+  const double tol = (double)s.M * 1.1102230246251565e-16;
+  const double be = G[j + j * Mp];
+  unsigned n = 0, nw = 0;
+  double best = kSmallAngle, sum = 0.0;
+  int bi = -1;
+  for (int64_t i = lane; i < Mp; i += 32) {
+    if (W) nw += !(fabs(W[i + j * Mp] - (i == j ? 1.0 : 0.0)) <= wtol);
+    if (i == j) continue;
+    const double al = G[i + i * Mp], ga = G[i + j * Mp];
+    const bool open = pair_open(al, be, ga, tol);
+    n += open && i < j;
+    const double t = fabs(pair_tangent(al, be, ga));
+    if (open && t > best) {
+      best = t;
+      bi = (int)i;
+    } else if (small_angle(open, t, (double)s.M)) {
+      sum += t;
+    }
+  }
+  sum = warp_sum(sum);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (oi >= 0 && (bi < 0 || ob > best || (ob == best && oi < bi))) {
+      best = ob;
+      bi = oi;
+    }
+  }
+  n = __reduce_add_sync(0xffffffffu, n);
+  nw = __reduce_add_sync(0xffffffffu, nw);
+  if (lane == 0) {
+    s.big[j] = bi >= 0 ? bi : sum <= limit ? -1 : -2;
+    if (n) atomicAdd(s.rot32 + kJOpen + c, n);
+    if (nw) atomicAdd(bad, nw);
+  }
+}
+
+// K = the antisymmetric small angles, L = K - E and B = I + K - E / 2 with
+// E = W - I, W = V^T V, so that Q = B + L K / 2 = (I - E / 2)(I + K + K^2 / 2)
+// up to E K^2.  B may overwrite W.
+// Two columns that are each other's largest angle get their exact rotation
+// in B (multiple singular values: the angle is anything up to 45 degrees)
+// and no other angle this time.
+__global__ void jacobi_angles_kernel(SvdState s, const double* G, const double* W, double* K, double* L,
+                                     double* B, const unsigned* skip) {
+  if (skip && *skip == 0) return;
+  const int64_t Mp = s.Mp;
+  const double tol = (double)s.M * 1.1102230246251565e-16;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mp * Mp;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % Mp, j = idx / Mp;
+    const int bi = s.big[i], bj = s.big[j];
+    double t = 0.0, x = 0.0;
+    if (i != j) {
+      if (bi == j && bj == i) {
+        const double tt = pair_tangent(G[i + i * Mp], G[j + j * Mp], G[idx]);
+        x = tt / sqrt(1.0 + tt * tt);
+      } else if (bi == -1 && bj == -1) {
+        const double al = G[i + i * Mp], be = G[j + j * Mp], ga = G[idx];
+        t = pair_tangent(al, be, ga);
+        if (!small_angle(pair_open(al, be, ga, tol), t, (double)s.M)) t = 0.0;
+      }
+    } else {
+      x = 1.0;
+      if (bi >= 0 && s.big[bi] == i) {
+        const double tt = pair_tangent(G[i + i * Mp], G[bi + (int64_t)bi * Mp], G[i + bi * Mp]);
+        x = 1.0 / sqrt(1.0 + tt * tt);
+      }
+    }
+    const double E = W[idx] - (i == j ? 1.0 : 0.0);
+    K[idx] = t;
+    L[idx] = t - E;
+    B[idx] = x + t - 0.5 * E;
+  }
+}
+
+__global__ void jacobi_restart_kernel(SvdState s, const double* R, int64_t ldr, const unsigned* bad, unsigned* open) {
+  if (*bad == 0) return;
+  const int64_t M = s.M, Mp = s.Mp, na = M * Mp, nv = Mp * Mp;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < na + nv;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    if (idx < na) {
+      const int64_t i = idx % M, j = idx / M;
+      s.A[idx] = (j < M) ? R[j + i * ldr] : 0.0;
+    } else {
+      const int64_t v = idx - na;
+      s.V[v] = (v % Mp == v / Mp) ? 1.0 : 0.0;
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *open = 1;
 }
 
 size_t jacobi32_extra_bytes(int64_t M) {
   if (M < kJac32MinM) return 0;
   const int64_t Mp = M + (M & 1);
-  const int64_t Mb = (M + 2 * kJB - 1) / (2 * kJB) * (2 * kJB);
+  const int64_t Mb = (M + kJW - 1) / kJW * kJW;
   return align256(sizeof(float) * (size_t)M * Mb) + align256(sizeof(float) * (size_t)Mb * Mb) +
-         2 * align256(sizeof(double) * (size_t)Mp * Mp) + align256(sizeof(unsigned) * kJ32MaxSweeps) +
-         align256(matmul_ws_bytes(Mp, Mp, Mp) > matmul_ws_bytes(M, Mp, M) ? matmul_ws_bytes(Mp, Mp, Mp)
-                                                                           : matmul_ws_bytes(M, Mp, M));
+         5 * align256(sizeof(double) * (size_t)Mp * Mp) + align256(sizeof(unsigned) * kJWords) +
+         align256(sizeof(double) * (size_t)M * Mp) + align256(sizeof(int) * (size_t)Mp);
 }
 
 void jacobi32_carve(SvdState& s, char* p) {
   const int64_t M = s.M, Mp = s.Mp;
-  s.Mb = (M + 2 * kJB - 1) / (2 * kJB) * (2 * kJB);
+  const size_t sq = align256(sizeof(double) * (size_t)Mp * Mp);
+  s.Mb = (M + kJW - 1) / kJW * kJW;
   s.A32 = (float*)p;    p += align256(sizeof(float) * (size_t)M * s.Mb);
   s.V32 = (float*)p;    p += align256(sizeof(float) * (size_t)s.Mb * s.Mb);
-  s.G = (double*)p;     p += align256(sizeof(double) * (size_t)Mp * Mp);
-  s.Tm = (double*)p;    p += align256(sizeof(double) * (size_t)Mp * Mp);
-  s.rot32 = (unsigned*)p; p += align256(sizeof(unsigned) * kJ32MaxSweeps);
-  s.mmws = (double*)p;
+  for (int i = 0; i < 5; ++i) { s.T[i] = (double*)p; p += sq; }
+  s.rot32 = (unsigned*)p; p += align256(sizeof(unsigned) * kJWords);
+  s.A2 = (double*)p;    p += align256(sizeof(double) * (size_t)M * Mp);
+  s.big = (int*)p;
 }
 
-// Leaves s.A = R^T V and s.V = V (orthogonal), the starting point of the
-// binary64 sweeps.
-cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int64_t ldr, cudaStream_t st) {
-  const int64_t M = s.M, Mp = s.Mp;
-  cudaError_t e = cudaMemsetAsync(s.rot32, 0, sizeof(unsigned) * kJ32MaxSweeps, st);
-  if (e != cudaSuccess) return e;
-  jacobi32_init_kernel<<<256, 256, 0, st>>>(s, R, ldr);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const size_t smem = sizeof(float) * ((size_t)2 * kJB * M + 4 * kJB * kJB);
-  if ((e = ensure_dyn_smem((const void*)jacobi32_block_kernel, smem)) != cudaSuccess) return e;
+static cudaError_t stage32(const SvdState& s, int stage, cudaStream_t st) {
+  cudaError_t e;
+  const int64_t npairs = s.Mb / kJW;
+  SvdState a = s;
+  if (npairs <= kJClusterMax) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)npairs);
+    cfg.blockDim = dim3(kJ32Threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)npairs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, jacobi32_block_kernel<true>, a, stage);
+  }
   int dev = 0, sms = 0, per = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jacobi32_block_kernel, kJ32Threads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jacobi32_block_kernel<false>, kJ32Threads, 0);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorCooperativeLaunchTooLarge;
-  int64_t grid = (s.Mb / kJB) / 2;
-  if (grid > (int64_t)per * sms) grid = (int64_t)per * sms;
-  SvdState a = s;
-  void* args[] = {&a};
-  e = cudaLaunchCooperativeKernel((const void*)jacobi32_block_kernel, dim3((unsigned)grid), dim3(kJ32Threads), args,
-                                  smem, st);
+  int64_t grid = npairs;
+  if (grid > sms) grid = sms;
+  void* args[] = {&a, &stage};
+  return cudaLaunchCooperativeKernel((const void*)jacobi32_block_kernel<false>, dim3((unsigned)grid),
+                                     dim3(kJ32Threads), args, 0, st);
+}
+
+// Leaves s.A = R^T V and s.V = V (orthogonal), the starting point of the
+// binary64 sweeps; **open_pairs (device) is 0 when nothing is left for them.
+cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int64_t ldr, const unsigned** open_pairs,
+                                         cudaStream_t st) {
+  const int64_t M = s.M, Mp = s.Mp;
+  const int gr = M <= 64 ? 16 : M <= 256 ? 128 : 304;
+  cudaError_t e = cudaMemsetAsync(s.rot32, 0, sizeof(unsigned) * kJWords, st);
   if (e != cudaSuccess) return e;
-  jacobi32_widen_kernel<<<256, 256, 0, st>>>(s);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  for (int it = 0; it < 2; ++it) {
-    e = launch_matmul_fp64(1, s.V, s.V, s.G, Mp, Mp, Mp, Mp, Mp, Mp, s.mmws, st);   // G = V^T V
+  double *T0 = s.T[0], *T1 = s.T[1], *T2 = s.T[2], *T3 = s.T[3], *T4 = s.T[4];
+  unsigned* open = s.rot32 + kJOpen;
+  // a product whose left factor op(A) has `m` rows and K = `k` (B then has
+  // leading dimension k, C and D m)
+  auto mm = [&](int ta, int64_t m, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
+                double beta, const double* D, double* C) {
+    return SmallGemm{ta, m, Mp, k, A, lda, B, k, alpha, beta, D, C};
+  };
+  auto one = [&](const SmallGemm& g, const unsigned* skip = nullptr) {
+    if (e == cudaSuccess) e = small_gemms(SmallGemms{{g, g}, skip}, 1, st);
+  };
+  auto two = [&](const SmallGemm& g, const SmallGemm& h, const unsigned* skip = nullptr) {
+    if (e == cudaSuccess) e = small_gemms(SmallGemms{{g, h}, skip}, 2, st);
+  };
+  jacobi32_scale_kernel<<<gr, 256, 0, st>>>(s, R, ldr);
+  jacobi32_init_kernel<<<gr, 256, 0, st>>>(s, R, ldr, 1);
+  if ((e = cudaGetLastError()) != cudaSuccess || (e = stage32(s, 0, st)) != cudaSuccess) return e;
+  jacobi32_widen_kernel<<<gr, 256, 0, st>>>(s, T0);
+  e = cudaGetLastError();
+  one(mm(1, Mp, Mp, 1.0, T0, Mp, T0, 0.0, nullptr, T1));                             // V^T V
+  one(mm(0, Mp, Mp, -0.5, T0, Mp, T1, 1.5, T0, T3));                                 // V <- 1.5 V - 0.5 V V^T V
+  one(SmallGemm{1, M, Mp, M, R, ldr, T3, Mp, 1.0, 0.0, nullptr, s.A2});              // A = R^T V (rows of V past M meet no row of R)
+  if (e != cudaSuccess) return e;
+  jacobi32_init_kernel<<<gr, 256, 0, st>>>(s, s.A2, M, 0);
+  if ((e = cudaGetLastError()) != cudaSuccess || (e = stage32(s, 1, st)) != cudaSuccess) return e;
+  jacobi32_widen_kernel<<<gr, 256, 0, st>>>(s, T0);
+  e = cudaGetLastError();
+  two(mm(0, Mp, Mp, 1.0, T3, Mp, T0, 0.0, nullptr, s.V), mm(0, M, Mp, 1.0, s.A2, M, T0, 0.0, nullptr, s.A));
+  // steps of simultaneous rotations, (A, V) -> (A2, T3) -> (A, V) and, if
+  // pairs are still open, the same again; V's departure from orthogonality
+  // goes 1e-6 -> 1e-12 -> rounding
+  const unsigned gc = (unsigned)((Mp * 32 + 255) / 256);
+  for (int it = 0; it < kJSteps; ++it) {
+    const bool fwd = (it & 1) == 0;
+    const double *Ai = fwd ? s.A : s.A2, *Vi = fwd ? s.V : T3;
+    double *Ao = fwd ? s.A2 : s.A, *Vo = fwd ? T3 : s.V;
+    const unsigned* skip = it < 2 ? nullptr : open + 2;
+    two(mm(1, Mp, M, 1.0, Ai, M, Ai, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, Vi, Mp, Vi, 0.0, nullptr, T1),
+        it == 2 ? nullptr : skip);
     if (e != cudaSuccess) return e;
-    e = launch_matmul_fp64(0, s.V, s.G, s.Tm, Mp, Mp, Mp, Mp, Mp, Mp, s.mmws, st);  // T = V G
-    if (e != cudaSuccess) return e;
-    newton_schulz_kernel<<<256, 256, 0, st>>>(s.V, s.Tm, Mp * Mp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // (a step of angle sum a leaves V off orthogonality by a^4 / 4, which the
+    // next one repairs: the last one takes tiny angles only)
+    jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, it == 2 ? T1 : nullptr, 1e-14, open + 2, it,
+                                            it == kJSteps - 1 ? 2e-4 : 0.05, it == 2 ? nullptr : skip);
+    jacobi_angles_kernel<<<gr, 256, 0, st>>>(s, T0, T1, T2, T4, T1, skip);
+    e = cudaGetLastError();
+    one(mm(0, Mp, Mp, 0.5, T4, Mp, T2, 1.0, T1, T0), skip);                          // Q
+    two(mm(0, M, Mp, 1.0, Ai, M, T0, 0.0, nullptr, Ao), mm(0, Mp, Mp, 1.0, Vi, Mp, T0, 0.0, nullptr, Vo), skip);
   }
-  // A = R^T V (M x Mp; rows of V beyond M meet no row of R)
-  return launch_matmul_fp64(1, R, s.V, s.A, M, Mp, M, ldr, Mp, M, s.mmws, st);
+  two(mm(1, Mp, M, 1.0, s.A, M, s.A, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, s.V, Mp, s.V, 0.0, nullptr, T1), open + 2);
+  if (e != cudaSuccess) return e;
+  const double wtol = (double)M * 1.1102230246251565e-16;
+  jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, T1, wtol > 1e-14 ? wtol : 1e-14, open + kJSteps + 1, kJSteps, 0.05,
+                                          open + 2);
+  // a V that is not orthogonal after all: the binary64 sweeps start from R^T
+  jacobi_restart_kernel<<<gr, 256, 0, st>>>(s, R, ldr, open + kJSteps + 1, open + kJSteps);
+  *open_pairs = open + kJSteps;
+  return cudaGetLastError();
 }
 
 }  // namespace pylom
