@@ -178,4 +178,230 @@ __device__ __forceinline__ bool mbar_wait_fast(uint64_t* mbar, uint32_t parity) 
   return done ? true : tc05::mbar_wait(mbar, parity);
 }
 
+// ---------------------------------------------------------------------------
+// the two pipelines (512 threads, one block per SM)
+// ---------------------------------------------------------------------------
+constexpr int kDigThreads = 512;   // 128 registers a thread: 64 hold the integer sums
+
+template <int NST>
+struct DigitBarriers {
+  uint64_t full[NST], empty[NST], dfull, dempty, fin;
+  uint32_t tmem;
+  // all threads; `extra`: arrivals on a full barrier besides one per warp
+  __device__ __forceinline__ void open(int extra) {
+    if (threadIdx.x == 0) {
+      for (int b = 0; b < NST; ++b) {
+        tc05::mbar_init(full + b, kDigThreads / 32 + extra);
+        tc05::mbar_init(empty + b, 1);
+      }
+      tc05::mbar_init(&dfull, 1);
+      tc05::mbar_init(&dempty, kDigThreads / 32);
+      tc05::mbar_init(&fin, 1);
+    }
+    if (threadIdx.x < 32) tc05::tmem_alloc(&tmem, 512);
+    tc05::fence_before();
+    __syncthreads();
+    tc05::fence_after();
+  }
+  // all threads: nothing of this block is in flight when it gives its memory back
+  __device__ __forceinline__ void close(bool ok, WsHeader* hdr) {
+    if (threadIdx.x == kDigThreads - 32) {
+      tc05::commit(&fin);
+      if (!mbar_wait_fast(&fin, 0)) ok = false;
+    }
+    if (!ok) raise_status(hdr, PYLOM_ERR_TIMEOUT);
+    tc05::fence_before();
+    __syncthreads();
+    if (threadIdx.x < 32) tc05::tmem_dealloc(tmem, 512);
+  }
+};
+
+// Sums over a range of rows: `nstage` stages of kStK rows, read out every
+// kStagesPerSum of them.  fill(j, stage) writes this thread's part of stage
+// j; issue(stage address, first) issues its MMAs (one thread); flush(acc0,
+// acc1) hands on the 64-bit sums of this thread's row and 16 columns.  The
+// accumulators are read only after the next NST stages have been filled, so
+// the warps work while the last MMAs of a sum run.
+template <int NST, class Fill, class Issue, class Flush>
+__device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int stage_bytes, int64_t nstage,
+                                              int nslots, WsHeader* hdr, Fill fill, Issue issue, Flush flush) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  bar.open(0);
+  const uint32_t tmem = bar.tmem;
+  const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16;
+  bool ok = true;
+  int64_t acc0[16], acc1[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
+  int64_t issued = 0, drained = 0;
+  for (int64_t j = 0; j <= nstage; ++j) {
+    const int b = (int)(j % NST);
+    if (j < nstage) {
+      if (j >= NST) {
+        ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + b, (uint32_t)((j / NST - 1) & 1)));
+        if (!ok) break;
+      }
+      fill(j, gsm + b * stage_bytes);
+      tc05::fence_smem_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar.full + b);
+    }
+    // the sums of the 128 rows before, once the stages ahead are filled
+    const bool due = (j % kStagesPerSum == NST - 1 && j >= kStagesPerSum && j < nstage) ||
+                     (j == nstage && nstage > 0);
+    if (due) {
+      ok = __all_sync(0xffffffffu, mbar_wait_fast(&bar.dfull, (uint32_t)(drained & 1)));
+      if (!ok) break;
+      tc05::fence_after();
+      drain_slots(taddr, nslots, acc0, acc1);
+      tc05::fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar.dempty);
+      ++drained;
+      if ((drained & 8191) == 0) flush(acc0, acc1);
+    }
+    // MMAs of the stages that are filled; those of a new sum wait until the
+    // last one has been read
+    const bool held = j >= kStagesPerSum && j % kStagesPerSum < NST - 1;
+    if (warp == kDigThreads / 32 - 1 && lane == 0 && j < nstage && !held) {
+      for (; issued <= j && ok; ++issued) {
+        const int ib = (int)(issued % NST);
+        const int64_t sum = issued / kStagesPerSum;
+        const bool first = issued % kStagesPerSum == 0;
+        ok = mbar_wait_fast(bar.full + ib, (uint32_t)((issued / NST) & 1));
+        if (ok && first && sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((sum - 1) & 1));
+        if (!ok) break;
+        tc05::fence_after();
+        issue(tmem, tc05::smem_u32(gsm) + ib * stage_bytes, first);
+        tc05::commit(bar.empty + ib);
+        if (issued % kStagesPerSum == kStagesPerSum - 1) tc05::commit(&bar.dfull);
+      }
+    }
+    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+    if (!ok) break;
+  }
+  if (ok) flush(acc0, acc1);
+  bar.close(ok, hdr);
+}
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               :: "r"(tc05::smem_u32(dst)), "l"((uint64_t)__cvta_generic_to_global(src)), "r"(bytes),
+                  "r"(tc05::smem_u32(mbar))
+               : "memory");
+}
+
+// Products of `mine` output tiles of 128 rows x 64 columns, K = `stages`
+// stages of kStK elements each, as one sequence of stages: fill(tile, js,
+// stage) writes the left factor's digits, the right factor's planes come by
+// a bulk copy from bsrc(tile, js), store(tile, acc0, acc1) writes this
+// thread's row and 16 columns.  `tile` counts 0 .. mine - 1.  LB: lowest
+// level that is kept.
+template <int S, int NST, int LB, class Fill, class Src, class Store>
+__device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int64_t mine, int64_t stages,
+                                                 WsHeader* hdr, Fill fill, Src bsrc, Store store) {
+  constexpr int kStage = S * (kPlaneA + kPlaneB);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bar.open(1);
+  const uint32_t tmem = bar.tmem;
+  const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16;
+  const int64_t sums = (stages + kStagesPerSum - 1) / kStagesPerSum;
+  const int64_t total = mine * stages, nsum = mine * sums;
+  bool ok = true;
+  int64_t acc0[16], acc1[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
+  int64_t issued = 0, issued_sum = 0, drained = 0;
+  int64_t tile = 0, js = 0, begun = 0;   // the stage being filled; sums whose first stage has been filled
+  int ahead = 0;                         // stages filled of the current sum
+  int64_t is_js = 0, dr_tile = 0, dr_sum = 0;
+  for (int64_t j = 0; j <= total; ++j) {
+    const int b = (int)(j % NST);
+    if (j < total) {
+      if (j >= NST) {
+        ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + b, (uint32_t)((j / NST - 1) & 1)));
+        if (!ok) break;
+      }
+      unsigned char* st = gsm + b * kStage;
+      if (tid == 0) {
+        tc05::mbar_arrive_expect_tx(bar.full + b, S * kPlaneB);
+        bulk_load(st + S * kPlaneA, bsrc(tile, js), S * kPlaneB, bar.full + b);
+      }
+      fill(tile, js, st);
+      tc05::fence_smem_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar.full + b);
+      if (js % kStagesPerSum == 0) {
+        ++begun;
+        ahead = 0;
+      }
+      ++ahead;
+      if (++js == stages) {
+        js = 0;
+        ++tile;
+      }
+    }
+    // read the sums that are complete: all of them at the end; before that,
+    // the one before the sum being filled, as soon as NST stages (or the
+    // whole sum) are filled ahead of it
+    const bool whole = j < total && (js == 0 || js % kStagesPerSum == 0);
+    const int64_t upto = j == total ? nsum : (ahead >= NST || whole) ? begun - 1 : drained;
+    while (drained < upto) {
+      ok = __all_sync(0xffffffffu, mbar_wait_fast(&bar.dfull, (uint32_t)(drained & 1)));
+      if (!ok) break;
+      tc05::fence_after();
+      drain_slots(taddr, kSlots, acc0, acc1);
+      tc05::fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar.dempty);
+      ++drained;
+      if (++dr_sum == sums) {
+        store(dr_tile, acc0, acc1);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
+        dr_sum = 0;
+        ++dr_tile;
+      }
+    }
+    if (!ok) break;
+    // MMAs of filled stages, up to the first sum whose accumulators are still unread
+    if (warp == kDigThreads / 32 - 1) {
+      if (lane == 0) {
+        while (issued <= j && issued < total) {
+          const bool first = is_js % kStagesPerSum == 0;
+          if (first && issued_sum > drained) break;      // this warp has not read the sum before
+          const int ib = (int)(issued % NST);
+          ok = mbar_wait_fast(bar.full + ib, (uint32_t)((issued / NST) & 1));
+          if (ok && first && issued_sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((issued_sum - 1) & 1));
+          if (!ok) break;
+          if (first) ++issued_sum;
+          tc05::fence_after();
+          const uint32_t sa = tc05::smem_u32(gsm) + ib * kStage;
+          issue_stage<S, LB>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo),
+                             kPlaneB, first);
+          tc05::commit(bar.empty + ib);
+          ++issued;
+          if (++is_js == stages) is_js = 0;
+          if (is_js % kStagesPerSum == 0) tc05::commit(&bar.dfull);
+        }
+      }
+      ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+      if (!ok) break;
+    }
+  }
+  // bulk copies of stages that were never consumed (after a timeout) land
+  // before the block ends
+  if (!ok && tid == 0)
+    for (int b = 0; b < NST; ++b) tc05::mbar_wait(bar.full + b, 0, 1000000ull);
+  bar.close(ok, hdr);
+}
+
+// one integer sum into the global groups: the low 32 bits to group g, the
+// carry to group g + 1 (so no group can overflow)
+__device__ __forceinline__ void add_group(unsigned long long* G, int64_t MM, int64_t at, int g, int64_t v) {
+  if (v == 0) return;
+  atomicAdd(G + g * MM + at, (unsigned long long)(v & 0xffffffffll));
+  atomicAdd(G + (g + 1) * MM + at, (unsigned long long)(v >> 32));
+}
+
 }  // namespace pylom

@@ -178,8 +178,6 @@ __global__ void __launch_bounds__(kPrThreads) gram_prologue_kernel(PrologueArgs 
 // MMAs of the sum run), and at the end those go to the global sums by
 // integer atomics, so the result does not depend on the order.
 
-constexpr int kGrThreads = 512;   // 128 registers a thread: 64 hold the integer sums
-
 struct GramArgs {
   const void* Y;
   int64_t ldy, N, M;
@@ -230,21 +228,11 @@ __device__ __forceinline__ void put_column8(const TY* Y, int64_t ldy, int64_t ro
   store_digits<S>(w, dst, plane);
 }
 
-// one integer sum into the global groups: the low 32 bits to group g, the
-// carry to group g + 1 (so no group can overflow)
-__device__ __forceinline__ void add_group(unsigned long long* G, int64_t MM, int64_t at, int g, int64_t v) {
-  if (v == 0) return;
-  atomicAdd(G + g * MM + at, (unsigned long long)(v & 0xffffffffll));
-  atomicAdd(G + (g + 1) * MM + at, (unsigned long long)(v >> 32));
-}
-
 template <typename TY>
-__global__ void __launch_bounds__(kGrThreads, 1) gram_kernel(GramArgs a) {
+__global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST;
-  constexpr int kStage = S * (kPlaneA + kPlaneB);
   extern __shared__ __align__(1024) unsigned char gsm[];
-  __shared__ __align__(8) uint64_t full[NST], empty[NST], dfull, dempty, fin;
-  __shared__ uint32_t tmem_base;
+  __shared__ __align__(8) DigitBarriers<NST> bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int item = blockIdx.x % a.items, split = blockIdx.x / a.items;
   const int half = item % Dig<TY>::HALVES;
@@ -257,22 +245,6 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_kernel(GramArgs a) {
   const bool diag = (J >> 1) == I;       // B's columns are among A's
   const int64_t nsum = (a.N + 127) / 128;
   const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
-  const int64_t nstage = (q1 - q0) * kStagesPerSum;
-  if (tid == 0) {
-    for (int b = 0; b < NST; ++b) {
-      tc05::mbar_init(full + b, kGrThreads / 32);
-      tc05::mbar_init(empty + b, 1);
-    }
-    tc05::mbar_init(&dfull, 1);
-    tc05::mbar_init(&dempty, kGrThreads / 32);
-    tc05::mbar_init(&fin, 1);
-  }
-  if (warp == 0) tc05::tmem_alloc(&tmem_base, 512);
-  tc05::fence_before();
-  __syncthreads();
-  tc05::fence_after();
-  const uint32_t tmem = tmem_base;
-  bool ok = true;
   const TY* Y = (const TY*)a.Y;
   const int c8 = lane & 7, kg = lane >> 3;
   const int ca = warp * 8 + c8;                  // A: 16 warps x 8 columns
@@ -282,17 +254,26 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_kernel(GramArgs a) {
   const bool doB = !diag && warp < 8;            // B: 8 warps x 8 columns
   const int64_t colB = (int64_t)J * 64 + ca;
   const int EB = (doB && colB < a.M) ? a.colE[colB] : 1;
-  const int qd = warp & 3, cp = warp >> 2;       // tensor-memory lane quadrant, 16-column part
-  const uint32_t taddr = tmem + ((uint32_t)(qd * 32) << 16) + cp * 16;
-  const int nslots = (sizeof(TY) == 8 && half == 1) ? 7 : 8;
-  int64_t acc0[16], acc1[16];
-#pragma unroll
-  for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
-  auto flush = [&]() {
-    const int64_t gi = (int64_t)I * 128 + qd * 32 + lane;
+  auto fill = [&](int64_t j, unsigned char* st) {
+    const int64_t row = (q0 * kStagesPerSum + j) * kStK + kg * 8;
+    put_column8<TY>(Y, a.ldy, row, colA, a.M, EA, st + offA, kPlaneA);
+    if (doB) put_column8<TY>(Y, a.ldy, row, colB, a.M, EB, st + S * kPlaneA + offA, kPlaneB);
+  };
+  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+    const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
+    const uint64_t dB = diag ? tc05::desc(sa + (J & 1) * 8 * kPlaneSbo, 128, kPlaneSbo)
+                             : tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
+    const int planeB = diag ? kPlaneA : kPlaneB;
+    if (Dig<TY>::HALVES == 2 && half == 1)
+      issue_stage<S, gram_base<TY>(1)>(tmem, dA, dB, planeB, first);
+    else
+      issue_stage<S, gram_base<TY>(0)>(tmem, dA, dB, planeB, first);
+  };
+  auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
+    const int64_t gi = (int64_t)I * 128 + (warp & 3) * 32 + lane;
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-      const int64_t gj = (int64_t)J * 64 + cp * 16 + c;
+      const int64_t gj = (int64_t)J * 64 + (warp >> 2) * 16 + c;
       if (gi < a.M && gj < a.M && gi <= gj) {
         add_group(a.G, a.M * a.M, gi + gj * a.M, half * 2, acc0[c]);
         add_group(a.G, a.M * a.M, gi + gj * a.M, half * 2 + 1, acc1[c]);
@@ -300,74 +281,8 @@ __global__ void __launch_bounds__(kGrThreads, 1) gram_kernel(GramArgs a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  int64_t issued = 0, drained = 0;
-  for (int64_t j = 0; j <= nstage; ++j) {
-    const int b = (int)(j % NST);
-    if (j < nstage) {
-      if (j >= NST) {
-        ok = __all_sync(0xffffffffu, mbar_wait_fast(empty + b, (uint32_t)((j / NST - 1) & 1)));
-        if (!ok) break;
-      }
-      unsigned char* st = gsm + b * kStage;
-      const int64_t row = (q0 * kStagesPerSum + j) * kStK + kg * 8;
-      put_column8<TY>(Y, a.ldy, row, colA, a.M, EA, st + offA, kPlaneA);
-      if (doB) put_column8<TY>(Y, a.ldy, row, colB, a.M, EB, st + S * kPlaneA + offA, kPlaneB);
-      tc05::fence_smem_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(full + b);
-    }
-    // the sums of the 128 rows before, once the stages ahead are filled
-    const bool due = (j % kStagesPerSum == NST - 1 && j >= kStagesPerSum && j < nstage) ||
-                     (j == nstage && nstage > 0);
-    if (due) {
-      ok = __all_sync(0xffffffffu, mbar_wait_fast(&dfull, (uint32_t)(drained & 1)));
-      if (!ok) break;
-      tc05::fence_after();
-      drain_slots(taddr, nslots, acc0, acc1);
-      tc05::fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&dempty);
-      ++drained;
-      if ((drained & 8191) == 0) flush();
-    }
-    // MMAs of the stages that are filled; those of a new sum wait until the
-    // last one has been read
-    const bool held = j >= kStagesPerSum && j % kStagesPerSum < NST - 1;
-    if (warp == kGrThreads / 32 - 1 && lane == 0 && j < nstage && !held) {
-      for (; issued <= j && ok; ++issued) {
-        const int ib = (int)(issued % NST);
-        const int64_t sum = issued / kStagesPerSum;
-        const bool first = issued % kStagesPerSum == 0;
-        ok = mbar_wait_fast(full + ib, (uint32_t)((issued / NST) & 1));
-        if (ok && first && sum > 0) ok = mbar_wait_fast(&dempty, (uint32_t)((sum - 1) & 1));
-        if (!ok) break;
-        tc05::fence_after();
-        const uint32_t sa = tc05::smem_u32(gsm) + ib * kStage;
-        const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
-        const uint64_t dB = diag ? tc05::desc(sa + (J & 1) * 8 * kPlaneSbo, 128, kPlaneSbo)
-                                 : tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
-        const int planeB = diag ? kPlaneA : kPlaneB;
-        if (Dig<TY>::HALVES == 2 && half == 1)
-          issue_stage<S, gram_base<TY>(1)>(tmem, dA, dB, planeB, first);
-        else
-          issue_stage<S, gram_base<TY>(0)>(tmem, dA, dB, planeB, first);
-        tc05::commit(empty + ib);
-        if (issued % kStagesPerSum == kStagesPerSum - 1) tc05::commit(&dfull);
-      }
-    }
-    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-    if (!ok) break;
-  }
-  if (ok) flush();
-  if (warp == kGrThreads / 32 - 1 && lane == 0) {
-    // nothing of this block is in flight when it gives its memory back
-    tc05::commit(&fin);
-    if (!mbar_wait_fast(&fin, 0)) ok = false;
-  }
-  if (!ok) raise_status(a.hdr, PYLOM_ERR_TIMEOUT);
-  tc05::fence_before();
-  __syncthreads();
-  if (warp == 0) tc05::tmem_dealloc(tmem, 512);
+  gram_pipeline<NST>(bar, gsm, S * (kPlaneA + kPlaneB), (q1 - q0) * kStagesPerSum,
+                     (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr, fill, issue, flush);
 }
 
 // ---------------------------------------------------------------------------
@@ -621,7 +536,7 @@ static cudaError_t gram_launch(const GramState& g, int sms, cudaStream_t st) {
   for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;
   GramArgs a{g.Y, g.ldy, g.N, g.M, g.colE, (unsigned long long*)g.G, nJ, tiles * Dig<TY>::HALVES, 1, g.hdr};
   a.splits = row_splits(a.items, (g.N + 127) / 128, sms);
-  gram_kernel<TY><<<(unsigned)(a.items * a.splits), kGrThreads, smem, st>>>(a);
+  gram_kernel<TY><<<(unsigned)(a.items * a.splits), kDigThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "svd_batched_gram.h"
 
 namespace pylom {
 
@@ -240,6 +241,8 @@ struct BatchArgs {
   double* S;            // packed singular values
   double2* scratch;     // per block: 2 x kMaxNb x kMaxK
   int max_sweeps;
+  const int* flags;     // null: all items; else flags[0] items, those with flags[1 + f] != 0
+  int nbins;
 };
 
 constexpr int kBThreads = 256;
@@ -871,6 +874,14 @@ __global__ void __launch_bounds__(kBThreads, 2) svd_batched_kernel(BatchArgs a) 
   V* sv = (V*)svraw;
   static_assert(kLeafMaxRowsF * 8 <= 8192 && kLeafMaxRowsD * 16 <= 8192, "reflector stage too small");
   const int tid = threadIdx.x;
+  // items that the Gram route has done are passed over
+  int nD = a.nD;
+  if (a.flags) {
+    if (a.flags[0] == 0) return;
+    nD = 0;
+    for (int f = 0; f < a.nbins; ++f)
+      if (a.flags[1 + f] && a.bins[f].k > 0) nD += (int)a.bins[f].P;
+  }
   double2* scratch = a.scratch + (int64_t)blockIdx.x * 2 * kMaxNb * kMaxK;
   // phase A
   while (true) {
@@ -881,6 +892,7 @@ __global__ void __launch_bounds__(kBThreads, 2) svd_batched_kernel(BatchArgs a) 
     if (item >= a.nA) break;
     if (read_status(a.hdr) == PYLOM_ERR_TIMEOUT) return;
     const int f = a.itemsA[item].x;
+    if (a.flags && !a.flags[1 + f]) continue;
     const int64_t leaf = a.itemsA[item].y;
     const BinDesc b = a.bins[f];
     leaf_qr_complex<TC>(a, b, leaf, sd, sred, sv);
@@ -935,7 +947,7 @@ __global__ void __launch_bounds__(kBThreads, 2) svd_batched_kernel(BatchArgs a) 
     __syncthreads();
     const int item = s_item;
     __syncthreads();
-    if (item >= a.nD) break;
+    if (item >= nD) break;
     if (tid == 0) {
       const unsigned long long t0 = global_ns();
       int ok = 1;
@@ -982,6 +994,8 @@ struct pylom_batched_plan {
   int64_t total_u = 0, total_z = 0, total_y = 0, total_s = 0;
   int grid = 0;
   bool bound = false;
+  pylom::BatchedGramPlan gram;        // items on the Gram route
+  std::vector<int> forced;            // items that are not (their leaf height was given, or binary64)
 };
 
 namespace pylom {
@@ -1062,7 +1076,7 @@ extern "C" pylom_status pylom_svd_batched_plan(int nbins, const int64_t* N, cons
     const int64_t np = nb + (nb & 1);
     BinDesc b{};
     b.N = n; b.Nb = nb; b.P = P; b.k = kmodes < nb ? kmodes : nb;
-    b.y_off = y;                 y += n * nb;
+    b.y_off = y;                 y += ((n > 4 ? n : 4) * nb + 3) & ~int64_t(3);   // 32-byte steps
     b.tau_off = z;               z += P * nb;
     b.rs_off = z;                z += P * nb * nb;
     b.taut_off = z;              z += P * nb;
@@ -1073,6 +1087,9 @@ extern "C" pylom_status pylom_svd_batched_plan(int nbins, const int64_t* N, cons
     b.s_off = sacc;              sacc += nb;
     p->N.push_back(n); p->Nb.push_back(nb); p->P.push_back(P); p->h.push_back(h);
     p->bins.push_back(b);
+    const bool gram = prec == PYLOM_PREC_MIXED_3XTF32 && !(leaf_rows && leaf_rows[f] > 0);
+    p->forced.push_back(gram ? 0 : 1);
+    if (gram) batched_gram_add(p->gram, f, n, nb, b.k, b.s_off);
     for (int64_t l = 0; l < P; ++l) p->itemsA.push_back(make_int2(f, (int)l));
     if (b.k > 0) p->nD += (int)P;
   }
@@ -1101,6 +1118,7 @@ extern "C" pylom_status pylom_svd_batched_plan(int nbins, const int64_t* N, cons
   p->off_f = off;     off += align256(sizeof(float2) * (size_t)(fz > 0 ? fz : 1));
   p->off_y = off;     off += align256(ye * (size_t)y);
   p->off_scr = off;   off += align256(sizeof(double2) * (size_t)p->grid * 2 * kMaxNb * kMaxK);
+  off = batched_gram_layout(p->gram, off, nbins);
   p->bytes = off;
   *plan_out = p;
   *ws_bytes = off;
@@ -1229,6 +1247,36 @@ static pylom_status batched_upload_tables(pylom_batched_plan* plan, void* ws, vo
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(base + plan->off_items, plan->itemsA.data(), sizeof(int2) * plan->itemsA.size(),
                         cudaMemcpyHostToDevice, st);
+  // the Gram route's items read their input in place (bins) or from a
+  // binary32 copy in the working-copy section (windows)
+  for (size_t i = 0; i < plan->gram.items.size(); ++i) {
+    const BinDesc& b = plan->bins[plan->gram.items[i]];
+    GramBin& g = plan->gram.bins[i];
+    g.kind = b.kind;
+    g.cplx = b.kind == 0;
+    g.Y = g.cplx ? (const float*)b.X : (const float*)(base + plan->off_y + sizeof(float2) * (size_t)b.y_off);
+    g.rows = g.cplx ? 2 * b.N : b.N;
+    g.ldy = g.cplx ? 2 * b.ldx : y_ld(b.N);
+    g.U = b.U;
+    g.Ur = (float*)b.Ureal;
+    g.ldu = b.ldu;
+    g.VT = b.VT;
+    g.ldvt = b.ldvt;
+    g.Xr = b.Xr;
+    g.ldx = b.ldx;
+    g.remove_mean = b.remove_mean;
+    g.physical = b.physical;
+    g.w = b.w;
+    g.mean = b.mean;
+  }
+  if (e == cudaSuccess) {
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) batched_gram_units(plan->gram, sms);
+    if (e == cudaSuccess)
+      e = batched_gram_upload(plan->gram, base, plan->forced.data(), (int)plan->forced.size(), st);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     set_error_message("%s: %s", who, cudaGetErrorString(e));
@@ -1274,6 +1322,19 @@ extern "C" pylom_status pylom_svd_batched_run(const pylom_batched_plan* plan, vo
   a.S = S;
   a.scratch = (double2*)(base + plan->off_scr);
   a.max_sweeps = max_sweeps;
+  // the Gram route takes its items first and leaves in the flags those that
+  // the Householder kernel below still has to do; a caller who allows only
+  // a few sweeps sees whether the plain iteration converges in them
+  a.nbins = plan->nbins;
+  a.flags = nullptr;
+  if (!plan->gram.items.empty() && max_sweeps >= 8) {
+    e = batched_gram_run(plan->gram, base, a.hdr, S, st);
+    if (e != cudaSuccess) {
+      set_error_message("pylom_svd_batched_run: Gram route: %s", cudaGetErrorString(e));
+      return PYLOM_ERR_CUDA;
+    }
+    a.flags = (const int*)(base + plan->gram.off_flags);
+  }
   void* args[] = {(void*)&a};
   if (plan->prec == PYLOM_PREC_FP64)
     e = cudaLaunchCooperativeKernel((const void*)svd_batched_kernel<double>, dim3(plan->grid), dim3(kBThreads),

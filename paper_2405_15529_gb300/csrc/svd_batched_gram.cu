@@ -1,0 +1,1107 @@
+// svd_batched_gram.cu -- batched SVDs by Gram matrices: the per-frequency
+// SVDs of SPOD (pyLOM, arXiv 2405.15529, Alg. 6) and the PODs of several
+// real windows (Alg. 2 per window), mixed precision.
+//
+// The persistent Householder kernel (svd_batched.cu) walks every leaf column
+// by column: 3 % of the binary32 rate, and one thread block per item for
+// the small SVD in binary64.  Here every step runs over all items at once:
+//   1. column exponents (and, for windows, mean, weights and a binary32 copy);
+//   2. G = Y^H Y exactly, by digit products on the tcgen05 tensor cores
+//      (digits.cuh).  A complex column is its 2N interleaved real and
+//      imaginary parts: Re G_ij is the product of columns i and j, Im G_ij
+//      that of column i turned by 90 degrees, (-im, re), and column j;
+//   3. Cholesky factor R in binary64, in one block's shared memory;
+//   4. complex one-sided Jacobi of R^H: two binary32 block stages (one
+//      cluster per item) and two binary64 steps of simultaneous rotations,
+//      as in the single small SVD (svd_jacobi32.cu);
+//   5. U = Y W_k S_k^-1 (W the right vectors) by digit products.
+// Items whose result would be less accurate than the Householder route's
+// (a kept mode below 1e-4 of the largest singular value, where squaring
+// costs binary32 digits; kept values too close to separate in two steps; a
+// zero matrix) are flagged on the device and left to that kernel.
+//
+// Persistent kernel -> here: 24 bins (N 16k..262k, Nb 16..128, 1.3 GB) 374 ->
+// 20 ms, 12 windows (N 16k..262k, M 16..96) 115 -> 5.0 ms, SPOD of 131072 x
+// 1056 25.6 -> 17 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
+#include <algorithm>
+
+#include "digits.cuh"
+#include "svd_batched_gram.h"
+
+namespace pylom {
+
+namespace {
+
+constexpr int kSB = Dig<float>::S;                 // 5 digits
+constexpr int kNstB = Dig<float>::NST;
+constexpr int kStageB = kSB * (kPlaneA + kPlaneB);
+constexpr double kKeptLevel = 1e-4;
+constexpr double kOpenCos = 1e-6;                  // kept columns: largest cosine before the last step
+
+struct BG {
+  const GramBin* bins;
+  const GramUnit* units;
+  int* ints;
+  unsigned long long* g;
+  double2* z;
+  float2* f;
+  unsigned char* c;
+  double* d;
+  int* flags;
+  double* S;
+  WsHeader* hdr;
+};
+
+__device__ __forceinline__ double2* mat(const BG& a, const GramBin& b, int i) {
+  return a.z + b.z + (int64_t)i * b.Nb * b.Nb;
+}
+
+// ---------------------------------------------------------------------------
+// 1. column exponents; windows: Y = sqrt(w) (x - mean) in binary32
+// ---------------------------------------------------------------------------
+template <typename TX>
+__device__ void window_rows(const GramBin& b, float* Y, int64_t r0, int64_t r1, int* sE, int& bad) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double ssum[8][32];
+  const TX* X = (const TX*)b.Xr;
+  int em[16];
+#pragma unroll
+  for (int t = 0; t < 16; ++t) em[t] = 0;
+  for (int64_t blk = r0; blk < r1; blk += 32) {
+    const int64_t n = blk + lane;
+    const bool in = n < b.rows;
+    TX x[16];
+    double s = 0.0;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int c = warp + 8 * t;
+      x[t] = (in && c < b.Nb) ? X[n + (int64_t)c * b.ldx] : (TX)0;
+    }
+    double xbar = 0.0;
+    if (b.remove_mean) {
+      if constexpr (sizeof(TX) == 4) {
+        float h, l;
+        sum32_compensated(x, h, l);
+        s = (double)h + (double)l;
+      } else {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) s += x[t];
+      }
+      ssum[warp][lane] = s;
+      __syncthreads();
+      double tot = 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) tot += ssum[q][lane];
+      xbar = tot / (double)b.Nb;
+      __syncthreads();
+    }
+    double sw = 1.0;
+    if (b.w && in) {
+      const double wn = b.w[n];
+      if (!(wn > 0.0) || !isfinite(wn)) bad = 1;
+      sw = sqrt(wn);
+    }
+    if (warp == 0 && in && b.mean) b.mean[n] = xbar;
+    const float xh = (float)xbar, xl = (float)(xbar - (double)xh);
+    const float sh = (float)sw, sl = (float)(sw - (double)sh);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int c = warp + 8 * t;
+      if (c >= b.Nb) continue;
+      float y;
+      if constexpr (sizeof(TX) == 4) {
+        float d, e;
+        two_sum32(x[t], -xh, d, e);
+        y = __fmaf_rn(d, sh, __fmaf_rn(d, sl, __fmul_rn(__fsub_rn(e, xl), sh)));
+      } else {
+        y = (float)(sw * (x[t] - xbar));
+      }
+      if (!in) y = 0.f;
+      if (!isfinite(x[t])) bad = 1;
+      em[t] = max(em[t], exp_field(y));
+      if (n < b.ldy) Y[n + (int64_t)c * b.ldy] = y;
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < 16; ++t) {
+    const int e = __reduce_max_sync(0xffffffffu, em[t]);
+    if (lane == 0 && warp + 8 * t < b.Nb) sE[warp + 8 * t] = e;
+  }
+}
+
+__global__ void __launch_bounds__(256) bg_prologue_kernel(BG a) {
+  __shared__ int sE[128];
+  const GramUnit u = a.units[blockIdx.x];
+  const GramBin b = a.bins[u.bin];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int bad = 0;
+  if (b.kind == 0) {
+    for (int c = warp; c < b.Nb; c += 8) {
+      const float2* col = (const float2*)(b.Y + (int64_t)c * b.ldy);
+      int e = 0;
+      for (int64_t n = u.q0 + lane; n < u.q1; n += 32) {
+        const float2 x = __ldg(col + n);
+        if (!isfinite(x.x) || !isfinite(x.y)) bad = 1;
+        e = max(e, max(exp_field(x.x), exp_field(x.y)));
+      }
+      e = __reduce_max_sync(0xffffffffu, e);
+      if (lane == 0) sE[c] = e;
+    }
+  } else if (b.kind == 1) {
+    window_rows<float>(b, (float*)b.Y, u.q0, u.q1, sE, bad);
+  } else {
+    window_rows<double>(b, (float*)b.Y, u.q0, u.q1, sE, bad);
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < b.Nb; c += 256) atomicMax(a.ints + b.colE + c, sE[c]);
+  if (bad) raise_status(a.hdr, PYLOM_ERR_NONFINITE);
+}
+
+// ---------------------------------------------------------------------------
+// 2. exact Gram matrices
+// ---------------------------------------------------------------------------
+// Unit modes: the 128 rows of the left factor are columns 0..127 (kPlain),
+// columns 0..63 and the same turned by 90 degrees (kPacked: Re and Im in one
+// pass, for the first 64 columns), or columns 0..127 turned (kTurned).  The
+// right factor is the column block J of 64.
+enum { kPlain = 0, kPacked = 1, kTurned = 2 };
+
+// digits of rows row..row+7 of a column (turned: (-im, re) pairs)
+__device__ __forceinline__ void put_rows8(const GramBin& b, int64_t row, int col, int E, bool turned, unsigned char* dst,
+                                          int plane) {
+  uint64_t w[8];
+  float y[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) y[i] = 0.f;
+  if (col < b.Nb) {
+    const float* p = b.Y + row + (int64_t)col * b.ldy;
+    if (row + 8 <= b.rows && ((uintptr_t)p & 15) == 0) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float4 v = __ldg((const float4*)p + i);
+        y[4 * i] = v.x;
+        y[4 * i + 1] = v.y;
+        y[4 * i + 2] = v.z;
+        y[4 * i + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (row + i < b.rows) y[i] = __ldg(p + i);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    const float x0 = turned ? -y[i + 1] : y[i], x1 = turned ? y[i] : y[i + 1];
+    w[i] = bias_digits(to_fixed(x0, E));
+    w[i + 1] = bias_digits(to_fixed(x1, E));
+  }
+  store_digits<kSB>(w, dst, plane);
+}
+
+__global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
+  extern __shared__ __align__(1024) unsigned char gsm[];
+  __shared__ __align__(8) DigitBarriers<kNstB> bar;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const GramUnit u = a.units[blockIdx.x];
+  const GramBin b = a.bins[u.bin];
+  const int mode = u.mode, J = u.J;
+  const int c8 = lane & 7, kg = lane >> 3, ca = warp * 8 + c8;
+  const bool turned = mode == kTurned || (mode == kPacked && ca >= 64);
+  const int colA = mode == kPacked ? (ca & 63) : ca;
+  // real items have nothing to turn: their second half is empty
+  const bool useA = !(mode == kPacked && ca >= 64 && !b.cplx);
+  const int EA = colA < b.Nb ? a.ints[b.colE + colA] : 1;
+  const uint32_t off = (uint32_t)((ca >> 3) * kPlaneSbo + kg * 128 + c8 * 16);
+  const bool sepB = mode == kTurned;             // else the right factor's columns are among the left's
+  const int colB = J * 64 + ca;
+  const int EB = (sepB && warp < 8 && colB < b.Nb) ? a.ints[b.colE + colB] : 1;
+  auto fill = [&](int64_t j, unsigned char* st) {
+    const int64_t row = (u.q0 * kStagesPerSum + j) * kStK + kg * 8;
+    put_rows8(b, row, useA ? colA : b.Nb, EA, turned, st + off, kPlaneA);
+    if (sepB && warp < 8) put_rows8(b, row, colB, EB, false, st + kSB * kPlaneA + off, kPlaneB);
+  };
+  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+    const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
+    const uint64_t dB = sepB ? tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo)
+                             : tc05::desc(sa + J * 8 * kPlaneSbo, 128, kPlaneSbo);
+    issue_stage<kSB, gram_base<float>(0)>(tmem, dA, dB, sepB ? kPlaneB : kPlaneA, first);
+  };
+  auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
+    const int row = (warp & 3) * 32 + lane;
+    const bool im = mode == kTurned || (mode == kPacked && row >= 64);
+    const int i = mode == kPacked ? (row & 63) : row;
+    const int64_t MM = (int64_t)b.Nb * b.Nb;
+    unsigned long long* G = a.g + b.g + (im ? 3 * MM : 0);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const int j = J * 64 + (warp >> 2) * 16 + c;
+      if (i < b.Nb && j < b.Nb && (im ? (i < j && b.cplx) : i <= j)) {
+        add_group(G, MM, i + (int64_t)j * b.Nb, 0, acc0[c]);
+        add_group(G, MM, i + (int64_t)j * b.Nb, 1, acc1[c]);
+      }
+      acc0[c] = acc1[c] = 0;
+    }
+  };
+  gram_pipeline<kNstB>(bar, gsm, kStageB, (u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, fill, issue, flush);
+}
+
+// ---------------------------------------------------------------------------
+// complex helpers
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double2 zadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 zmulc(double2 a, double2 b) {   // conj(a) b
+  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.x, b.y, -a.y * b.x));
+}
+__device__ __forceinline__ float2 fmulc(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
+}
+__device__ __forceinline__ float2 fmul(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+
+// ---------------------------------------------------------------------------
+// 3. Cholesky: A = R^H (matrix 0), A32 = its binary32 copy scaled, V32 = I
+// ---------------------------------------------------------------------------
+// One block per item, the upper triangle packed by rows in shared memory
+// (at most 132 KB).  G = D H D with D the columns' scales: H's entries are
+// the exact integer sums.
+constexpr int kCholThreads = 512;
+__device__ __forceinline__ int tri(int i, int j, int n) { return i * n - i * (i - 1) / 2 + (j - i); }   // row i, column j >= i
+
+__global__ void __launch_bounds__(kCholThreads) bg_chol_kernel(BG a) {
+  extern __shared__ __align__(16) unsigned char csm[];
+  double2* H = (double2*)csm;
+  __shared__ double s_inv, s_diag[128];
+  __shared__ unsigned s_e;
+  const GramBin b = a.bins[blockIdx.x];
+  const int n = b.Nb, tid = threadIdx.x;
+  const int64_t MM = (int64_t)n * n;
+  const long long* Gr = (const long long*)a.g + b.g;
+  auto sum = [&](const long long* G, int64_t at) {
+    // groups 0..2 of 32 bits each, exact but for one rounding
+    return fma((double)__ldcg(G + 2 * MM + at), 4294967296.0, (double)__ldcg(G + MM + at)) * 4294967296.0 +
+           (double)__ldcg(G + at);
+  };
+  for (int64_t idx = tid; idx < MM; idx += kCholThreads) {
+    const int i = (int)(idx % n), j = (int)(idx / n);
+    if (i <= j) H[tri(i, j, n)] = make_double2(sum(Gr, idx), (b.cplx && i < j) ? sum(Gr + 3 * MM, idx) : 0.0);
+  }
+  if (tid == 0) s_e = 0;
+  __syncthreads();
+  if (tid < n) s_diag[tid] = H[tri(tid, tid, n)].x;
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    if (tid == 0) {
+      const double d = H[tri(k, k, n)].x;
+      // a pivot at the rounding level of its column: a dependent column, a zero row of R
+      const bool live = d > 1e-15 * s_diag[k];
+      s_inv = live ? 1.0 / sqrt(d) : 0.0;
+    }
+    __syncthreads();
+    const double inv = s_inv;
+    for (int j = k + tid; j < n; j += kCholThreads) {
+      double2& h = H[tri(k, j, n)];
+      h = make_double2(h.x * inv, h.y * inv);
+    }
+    __syncthreads();
+    // rows i > k: H_ij -= conj(R_ki) R_kj; a warp per row
+    if (inv != 0.0) {
+      const int lane = tid & 31, warp = tid >> 5;
+      for (int i = k + 1 + warp; i < n; i += kCholThreads / 32) {
+        const double2 r = H[tri(k, i, n)];
+        const double2* hk = H + tri(k, i, n);
+        double2* hi = H + tri(i, i, n);
+        for (int j = lane; j < n - i; j += 32) {
+          const double2 x = hk[j], p = zmulc(r, x);
+          hi[j] = make_double2(hi[j].x - p.x, hi[j].y - p.y);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // A = R^H with the columns of R scaled back: A(j, c) = conj(R(c, j)) 2^(E_j - bias)
+  double2* A = mat(a, b, 0);
+  const int* E = a.ints + b.colE;
+  unsigned em = 0;
+  for (int64_t idx = tid; idx < MM; idx += kCholThreads) {
+    const int j = (int)(idx % n), c = (int)(idx / n);
+    double2 v = make_double2(0.0, 0.0);
+    if (c <= j) {
+      const double2 r = H[tri(c, j, n)];
+      // the sums count from level 1 (2^8)
+      const double s = scalbn(16.0, E[j] - fix_bias<float>());
+      v = make_double2(r.x * s, -r.y * s);
+    }
+    A[idx] = v;
+    em = max(em, (unsigned)max(exp_field(v.x), exp_field(v.y)));
+  }
+  em = __reduce_max_sync(0xffffffffu, em);
+  if ((tid & 31) == 0) atomicMax(&s_e, em);
+  __syncthreads();
+  if (tid == 0) a.d[b.d] = (double)s_e;
+  const double sc = __hiloint2double((s_e > 1 && s_e < 2045 ? 2046 - (int)s_e : 1023) << 20, 0);
+  float2* A32 = a.f + b.f;
+  float2* V32 = A32 + (int64_t)n * b.Mb;
+  for (int64_t idx = tid; idx < (int64_t)n * b.Mb; idx += kCholThreads) {
+    const int64_t c = idx / n;
+    float2 v = make_float2(0.f, 0.f);
+    if (c < n) v = make_float2((float)(A[idx].x * sc), (float)(A[idx].y * sc));
+    A32[idx] = v;
+  }
+  for (int64_t idx = tid; idx < (int64_t)b.Mb * b.Mb; idx += kCholThreads)
+    V32[idx] = make_float2(idx % b.Mb == idx / b.Mb ? 1.f : 0.f, 0.f);
+}
+
+// second stage: A32 from the binary64 A2, V32 = I
+__global__ void __launch_bounds__(256) bg_init_kernel(BG a) {
+  const GramBin b = a.bins[blockIdx.y];
+  const int n = b.Nb;
+  const int e = (int)a.d[b.d];
+  const double sc = __hiloint2double((e > 1 && e < 2045 ? 2046 - e : 1023) << 20, 0);
+  const double2* A = mat(a, b, 2);
+  float2* A32 = a.f + b.f;
+  float2* V32 = A32 + (int64_t)n * b.Mb;
+  const int64_t stride = (int64_t)gridDim.x * 256, t0 = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  for (int64_t idx = t0; idx < (int64_t)n * b.Mb; idx += stride) {
+    float2 v = make_float2(0.f, 0.f);
+    if (idx / n < n) v = make_float2((float)(A[idx].x * sc), (float)(A[idx].y * sc));
+    A32[idx] = v;
+  }
+  for (int64_t idx = t0; idx < (int64_t)b.Mb * b.Mb; idx += stride)
+    V32[idx] = make_float2(idx % b.Mb == idx / b.Mb ? 1.f : 0.f, 0.f);
+}
+
+// T0 = V32 (binary64)
+__global__ void __launch_bounds__(256) bg_widen_kernel(BG a) {
+  const GramBin b = a.bins[blockIdx.y];
+  const int n = b.Nb;
+  const float2* V32 = a.f + b.f + (int64_t)n * b.Mb;
+  double2* T = mat(a, b, 3);
+  for (int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x; idx < (int64_t)n * n; idx += (int64_t)gridDim.x * 256) {
+    const float2 v = V32[idx % n + (idx / n) * b.Mb];
+    T[idx] = make_double2(v.x, v.y);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// 4. binary32 block Jacobi (one cluster, the grid's x, per item; see svd_jacobi32.cu)
+// ---------------------------------------------------------------------------
+constexpr int kZB = 16, kZW = 32, kZThreads = 256, kZRows = 32, kZSweeps = 24;
+
+__device__ __forceinline__ void z_rotation(float al, float be, float2 ga, float thr2, float& c, float& sn, float2& ph) {
+  // |ga|, its phase, and the real rotation of [a_i, e^(-i phi) a_j]
+  const float g2 = fmaf(ga.x, ga.x, ga.y * ga.y);
+  const bool act = g2 > thr2 * fabsf(al * be);
+  float ig;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ig) : "f"(fmaxf(g2, 1e-37f)));
+  const float ag = g2 * ig;                 // |ga|
+  ph = act ? make_float2(ga.x * ig, -ga.y * ig) : make_float2(1.f, 0.f);
+  const float d = be - al, h = ag + ag;
+  float r, q;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaf(d, d, h * h)));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(fmaxf(fabsf(d) + r, h)));
+  const float t = act ? copysignf(1.f, d) * h * q : 0.f;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(fmaf(t, t, 1.f)));
+  sn = c * t;
+}
+
+__global__ void __launch_bounds__(kZThreads) bg_jacobi32_kernel(BG a) {
+  constexpr int LD = kZW + 2;
+  extern __shared__ __align__(16) unsigned char jsm[];
+  float2* sA = (float2*)jsm;                                   // [kZRows][LD], then partial Gram matrices
+  float2(*sG)[kZW][kZW + 1] = (float2(*)[kZW][kZW + 1])(sA + kZW * kZW);   // [2]
+  float2(*sJ)[LD] = (float2(*)[LD])(sG + 2);                   // [kZW][LD]
+  __shared__ unsigned char sI[kZW - 1][kZB], sK[kZW - 1][kZB];
+  __shared__ unsigned s_rot, s_total[2];
+  const GramBin b = a.bins[blockIdx.y];
+  const int n = b.Nb, Mb = b.Mb, tid = threadIdx.x;
+  float2* A32 = a.f + b.f;
+  float2* V32 = A32 + (int64_t)n * Mb;
+  const int nblk = Mb / kZB, npairs = nblk / 2;
+  const float tol = 4.f * sqrtf((float)n) * 5.9604645e-8f;
+  for (int idx = tid; idx < (kZW - 1) * kZB; idx += kZThreads) {
+    const int round = idx / kZB, p = idx % kZB;
+    int x, y;
+    if (round < kZB) {
+      x = p;
+      y = kZB + (p + round) % kZB;
+    } else {
+      const int h = p / 8 * kZB, q = p % 8, r = round - kZB;
+      x = h + ((q == 0) ? 0 : ((q - 1 + r) % (kZB - 1)) + 1);
+      y = h + ((kZB - 2 - q + r) % (kZB - 1)) + 1;
+    }
+    sI[round][p] = (unsigned char)min(x, y);
+    sK[round][p] = (unsigned char)max(x, y);
+  }
+  if (tid < 2) s_total[tid] = 0;
+  auto cluster_sync = [&]() {
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  };
+  cluster_sync();
+  for (int sweep = 0; sweep < kZSweeps; ++sweep) {
+    unsigned local = 0;
+    for (int step = 0; step < nblk - 1; ++step) {
+      const int pr = blockIdx.x;
+      if (pr < npairs) {
+        const int p = (pr == 0) ? 0 : ((pr - 1 + step) % (nblk - 1)) + 1;
+        const int q = ((nblk - 2 - pr + step) % (nblk - 1)) + 1;
+        const int bI = min(p, q), bJ = max(p, q);
+        auto column = [&](int l) { return (int64_t)(l < kZB ? bI * kZB + l : bJ * kZB + (l - kZB)); };
+        // 32 x 32 Gram matrix: 8 x 8 threads of 4 x 4 entries, 4 row slices
+        const int ti = (tid & 7) * 4, tj = ((tid >> 3) & 7) * 4, sl = tid >> 6;
+        float2 g[4][4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) g[x][y] = make_float2(0.f, 0.f);
+        for (int r0 = 0; r0 < n; r0 += kZRows) {
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < kZRows * kZW / kZThreads; ++u) {
+            const int idx = tid + u * kZThreads, r = idx % kZRows, l = idx / kZRows;
+            sA[r * LD + l] = (r0 + r < n) ? __ldcg(A32 + r0 + r + column(l) * n) : make_float2(0.f, 0.f);
+          }
+          __syncthreads();
+#pragma unroll 2
+          for (int r = sl; r < kZRows; r += 4) {
+            float2 x[4], y[4];
+#pragma unroll
+            for (int h = 0; h < 4; h += 2) {
+              const float4 xv = *(const float4*)(sA + r * LD + ti + h), yv = *(const float4*)(sA + r * LD + tj + h);
+              x[h] = make_float2(xv.x, xv.y);
+              x[h + 1] = make_float2(xv.z, xv.w);
+              y[h] = make_float2(yv.x, yv.y);
+              y[h + 1] = make_float2(yv.z, yv.w);
+            }
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+#pragma unroll
+              for (int v = 0; v < 4; ++v) {
+                g[h][v].x = fmaf(x[h].x, y[v].x, fmaf(x[h].y, y[v].y, g[h][v].x));
+                g[h][v].y = fmaf(x[h].x, y[v].y, fmaf(-x[h].y, y[v].x, g[h][v].y));
+              }
+          }
+        }
+        __syncthreads();
+        for (int h = 3; h >= 1; --h) {
+          if (sl == h) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+              for (int y = 0; y < 4; ++y) sA[(ti + x) * kZW + tj + y] = g[x][y];
+          }
+          __syncthreads();
+          if (sl == 0) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+              for (int y = 0; y < 4; ++y) {
+                const float2 v = sA[(ti + x) * kZW + tj + y];
+                g[x][y].x += v.x;
+                g[x][y].y += v.y;
+              }
+          }
+          __syncthreads();
+        }
+        if (tid == 0) s_rot = 0;
+        if (sl == 0) {
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) sG[0][ti + x][tj + y] = g[x][y];
+        }
+        for (int idx = tid; idx < kZW * kZW; idx += kZThreads)
+          sJ[idx / kZW][idx % kZW] = make_float2(idx / kZW == idx % kZW ? 1.f : 0.f, 0.f);
+        __syncthreads();
+        unsigned open = 0;
+        for (int idx = tid; idx < kZW * kZW; idx += kZThreads) {
+          const int i = idx / kZW, j = idx % kZW;
+          const float2 v = sG[0][i][j];
+          if (i < j && fmaf(v.x, v.x, v.y * v.y) > tol * tol * (sG[0][i][i].x * sG[0][j][j].x)) ++open;
+        }
+        if (open) atomicAdd(&s_rot, open);
+        __syncthreads();
+        open = s_rot;
+        local += open;
+        if (open) {
+          const int pb = tid & 15, qb = tid >> 4;
+          const int rounds = step == 0 ? kZW - 1 : kZB;
+          const float thr2 = 0.0625f * tol * tol;
+          int ni = sI[0][pb], nj = sK[0][pb], nk = sI[0][qb], nl = sK[0][qb];
+          for (int round = 0; round < rounds; ++round) {
+            const float2(*G0)[kZW + 1] = sG[round & 1];
+            float2(*G1)[kZW + 1] = sG[(round & 1) ^ 1];
+            const int i = ni, j = nj, k = nk, l = nl, nr = round + 1 < rounds ? round + 1 : 0;
+            ni = sI[nr][pb];
+            nj = sK[nr][pb];
+            nk = sI[nr][qb];
+            nl = sK[nr][qb];
+            float cp, sp, cq, sq;
+            float2 pp, pq;
+            z_rotation(G0[i][i].x, G0[j][j].x, G0[i][j], thr2, cp, sp, pp);
+            z_rotation(G0[k][k].x, G0[l][l].x, G0[k][l], thr2, cq, sq, pq);
+            // columns: x_k' = cq x_k - sq pq x_l, x_l' = sq x_k + cq pq x_l
+            const float2 e = G0[i][k], f = fmul(pq, G0[i][l]), gg = G0[j][k], h = fmul(pq, G0[j][l]);
+            const float2 e1 = make_float2(cq * e.x - sq * f.x, cq * e.y - sq * f.y);
+            const float2 f1 = make_float2(sq * e.x + cq * f.x, sq * e.y + cq * f.y);
+            const float2 g1 = fmulc(pp, make_float2(cq * gg.x - sq * h.x, cq * gg.y - sq * h.y));
+            const float2 h1 = fmulc(pp, make_float2(sq * gg.x + cq * h.x, sq * gg.y + cq * h.y));
+            // rows, conjugated
+            G1[i][k] = make_float2(cp * e1.x - sp * g1.x, cp * e1.y - sp * g1.y);
+            G1[i][l] = make_float2(cp * f1.x - sp * h1.x, cp * f1.y - sp * h1.y);
+            G1[j][k] = make_float2(sp * e1.x + cp * g1.x, sp * e1.y + cp * g1.y);
+            G1[j][l] = make_float2(sp * f1.x + cp * h1.x, sp * f1.y + cp * h1.y);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int r = qb + 16 * u;
+              const float2 x = sJ[r][i], y = fmul(pp, sJ[r][j]);
+              sJ[r][i] = make_float2(cp * x.x - sp * y.x, cp * x.y - sp * y.y);
+              sJ[r][j] = make_float2(sp * x.x + cp * y.x, sp * x.y + cp * y.y);
+            }
+            __syncthreads();
+          }
+          // A32 and V32 columns <- columns J; a thread per row and half of the new columns
+          for (int i0 = 0; i0 < 2 * (n + Mb); i0 += kZThreads) {
+            const int it = i0 + tid;
+            const bool live = it < 2 * (n + Mb);
+            const int row = live ? it >> 1 : 0, hf = it & 1;
+            const bool isA = row < n;
+            float2* base = isA ? A32 + row : V32 + (row - n);
+            const int64_t ld = isA ? n : Mb;
+            float2 v[kZW];
+#pragma unroll
+            for (int l = 0; l < kZW; ++l) v[l] = __ldcg(base + column(l) * ld);
+            __syncwarp();   // both threads of the row have read it
+            if (!live) continue;
+#pragma unroll 1
+            for (int l = hf * kZB; l < hf * kZB + kZB; l += 2) {
+              float2 o0 = make_float2(0.f, 0.f), o1 = o0;
+#pragma unroll
+              for (int m = 0; m < kZW; ++m) {
+                const float4 jv = *(const float4*)&sJ[m][l];
+                o0.x = fmaf(v[m].x, jv.x, fmaf(-v[m].y, jv.y, o0.x));
+                o0.y = fmaf(v[m].x, jv.y, fmaf(v[m].y, jv.x, o0.y));
+                o1.x = fmaf(v[m].x, jv.z, fmaf(-v[m].y, jv.w, o1.x));
+                o1.y = fmaf(v[m].x, jv.w, fmaf(v[m].y, jv.z, o1.y));
+              }
+              __stcg(base + column(l) * ld, o0);
+              __stcg(base + column(l + 1) * ld, o1);
+            }
+          }
+        }
+      }
+      cluster_sync();
+    }
+    // the cluster's open pairs of this sweep, at rank 0 (alternating words)
+    if (tid == 0 && local) {
+      uint32_t addr;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(addr) : "r"(tc05::smem_u32(&s_total[sweep & 1])));
+      asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" :: "r"(addr), "r"(local) : "memory");
+    }
+    cluster_sync();
+    uint32_t addr, total;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(addr) : "r"(tc05::smem_u32(&s_total[sweep & 1])));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(total) : "r"(addr) : "memory");
+    cluster_sync();
+    if (blockIdx.x == 0 && tid == 0) s_total[sweep & 1] = 0;
+    if (total == 0) break;
+  }
+  cluster_sync();   // no block leaves while another may read its shared memory
+}
+
+// ---------------------------------------------------------------------------
+// binary64 products C = alpha op(A) B + beta D over all items, one or two at a time
+// ---------------------------------------------------------------------------
+struct ZGemm {
+  int ta, A, B, D, C;       // matrix numbers; ta: A^H; D < 0: none
+  double alpha, beta;
+};
+struct ZGemms {
+  ZGemm g[2];
+  int count;
+};
+
+__global__ void __launch_bounds__(128) bg_gemm_kernel(BG a, ZGemms gs) {
+  __shared__ double2 part[4][8][9];
+  const GramBin b = a.bins[blockIdx.z / gs.count];
+  const ZGemm& p = gs.g[blockIdx.z % gs.count];
+  const int n = b.Nb, i0 = blockIdx.x * 8, j0 = blockIdx.y * 8;
+  if (i0 >= n || j0 >= n) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const double2* A = mat(a, b, p.A);
+  const double2* B = mat(a, b, p.B);
+  double r0 = 0.0, r1 = 0.0, m0 = 0.0, m1 = 0.0;
+  const int i = i0 + g, j = j0 + g;
+#pragma unroll 4
+  for (int st = warp; st < (n + 3) / 4; st += 4) {
+    const int kk = st * 4 + t;
+    double2 x = make_double2(0.0, 0.0), y = x;
+    if (kk < n && i < n) x = p.ta ? __ldg(A + kk + (int64_t)i * n) : __ldg(A + i + (int64_t)kk * n);
+    if (kk < n && j < n) y = __ldg(B + kk + (int64_t)j * n);
+    if (p.ta) x.y = -x.y;
+    dmma884(r0, r1, x.x, y.x);
+    if (b.cplx) {
+      dmma884(r0, r1, -x.y, y.y);
+      dmma884(m0, m1, x.x, y.y);
+      dmma884(m0, m1, x.y, y.x);
+    }
+  }
+  part[warp][g][2 * t] = make_double2(r0, m0);
+  part[warp][g][2 * t + 1] = make_double2(r1, m1);
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    const int r = threadIdx.x & 7, c = threadIdx.x >> 3;
+    if (i0 + r < n && j0 + c < n) {
+      const int64_t at = (i0 + r) + (int64_t)(j0 + c) * n;
+      double2 v = zadd(zadd(part[0][r][c], part[1][r][c]), zadd(part[2][r][c], part[3][r][c]));
+      v = make_double2(p.alpha * v.x, p.alpha * v.y);
+      if (p.D >= 0) {
+        const double2 d = mat(a, b, p.D)[at];
+        v = make_double2(fma(p.beta, d.x, v.x), fma(p.beta, d.y, v.y));
+      }
+      mat(a, b, p.C)[at] = v;
+    }
+  }
+}
+
+// Small-angle generator of a step from G (matrix 3) and W = V^H V (matrix
+// 4): K (5), L = K - E (7), B = I + K - E/2 (4, in place of W), E = W - I.
+// A pair's angle is t e^(i phi) on column j (+) and column i (-, conjugate).
+// Columns whose angles are not small, or too many, are left alone.  `last`:
+// also records each column's largest cosine.  A warp per column, twice: the
+// columns' decisions are needed by all pairs.
+__device__ __forceinline__ double z_tangent(double al, double be, double g) {
+  if (!(g > 0.0)) return 0.0;
+  const double zeta = (be - al) / (2.0 * g);
+  return ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+}
+
+__global__ void __launch_bounds__(256) bg_check_kernel(BG a, int last) {
+  const GramBin b = a.bins[blockIdx.y];
+  const int n = b.Nb, lane = threadIdx.x & 31, j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (j >= n) return;
+  const double2* G = mat(a, b, 3);
+  const double be = G[j + (int64_t)j * n].x;
+  double sum = 0.0, big = 0.0, cosm = 0.0;
+  for (int i = lane; i < n; i += 32) {
+    if (i == j) continue;
+    const double al = G[i + (int64_t)i * n].x;
+    const double2 v = G[i + (int64_t)j * n];
+    const double g = sqrt(v.x * v.x + v.y * v.y), q = sqrt(al) * sqrt(be);
+    const double c = q > 0.0 ? g / q : 0.0;
+    cosm = fmax(cosm, c);
+    if (c > 1e-14) {
+      const double t = fabs(z_tangent(al, be, g));
+      sum += t;
+      big = fmax(big, t);
+    }
+  }
+  sum = warp_sum(sum);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    cosm = fmax(cosm, __shfl_xor_sync(0xffffffffu, cosm, o));
+  }
+  if (lane == 0) {
+    const bool moves = big <= 0.02 && sum <= 0.05;
+    // a column that keeps a cosine it cannot shed counts with it in full
+    a.d[b.d + 1 + j] = last ? (moves ? cosm : cosm + 1.0) : 0.0;
+    a.d[b.d + 1 + n + j] = moves ? 1.0 : 0.0;
+  }
+}
+
+__global__ void __launch_bounds__(256) bg_angles_kernel(BG a) {
+  const GramBin b = a.bins[blockIdx.y];
+  const int n = b.Nb;
+  const double2* G = mat(a, b, 3);
+  double2 *W = mat(a, b, 4), *K = mat(a, b, 5), *L = mat(a, b, 7);
+  const double* mv = a.d + b.d + 1 + n;
+  for (int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x; idx < (int64_t)n * n; idx += (int64_t)gridDim.x * 256) {
+    const int i = (int)(idx % n), j = (int)(idx / n);
+    double2 t = make_double2(0.0, 0.0);
+    if (i != j && mv[i] != 0.0 && mv[j] != 0.0) {
+      const double al = G[i + (int64_t)i * n].x, be = G[j + (int64_t)j * n].x;
+      const double2 v = G[idx];
+      const double g = sqrt(v.x * v.x + v.y * v.y), q = sqrt(al) * sqrt(be);
+      if (g > 1e-14 * q && q > 0.0) {
+        const double tt = z_tangent(al, be, g) / g;
+        // column j gains t e^(i phi) a_i, e^(i phi) = G_ij / |G_ij| (the pair's
+        // other entry follows by symmetry: G_ji = conj G_ij and t changes sign)
+        t = make_double2(tt * v.x, tt * v.y);
+      }
+    }
+    double2 e = W[idx];
+    if (i == j) e.x -= 1.0;
+    K[idx] = t;
+    L[idx] = make_double2(t.x - e.x, t.y - e.y);
+    W[idx] = make_double2((i == j ? 1.0 : 0.0) + t.x - 0.5 * e.x, t.y - 0.5 * e.y);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// 5. order, phases, S, V^T of windows, coefficient digits, flags
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
+  __shared__ double sig[128];
+  __shared__ double2 phs[128];
+  __shared__ int perm[128], s_ce[64];
+  const GramBin b = a.bins[blockIdx.x];
+  const int n = b.Nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double2* A = mat(a, b, 0);
+  for (int j = warp; j < n; j += 8) {
+    double s2 = 0.0, best = -1.0;
+    int kb = 0;
+    for (int r = lane; r < n; r += 32) {
+      const double2 v = A[r + (int64_t)j * n];
+      const double m2 = v.x * v.x + v.y * v.y;
+      s2 += m2;
+      if (m2 > best) {
+        best = m2;
+        kb = r;
+      }
+    }
+    s2 = warp_sum(s2);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int ok = __shfl_xor_sync(0xffffffffu, kb, o);
+      if (ob > best || (ob == best && ok < kb)) {
+        best = ob;
+        kb = ok;
+      }
+    }
+    if (lane == 0) {
+      sig[j] = sqrt(s2);
+      const double2 v = A[kb + (int64_t)j * n];
+      const double m = sqrt(v.x * v.x + v.y * v.y);
+      phs[j] = m > 0.0 ? make_double2(v.x / m, -v.y / m) : make_double2(1.0, 0.0);
+    }
+  }
+  __syncthreads();
+  if (tid < n) {
+    const double sj = (sig[tid] == sig[tid]) ? sig[tid] : -1.0;
+    int rank = 0;
+    for (int q = 0; q < n; ++q) {
+      const double sq = (sig[q] == sig[q]) ? sig[q] : -1.0;
+      rank += (sq > sj) || (sq == sj && q < tid);
+    }
+    perm[rank] = tid;
+    a.S[b.s_off + rank] = sig[tid];
+  }
+  if (tid < 64) s_ce[tid] = 1;
+  __syncthreads();
+  // leave the item to the Householder route?
+  if (tid == 0) {
+    const double s1 = sig[perm[0]];
+    bool bad = !(s1 > 0.0);
+    for (int c = 0; c < b.k; ++c) {
+      const int j = perm[c];
+      bad = bad || !(sig[j] >= kKeptLevel * s1) || !(a.d[b.d + 1 + j] <= kOpenCos);
+    }
+    if (bad) {
+      a.flags[b.flag] = 1;
+      atomicAdd(a.flags - 1, 1);
+    }
+  }
+  if (b.VT && b.kind != 0) {
+    for (int64_t idx = tid; idx < (int64_t)n * n; idx += 256) {
+      const int c = (int)(idx % n), r = (int)(idx / n), j = perm[c];
+      const double2 v = A[r + (int64_t)j * n], p = phs[j];
+      b.VT[c + r * b.ldvt] = sig[j] > 0.0 ? (v.x * p.x - v.y * p.y) / sig[j] : 0.0;
+    }
+  }
+  if (b.k == 0) return;
+  // C = W_k S_k^-1 2^(E - bias): column c (real items) or columns 2c (re),
+  // 2c + 1 (im) of the planes
+  const int* E = a.ints + b.colE;
+  int* Ce = a.ints + b.colE + n;
+  const int ncol = b.cplx ? 2 * b.k : b.k;
+  const int stages = (n + kStK - 1) / kStK;
+  auto value = [&](int r, int col) {
+    const int c = b.cplx ? col >> 1 : col;
+    if (r >= n || col >= ncol) return 0.0;
+    const int j = perm[c];
+    const double2 v = A[r + (int64_t)j * n], p = phs[j];
+    const double x = (b.cplx && (col & 1)) ? v.x * p.y + v.y * p.x : v.x * p.x - v.y * p.y;
+    return scalbn(x / sig[j] / sig[j], E[r] - fix_bias<float>());
+  };
+  for (int col = warp; col < ncol; col += 8) {
+    int e = 1;
+    for (int r = lane; r < n; r += 32) e = max(e, exp_field(value(r, col)));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) s_ce[col] = e;
+  }
+  __syncthreads();
+  if (tid < 64) Ce[tid] = s_ce[tid];
+  for (int it = tid; it < 64 * stages * (kStK / 8); it += 256) {
+    const int col = it & 63, j0 = (it >> 6) * 8;
+    uint64_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = bias_digits((to_fixed(value(j0 + i, col), s_ce[col]) + (1ll << 23)) >> 24);
+    unsigned char* dst = a.c + b.c + (int64_t)(j0 / kStK) * kSB * kPlaneB + (col >> 3) * kPlaneSbo + ((j0 % kStK) >> 3) * 128 +
+                         (col & 7) * 16;
+    store_digits<kSB>(w, dst, kPlaneB);
+  }
+}
+
+// U = Y C
+__global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
+  constexpr int LB = Dig<float>::LBM;
+  extern __shared__ __align__(1024) unsigned char gsm[];
+  __shared__ __align__(8) DigitBarriers<kNstB> bar;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const GramUnit u = a.units[blockIdx.x];
+  const GramBin b = a.bins[u.bin];
+  const int n = b.Nb, stages = (n + kStK - 1) / kStK;
+  const int rl = tid & 127, kg = tid >> 7;
+  const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + kg * 128 + (rl & 7) * 16);
+  const int* E = a.ints + b.colE;
+  const int* Ce = a.ints + b.colE + n;
+  auto fill = [&](int64_t t, int64_t js, unsigned char* st) {
+    const int64_t row = (u.q0 + t) * 128 + rl;
+    const int c0 = (int)js * kStK + kg * 8;
+    uint64_t wv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int c = c0 + i;
+      const float y = (c < n && row < b.rows) ? __ldg(b.Y + row + (int64_t)c * b.ldy) : 0.f;
+      wv[i] = bias_digits(to_fixed(y, c < n ? __ldg(E + c) : 1));
+    }
+    store_digits<kSB>(wv, st + offA, kPlaneA);
+  };
+  auto bsrc = [&](int64_t, int64_t js) { return a.c + b.c + js * kSB * (int64_t)kPlaneB; };
+  auto store = [&](int64_t t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
+    const int64_t row = (u.q0 + t) * 128 + (warp & 3) * 32 + lane;
+    const int k0 = (warp >> 2) * 16;
+    const double iw = (b.physical && b.w && row < b.rows) ? 1.0 / sqrt(b.w[row]) : 1.0;
+    auto value = [&](int c) {
+      const int pk = 8 * LB + __ldg(Ce + k0 + c) - fix_bias<double>() + 24;
+      const double x = __fma_rn((double)acc1[c], 4294967296.0, (double)acc0[c]);
+      return (pk > -900 && pk < 900) ? x * __hiloint2double((pk + 1023) << 20, 0) : scalbn(x, pk);
+    };
+    if (b.cplx) {
+      // rows 2m, 2m + 1 hold re, im of point m times the coefficients' parts
+#pragma unroll
+      for (int c = 0; c < 16; c += 2) {
+        if (((k0 + c) >> 1) >= b.k) break;     // uniform over the warp; binary64 conversions are dear
+        const double vr = value(c), vi = value(c + 1);
+        const double pr = __shfl_xor_sync(0xffffffffu, vr, 1), pi = __shfl_xor_sync(0xffffffffu, vi, 1);
+        const int k = (k0 + c) >> 1;
+        if (!(lane & 1) && k < b.k && row < b.rows)
+          b.U[(row >> 1) + (int64_t)k * b.ldu] = make_float2((float)(vr - pi), (float)(vi + pr));
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        if (k0 + c < b.k && row < b.rows) b.Ur[row + (int64_t)(k0 + c) * b.ldu] = (float)(value(c) * iw);
+    }
+  };
+  product_pipeline<kSB, kNstB, LB>(bar, gsm, u.q1 - u.q0, stages, a.hdr, fill, bsrc, store);
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+
+void batched_gram_add(BatchedGramPlan& p, int item, int64_t N, int64_t Nb, int64_t k, int64_t s_off) {
+  GramBin b{};
+  b.Nb = (int)Nb;
+  b.Mb = (int)((Nb + kZW - 1) / kZW * kZW);
+  b.k = (int)k;
+  b.rows = N;                       // points; doubled at bind for complex items
+  b.colE = p.n_i;                   p.n_i += Nb + 64;
+  b.g = p.n_g;                      p.n_g += 6 * Nb * Nb;
+  b.z = p.n_z;                      p.n_z += (int64_t)kBinMats * Nb * Nb;
+  b.f = p.n_f;                      p.n_f += Nb * b.Mb + (int64_t)b.Mb * b.Mb;
+  b.c = p.n_c;                      p.n_c += (Nb + kStK - 1) / kStK * kSB * (int64_t)kPlaneB;
+  b.d = p.n_d;                      p.n_d += 1 + 2 * Nb;
+  b.s_off = s_off;
+  b.flag = item;
+  p.items.push_back(item);
+  p.bins.push_back(b);
+  p.maxNb = std::max(p.maxNb, b.Nb);
+  p.maxpairs = std::max(p.maxpairs, b.Mb / kZW);
+  p.kmax = std::max(p.kmax, b.k);
+}
+
+// Units hold at most this many per item: the tables' sizes must not depend on
+// what bind learns (real or complex items).
+static int64_t max_units(int64_t nitems) { return 16 * nitems + 2048; }
+
+size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems) {
+  const int64_t nb = (int64_t)p.bins.size();
+  p.nitems = nitems;
+  p.off_flags = off; off += align256(sizeof(int) * ((size_t)nitems + 1) * 2);
+  if (nb == 0) return off;
+  p.off_bins = off;  off += align256(sizeof(GramBin) * (size_t)nb);
+  p.off_units = off; off += align256(sizeof(GramUnit) * 3 * (size_t)max_units(nb));
+  p.off_i = off;     off += align256(sizeof(int) * (size_t)p.n_i);
+  p.off_g = off;     off += align256(sizeof(long long) * (size_t)p.n_g);
+  p.off_z = off;     off += align256(sizeof(double2) * (size_t)p.n_z);
+  p.off_f = off;     off += align256(sizeof(float2) * (size_t)p.n_f);
+  p.off_c = off;     off += align256((size_t)p.n_c);
+  p.off_d = off;     off += align256(sizeof(double) * (size_t)p.n_d);
+  return off;
+}
+
+// Units of about equal cost, about four waves of them: an item's tiles (cost
+// tiles x rows) are cut into row ranges.
+void batched_gram_units(BatchedGramPlan& p, int sms) {
+  p.pro.clear();
+  p.gram.clear();
+  p.mod.clear();
+  double total = 0.0, mtotal = 0.0, ptotal = 0.0;
+  auto passes = [](const GramBin& b) { return b.Nb <= 64 ? 1 : b.cplx ? 3 : 2; };
+  auto mcost = [](const GramBin& b) { return (double)((b.Nb + kStK - 1) / kStK); };
+  for (const GramBin& b : p.bins) {
+    total += (double)b.rows * passes(b);
+    if (b.k > 0) mtotal += (double)b.rows * mcost(b);
+    ptotal += (double)b.rows * b.Nb;
+  }
+  const int64_t cap = max_units((int64_t)p.bins.size()) - 4 * (int64_t)p.bins.size();
+  const double want = (double)std::min<int64_t>(4 * (int64_t)sms, cap / 2);
+  for (size_t f = 0; f < p.bins.size(); ++f) {
+    const GramBin& b = p.bins[f];
+    const int64_t sums = (b.rows + 127) / 128;
+    auto cut = [&](std::vector<GramUnit>& v, double share, int mode, int J, int64_t n) {
+      int64_t s = (int64_t)(share + 0.5);
+      s = std::max<int64_t>(1, std::min(s, n));
+      for (int64_t i = 0; i < s; ++i) v.push_back(GramUnit{(int)f, mode, J, 0, n * i / s, n * (i + 1) / s});
+    };
+    const double share = want * (double)b.rows / total;
+    cut(p.gram, share, kPacked, 0, sums);
+    if (b.Nb > 64) {
+      cut(p.gram, share, kPlain, 1, sums);
+      if (b.cplx) cut(p.gram, share, kTurned, 1, sums);
+    }
+    if (b.k > 0) cut(p.mod, want * (double)b.rows * mcost(b) / mtotal, 0, 0, sums);
+    // prologue: points (bins) or rows rounded to 32 (windows)
+    const int64_t pts = b.cplx ? b.rows / 2 : b.ldy;
+    const int64_t blk = (pts + 31) / 32;
+    const size_t first = p.pro.size();
+    cut(p.pro, want * (double)b.rows * b.Nb / ptotal, 0, 0, blk);
+    for (size_t i = first; i < p.pro.size(); ++i) {
+      p.pro[i].q0 *= 32;
+      p.pro[i].q1 = std::min(p.pro[i].q1 * 32, pts);
+    }
+  }
+  auto longest = [](const GramUnit& x, const GramUnit& y) { return x.q1 - x.q0 > y.q1 - y.q0; };
+  std::stable_sort(p.gram.begin(), p.gram.end(), longest);
+  std::stable_sort(p.mod.begin(), p.mod.end(), [&](const GramUnit& x, const GramUnit& y) {
+    return (double)(x.q1 - x.q0) * mcost(p.bins[x.bin]) > (double)(y.q1 - y.q0) * mcost(p.bins[y.bin]);
+  });
+}
+
+cudaError_t batched_gram_upload(const BatchedGramPlan& p, char* ws, const int* forced, int nitems, cudaStream_t st) {
+  // flags: [count, flags of the items] in use, then the same as given
+  std::vector<int> fl((size_t)nitems + 1, 0);
+  for (int i = 0; i < nitems; ++i) {
+    fl[i + 1] = forced[i];
+    fl[0] += forced[i] != 0;
+  }
+  cudaError_t e = cudaMemcpyAsync(ws + p.off_flags + sizeof(int) * ((size_t)nitems + 1), fl.data(),
+                                  sizeof(int) * fl.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess || p.bins.empty()) return e;
+  const size_t m = (size_t)max_units((int64_t)p.bins.size());
+  e = cudaMemcpyAsync(ws + p.off_bins, p.bins.data(), sizeof(GramBin) * p.bins.size(), cudaMemcpyHostToDevice, st);
+  const std::vector<GramUnit>* lists[3] = {&p.pro, &p.gram, &p.mod};
+  for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
+    if (lists[i]->size() > m) return cudaErrorInvalidValue;
+    if (!lists[i]->empty())
+      e = cudaMemcpyAsync(ws + p.off_units + sizeof(GramUnit) * m * i, lists[i]->data(),
+                          sizeof(GramUnit) * lists[i]->size(), cudaMemcpyHostToDevice, st);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  return e;
+}
+
+cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, double* S, cudaStream_t st) {
+  if (p.bins.empty()) return cudaSuccess;
+  cudaError_t e;
+  const size_t m = (size_t)max_units((int64_t)p.bins.size());
+  BG a{};
+  a.bins = (const GramBin*)(ws + p.off_bins);
+  const GramUnit* units = (const GramUnit*)(ws + p.off_units);
+  a.ints = (int*)(ws + p.off_i);
+  a.g = (unsigned long long*)(ws + p.off_g);
+  a.z = (double2*)(ws + p.off_z);
+  a.f = (float2*)(ws + p.off_f);
+  a.c = (unsigned char*)(ws + p.off_c);
+  a.d = (double*)(ws + p.off_d);
+  a.flags = (int*)(ws + p.off_flags) + 1;
+  a.S = S;
+  a.hdr = hdr;
+  const unsigned nb = (unsigned)p.bins.size();
+  const size_t smem = (size_t)kNstB * kStageB;
+  const size_t csmem = sizeof(double2) * ((size_t)p.maxNb * (p.maxNb + 1) / 2);
+  const size_t jsmem = sizeof(float2) * ((size_t)kZW * kZW + 2 * kZW * (kZW + 1) + kZW * (kZW + 2) + 64);
+  if ((e = ensure_dyn_smem((const void*)bg_gram_kernel, smem)) != cudaSuccess) return e;
+  if ((e = ensure_dyn_smem((const void*)bg_modes_kernel, smem)) != cudaSuccess) return e;
+  if ((e = ensure_dyn_smem((const void*)bg_chol_kernel, sizeof(double2) * 128 * 129 / 2)) != cudaSuccess) return e;
+  if ((e = ensure_dyn_smem((const void*)bg_jacobi32_kernel, jsmem)) != cudaSuccess) return e;
+  const size_t nfl = (size_t)p.nitems + 1;
+  e = cudaMemcpyAsync(a.flags - 1, a.flags - 1 + nfl, sizeof(int) * nfl, cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) return e;
+  // column exponents and integer sums are neighbours: one clear
+  e = cudaMemsetAsync(a.ints, 0, (size_t)((char*)a.z - (char*)a.ints), st);
+  if (e != cudaSuccess) return e;
+  BG au = a;
+  au.units = units;
+  bg_prologue_kernel<<<(unsigned)p.pro.size(), 256, 0, st>>>(au);
+  au.units = units + m;
+  bg_gram_kernel<<<(unsigned)p.gram.size(), kDigThreads, smem, st>>>(au);
+  bg_chol_kernel<<<nb, kCholThreads, csmem, st>>>(a);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const unsigned tiles = (unsigned)((p.maxNb + 7) / 8), el = (unsigned)std::max(1, p.maxNb * p.maxNb / 2048);
+  auto stage = [&]() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.maxpairs, nb);
+    cfg.blockDim = dim3(kZThreads);
+    cfg.dynamicSmemBytes = jsmem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)p.maxpairs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, bg_jacobi32_kernel, a);
+  };
+  auto gemm = [&](const ZGemm& x) {
+    bg_gemm_kernel<<<dim3(tiles, tiles, nb), 128, 0, st>>>(a, ZGemms{{x, x}, 1});
+  };
+  auto gemm2 = [&](const ZGemm& x, const ZGemm& y) {
+    bg_gemm_kernel<<<dim3(tiles, tiles, 2 * nb), 128, 0, st>>>(a, ZGemms{{x, y}, 2});
+  };
+  enum { A = 0, V = 1, A2 = 2, T0 = 3, T1 = 4, T2 = 5, T3 = 6, T4 = 7 };
+  if ((e = stage()) != cudaSuccess) return e;
+  bg_widen_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
+  gemm(ZGemm{1, T0, T0, -1, T1, 1.0, 0.0});                 // V^H V
+  gemm(ZGemm{0, T0, T1, T0, T3, -0.5, 1.5});                // V <- 1.5 V - 0.5 V V^H V
+  gemm(ZGemm{0, A, T3, -1, A2, 1.0, 0.0});                  // A = R^H V
+  bg_init_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
+  if ((e = cudaGetLastError()) != cudaSuccess || (e = stage()) != cudaSuccess) return e;
+  bg_widen_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
+  gemm2(ZGemm{0, T3, T0, -1, V, 1.0, 0.0}, ZGemm{0, A2, T0, -1, A, 1.0, 0.0});
+  for (int it = 0; it < 2; ++it) {
+    const int Ai = it ? A2 : A, Vi = it ? T3 : V, Ao = it ? A : A2, Vo = it ? V : T3;
+    gemm2(ZGemm{1, Ai, Ai, -1, T0, 1.0, 0.0}, ZGemm{1, Vi, Vi, -1, T1, 1.0, 0.0});
+    bg_check_kernel<<<dim3((unsigned)((p.maxNb + 7) / 8), nb), 256, 0, st>>>(a, it);
+    bg_angles_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
+    gemm(ZGemm{0, T4, T2, T1, T0, 0.5, 1.0});               // Q
+    gemm2(ZGemm{0, Ai, T0, -1, Ao, 1.0, 0.0}, ZGemm{0, Vi, T0, -1, Vo, 1.0, 0.0});
+  }
+  bg_finalize_kernel<<<nb, 256, 0, st>>>(a);
+  if (!p.mod.empty()) {
+    au.units = units + 2 * m;
+    bg_modes_kernel<<<(unsigned)p.mod.size(), kDigThreads, smem, st>>>(au);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace pylom
