@@ -46,63 +46,118 @@ template <typename TY> __host__ __device__ constexpr int gram_base(int half) { r
 // y = v 2^(E - kFixBias): the fixed-point value v of an element of a column with exponent field E
 template <typename TY> __host__ __device__ constexpr int fix_bias() { return sizeof(TY) == 8 ? 1084 : 164; }
 
-// biased exponent field of |y| (at least 1, so subnormals share the lowest one)
+// Exponent field that a column's scale is taken from, of one element: the
+// biased exponent, from a floor on (elements below it count as zero in
+// binary64; in binary32 the floor keeps the scale finite and loses nothing).
+constexpr int kMinField64 = 64, kMinField32 = 8;
 __device__ __forceinline__ int exp_field(double y) {
   const int e = (__double2hiint(y) >> 20) & 0x7ff;
-  return e > 1 ? e : 1;
+  return e > kMinField64 ? e : kMinField64;
 }
 __device__ __forceinline__ int exp_field(float y) {
   const int e = (__float_as_int(y) >> 23) & 0xff;
-  return e > 1 ? e : 1;
-}
-// fixed-point value of y in a column whose largest exponent field is E: |v| < 2^62 (binary64), < 2^38 (binary32)
-__device__ __forceinline__ int64_t to_fixed(double y, int E) {
-  const uint32_t hi = (uint32_t)__double2hiint(y), lo = (uint32_t)__double2loint(y);
-  const int e = (hi >> 20) & 0x7ff;
-  const uint32_t mh = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
-  uint64_t m = (((uint64_t)mh << 32) | lo) << 9;
-  const int sh = E - (e > 1 ? e : 1);
-  m = sh < 63 ? m >> sh : 0;
-  const int64_t sg = -(int64_t)(hi >> 31);
-  return ((int64_t)m ^ sg) - sg;
-}
-__device__ __forceinline__ int64_t to_fixed(float y, int E) {
-  const uint32_t b = (uint32_t)__float_as_int(y);
-  const int e = (b >> 23) & 0xff;
-  uint64_t m = (uint64_t)((b & 0x7fffffu) | (e ? 0x800000u : 0u)) << 14;
-  const int sh = E - (e > 1 ? e : 1);
-  m = sh < 63 ? m >> sh : 0;
-  const int64_t sg = -(int64_t)(b >> 31);
-  return ((int64_t)m ^ sg) - sg;
+  return e > kMinField32 ? e : kMinField32;
 }
 
-// Signed digits of v: v + B with 0x80 in every byte, byte k minus 128 is
-// digit k in [-128, 127] (the top one in [-64, 64]).
-__device__ __forceinline__ uint64_t bias_digits(int64_t v) { return (uint64_t)v + 0x8080808080808080ull; }
-// digit k of two biased values as a binary16 pair: 1024 + byte by bit
-// pattern, minus 1152
-__device__ __forceinline__ uint32_t digit_pair(uint32_t wa, uint32_t wb, uint32_t sel) {
-  const uint32_t x = (__byte_perm(wa, wb, sel) & 0x00ff00ffu) | 0x64006400u;
+// Fixed-point value of y in a column whose largest exponent field is E, with
+// 0x80 added to every byte: |v| < 2^62, and byte k minus 128 is the signed
+// digit k in [-128, 127] (the top one in [-64, 64]).  An element of exponent
+// field 0 (zero, subnormal) is shifted out.
+constexpr uint32_t kDigitBias = 0x80808080u;
+__device__ __forceinline__ uint2 biased_fixed(double y, int E) {
+  const uint32_t hi = (uint32_t)__double2hiint(y), lo = (uint32_t)__double2loint(y);
+  // E - e: the mantissa bits cannot borrow from the exponent's
+  const uint32_t sh = min((((uint32_t)E << 20 | 0xfffffu) - (hi & 0x7fffffffu)) >> 20, 63u);
+  uint32_t m1 = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 9), m0 = lo << 9;
+  const bool far = sh >= 32;
+  m0 = far ? m1 : m0;
+  m1 = far ? 0u : m1;
+  m0 = __funnelshift_r(m0, m1, sh);          // by sh mod 32
+  m1 >>= (sh & 31);
+  const uint32_t sg = (uint32_t)((int32_t)hi >> 31);       // 0 or all ones
+  // (m ^ sg) - sg + bias
+  uint2 w;
+  asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, %5;"
+      : "=r"(w.x), "=r"(w.y)
+      : "r"(m0 ^ sg), "r"(m1 ^ sg), "r"(kDigitBias - sg), "r"(kDigitBias));
+  return w;
+}
+constexpr uint64_t kDigitBias64 = ((uint64_t)kDigitBias << 32) | kDigitBias;
+__device__ __forceinline__ uint2 bias_digits(int64_t v) {
+  const uint64_t w = (uint64_t)v + kDigitBias64;
+  return make_uint2((uint32_t)w, (uint32_t)(w >> 32));
+}
+__device__ __forceinline__ int64_t to_fixed(double y, int E) {
+  const uint2 w = biased_fixed(y, E);
+  return (int64_t)((((uint64_t)w.y << 32) | w.x) - kDigitBias64);
+}
+
+// All digits of eight values, digit s as one 16-byte store at dst + s * plane.
+// A digit of two values becomes a binary16 pair by its bit pattern (1024 +
+// byte: 0x64 above the byte) minus 1152.
+__device__ __forceinline__ uint32_t sub_1152(uint32_t x) {
   uint32_t r;
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(0x64806480u));
   return r;
 }
-// all digits of eight values, digit s as one 16-byte store at dst + s * plane
 template <int S>
-__device__ __forceinline__ void store_digits(const uint64_t (&w)[8], unsigned char* dst, int plane) {
+__device__ __forceinline__ void store_digits(const uint2 (&w)[8], unsigned char* dst, int plane) {
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const uint32_t sel = (uint32_t)((s & 3) | ((4 + (s & 3)) << 8));
-    uint32_t d[4];
+  for (int s = 0; s < S; s += 2) {
+    uint32_t d0[4], d1[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const uint32_t a = s < 4 ? (uint32_t)w[2 * i] : (uint32_t)(w[2 * i] >> 32);
-      const uint32_t b = s < 4 ? (uint32_t)w[2 * i + 1] : (uint32_t)(w[2 * i + 1] >> 32);
-      // bytes: [a.k, a.0, b.k, b.0]; the odd ones are masked off
-      d[i] = digit_pair(a, b, (sel & 0xfu) | ((sel >> 8) & 0xfu) << 8);
+      const uint32_t a = s < 4 ? w[2 * i].x : w[2 * i].y, b = s < 4 ? w[2 * i + 1].x : w[2 * i + 1].y;
+      const uint32_t x = __byte_perm(a, b, (s & 2) ? 0x7632 : 0x5410);   // [a.s, a.s+1, b.s, b.s+1]
+      d0[i] = sub_1152(__byte_perm(x, 0x64646464u, 0x4240));
+      if (s + 1 < S) d1[i] = sub_1152(__byte_perm(x, 0x64646464u, 0x4341));
     }
-    *(uint4*)(dst + s * plane) = make_uint4(d[0], d[1], d[2], d[3]);
+    *(uint4*)(dst + s * plane) = make_uint4(d0[0], d0[1], d0[2], d0[3]);
+    if (s + 1 < S) *(uint4*)(dst + (s + 1) * plane) = make_uint4(d1[0], d1[1], d1[2], d1[3]);
   }
+}
+
+// Eight elements of one column (scale E) as digits in a stage.
+__device__ __forceinline__ void put_digits(const double (&y)[8], int E, unsigned char* dst, int plane) {
+  uint2 w[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) w[i] = biased_fixed(y[i], E);
+  store_digits<Dig<double>::S>(w, dst, plane);
+}
+// Binary32: digits by rounding, top down, in binary32 itself (d = rint(r),
+// r <- 256 (r - d), every step exact): three operations a digit on the
+// full-rate pipe instead of a 64-bit shift and byte selection on the
+// half-rate one.  The top digit is rint(y 2^(132 - E)), at most 64.
+__device__ __forceinline__ void put_digits(const float (&y)[8], const int (&E)[8], unsigned char* dst, int plane) {
+  constexpr int S = Dig<float>::S;
+  constexpr float kRound = 12582912.f;   // 1.5 2^23: adding it rounds to an integer
+  float r[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r[i] = y[i] * __int_as_float((132 - E[i] + 127) << 23);
+#pragma unroll
+  for (int s = S - 1; s >= 0; --s) {
+    float d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float t = s == S - 1 ? __fadd_rn(r[i], kRound) : __fmaf_rn(r[i], 256.f, kRound);
+      d[i] = __fsub_rn(t, kRound);
+      r[i] = s == S - 1 ? __fsub_rn(r[i], d[i]) : __fmaf_rn(r[i], 256.f, -d[i]);
+    }
+    uint32_t p[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(p[i]) : "f"(d[2 * i + 1]), "f"(d[2 * i]));
+    *(uint4*)(dst + s * plane) = make_uint4(p[0], p[1], p[2], p[3]);
+  }
+}
+__device__ __forceinline__ void put_digits(const float (&y)[8], int E, unsigned char* dst, int plane) {
+  const int e[8] = {E, E, E, E, E, E, E, E};
+  put_digits(y, e, dst, plane);
+}
+__device__ __forceinline__ void put_digits(const double (&y)[8], const int (&E)[8], unsigned char* dst, int plane) {
+  uint2 w[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) w[i] = biased_fixed(y[i], E[i]);
+  store_digits<Dig<double>::S>(w, dst, plane);
 }
 
 // instruction descriptor of kind::f16: D binary32, A and B binary16, K-major
@@ -119,26 +174,22 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc05::smem_u32(mbar)) : "memory");
 }
 
-// One thread: all digit products of one stage with level LB <= s + t < LB + 8
-// into the eight accumulators of 64 columns; `first`: the stage starts new
-// sums.  Descriptors advance 256 bytes per K = 16 step.
-template <int S, int LB>
-__device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t dA, uint64_t dB, int planeB, bool first) {
+// One thread: the digit products of one stage with level s + t = l into
+// one accumulator of 64 columns; `first`: the stage starts new sums.
+// Descriptors advance 256 bytes per K = 16 step.  The eight accumulators are
+// issued by eight warps: one thread issuing all 72 MMAs of a binary64 stage
+// took longer than the MMAs.
+template <int S>
+__device__ __forceinline__ void issue_level(uint32_t dtmem, uint64_t dA, uint64_t dB, int planeB, int l, bool first) {
   constexpr uint32_t id = idesc_f16(128, 64);
+  bool acc = !first;
+  const int s0 = l < S ? 0 : l - S + 1, s1 = l < S ? l : S - 1;
+  for (int s = s0; s <= s1; ++s) {
+    const uint64_t a = dA + (uint64_t)((s * kPlaneA) >> 4), b = dB + (uint64_t)(((l - s) * planeB) >> 4);
 #pragma unroll
-  for (int sl = 0; sl < kSlots; ++sl) {
-    const int l = LB + sl;
-    bool acc = !first;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const int t = l - s;
-      if (t < 0 || t >= S) continue;
-#pragma unroll
-      for (int ks = 0; ks < kStK / 16; ++ks) {
-        mma_f16(tmem + sl * 64, dA + (uint64_t)((s * kPlaneA + ks * 256) >> 4),
-                dB + (uint64_t)((t * planeB + ks * 256) >> 4), id, acc);
-        acc = true;
-      }
+    for (int ks = 0; ks < kStK / 16; ++ks) {
+      mma_f16(dtmem, a + (uint64_t)((ks * 256) >> 4), b + (uint64_t)((ks * 256) >> 4), id, acc);
+      acc = true;
     }
   }
 }
@@ -187,16 +238,16 @@ template <int NST>
 struct DigitBarriers {
   uint64_t full[NST], empty[NST], dfull, dempty, fin;
   uint32_t tmem;
-  // all threads; `extra`: arrivals on a full barrier besides one per warp
+  // all threads; `extra`: arrivals on a full barrier besides one per warp of a group
   __device__ __forceinline__ void open(int extra) {
     if (threadIdx.x == 0) {
       for (int b = 0; b < NST; ++b) {
-        tc05::mbar_init(full + b, kDigThreads / 32 + extra);
-        tc05::mbar_init(empty + b, 1);
+        tc05::mbar_init(full + b, kDigThreads / 64 + extra);
+        tc05::mbar_init(empty + b, kSlots);
       }
-      tc05::mbar_init(&dfull, 1);
+      tc05::mbar_init(&dfull, kSlots);
       tc05::mbar_init(&dempty, kDigThreads / 32);
-      tc05::mbar_init(&fin, 1);
+      tc05::mbar_init(&fin, kDigThreads / 32);
     }
     if (threadIdx.x < 32) tc05::tmem_alloc(&tmem, 512);
     tc05::fence_before();
@@ -205,10 +256,8 @@ struct DigitBarriers {
   }
   // all threads: nothing of this block is in flight when it gives its memory back
   __device__ __forceinline__ void close(bool ok, WsHeader* hdr) {
-    if (threadIdx.x == kDigThreads - 32) {
-      tc05::commit(&fin);
-      if (!mbar_wait_fast(&fin, 0)) ok = false;
-    }
+    if ((threadIdx.x & 31) == 0) tc05::commit(&fin);
+    if (threadIdx.x == 0 && !mbar_wait_fast(&fin, 0)) ok = false;
     if (!ok) raise_status(hdr, PYLOM_ERR_TIMEOUT);
     tc05::fence_before();
     __syncthreads();
@@ -216,70 +265,112 @@ struct DigitBarriers {
   }
 };
 
+// Both pipelines: the stages alternate between two groups of eight warps.  A
+// group fills its stage (fills wait on loads and on the integer pipe), waits
+// for its eight warps, and each of them issues one accumulator's MMAs; the
+// other group fills meanwhile.  A stage's MMAs start after those of the stage
+// before are complete, since they go to the same accumulators from other
+// threads.  At the end of a sum all sixteen warps read the accumulators; the
+// group that fills the next sum's first stage does so before it reads.  (All
+// sixteen warps filling every stage together, one thread issuing: 25.8 ms for
+// the Gram matrix of 2,097,152 x 256 binary64; this way 20.)
+//
+// Deadlock freedom: a group waits for (1) the MMAs of an earlier stage,
+// (2) the reads of an earlier sum by the other group, which reads before it
+// fills unless it opens the sum itself, (3) the MMAs of the sum it reads,
+// issued once (2) holds for the sums before.  All are earlier in the order of
+// stages, and every wait is bounded.
+// (Counters are 32-bit and stage numbers advance without divisions.)
+template <int NST>
+struct StageSlot {      // buffer and phase parity of a stage number
+  int b;
+  uint32_t par;
+  __device__ __forceinline__ void advance2() {
+    b += 2;
+    if (b >= NST) {
+      b -= NST;
+      par ^= 1u;
+    }
+  }
+};
+
+// One group's part of issuing a stage (every lane calls; lane 0 of each warp
+// issues): `cur` the stage, `prev` the one before it (j: its number).
+template <int NST, class Issue>
+__device__ __forceinline__ bool issue_turn(DigitBarriers<NST>& bar, const StageSlot<NST>& cur, const StageSlot<NST>& prev,
+                                           int j, int sum, bool first, bool last, uint32_t sa, Issue issue) {
+  bool ok = true;
+  if ((threadIdx.x & 31) == 0) {
+    ok = mbar_wait_fast(bar.full + cur.b, cur.par);
+    if (ok && j > 0) ok = mbar_wait_fast(bar.empty + prev.b, prev.par);
+    if (ok && first && sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((sum - 1) & 1));
+    if (ok) {
+      tc05::fence_after();
+      issue(bar.tmem, sa, (int)(threadIdx.x >> 5) & 7, first);
+      tc05::commit(bar.empty + cur.b);
+      if (last) tc05::commit(&bar.dfull);
+    }
+  }
+  return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+}
+
+template <int NST>
+__device__ __forceinline__ bool drain_turn(DigitBarriers<NST>& bar, int& drained, int nslots, int64_t (&acc0)[16],
+                                           int64_t (&acc1)[16]) {
+  const int warp = threadIdx.x >> 5;
+  if (!__all_sync(0xffffffffu, mbar_wait_fast(&bar.dfull, (uint32_t)(drained & 1)))) return false;
+  tc05::fence_after();
+  drain_slots(bar.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16, nslots, acc0, acc1);
+  tc05::fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&bar.dempty);
+  ++drained;
+  return true;
+}
+
 // Sums over a range of rows: `nstage` stages of kStK rows, read out every
 // kStagesPerSum of them.  fill(j, stage) writes this thread's part of stage
-// j; issue(stage address, first) issues its MMAs (one thread); flush(acc0,
-// acc1) hands on the 64-bit sums of this thread's row and 16 columns.  The
-// accumulators are read only after the next NST stages have been filled, so
-// the warps work while the last MMAs of a sum run.
+// j; issue(tensor memory, stage address, slot, first) issues one
+// accumulator's MMAs; flush(acc0, acc1) hands on the 64-bit sums of this
+// thread's row and 16 columns.
 template <int NST, class Fill, class Issue, class Flush>
-__device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int stage_bytes, int64_t nstage,
+__device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int stage_bytes, int nstage,
                                               int nslots, WsHeader* hdr, Fill fill, Issue issue, Flush flush) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, group = threadIdx.x >> 8;
   bar.open(0);
-  const uint32_t tmem = bar.tmem;
-  const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16;
+  const uint32_t base = tc05::smem_u32(gsm);
   bool ok = true;
   int64_t acc0[16], acc1[16];
 #pragma unroll
   for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
-  int64_t issued = 0, drained = 0;
-  for (int64_t j = 0; j <= nstage; ++j) {
-    const int b = (int)(j % NST);
-    if (j < nstage) {
-      if (j >= NST) {
-        ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + b, (uint32_t)((j / NST - 1) & 1)));
-        if (!ok) break;
-      }
-      fill(j, gsm + b * stage_bytes);
-      tc05::fence_smem_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar.full + b);
-    }
-    // the sums of the 128 rows before, once the stages ahead are filled
-    const bool due = (j % kStagesPerSum == NST - 1 && j >= kStagesPerSum && j < nstage) ||
-                     (j == nstage && nstage > 0);
-    if (due) {
-      ok = __all_sync(0xffffffffu, mbar_wait_fast(&bar.dfull, (uint32_t)(drained & 1)));
+  int drained = 0;
+  StageSlot<NST> cur{group, 0u}, prev{group ? 0 : NST - 1, group ? 0u : 1u};
+  for (int j = group; j < nstage; j += 2) {
+    const int sum = j / kStagesPerSum, js = j % kStagesPerSum;
+    if (js != 0 && drained < sum) {
+      ok = drain_turn(bar, drained, nslots, acc0, acc1);
       if (!ok) break;
-      tc05::fence_after();
-      drain_slots(taddr, nslots, acc0, acc1);
-      tc05::fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar.dempty);
-      ++drained;
-      if ((drained & 8191) == 0) flush(acc0, acc1);
     }
-    // MMAs of the stages that are filled; those of a new sum wait until the
-    // last one has been read
-    const bool held = j >= kStagesPerSum && j % kStagesPerSum < NST - 1;
-    if (warp == kDigThreads / 32 - 1 && lane == 0 && j < nstage && !held) {
-      for (; issued <= j && ok; ++issued) {
-        const int ib = (int)(issued % NST);
-        const int64_t sum = issued / kStagesPerSum;
-        const bool first = issued % kStagesPerSum == 0;
-        ok = mbar_wait_fast(bar.full + ib, (uint32_t)((issued / NST) & 1));
-        if (ok && first && sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((sum - 1) & 1));
-        if (!ok) break;
-        tc05::fence_after();
-        issue(tmem, tc05::smem_u32(gsm) + ib * stage_bytes, first);
-        tc05::commit(bar.empty + ib);
-        if (issued % kStagesPerSum == kStagesPerSum - 1) tc05::commit(&bar.dfull);
-      }
+    if (j >= NST) {
+      ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + cur.b, cur.par ^ 1u));
+      if (!ok) break;
     }
-    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+    fill(j, gsm + cur.b * stage_bytes);
+    tc05::fence_smem_async();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar.full + cur.b);
+    if (js == 0 && drained < sum) {
+      ok = drain_turn(bar, drained, nslots, acc0, acc1);
+      if (!ok) break;
+    }
+    // (64-bit sums of at most 2^20 rows)
+    if (drained > 0 && (drained & 8191) == 0 && js < 2) flush(acc0, acc1);
+    ok = issue_turn(bar, cur, prev, j, sum, js == 0, js == kStagesPerSum - 1, base + cur.b * stage_bytes, issue);
     if (!ok) break;
+    cur.advance2();
+    prev.advance2();
   }
+  while (ok && drained * kStagesPerSum < nstage) ok = drain_turn(bar, drained, nslots, acc0, acc1);
   if (ok) flush(acc0, acc1);
   bar.close(ok, hdr);
 }
@@ -298,63 +389,22 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 // thread's row and 16 columns.  `tile` counts 0 .. mine - 1.  LB: lowest
 // level that is kept.
 template <int S, int NST, int LB, class Fill, class Src, class Store>
-__device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int64_t mine, int64_t stages,
+__device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int mine, int stages,
                                                  WsHeader* hdr, Fill fill, Src bsrc, Store store) {
   constexpr int kStage = S * (kPlaneA + kPlaneB);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, group = tid >> 8;
   bar.open(1);
-  const uint32_t tmem = bar.tmem;
-  const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16;
-  const int64_t sums = (stages + kStagesPerSum - 1) / kStagesPerSum;
-  const int64_t total = mine * stages, nsum = mine * sums;
+  const uint32_t base = tc05::smem_u32(gsm);
+  const int sums = (stages + kStagesPerSum - 1) / kStagesPerSum;
   bool ok = true;
   int64_t acc0[16], acc1[16];
 #pragma unroll
   for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
-  int64_t issued = 0, issued_sum = 0, drained = 0;
-  int64_t tile = 0, js = 0, begun = 0;   // the stage being filled; sums whose first stage has been filled
-  int ahead = 0;                         // stages filled of the current sum
-  int64_t is_js = 0, dr_tile = 0, dr_sum = 0;
-  for (int64_t j = 0; j <= total; ++j) {
-    const int b = (int)(j % NST);
-    if (j < total) {
-      if (j >= NST) {
-        ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + b, (uint32_t)((j / NST - 1) & 1)));
-        if (!ok) break;
-      }
-      unsigned char* st = gsm + b * kStage;
-      if (tid == 0) {
-        tc05::mbar_arrive_expect_tx(bar.full + b, S * kPlaneB);
-        bulk_load(st + S * kPlaneA, bsrc(tile, js), S * kPlaneB, bar.full + b);
-      }
-      fill(tile, js, st);
-      tc05::fence_smem_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar.full + b);
-      if (js % kStagesPerSum == 0) {
-        ++begun;
-        ahead = 0;
-      }
-      ++ahead;
-      if (++js == stages) {
-        js = 0;
-        ++tile;
-      }
-    }
-    // read the sums that are complete: all of them at the end; before that,
-    // the one before the sum being filled, as soon as NST stages (or the
-    // whole sum) are filled ahead of it
-    const bool whole = j < total && (js == 0 || js % kStagesPerSum == 0);
-    const int64_t upto = j == total ? nsum : (ahead >= NST || whole) ? begun - 1 : drained;
-    while (drained < upto) {
-      ok = __all_sync(0xffffffffu, mbar_wait_fast(&bar.dfull, (uint32_t)(drained & 1)));
-      if (!ok) break;
-      tc05::fence_after();
-      drain_slots(taddr, kSlots, acc0, acc1);
-      tc05::fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar.dempty);
-      ++drained;
+  int drained = 0, dr_tile = 0, dr_sum = 0;
+  auto read_upto = [&](int upto) {
+    while (ok && drained < upto) {
+      ok = drain_turn(bar, drained, kSlots, acc0, acc1);
+      if (!ok) return;
       if (++dr_sum == sums) {
         store(dr_tile, acc0, acc1);
 #pragma unroll
@@ -363,32 +413,46 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
         ++dr_tile;
       }
     }
-    if (!ok) break;
-    // MMAs of filled stages, up to the first sum whose accumulators are still unread
-    if (warp == kDigThreads / 32 - 1) {
-      if (lane == 0) {
-        while (issued <= j && issued < total) {
-          const bool first = is_js % kStagesPerSum == 0;
-          if (first && issued_sum > drained) break;      // this warp has not read the sum before
-          const int ib = (int)(issued % NST);
-          ok = mbar_wait_fast(bar.full + ib, (uint32_t)((issued / NST) & 1));
-          if (ok && first && issued_sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((issued_sum - 1) & 1));
-          if (!ok) break;
-          if (first) ++issued_sum;
-          tc05::fence_after();
-          const uint32_t sa = tc05::smem_u32(gsm) + ib * kStage;
-          issue_stage<S, LB>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo),
-                             kPlaneB, first);
-          tc05::commit(bar.empty + ib);
-          ++issued;
-          if (++is_js == stages) is_js = 0;
-          if (is_js % kStagesPerSum == 0) tc05::commit(&bar.dfull);
-        }
-      }
-      ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-      if (!ok) break;
-    }
+  };
+  auto issue = [&](uint32_t tmem, uint32_t sa, int slot, bool first) {
+    issue_level<S>(tmem + slot * 64, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo),
+                   kPlaneB, LB + slot, first);
+  };
+  StageSlot<NST> cur{group, 0u}, prev{group ? 0 : NST - 1, group ? 0u : 1u};
+  int tile = 0, js = group, j = group;
+  while (js >= stages) {
+    js -= stages;
+    ++tile;
   }
+  for (; tile < mine; j += 2) {
+    const int sum = tile * sums + js / kStagesPerSum;
+    const bool first = js % kStagesPerSum == 0;
+    if (!first) read_upto(sum);
+    if (ok && j >= NST) ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + cur.b, cur.par ^ 1u));
+    if (!ok) break;
+    unsigned char* st = gsm + cur.b * kStage;
+    if ((tid & 255) == 0) {
+      tc05::mbar_arrive_expect_tx(bar.full + cur.b, S * kPlaneB);
+      bulk_load(st + S * kPlaneA, bsrc(tile, js), S * kPlaneB, bar.full + cur.b);
+    }
+    fill(tile, js, st);
+    tc05::fence_smem_async();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar.full + cur.b);
+    if (first) read_upto(sum);
+    if (!ok) break;
+    ok = issue_turn(bar, cur, prev, j, sum, first, js % kStagesPerSum == kStagesPerSum - 1 || js == stages - 1,
+                    base + cur.b * kStage, issue);
+    if (!ok) break;
+    js += 2;
+    while (js >= stages) {
+      js -= stages;
+      ++tile;
+    }
+    cur.advance2();
+    prev.advance2();
+  }
+  read_upto(mine * sums);
   // bulk copies of stages that were never consumed (after a timeout) land
   // before the block ends
   if (!ok && tid == 0)

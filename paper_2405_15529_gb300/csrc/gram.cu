@@ -13,9 +13,9 @@
 // does at 1/60 of its binary32 rate.
 //
 // Measured (4,194,304 x 256, binary64): Householder leaves + tree 554 + 13
-// ms; here Y 8.2, Gram matrix 51.5, Cholesky factor 1.3 ms.  1,048,576 x 128
+// ms; here Y 8.2, Gram matrix 40, Cholesky factor 1.3 ms.  1,048,576 x 128
 // leaves + tree 39 + 3.8 ms.  Binary32 leaves (mixed, 4,194,304 x 256) 57.7 +
-// 8.8 ms; here 6.4, 18.6 and 1.3 ms.
+// 8.8 ms; here 6.4, 16.7 and 1.3 ms.
 #include <atomic>
 
 #include "digits.cuh"
@@ -210,22 +210,17 @@ __device__ __forceinline__ void load8<float>(const float* p, float (&y)[8]) {
   }
 }
 
-// digits of 8 rows of one column into a stage plane (zeros outside Y)
+// digits of the 8 rows at p of one column into a stage plane (zeros if !in)
 template <typename TY>
-__device__ __forceinline__ void put_column8(const TY* Y, int64_t ldy, int64_t row, int64_t col, int64_t M, int E,
-                                            unsigned char* dst, int plane) {
-  constexpr int S = Dig<TY>::S;
-  uint64_t w[8];
-  if (col < M && row < ldy) {
-    TY y[8];
-    load8(Y + row + col * ldy, y);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = bias_digits(to_fixed(y[i], E));
+__device__ __forceinline__ void put_column8(const TY* p, bool in, int E, unsigned char* dst, int plane) {
+  TY y[8];
+  if (in) {
+    load8(p, y);
   } else {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = bias_digits(0);
+    for (int i = 0; i < 8; ++i) y[i] = (TY)0;
   }
-  store_digits<S>(w, dst, plane);
+  put_digits(y, E, dst, plane);
 }
 
 template <typename TY>
@@ -247,27 +242,30 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
   const TY* Y = (const TY*)a.Y;
   const int c8 = lane & 7, kg = lane >> 3;
-  const int ca = warp * 8 + c8;                  // A: 16 warps x 8 columns
-  const int64_t colA = (int64_t)I * 128 + ca;
-  const int EA = colA < a.M ? a.colE[colA] : 1;
-  const uint32_t offA = (uint32_t)((ca >> 3) * kPlaneSbo + kg * 128 + c8 * 16);
-  const bool doB = !diag && warp < 8;            // B: 8 warps x 8 columns
-  const int64_t colB = (int64_t)J * 64 + ca;
-  const int EB = (doB && colB < a.M) ? a.colE[colB] : 1;
-  auto fill = [&](int64_t j, unsigned char* st) {
-    const int64_t row = (q0 * kStagesPerSum + j) * kStK + kg * 8;
-    put_column8<TY>(Y, a.ldy, row, colA, a.M, EA, st + offA, kPlaneA);
-    if (doB) put_column8<TY>(Y, a.ldy, row, colB, a.M, EB, st + S * kPlaneA + offA, kPlaneB);
+  const int gw = warp & 7;                       // a stage's eight warps: 16 columns of A and 8 of B each
+  const int64_t colA = (int64_t)I * 128 + gw * 16 + c8, colB = (int64_t)J * 64 + gw * 8 + c8;
+  const int E0 = colA < a.M ? a.colE[colA] : 128, E1 = colA + 8 < a.M ? a.colE[colA + 8] : 128;
+  const int EB = (!diag && colB < a.M) ? a.colE[colB] : 128;
+  const uint32_t off = (uint32_t)(kg * 128 + c8 * 16);
+  // this thread's first row of the unit, and how many stages hold rows of Y
+  const int64_t row0 = q0 * 128 + kg * 8;
+  const int jin = (int)((a.ldy - row0 + kStK - 1) / kStK);
+  const TY* pA = Y + row0 + (colA < a.M ? colA : 0) * a.ldy;
+  const TY* pA8 = Y + row0 + (colA + 8 < a.M ? colA + 8 : 0) * a.ldy;
+  const TY* pB = Y + row0 + (colB < a.M ? colB : 0) * a.ldy;
+  const int jA = colA < a.M ? jin : 0, jA8 = colA + 8 < a.M ? jin : 0, jB = colB < a.M ? jin : 0;
+  auto fill = [&](int j, unsigned char* st) {
+    unsigned char* d = st + off + 2 * gw * kPlaneSbo;
+    put_column8<TY>(pA + j * kStK, j < jA, E0, d, kPlaneA);
+    put_column8<TY>(pA8 + j * kStK, j < jA8, E1, d + kPlaneSbo, kPlaneA);
+    if (!diag) put_column8<TY>(pB + j * kStK, j < jB, EB, st + S * kPlaneA + off + gw * kPlaneSbo, kPlaneB);
   };
-  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+  auto issue = [&](uint32_t tmem, uint32_t sa, int slot, bool first) {
     const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
     const uint64_t dB = diag ? tc05::desc(sa + (J & 1) * 8 * kPlaneSbo, 128, kPlaneSbo)
                              : tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
     const int planeB = diag ? kPlaneA : kPlaneB;
-    if (Dig<TY>::HALVES == 2 && half == 1)
-      issue_stage<S, gram_base<TY>(1)>(tmem, dA, dB, planeB, first);
-    else
-      issue_stage<S, gram_base<TY>(0)>(tmem, dA, dB, planeB, first);
+    issue_level<S>(tmem + slot * 64, dA, dB, planeB, gram_base<TY>(half) + slot, first);
   };
   auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
     const int64_t gi = (int64_t)I * 128 + (warp & 3) * 32 + lane;
@@ -281,7 +279,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<NST>(bar, gsm, S * (kPlaneA + kPlaneB), (q1 - q0) * kStagesPerSum,
+  gram_pipeline<NST>(bar, gsm, S * (kPlaneA + kPlaneB), (int)(q1 - q0) * kStagesPerSum,
                      (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr, fill, issue, flush);
 }
 

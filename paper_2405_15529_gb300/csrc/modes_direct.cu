@@ -5,7 +5,7 @@
 // multiplied without rounding on the tcgen05 tensor cores; digit products
 // below the level of a binary64 (binary32) rounding of the sum are left out.
 // Measured (4,194,304 x 256, r = 43): top-down pass + reflectors 7.3 + 209 ms
-// in binary64, 5.2 + 16.7 ms mixed; here 11.3 and 7.8 ms.
+// in binary64, 5.2 + 16.7 ms mixed; here 8.4 and 7.5 ms.
 //
 // A block takes tiles of 128 rows x 64 columns of U.  16 warps cut 32
 // columns of the tile's rows of Y into digit planes per stage (a thread
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(GramState g, const dou
   const int64_t k = blockIdx.x, r = g.hdr->r, M = g.M;
   if (k >= (r + 63) / 64 * 64) return;
   const int64_t stages = (M + kStK - 1) / kStK;
-  if (threadIdx.x == 0) s_e = 1;
+  if (threadIdx.x == 0) s_e = kMinField64;
   __syncthreads();
   const double sk = (!C && k < r) ? S[k] : 1.0;
   auto value = [&](int64_t j) {
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(GramState g, const dou
     const double c = C ? C[j + k * M] : VT[k + j * ldvt] / sk;
     return scalbn(c, g.colE[j] - fix_bias<TY>());
   };
-  int e = 1;
+  int e = kMinField64;
   for (int64_t j = threadIdx.x; j < M; j += blockDim.x) {
     const int ej = exp_field(value(j));
     e = ej > e ? ej : e;
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(GramState g, const dou
   e = s_e;
   if (threadIdx.x == 0) g.Ce[k] = e;
   for (int64_t j0 = (int64_t)threadIdx.x * 8; j0 < stages * kStK; j0 += (int64_t)blockDim.x * 8) {
-    uint64_t w[8];
+    uint2 w[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       int64_t v = to_fixed(value(j0 + i), e);
@@ -77,39 +77,47 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(GramState 
   const bool zero = S0 && S0[0] == 0.0;
   if (blockIdx.x == 0 && tid == 0 && r_out) *r_out = r;
   const int64_t ktiles = (r + 63) / 64, tiles = (N + 127) / 128 * ktiles;
-  const int64_t stages = (M + kStK - 1) / kStK;
+  const int stages = (int)((M + kStK - 1) / kStK), m32 = (int)M;
+  const uint32_t kt32 = (uint32_t)ktiles;
   const TY* Y = (const TY*)g.Y;
-  const int rl = tid & 127, kg = tid >> 7;       // row of the tile, group of 8 columns of the stage
-  const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + kg * 128 + (rl & 7) * 16);
-  const int64_t mine = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  auto fill = [&](int64_t t, int64_t js, unsigned char* st) {
-    const int64_t tile = blockIdx.x + t * gridDim.x;
-    const int64_t row = tile / ktiles * 128 + rl, c0 = js * kStK + kg * 8;
-    uint64_t wv[8];
+  const int rl = tid & 127, kh = (tid >> 7) & 1; // row of the tile, half of the stage's columns
+  const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
+  const int mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+  auto fill = [&](int t, int js, unsigned char* st) {
+    const uint32_t tile = blockIdx.x + t * gridDim.x;
+    const int64_t row = (int64_t)(tile / kt32) * 128 + rl;
+    const bool rin = row < N;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int64_t c = c0 + i;
-      const bool in = c < M && row < N;
-      const TY y = in ? __ldg(Y + row + c * g.ldy) : (TY)0;
-      const int E = c < M ? __ldg(g.colE + c) : 1;
-      wv[i] = bias_digits(to_fixed(y, E));
+    for (int h = 0; h < 2; ++h) {
+      const int kg = 2 * kh + h;
+      const int c0 = js * kStK + kg * 8;
+      const TY* p = Y + row + c0 * g.ldy;
+      TY y[8];
+      int E[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const bool in = c0 + i < m32;
+        y[i] = (in && rin) ? __ldg(p + i * g.ldy) : (TY)0;
+        E[i] = in ? __ldg(g.colE + c0 + i) : 128;
+      }
+      put_digits(y, E, st + offA + kg * 128, kPlaneA);
     }
-    store_digits<S>(wv, st + offA, kPlaneA);
   };
-  auto bsrc = [&](int64_t t, int64_t js) {
-    const int64_t tile = blockIdx.x + t * gridDim.x;
-    return g.Cd + (((tile % ktiles) * stages + js) * S) * (int64_t)kPlaneB;
+  auto bsrc = [&](int t, int js) {
+    const uint32_t tile = blockIdx.x + t * gridDim.x;
+    return g.Cd + ((int64_t)(tile % kt32) * stages + js) * (S * kPlaneB);
   };
-  auto store = [&](int64_t t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
+  auto store = [&](int t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
     // the tile's rows of U: lanes hold consecutive rows
-    const int64_t tile = blockIdx.x + t * gridDim.x;
-    const int64_t row = tile / ktiles * 128 + (warp & 3) * 32 + lane;
-    const int64_t k0 = tile % ktiles * 64 + (warp >> 2) * 16;
+    const uint32_t tile = blockIdx.x + t * gridDim.x;
+    const int64_t row = (int64_t)(tile / kt32) * 128 + (warp & 3) * 32 + lane;
+    const int k0 = (int)(tile % kt32) * 64 + (warp >> 2) * 16;
     const double iw = (physical && w && row < N) ? 1.0 / sqrt(w[row]) : 1.0;
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-      const int64_t k = k0 + c;
-      if (k < r && row < N) {
+      const int k = k0 + c;
+      if (k >= r) break;     // uniform over the warp
+      if (row < N) {
         const int pk = 8 * LB + __ldg(g.Ce + k) - fix_bias<double>() + (S == 5 ? 24 : 0);
         double v = __fma_rn((double)acc1[c], 4294967296.0, (double)acc0[c]);
         v = (pk > -900 && pk < 900) ? v * __hiloint2double((pk + 1023) << 20, 0) : scalbn(v, pk);

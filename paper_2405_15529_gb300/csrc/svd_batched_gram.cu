@@ -21,8 +21,8 @@
 // zero matrix) are flagged on the device and left to that kernel.
 //
 // Persistent kernel -> here: 24 bins (N 16k..262k, Nb 16..128, 1.3 GB) 374 ->
-// 20 ms, 12 windows (N 16k..262k, M 16..96) 115 -> 5.0 ms, SPOD of 131072 x
-// 1056 25.6 -> 17 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
+// 14.5 ms, 12 windows (N 16k..262k, M 16..96) 115 -> 4.9 ms, SPOD of 131072 x
+// 1056 25.6 -> 9.7 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
 #include <algorithm>
 
 #include "digits.cuh"
@@ -169,7 +169,6 @@ enum { kPlain = 0, kPacked = 1, kTurned = 2 };
 // digits of rows row..row+7 of a column (turned: (-im, re) pairs)
 __device__ __forceinline__ void put_rows8(const GramBin& b, int64_t row, int col, int E, bool turned, unsigned char* dst,
                                           int plane) {
-  uint64_t w[8];
   float y[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) y[i] = 0.f;
@@ -190,13 +189,15 @@ __device__ __forceinline__ void put_rows8(const GramBin& b, int64_t row, int col
         if (row + i < b.rows) y[i] = __ldg(p + i);
     }
   }
+  if (turned) {
 #pragma unroll
-  for (int i = 0; i < 8; i += 2) {
-    const float x0 = turned ? -y[i + 1] : y[i], x1 = turned ? y[i] : y[i + 1];
-    w[i] = bias_digits(to_fixed(x0, E));
-    w[i + 1] = bias_digits(to_fixed(x1, E));
+    for (int i = 0; i < 8; i += 2) {
+      const float x = y[i];
+      y[i] = -y[i + 1];
+      y[i + 1] = x;
+    }
   }
-  store_digits<kSB>(w, dst, plane);
+  put_digits(y, E, dst, plane);
 }
 
 __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
@@ -206,26 +207,27 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
   const GramUnit u = a.units[blockIdx.x];
   const GramBin b = a.bins[u.bin];
   const int mode = u.mode, J = u.J;
-  const int c8 = lane & 7, kg = lane >> 3, ca = warp * 8 + c8;
-  const bool turned = mode == kTurned || (mode == kPacked && ca >= 64);
-  const int colA = mode == kPacked ? (ca & 63) : ca;
+  // a stage's eight warps: 16 rows of the left factor (columns of Y) and 8 of the right each
+  const int c8 = lane & 7, kg = lane >> 3, gw = warp & 7, ca = gw * 16 + c8;
+  const bool turned = mode == kTurned || (mode == kPacked && gw >= 4);
   // real items have nothing to turn: their second half is empty
-  const bool useA = !(mode == kPacked && ca >= 64 && !b.cplx);
-  const int EA = colA < b.Nb ? a.ints[b.colE + colA] : 1;
-  const uint32_t off = (uint32_t)((ca >> 3) * kPlaneSbo + kg * 128 + c8 * 16);
+  const int colA = (mode == kPacked && gw >= 4 && !b.cplx) ? 128 : mode == kPacked ? (ca & 63) : ca;
+  const int E0 = colA < b.Nb ? a.ints[b.colE + colA] : 128, E1 = colA + 8 < b.Nb ? a.ints[b.colE + colA + 8] : 128;
   const bool sepB = mode == kTurned;             // else the right factor's columns are among the left's
-  const int colB = J * 64 + ca;
-  const int EB = (sepB && warp < 8 && colB < b.Nb) ? a.ints[b.colE + colB] : 1;
-  auto fill = [&](int64_t j, unsigned char* st) {
+  const int colB = J * 64 + gw * 8 + c8;
+  const int EB = (sepB && colB < b.Nb) ? a.ints[b.colE + colB] : 128;
+  const uint32_t off = (uint32_t)(kg * 128 + c8 * 16);
+  auto fill = [&](int j, unsigned char* st) {
     const int64_t row = (u.q0 * kStagesPerSum + j) * kStK + kg * 8;
-    put_rows8(b, row, useA ? colA : b.Nb, EA, turned, st + off, kPlaneA);
-    if (sepB && warp < 8) put_rows8(b, row, colB, EB, false, st + kSB * kPlaneA + off, kPlaneB);
+    put_rows8(b, row, colA, E0, turned, st + off + 2 * gw * kPlaneSbo, kPlaneA);
+    put_rows8(b, row, colA + 8, E1, turned, st + off + (2 * gw + 1) * kPlaneSbo, kPlaneA);
+    if (sepB) put_rows8(b, row, colB, EB, false, st + kSB * kPlaneA + off + gw * kPlaneSbo, kPlaneB);
   };
-  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+  auto issue = [&](uint32_t tmem, uint32_t sa, int slot, bool first) {
     const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
     const uint64_t dB = sepB ? tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo)
                              : tc05::desc(sa + J * 8 * kPlaneSbo, 128, kPlaneSbo);
-    issue_stage<kSB, gram_base<float>(0)>(tmem, dA, dB, sepB ? kPlaneB : kPlaneA, first);
+    issue_level<kSB>(tmem + slot * 64, dA, dB, sepB ? kPlaneB : kPlaneA, gram_base<float>(0) + slot, first);
   };
   auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
     const int row = (warp & 3) * 32 + lane;
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<kNstB>(bar, gsm, kStageB, (u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, fill, issue, flush);
+  gram_pipeline<kNstB>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, fill, issue, flush);
 }
 
 // ---------------------------------------------------------------------------
@@ -790,7 +792,7 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
     perm[rank] = tid;
     a.S[b.s_off + rank] = sig[tid];
   }
-  if (tid < 64) s_ce[tid] = 1;
+  if (tid < 64) s_ce[tid] = kMinField64;
   __syncthreads();
   // leave the item to the Householder route?
   if (tid == 0) {
@@ -828,7 +830,7 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
     return scalbn(x / sig[j] / sig[j], E[r] - fix_bias<float>());
   };
   for (int col = warp; col < ncol; col += 8) {
-    int e = 1;
+    int e = kMinField64;
     for (int r = lane; r < n; r += 32) e = max(e, exp_field(value(r, col)));
     e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0) s_ce[col] = e;
@@ -837,7 +839,7 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
   if (tid < 64) Ce[tid] = s_ce[tid];
   for (int it = tid; it < 64 * stages * (kStK / 8); it += 256) {
     const int col = it & 63, j0 = (it >> 6) * 8;
-    uint64_t w[8];
+    uint2 w[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = bias_digits((to_fixed(value(j0 + i, col), s_ce[col]) + (1ll << 23)) >> 24);
     unsigned char* dst = a.c + b.c + (int64_t)(j0 / kStK) * kSB * kPlaneB + (col >> 3) * kPlaneSbo + ((j0 % kStK) >> 3) * 128 +
@@ -855,24 +857,30 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
   const GramUnit u = a.units[blockIdx.x];
   const GramBin b = a.bins[u.bin];
   const int n = b.Nb, stages = (n + kStK - 1) / kStK;
-  const int rl = tid & 127, kg = tid >> 7;
-  const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + kg * 128 + (rl & 7) * 16);
+  const int rl = tid & 127, kh = (tid >> 7) & 1;
+  const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
   const int* E = a.ints + b.colE;
   const int* Ce = a.ints + b.colE + n;
-  auto fill = [&](int64_t t, int64_t js, unsigned char* st) {
+  auto fill = [&](int t, int js, unsigned char* st) {
     const int64_t row = (u.q0 + t) * 128 + rl;
-    const int c0 = (int)js * kStK + kg * 8;
-    uint64_t wv[8];
+    const bool rin = row < b.rows;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int c = c0 + i;
-      const float y = (c < n && row < b.rows) ? __ldg(b.Y + row + (int64_t)c * b.ldy) : 0.f;
-      wv[i] = bias_digits(to_fixed(y, c < n ? __ldg(E + c) : 1));
+    for (int h = 0; h < 2; ++h) {
+      const int kg = 2 * kh + h, c0 = js * kStK + kg * 8;
+      const float* p = b.Y + row + c0 * b.ldy;
+      float y[8];
+      int e[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int c = c0 + i;
+        y[i] = (c < n && rin) ? __ldg(p + i * b.ldy) : 0.f;
+        e[i] = c < n ? __ldg(E + c) : 128;
+      }
+      put_digits(y, e, st + offA + kg * 128, kPlaneA);
     }
-    store_digits<kSB>(wv, st + offA, kPlaneA);
   };
-  auto bsrc = [&](int64_t, int64_t js) { return a.c + b.c + js * kSB * (int64_t)kPlaneB; };
-  auto store = [&](int64_t t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
+  auto bsrc = [&](int, int js) { return a.c + b.c + js * kSB * (int64_t)kPlaneB; };
+  auto store = [&](int t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
     const int64_t row = (u.q0 + t) * 128 + (warp & 3) * 32 + lane;
     const int k0 = (warp >> 2) * 16;
     const double iw = (b.physical && b.w && row < b.rows) ? 1.0 / sqrt(b.w[row]) : 1.0;
@@ -898,7 +906,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
         if (k0 + c < b.k && row < b.rows) b.Ur[row + (int64_t)(k0 + c) * b.ldu] = (float)(value(c) * iw);
     }
   };
-  product_pipeline<kSB, kNstB, LB>(bar, gsm, u.q1 - u.q0, stages, a.hdr, fill, bsrc, store);
+  product_pipeline<kSB, kNstB, LB>(bar, gsm, (int)(u.q1 - u.q0), stages, a.hdr, fill, bsrc, store);
 }
 
 }  // namespace
