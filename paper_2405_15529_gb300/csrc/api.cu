@@ -175,15 +175,22 @@ static size_t pod_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, int prec
 
 // Which route gives R and the modes.  The Gram route (gram.cu) needs no
 // leaves and no tree; its modes Y V_r S_r^-1 are as orthonormal as Q U_r up
-// to a factor sigma_1 / sigma_r, which an energy share of at most 1 - 1e-4
-// bounds by sqrt(M / 1e-4) (the share left out is at least that, so the last
-// kept value is no smaller than its mean).  Everything else -- all modes
-// kept, where sigma_r may be at the rounding level, a leaf height or a tree
-// that the caller asks for -- takes the Householder TSQR.  Whole calls, Householder /
-// Gram: 4096 x 32 3.8 / 2.3 ms, 65537 x 63 10.0 / 5.0 ms, 4194304 x 256 799 /
-// 86 ms; mixed 262144 x 100 13.8 / 8.6 ms, 4194304 x 256 102 / 48 ms.
-static bool use_gram_route(int64_t leaf_rows, double energy) {
-  return leaf_rows == 0 && energy > 0.0 && energy <= 1.0 - 1e-4 && !tree_requested();
+// to a factor sigma_1 / sigma_r.  An energy share of at most 1 - 1e-4 bounds
+// that by sqrt(M / 1e-4) (the share left out is at least that, so the last
+// kept value is no smaller than its mean).  With r_max < M columns asked for
+// instead, the device looks at sigma_r and has the Householder route done
+// behind it where it is too small (about 15 launches that return at once
+// otherwise, 25 us).  All modes, where sigma_M is usually at the rounding
+// level, a leaf height or a tree that the caller asks for take the
+// Householder TSQR directly.  Whole calls, Householder / Gram: 4096 x 32
+// 3.8 / 0.7 ms, 65537 x 63 10.0 / 1.2 ms, 1048576 x 128 (r_max 40) 78 / 7 ms,
+// 4194304 x 256 799 / 65 ms; mixed 262144 x 100 13.8 / 2.5 ms, 4194304 x 256
+// 102 / 36 ms.
+enum Route { kHouseholder, kGram, kGramChecked };
+static Route pod_route(int64_t leaf_rows, double energy, int64_t r_max, int64_t M) {
+  if (leaf_rows != 0 || tree_requested()) return kHouseholder;
+  if (energy > 0.0 && energy <= 1.0 - 1e-4) return kGram;
+  return r_max < M ? kGramChecked : kHouseholder;
 }
 
 extern "C" size_t pylom_pod_workspace_size(int64_t N, int64_t M, int64_t leaf_rows, int64_t r_max,
@@ -247,7 +254,8 @@ extern "C" pylom_status pylom_pod(const void* X, int64_t N, int64_t M, int64_t l
   e = cudaMemsetAsync(ts.arrive, 0, sizeof(unsigned) * (size_t)P, st);
   if (e != cudaSuccess) return cuda_fail(e, "pylom_pod: counter clear");
   if (prof && (e = cudaEventRecord(g_prof.at(call, 0), st)) != cudaSuccess) return cuda_fail(e, "profile");
-  const bool gram = use_gram_route(leaf_rows, energy);
+  const Route route = pod_route(leaf_rows, energy, r_max, M);
+  const bool gram = route != kHouseholder;
   GramState gs;
   if (gram) {
     gs.hdr = hdr;
@@ -265,9 +273,23 @@ extern "C" pylom_status pylom_pod(const void* X, int64_t N, int64_t M, int64_t l
   e = launch_svd_fp64(ss, ts.Rs, M, UR, M, S, VT, ldvt, 60, energy, r_max, st);
   if (e != cudaSuccess) return cuda_fail(e, "pylom_pod: small SVD");
   if (prof && (e = cudaEventRecord(g_prof.at(call, 3), st)) != cudaSuccess) return cuda_fail(e, "profile");
-  if (gram)
+  if (gram) {
+    if (route == kGramChecked && (e = launch_gram_check(gs, S, st)) != cudaSuccess)
+      return cuda_fail(e, "pylom_pod: modes");
     e = launch_modes_direct(gs, nullptr, S, VT, ldvt, w, mode_kind == PYLOM_MODES_PHYSICAL, U, ldu, r_out, st,
                             prof ? g_prof.at(call, 4) : nullptr);
+    if (route == kGramChecked) {
+      ts.run_if = &hdr->gram_redo;
+      if (e == cudaSuccess)
+        e = mixed ? launch_tsqr_mixed(ts, extra, X, ldx, xtype, w, remove_mean, mean, st)
+                  : launch_tsqr_fp64(ts, X, ldx, xtype, w, remove_mean, mean, st);
+      if (e == cudaSuccess) e = launch_sign_ur(ts, UR, st);
+      if (e == cudaSuccess)
+        e = mixed ? launch_modes_mixed(ts, extra, UR, M, -1, w, mode_kind == PYLOM_MODES_PHYSICAL, (float*)U, ldu,
+                                       r_out, st, nullptr)
+                  : launch_modes_fp64(ts, UR, M, -1, w, mode_kind == PYLOM_MODES_PHYSICAL, (double*)U, ldu, r_out, st);
+    }
+  }
   else if (mixed)
     e = launch_modes_mixed(ts, extra, UR, M, -1, w, mode_kind == PYLOM_MODES_PHYSICAL, (float*)U, ldu, r_out, st,
                            prof ? g_prof.at(call, 4) : nullptr);
@@ -333,7 +355,9 @@ extern "C" size_t pylom_pod_backward_workspace_size(int64_t N, int64_t M, int64_
   // the forward's r_max enters the layout last, so any value gives the same
   // offsets of what is refactored: r is at most r_max
   return pod_backward_bytes(N, M, P, r) +
-         (leaf_rows == 0 ? pod_refactor_bytes(N, M, P, 0, prec == PYLOM_PREC_MIXED_3XTF32) : 0);
+         (leaf_rows == 0 ? pod_refactor_bytes(N, M, P, 0, prec == PYLOM_PREC_MIXED_3XTF32) +
+                               pod_backward_gram_bytes(N, M, r)
+                         : 0);
 }
 
 extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_bytes, int64_t N, int64_t M,
@@ -376,11 +400,29 @@ extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_byt
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(WsHeader), st);
   if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward: header clear");
   if (leaf_rows == 0) {
-    // the forward may have left Y unfactored (its header says so)
+    // the forward may have left Y unfactored (its header says so): then the
+    // form with two products of Y does the call, where the singular values
+    // to invert allow it; else, on a device flag, the Householder form below
+    GramState gs{};
+    gs.hdr = fs.hdr;
+    gs.N = N;
+    gs.ldy = y_ld(N);
+    gs.Y = mixed ? (void*)extra : (void*)fs.Y;
+    gs.f32 = mixed;
+    gram_carve(gs, p2 + svd_state_bytes(M) + align256(sizeof(double) * (size_t)M * M) +
+                       (mixed ? mixed_extra_bytes(N, M, P) : 0), M, r_max);
+    char* bws = (char*)ws + pod_backward_bytes(N, M, P, r);
+    void* dY = pod_backward_dy((char*)ws, N, M, P, r);
+    e = launch_pod_backward_gram(gs, (WsHeader*)ws, S, VT, ldvt, dU, lddu, dS, dVT, lddvt, w,
+                                 mode_kind == PYLOM_MODES_PHYSICAL, r, dY, bws + pod_refactor_bytes(N, M, P, 0, mixed),
+                                 st);
+    if (e == cudaSuccess)
+      e = launch_bw_finalize_gram(dY, mixed, w, remove_mean, dX, lddx, dxtype, N, M, &((WsHeader*)ws)->gram_redo, st);
+    if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward");
     TsqrState os;
     fs.rmax = 0;
     double* UR2 = nullptr;
-    e = launch_refactor(fs, extra, (char*)ws + pod_backward_bytes(N, M, P, r), (WsHeader*)ws, mixed, UR, os, &extra,
+    e = launch_refactor(fs, extra, bws, (WsHeader*)ws, mixed, UR, os, &extra,
                         &UR2, st);
     if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward: factorisation");
     fs = os;

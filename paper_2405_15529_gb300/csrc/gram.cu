@@ -185,6 +185,11 @@ struct GramArgs {
   unsigned long long* G;
   int nJ, items, splits;
   WsHeader* hdr;
+  // Y^T Z instead of Y^T Y: Z (N x NZ), its exponents, all tiles
+  const void* Z;
+  int64_t ldz, NZ;
+  const int* zE;
+  const unsigned* unless;
 };
 
 template <typename TY>
@@ -231,13 +236,22 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int item = blockIdx.x % a.items, split = blockIdx.x / a.items;
   const int half = item % Dig<TY>::HALVES;
+  if (a.unless && *a.unless) return;
   int I = 0, t = item / Dig<TY>::HALVES;
-  while (t >= a.nJ - 2 * I) {
-    t -= a.nJ - 2 * I;
-    ++I;
+  if (a.Z) {
+    I = t / a.nJ;
+    t %= a.nJ;
+  } else {
+    while (t >= a.nJ - 2 * I) {
+      t -= a.nJ - 2 * I;
+      ++I;
+    }
+    t += 2 * I;
   }
-  const int J = 2 * I + t;
-  const bool diag = (J >> 1) == I;       // B's columns are among A's
+  const int J = t;
+  const bool diag = !a.Z && (J >> 1) == I;       // B's columns are among A's
+  const TY* B = (const TY*)(a.Z ? a.Z : a.Y);
+  const int64_t ldb = a.Z ? a.ldz : a.ldy, nB = a.Z ? a.NZ : a.M;
   const int64_t nsum = (a.N + 127) / 128;
   const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
   const TY* Y = (const TY*)a.Y;
@@ -245,15 +259,15 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   const int gw = warp & 7;                       // a stage's eight warps: 16 columns of A and 8 of B each
   const int64_t colA = (int64_t)I * 128 + gw * 16 + c8, colB = (int64_t)J * 64 + gw * 8 + c8;
   const int E0 = colA < a.M ? a.colE[colA] : 128, E1 = colA + 8 < a.M ? a.colE[colA + 8] : 128;
-  const int EB = (!diag && colB < a.M) ? a.colE[colB] : 128;
+  const int EB = (!diag && colB < nB) ? (a.Z ? a.zE : a.colE)[colB] : 128;
   const uint32_t off = (uint32_t)(kg * 128 + c8 * 16);
   // this thread's first row of the unit, and how many stages hold rows of Y
   const int64_t row0 = q0 * 128 + kg * 8;
   const int jin = (int)((a.ldy - row0 + kStK - 1) / kStK);
   const TY* pA = Y + row0 + (colA < a.M ? colA : 0) * a.ldy;
   const TY* pA8 = Y + row0 + (colA + 8 < a.M ? colA + 8 : 0) * a.ldy;
-  const TY* pB = Y + row0 + (colB < a.M ? colB : 0) * a.ldy;
-  const int jA = colA < a.M ? jin : 0, jA8 = colA + 8 < a.M ? jin : 0, jB = colB < a.M ? jin : 0;
+  const TY* pB = B + row0 + (colB < nB ? colB : 0) * ldb;
+  const int jA = colA < a.M ? jin : 0, jA8 = colA + 8 < a.M ? jin : 0, jB = colB < nB ? jin : 0;
   auto fill = [&](int j, unsigned char* st) {
     unsigned char* d = st + off + 2 * gw * kPlaneSbo;
     put_column8<TY>(pA + j * kStK, j < jA, E0, d, kPlaneA);
@@ -272,9 +286,9 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
       const int64_t gj = (int64_t)J * 64 + (warp >> 2) * 16 + c;
-      if (gi < a.M && gj < a.M && gi <= gj) {
-        add_group(a.G, a.M * a.M, gi + gj * a.M, half * 2, acc0[c]);
-        add_group(a.G, a.M * a.M, gi + gj * a.M, half * 2 + 1, acc1[c]);
+      if (gi < a.M && gj < nB && (a.Z || gi <= gj)) {
+        add_group(a.G, a.M * nB, gi + gj * a.M, half * 2, acc0[c]);
+        add_group(a.G, a.M * nB, gi + gj * a.M, half * 2 + 1, acc1[c]);
       }
       acc0[c] = acc1[c] = 0;
     }
@@ -471,11 +485,9 @@ __global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
 // ---------------------------------------------------------------------------
 
 size_t gram_bytes(int64_t M, int64_t rmax) {
-  const int64_t kt = (rmax + 63) / 64, js = (M + kStK - 1) / kStK;
   return align256(sizeof(int) * (size_t)M) + align256(sizeof(long long) * (size_t)5 * M * M) +
          2 * align256(sizeof(double) * (size_t)M * M) + 2 * align256(sizeof(double) * (size_t)kNBC * M) +
-         align256((size_t)kt * js * 8 * kPlaneB) +
-         align256(sizeof(int) * (size_t)kt * 64);
+         product_planes_bytes(M, 0, rmax);
 }
 
 void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax) {
@@ -524,17 +536,46 @@ static int row_splits(int64_t items, int64_t nsum, int sms) {
 }
 
 template <typename TY>
-static cudaError_t gram_launch(const GramState& g, int sms, cudaStream_t st) {
+static cudaError_t gram_launch(const GramState& g, int sms, const void* Z, int64_t ldz, int64_t NZ, const int* zE,
+                               long long* G, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
   constexpr int S = Dig<TY>::S;
   constexpr size_t smem = (size_t)Dig<TY>::NST * S * (kPlaneA + kPlaneB);
   cudaError_t e = ensure_dyn_smem((const void*)gram_kernel<TY>, smem);
   if (e != cudaSuccess) return e;
-  const int nJ = (int)((g.M + 63) / 64), nI = (int)((g.M + 127) / 128);
+  const int nJ = (int)(((Z ? NZ : g.M) + 63) / 64), nI = (int)((g.M + 127) / 128);
   int tiles = 0;
-  for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;
-  GramArgs a{g.Y, g.ldy, g.N, g.M, g.colE, (unsigned long long*)g.G, nJ, tiles * Dig<TY>::HALVES, 1, g.hdr};
+  for (int I = 0; I < nI; ++I) tiles += Z ? nJ : nJ - 2 * I;
+  GramArgs a{g.Y, g.ldy, g.N, g.M, g.colE, (unsigned long long*)G, nJ, tiles * Dig<TY>::HALVES, 1, hdr, Z, ldz, NZ, zE,
+             unless};
   a.splits = row_splits(a.items, (g.N + 127) / 128, sms);
   gram_kernel<TY><<<(unsigned)(a.items * a.splits), kDigThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+// integers of Y^T Z -> W
+__global__ void cross_sum_kernel(GramState g, int64_t NZ, const int* zE, const long long* G, double* W, int groups, int lb,
+                                 int bias) {
+  const int64_t n = g.M * NZ;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
+    const dd s = group_sum(G, n, idx, groups, lb);
+    W[idx] = scalbn(scalbn(s.h + s.l, g.colE[idx % g.M] - bias), zE[idx / g.M] - bias + 64);
+  }
+}
+
+cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, long long* G,
+                         double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
+  cudaError_t e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int groups = g.f32 ? 3 : 5;
+  e = cudaMemsetAsync(G, 0, sizeof(long long) * (size_t)groups * g.M * NZ, st);
+  if (e != cudaSuccess) return e;
+  e = g.f32 ? gram_launch<float>(g, sms, Z, ldz, NZ, zE, G, unless, hdr, st)
+            : gram_launch<double>(g, sms, Z, ldz, NZ, zE, G, unless, hdr, st);
+  if (e != cudaSuccess) return e;
+  cross_sum_kernel<<<64, 256, 0, st>>>(g, NZ, zE, G, W, groups, g.f32 ? gram_base<float>(0) : 0,
+                                       g.f32 ? fix_bias<float>() : fix_bias<double>());
   return cudaGetLastError();
 }
 
@@ -552,7 +593,8 @@ cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xt
   if (g.f32) e = xtype == PYLOM_F32 ? prologue<float, float>(pa, sms, st) : prologue<double, float>(pa, sms, st);
   else e = xtype == PYLOM_F32 ? prologue<float, double>(pa, sms, st) : prologue<double, double>(pa, sms, st);
   if (e != cudaSuccess) return e;
-  e = g.f32 ? gram_launch<float>(g, sms, st) : gram_launch<double>(g, sms, st);
+  e = g.f32 ? gram_launch<float>(g, sms, nullptr, 0, 0, nullptr, g.G, nullptr, g.hdr, st)
+            : gram_launch<double>(g, sms, nullptr, 0, 0, nullptr, g.G, nullptr, g.hdr, st);
   if (e != cudaSuccess) return e;
   if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
   CholArgs c{g, R, groups, g.f32 ? gram_base<float>(0) : gram_base<double>(0),

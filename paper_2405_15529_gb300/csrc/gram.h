@@ -21,6 +21,26 @@ struct GramState {
   int64_t rmax;
 };
 
+// U = [Y Z] [C; D]: a second left factor Z (N x NZ, nullable) beside g.Y, the
+// coefficients given as doubles (C: M x cols, D: NZ x cols) or, C null, V_r
+// S_r^-1 from VT and S.  cols < 0: hdr->r columns.  Cd, Ce: digit planes and
+// exponents of the coefficients (product_planes_bytes).
+struct ProductArgs {
+  const void* Y;
+  int64_t ldy, N, M;
+  const int* colE;
+  const void* Z;
+  int64_t ldz, NZ;
+  const int* zE;
+  const double *C, *D, *S, *VT;
+  int64_t ldc, ldd, ldvt;
+  int64_t cols, cols_max;
+  unsigned char* Cd;
+  int* Ce;
+  const unsigned* unless;   // nullable: nothing to do when *unless is not 0
+  const WsHeader* hdr;
+};
+
 size_t gram_bytes(int64_t M, int64_t rmax);
 void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax);
 
@@ -35,5 +55,37 @@ cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xt
 cudaError_t launch_modes_direct(const GramState& g, const double* C, const double* S, const double* VT, int64_t ldvt,
                                 const double* w, int physical, void* U, int64_t ldu, int64_t* r_out,
                                 cudaStream_t st, cudaEvent_t mid);
+
+// W = Y^T Z (M x NZ, ld M) from the same integer products.  G: 5 M NZ integers.
+cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, long long* G,
+                         double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st);
+// The product above into U (binary32 if f32, else binary64; ld ldu).
+size_t product_planes_bytes(int64_t M, int64_t NZ, int64_t cols);
+cudaError_t launch_product(const ProductArgs& p, bool f32, void* U, int64_t ldu, WsHeader* hdr, cudaStream_t st);
+
+// The adjoint without reflectors (pod_backward_gram.cu); `f` the forward's
+// state.  hdr->gram_redo = 1 afterwards: nothing was done.
+size_t pod_backward_gram_bytes(int64_t N, int64_t M, int64_t r);
+cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const double* S, const double* VT, int64_t ldvt,
+                                     const double* dU, int64_t lddu, const double* dS, const double* dVT,
+                                     int64_t lddvt, const double* w, int physical, int64_t r, void* dY, char* base,
+                                     cudaStream_t st);
+// pod_backward.cu: C = alpha op(A) op(B) + beta C, and C = diag(1 / S) VT (rows of them), unless *unless
+cudaError_t launch_bw_gemm(int ta, int tb, int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda,
+                           const double* B, int64_t ldb, double beta, double* C, int64_t ldc, const unsigned* unless,
+                           cudaStream_t st);
+cudaError_t launch_bw_scale_rows(const double* VT, int64_t ldvt, const double* S, double* C, int64_t rows, int64_t M,
+                                 const unsigned* unless, cudaStream_t st);
+// pod_backward.cu: dX = W^(1/2) dY, minus row means, where *redo is 0
+cudaError_t launch_bw_finalize_gram(const void* dY, bool f32, const double* w, int remove_mean, void* dX, int64_t lddx,
+                                    int dxtype, int64_t N, int64_t M, const unsigned* redo, cudaStream_t st);
+
+// Whether the kept values are large enough for the direct product (hdr->r,
+// S known): else hdr->gram_redo = 1 and hdr->gram_y = 0, and the Householder
+// route on `ts` (ts.run_if = &hdr->gram_redo) gives the modes.
+cudaError_t launch_gram_check(const GramState& g, const double* S, cudaStream_t st);
+// The rows of U_R with the signs of the Householder R's diagonal (the Gram
+// route's R has a non-negative one), for the Householder route after a redo.
+cudaError_t launch_sign_ur(const TsqrState& ts, double* UR, cudaStream_t st);
 
 }  // namespace pylom

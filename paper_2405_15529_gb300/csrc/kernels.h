@@ -48,6 +48,9 @@ struct TsqrState {
   // (mixed extra region: `shiftx`) bytes away from these pointers
   const unsigned* gram_y;
   int64_t shift, shiftx;
+  // if given, the kernels on this state do nothing while *run_if is 0 (the
+  // Householder route behind the Gram route of the same call)
+  const unsigned* run_if;
 };
 
 // leading dimension of the working copies (binary64 Y, binary32 Yf): whole
@@ -57,6 +60,7 @@ __host__ __device__ __forceinline__ int64_t y_ld(int64_t N) { return (N + 7) & ~
 #ifdef __CUDACC__
 // kernels that factor Y: nothing to do when the forward has done it
 __device__ __forceinline__ bool already_factored(const TsqrState& s) { return s.gram_y && *s.gram_y == 0; }
+__device__ __forceinline__ bool passed_over(const TsqrState& s) { return s.run_if && *s.run_if == 0; }
 // kernels that apply the factorisation: take the forward's where it exists
 template <class T>
 __device__ __forceinline__ void shift_ptr(T*& p, int64_t bytes) {
@@ -150,6 +154,7 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
 // Room in the backward's workspace for a factorisation of the forward's Y
 // (forwards with the automatic leaf height may have left Y unfactored), and
 // its state: os (and *extra, mixed path) in the backward's workspace.
+void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r);
 size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed);
 cudaError_t launch_refactor(const TsqrState& fs, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
                             const double* UR, TsqrState& os, char** extra, double** UR_out, cudaStream_t st);

@@ -19,27 +19,35 @@
 
 namespace pylom {
 
-// Digit planes of C' = diag(2^(E_j - bias)) C, one block per column of C;
-// planes of column tile kt and stage js at ((kt * stages + js) * S) kPlaneB
-// bytes.  C null: C = V_r S_r^-1.
+__device__ __forceinline__ int64_t product_cols(const ProductArgs& p) { return p.cols >= 0 ? p.cols : (int64_t)p.hdr->r; }
+// stages of the two left factors: each starts a stage of its own
+__host__ __device__ __forceinline__ int product_stages(int64_t n) { return (int)((n + kStK - 1) / kStK); }
+
+// Digit planes of the coefficients times their rows' scales 2^(E - bias),
+// one block per column; planes of column tile kt and stage js at
+// ((kt * stages + js) * S) kPlaneB bytes.
 template <typename TY>
-__global__ void __launch_bounds__(128) coef_digits_kernel(GramState g, const double* C, const double* S,
-                                                         const double* VT, int64_t ldvt) {
+__global__ void __launch_bounds__(128) coef_digits_kernel(ProductArgs p) {
   constexpr int SD = Dig<TY>::S;
   __shared__ int s_e;
-  const int64_t k = blockIdx.x, r = g.hdr->r, M = g.M;
+  if (p.unless && *p.unless) return;
+  const int64_t k = blockIdx.x, r = product_cols(p);
   if (k >= (r + 63) / 64 * 64) return;
-  const int64_t stages = (M + kStK - 1) / kStK;
+  const int s1 = product_stages(p.M), stages = s1 + product_stages(p.NZ);
   if (threadIdx.x == 0) s_e = kMinField64;
   __syncthreads();
-  const double sk = (!C && k < r) ? S[k] : 1.0;
+  const double sk = (!p.C && k < r) ? p.S[k] : 1.0;
   auto value = [&](int64_t j) {
-    if (j >= M || k >= r) return 0.0;
-    const double c = C ? C[j + k * M] : VT[k + j * ldvt] / sk;
-    return scalbn(c, g.colE[j] - fix_bias<TY>());
+    if (k >= r) return 0.0;
+    if (j < (int64_t)s1 * kStK) {
+      if (j >= p.M) return 0.0;
+      return scalbn(p.C ? p.C[j + k * p.ldc] : p.VT[k + j * p.ldvt] / sk, p.colE[j] - fix_bias<TY>());
+    }
+    j -= (int64_t)s1 * kStK;
+    return j < p.NZ ? scalbn(p.D[j + k * p.ldd], p.zE[j] - fix_bias<TY>()) : 0.0;
   };
   int e = kMinField64;
-  for (int64_t j = threadIdx.x; j < M; j += blockDim.x) {
+  for (int64_t j = threadIdx.x; j < (int64_t)stages * kStK; j += blockDim.x) {
     const int ej = exp_field(value(j));
     e = ej > e ? ej : e;
   }
@@ -47,65 +55,67 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(GramState g, const dou
   if ((threadIdx.x & 31) == 0) atomicMax(&s_e, e);
   __syncthreads();
   e = s_e;
-  if (threadIdx.x == 0) g.Ce[k] = e;
-  for (int64_t j0 = (int64_t)threadIdx.x * 8; j0 < stages * kStK; j0 += (int64_t)blockDim.x * 8) {
+  if (threadIdx.x == 0) p.Ce[k] = e;
+  for (int64_t j0 = (int64_t)threadIdx.x * 8; j0 < (int64_t)stages * kStK; j0 += (int64_t)blockDim.x * 8) {
     uint2 w[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       int64_t v = to_fixed(value(j0 + i), e);
-      // binary32 Y: the coefficients keep 38 of the 62 bits (rounded)
+      // binary32 left factors: the coefficients keep 38 of the 62 bits (rounded)
       if (SD == 5) v = (v + (1ll << 23)) >> 24;
       w[i] = bias_digits(v);
     }
-    const int64_t js = j0 / kStK;
-    unsigned char* dst = g.Cd + (((k / 64) * stages + js) * SD) * (int64_t)kPlaneB + ((k & 63) >> 3) * kPlaneSbo +
+    unsigned char* dst = p.Cd + (((k / 64) * stages + j0 / kStK) * SD) * (int64_t)kPlaneB + ((k & 63) >> 3) * kPlaneSbo +
                          ((j0 % kStK) >> 3) * 128 + (k & 7) * 16;
     store_digits<SD>(w, dst, kPlaneB);
   }
 }
 
 template <typename TY>
-__global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(GramState g, const double* S0, const double* w,
+__global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArgs p, const double* S0, const double* w,
                                                                      int physical, TY* U, int64_t ldu,
-                                                                     int64_t* r_out) {
+                                                                     int64_t* r_out, WsHeader* hdr) {
   constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST, LB = Dig<TY>::LBM;
   extern __shared__ __align__(1024) unsigned char gsm[];
   __shared__ __align__(8) DigitBarriers<NST> bar;
+  if (p.unless && *p.unless) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t N = g.N, M = g.M, r = g.hdr->r;
+  const int64_t N = p.N, r = product_cols(p);
   // a zero matrix keeps all modes (there is no energy to share): unit vectors
   const bool zero = S0 && S0[0] == 0.0;
   if (blockIdx.x == 0 && tid == 0 && r_out) *r_out = r;
   const int64_t ktiles = (r + 63) / 64, tiles = (N + 127) / 128 * ktiles;
-  const int stages = (int)((M + kStK - 1) / kStK), m32 = (int)M;
+  const int s1 = product_stages(p.M), stages = s1 + product_stages(p.NZ);
   const uint32_t kt32 = (uint32_t)ktiles;
-  const TY* Y = (const TY*)g.Y;
   const int rl = tid & 127, kh = (tid >> 7) & 1; // row of the tile, half of the stage's columns
   const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
   const int mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
   auto fill = [&](int t, int js, unsigned char* st) {
     const uint32_t tile = blockIdx.x + t * gridDim.x;
     const int64_t row = (int64_t)(tile / kt32) * 128 + rl;
-    const bool rin = row < N;
+    const bool rin = row < N, second = js >= s1;
+    const TY* Y = (const TY*)(second ? p.Z : p.Y);
+    const int64_t ld = second ? p.ldz : p.ldy;
+    const int* ex = second ? p.zE : p.colE;
+    const int m32 = (int)(second ? p.NZ : p.M), j0 = (second ? js - s1 : js) * kStK;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int kg = 2 * kh + h;
-      const int c0 = js * kStK + kg * 8;
-      const TY* p = Y + row + c0 * g.ldy;
+      const int kg = 2 * kh + h, c0 = j0 + kg * 8;
+      const TY* q = Y + row + c0 * ld;
       TY y[8];
       int E[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const bool in = c0 + i < m32;
-        y[i] = (in && rin) ? __ldg(p + i * g.ldy) : (TY)0;
-        E[i] = in ? __ldg(g.colE + c0 + i) : 128;
+        y[i] = (in && rin) ? __ldg(q + i * ld) : (TY)0;
+        E[i] = in ? __ldg(ex + c0 + i) : 128;
       }
       put_digits(y, E, st + offA + kg * 128, kPlaneA);
     }
   };
   auto bsrc = [&](int t, int js) {
     const uint32_t tile = blockIdx.x + t * gridDim.x;
-    return g.Cd + ((int64_t)(tile % kt32) * stages + js) * (S * kPlaneB);
+    return p.Cd + ((int64_t)(tile % kt32) * stages + js) * (S * kPlaneB);
   };
   auto store = [&](int t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
     // the tile's rows of U: lanes hold consecutive rows
@@ -118,7 +128,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(GramState 
       const int k = k0 + c;
       if (k >= r) break;     // uniform over the warp
       if (row < N) {
-        const int pk = 8 * LB + __ldg(g.Ce + k) - fix_bias<double>() + (S == 5 ? 24 : 0);
+        const int pk = 8 * LB + __ldg(p.Ce + k) - fix_bias<double>() + (S == 5 ? 24 : 0);
         double v = __fma_rn((double)acc1[c], 4294967296.0, (double)acc0[c]);
         v = (pk > -900 && pk < 900) ? v * __hiloint2double((pk + 1023) << 20, 0) : scalbn(v, pk);
         if (zero) v = row == k ? 1.0 : 0.0;
@@ -127,35 +137,93 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(GramState 
       }
     }
   };
-  product_pipeline<S, NST, LB>(bar, gsm, mine, stages, g.hdr, fill, bsrc, store);
+  product_pipeline<S, NST, LB>(bar, gsm, mine, stages, hdr, fill, bsrc, store);
+}
+
+// Smallest kept value, relative to the largest, for which Y V_r S_r^-1 is
+// taken: its rounding grows by sigma_1 / sigma_r.
+constexpr double kKeptLevel64 = 1e-4, kKeptLevel32 = 1e-5;
+
+__global__ void gram_check_kernel(WsHeader* hdr, const double* S, double level) {
+  const long long r = hdr->r;
+  if (r >= 1 && S[0] > 0.0 && !(S[r - 1] >= level * S[0])) {
+    hdr->gram_redo = 1;
+    hdr->gram_y = 0;
+  }
+}
+
+cudaError_t launch_gram_check(const GramState& g, const double* S, cudaStream_t st) {
+  gram_check_kernel<<<1, 1, 0, st>>>(g.hdr, S, g.f32 ? kKeptLevel32 : kKeptLevel64);
+  return cudaGetLastError();
+}
+
+__global__ void sign_ur_kernel(TsqrState s, double* UR) {
+  if (passed_over(s)) return;
+  const int64_t M = s.M;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % M;
+    if (s.Rs[i + i * M] < 0.0) UR[idx] = -UR[idx];
+  }
+}
+
+cudaError_t launch_sign_ur(const TsqrState& ts, double* UR, cudaStream_t st) {
+  sign_ur_kernel<<<64, 256, 0, st>>>(ts, UR);
+  return cudaGetLastError();
 }
 
 template <typename TY>
-static cudaError_t run(const GramState& g, const double* C, const double* S, const double* VT, int64_t ldvt,
-                       const double* w, int physical, void* U, int64_t ldu, int64_t* r_out, int sms,
-                       cudaStream_t st, cudaEvent_t mid) {
+static cudaError_t run(const ProductArgs& p, const double* S0, const double* w, int physical, void* U, int64_t ldu,
+                       int64_t* r_out, WsHeader* hdr, cudaStream_t st, cudaEvent_t mid) {
   constexpr size_t smem = (size_t)Dig<TY>::NST * Dig<TY>::S * (kPlaneA + kPlaneB);
-  cudaError_t e = ensure_dyn_smem((const void*)modes_direct_kernel<TY>, smem);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const int64_t kt = (g.rmax + 63) / 64;
-  coef_digits_kernel<TY><<<(unsigned)(kt * 64), 128, 0, st>>>(g, C, S, VT, ldvt);
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = ensure_dyn_smem((const void*)modes_direct_kernel<TY>, smem)) != cudaSuccess) return e;
+  const int64_t kt = (p.cols_max + 63) / 64;
+  coef_digits_kernel<TY><<<(unsigned)(kt * 64), 128, 0, st>>>(p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
-  int64_t grid = (g.N + 127) / 128 * kt;
+  int64_t grid = (p.N + 127) / 128 * kt;
   if (grid > sms) grid = sms;
-  modes_direct_kernel<TY><<<(unsigned)grid, kDigThreads, smem, st>>>(g, C ? nullptr : S, w, physical, (TY*)U, ldu, r_out);
+  modes_direct_kernel<TY><<<(unsigned)grid, kDigThreads, smem, st>>>(p, S0, w, physical, (TY*)U, ldu, r_out, hdr);
   return cudaGetLastError();
+}
+
+size_t product_planes_bytes(int64_t M, int64_t NZ, int64_t cols) {
+  const int64_t kt = (cols + 63) / 64;
+  return align256((size_t)kt * (product_stages(M) + product_stages(NZ)) * 8 * kPlaneB) +
+         align256(sizeof(int) * (size_t)kt * 64);
+}
+
+cudaError_t launch_product(const ProductArgs& p, bool f32, void* U, int64_t ldu, WsHeader* hdr, cudaStream_t st) {
+  return f32 ? run<float>(p, nullptr, nullptr, 0, U, ldu, nullptr, hdr, st, nullptr)
+             : run<double>(p, nullptr, nullptr, 0, U, ldu, nullptr, hdr, st, nullptr);
 }
 
 cudaError_t launch_modes_direct(const GramState& g, const double* C, const double* S, const double* VT, int64_t ldvt,
                                 const double* w, int physical, void* U, int64_t ldu, int64_t* r_out,
                                 cudaStream_t st, cudaEvent_t mid) {
-  cudaError_t e;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  return g.f32 ? run<float>(g, C, S, VT, ldvt, w, physical, U, ldu, r_out, sms, st, mid)
-               : run<double>(g, C, S, VT, ldvt, w, physical, U, ldu, r_out, sms, st, mid);
+  ProductArgs p{};
+  p.Y = g.Y;
+  p.ldy = g.ldy;
+  p.N = g.N;
+  p.M = g.M;
+  p.colE = g.colE;
+  p.C = C;
+  p.ldc = g.M;
+  p.S = S;
+  p.VT = VT;
+  p.ldvt = ldvt;
+  p.cols = -1;
+  p.cols_max = g.rmax;
+  p.Cd = g.Cd;
+  p.Ce = g.Ce;
+  p.hdr = g.hdr;
+  const double* S0 = C ? nullptr : S;
+  return g.f32 ? run<float>(p, S0, w, physical, U, ldu, r_out, g.hdr, st, mid)
+               : run<double>(p, S0, w, physical, U, ldu, r_out, g.hdr, st, mid);
 }
 
 }  // namespace pylom

@@ -20,6 +20,7 @@
 // singular); in the composition R^-T cancels, and only the singular values
 // of modes that carry a cotangent are inverted.  Degenerate pairs
 // (s_i == s_j, i != j) contribute no coupling term.
+#include "gram.h"
 #include "kernels.h"
 #include "reflectors.cuh"
 
@@ -27,7 +28,8 @@ namespace pylom {
 
 // dU (N x r) -> C (N x r, ld N), with W^(-1/2) applied for physical modes.
 __global__ void bw_load_du_kernel(const double* dU, int64_t lddu, const double* w, int physical,
-                                  double* C, int64_t N, int64_t r) {
+                                  double* C, int64_t N, int64_t r, const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N * r; idx += stride) {
     const int64_t n = idx % N, c = idx / N;
@@ -50,6 +52,7 @@ __global__ void __launch_bounds__(kLeafThreads) bw_leaf_qt_kernel(TsqrState s, d
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  if (passed_over(s)) return;
   select_factors(s);
   const double* A = s.Y + r0;
   double* Cl = C + r0;
@@ -73,7 +76,7 @@ __global__ void __launch_bounds__(kLeafThreads) bw_leaf_qt_kernel(TsqrState s, d
 __global__ void __launch_bounds__(256) bw_up_pass_kernel(TsqrState s, double* Z, int64_t r, int64_t step) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int64_t left = (int64_t)blockIdx.x * 2 * step, right = left + step;
-  if (right >= s.P) return;
+  if (right >= s.P || passed_over(s)) return;
   select_factors(s);
   const int64_t col = (int64_t)blockIdx.y * nwarps + warp;
   if (col >= r) return;
@@ -98,7 +101,8 @@ __global__ void __launch_bounds__(256) bw_up_pass_kernel(TsqrState s, double* Z,
 // C = alpha op(A) op(B) + beta C, small FP64 matrices, 16 x 16 shared tiles.
 __global__ void bw_gemm_kernel(int ta, int tb, int64_t m, int64_t n, int64_t k, double alpha,
                                const double* A, int64_t lda, const double* B, int64_t ldb,
-                               double beta, double* C, int64_t ldc) {
+                               double beta, double* C, int64_t ldc, const unsigned* run_if, unsigned want) {
+  if (run_if && (*run_if != 0) != (want != 0)) return;
   __shared__ double sa[16][17], sb[16][17];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t i = (int64_t)blockIdx.y * 16 + ty;   // row of C
@@ -122,7 +126,8 @@ __global__ void bw_gemm_kernel(int ta, int tb, int64_t m, int64_t n, int64_t k, 
 
 // K = (F o G1) S + diag(dS) + S (F o G2) with G = A - A^T, in place of K.
 __global__ void bw_svd_core_kernel(const double* A1, const double* A2, const double* S,
-                                   const double* dS, double* K, int64_t M) {
+                                   const double* dS, double* K, int64_t M, const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M; idx += stride) {
     const int64_t i = idx % M, j = idx / M;
@@ -141,7 +146,8 @@ __global__ void bw_svd_core_kernel(const double* A1, const double* A2, const dou
 
 // C (rows x M, ld rows) = diag(1 / S[0:rows]) VT[0:rows, :].
 __global__ void bw_scale_rows_kernel(const double* VT, int64_t ldvt, const double* S, double* C,
-                                     int64_t rows, int64_t M) {
+                                     int64_t rows, int64_t M, const unsigned* run_if, unsigned want) {
+  if (run_if && (*run_if != 0) != (want != 0)) return;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < rows * M; idx += stride) {
     const int64_t i = idx % rows, j = idx / rows;
@@ -153,7 +159,8 @@ __global__ void bw_scale_rows_kernel(const double* VT, int64_t ldvt, const doubl
 // 8-row tiles and sweeps all 8-column tiles; k = r in steps of 4.
 __global__ void __launch_bounds__(256) bw_add_du_c_kernel(const double* dU, const double* Cm,
                                                           int64_t ldcm, double* dY, int64_t N,
-                                                          int64_t M, int64_t r) {
+                                                          int64_t M, int64_t r, const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -179,7 +186,8 @@ __global__ void __launch_bounds__(256) bw_add_du_c_kernel(const double* dU, cons
 // dX = W^(1/2) dY, then minus each row's mean (adjoint of mean removal).
 template <typename TX, typename TY>
 __global__ void bw_finalize_kernel(const TY* dY, const double* w, int remove_mean, TX* dX,
-                                   int64_t lddx, int64_t N, int64_t M) {
+                                   int64_t lddx, int64_t N, int64_t M, const unsigned* run_if, unsigned want) {
+  if (run_if && (*run_if != 0) != (want != 0)) return;
   for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N;
        n += (int64_t)gridDim.x * blockDim.x) {
     const double sw = w ? sqrt(w[n]) : 1.0;
@@ -195,7 +203,8 @@ __global__ void bw_finalize_kernel(const TY* dY, const double* w, int remove_mea
 
 // Mixed path: dU (N x r, binary64) -> C (FP32, ld N), W^(-1/2) for physical modes.
 __global__ void bw_load_du_f32_kernel(const double* dU, int64_t lddu, const double* w, int physical, float* C,
-                                      int64_t N, int64_t r) {
+                                      int64_t N, int64_t r, const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N * r; idx += stride) {
     const int64_t n = idx % N, c = idx / N;
@@ -209,7 +218,9 @@ __global__ void bw_load_du_f32_kernel(const double* dU, int64_t lddu, const doub
 // FP32; Cm staged per block in shared memory (r <= M <= 4096 columns are
 // taken 64 at a time).
 __global__ void __launch_bounds__(256) bw_add_du_c_f32_kernel(const float* C, const double* Cm, int64_t ldcm,
-                                                              float* dY, int64_t N, int64_t M, int64_t r) {
+                                                              float* dY, int64_t N, int64_t M, int64_t r,
+                                                              const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
   extern __shared__ float scm[];   // r x 64
   for (int64_t m0 = 0; m0 < M; m0 += 64) {
     const int64_t mw = (M - m0) < 64 ? (M - m0) : 64;
@@ -254,6 +265,7 @@ cudaError_t launch_refactor(const TsqrState& fs, const char* fwd_extra, char* ba
   char* oextra = mixed ? own + tsqr_state_bytes(fs.N, fs.M, fs.P, fs.rmax, false) : nullptr;
   tsqr_state_carve(os, own, fs.N, fs.M, fs.P, fs.rmax, !mixed);
   os.hdr = hdr;
+  os.run_if = &hdr->gram_redo;
   os.gram_y = &fs.hdr->gram_y;
   os.shift = (const char*)fs.tau - (const char*)os.tau;
   os.shiftx = mixed ? fwd_extra - oextra : 0;
@@ -308,11 +320,43 @@ static BwLayout carve_backward(char* base, int64_t N, int64_t M, int64_t P, int6
   return L;
 }
 
+// where the adjoint's dY (N x M) lies in the workspace
+void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r) {
+  return carve_backward(base, N, M, P, r).dY;
+}
+
 static cudaError_t gemm(int ta, int tb, int64_t m, int64_t n, int64_t k, double alpha, const double* A,
                         int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc,
-                        cudaStream_t st) {
+                        const unsigned* run_if, cudaStream_t st) {
   dim3 blk(16, 16), grd((unsigned)((n + 15) / 16), (unsigned)((m + 15) / 16));
-  bw_gemm_kernel<<<grd, blk, 0, st>>>(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  bw_gemm_kernel<<<grd, blk, 0, st>>>(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, run_if, 1u);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_bw_gemm(int ta, int tb, int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda,
+                           const double* B, int64_t ldb, double beta, double* C, int64_t ldc, const unsigned* unless,
+                           cudaStream_t st) {
+  dim3 blk(16, 16), grd((unsigned)((n + 15) / 16), (unsigned)((m + 15) / 16));
+  bw_gemm_kernel<<<grd, blk, 0, st>>>(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, unless, 0u);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_bw_scale_rows(const double* VT, int64_t ldvt, const double* S, double* C, int64_t rows, int64_t M,
+                                 const unsigned* unless, cudaStream_t st) {
+  bw_scale_rows_kernel<<<64, 256, 0, st>>>(VT, ldvt, S, C, rows, M, unless, 0u);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_bw_finalize_gram(const void* dY, bool f32, const double* w, int remove_mean, void* dX, int64_t lddx,
+                                    int dxtype, int64_t N, int64_t M, const unsigned* redo, cudaStream_t st) {
+  if (f32 && dxtype == PYLOM_F32)
+    bw_finalize_kernel<float, float><<<1024, 256, 0, st>>>((const float*)dY, w, remove_mean, (float*)dX, lddx, N, M, redo, 0u);
+  else if (f32)
+    bw_finalize_kernel<double, float><<<1024, 256, 0, st>>>((const float*)dY, w, remove_mean, (double*)dX, lddx, N, M, redo, 0u);
+  else if (dxtype == PYLOM_F32)
+    bw_finalize_kernel<float, double><<<1024, 256, 0, st>>>((const double*)dY, w, remove_mean, (float*)dX, lddx, N, M, redo, 0u);
+  else
+    bw_finalize_kernel<double, double><<<1024, 256, 0, st>>>((const double*)dY, w, remove_mean, (double*)dX, lddx, N, M, redo, 0u);
   return cudaGetLastError();
 }
 
@@ -322,6 +366,7 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
                                 int physical, int64_t r, void* dX, int64_t lddx, int dxtype,
                                 char* bw_base, char* mixed_extra, cudaStream_t st) {
   const int64_t N = fs.N, M = fs.M, P = fs.P;
+  const unsigned* run_if = fs.run_if;   // null: always
   BwLayout L = carve_backward(bw_base, N, M, P, r);
   const bool mixed = mixed_extra != nullptr;   // FP32 reflectors of a mixed-precision forward
   float* C32 = (float*)L.C;
@@ -329,7 +374,7 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
   cudaError_t e;
   // 1. Z = Q^T dU
   if (mixed && dU && r > 0) {
-    bw_load_du_f32_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, C32, N, r);
+    bw_load_du_f32_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, C32, N, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_leaf_qt_mixed(fs, mixed_extra, C32, r, L.Z, st)) != cudaSuccess) return e;
     for (int64_t step = 1; step < P; step <<= 1) {
@@ -339,7 +384,7 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
   } else if (dU && r > 0) {
-    bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r);
+    bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = ensure_dyn_smem((const void*)bw_leaf_qt_kernel, kLeafSmemBytes)) != cudaSuccess) return e;
     bw_leaf_qt_kernel<<<(unsigned)P, kLeafThreads, kLeafSmemBytes, st>>>(fs, L.C, L.Z, r);
@@ -356,56 +401,56 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
   }
   // 2. small algebra.  A1 = U_R^T Zt (only the first r columns are nonzero)
   if ((e = cudaMemsetAsync(L.A1, 0, sizeof(double) * (size_t)M * M, st)) != cudaSuccess) return e;
-  if (r > 0 && (e = gemm(1, 0, M, r, M, 1.0, UR, M, L.Z, M, 0.0, L.A1, M, st)) != cudaSuccess) return e;
+  if (r > 0 && (e = gemm(1, 0, M, r, M, 1.0, UR, M, L.Z, M, 0.0, L.A1, M, run_if, st)) != cudaSuccess) return e;
   // A2 = V^T dV = VT dVT^T
   if (dVT) {
-    if ((e = gemm(0, 1, M, M, M, 1.0, VT, ldvt, dVT, lddvt, 0.0, L.A2, M, st)) != cudaSuccess) return e;
+    if ((e = gemm(0, 1, M, M, M, 1.0, VT, ldvt, dVT, lddvt, 0.0, L.A2, M, run_if, st)) != cudaSuccess) return e;
   } else if ((e = cudaMemsetAsync(L.A2, 0, sizeof(double) * (size_t)M * M, st)) != cudaSuccess) {
     return e;
   }
-  bw_svd_core_kernel<<<256, 256, 0, st>>>(L.A1, L.A2, S, dS, L.K, M);
+  bw_svd_core_kernel<<<256, 256, 0, st>>>(L.A1, L.A2, S, dS, L.K, M, run_if);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // dR = U_R K V^T = U_R (K VT), into Bm
-  if ((e = gemm(0, 0, M, M, M, 1.0, L.K, M, VT, ldvt, 0.0, L.T1, M, st)) != cudaSuccess) return e;
-  if ((e = gemm(0, 0, M, M, M, 1.0, UR, M, L.T1, M, 0.0, L.Bm, M, st)) != cudaSuccess) return e;
+  if ((e = gemm(0, 0, M, M, M, 1.0, L.K, M, VT, ldvt, 0.0, L.T1, M, run_if, st)) != cudaSuccess) return e;
+  if ((e = gemm(0, 0, M, M, M, 1.0, UR, M, L.T1, M, 0.0, L.Bm, M, run_if, st)) != cudaSuccess) return e;
   if (r > 0) {
     // C = S_r^-1 V_r^T (r x M); B -= Zt S^-1 V^T = Z C
-    bw_scale_rows_kernel<<<256, 256, 0, st>>>(VT, ldvt, S, L.Cm, r, M);
+    bw_scale_rows_kernel<<<256, 256, 0, st>>>(VT, ldvt, S, L.Cm, r, M, run_if, 1u);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = gemm(0, 0, M, M, r, -1.0, L.Z, M, L.Cm, r, 1.0, L.Bm, M, st)) != cudaSuccess) return e;
+    if ((e = gemm(0, 0, M, M, r, -1.0, L.Z, M, L.Cm, r, 1.0, L.Bm, M, run_if, st)) != cudaSuccess) return e;
   }
   // 3. dY = Q [B; 0] (top-down pass + leaf products, r = M columns) ...
-  TsqrState ds = fs;
+  TsqrState ds = fs;   // (with fs.run_if)
   ds.B = L.B;
   ds.rmax = M;
   if (mixed) {
     e = launch_modes_mixed(ds, mixed_extra, L.Bm, M, M, nullptr, 0, dY32, N, nullptr, st, nullptr);
     if (e != cudaSuccess) return e;
     if (dU && r > 0) {
-      bw_load_du_f32_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, C32, N, r);
+      bw_load_du_f32_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, C32, N, r, run_if);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      bw_add_du_c_f32_kernel<<<1216, 256, sizeof(float) * (size_t)r * 64, st>>>(C32, L.Cm, r, dY32, N, M, r);
+      bw_add_du_c_f32_kernel<<<1216, 256, sizeof(float) * (size_t)r * 64, st>>>(C32, L.Cm, r, dY32, N, M, r, run_if);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (dxtype == PYLOM_F32)
-      bw_finalize_kernel<float, float><<<1024, 256, 0, st>>>(dY32, w, remove_mean, (float*)dX, lddx, N, M);
+      bw_finalize_kernel<float, float><<<1024, 256, 0, st>>>(dY32, w, remove_mean, (float*)dX, lddx, N, M, run_if, 1u);
     else
-      bw_finalize_kernel<double, float><<<1024, 256, 0, st>>>(dY32, w, remove_mean, (double*)dX, lddx, N, M);
+      bw_finalize_kernel<double, float><<<1024, 256, 0, st>>>(dY32, w, remove_mean, (double*)dX, lddx, N, M, run_if, 1u);
     return cudaGetLastError();
   }
   if ((e = launch_modes_fp64(ds, L.Bm, M, M, nullptr, 0, L.dY, N, nullptr, st)) != cudaSuccess) return e;
   // ... + dU_w C (dU reloaded: step 1 transformed its copy in place)
   if (dU && r > 0) {
-    bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r);
+    bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm, r, L.dY, N, M, r);
+    bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm, r, L.dY, N, M, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   // 4. dX = W^(1/2) dY (minus row means)
   if (dxtype == PYLOM_F32)
-    bw_finalize_kernel<float, double><<<1024, 256, 0, st>>>(L.dY, w, remove_mean, (float*)dX, lddx, N, M);
+    bw_finalize_kernel<float, double><<<1024, 256, 0, st>>>(L.dY, w, remove_mean, (float*)dX, lddx, N, M, run_if, 1u);
   else
-    bw_finalize_kernel<double, double><<<1024, 256, 0, st>>>(L.dY, w, remove_mean, (double*)dX, lddx, N, M);
+    bw_finalize_kernel<double, double><<<1024, 256, 0, st>>>(L.dY, w, remove_mean, (double*)dX, lddx, N, M, run_if, 1u);
   return cudaGetLastError();
 }
 

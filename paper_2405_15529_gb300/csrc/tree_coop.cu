@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kLeafThreads, 2) tree_coop_kernel(TsqrState s)
   double* sWp = sW + kSmW;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int64_t M = s.M, P = s.P, G = gridDim.x;
-  if (already_factored(s)) return;
+  if (already_factored(s) || passed_over(s)) return;
   const int64_t half = (P + 1) / 2;   // most merges a level can have
   for (int64_t step = 1; step < P; step <<= 1) {
     const int64_t m = (P - step + 2 * step - 1) / (2 * step);

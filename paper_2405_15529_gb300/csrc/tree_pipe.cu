@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kLeafThreads, 2) tree_pipe_kernel(TsqrState s)
   double* sW = sout + kSmOut;
   double* sWp = sW + kSmW;
   __shared__ int s_ok;
-  if (already_factored(s)) return;
+  if (already_factored(s) || passed_over(s)) return;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int64_t M = s.M, P = s.P, G = gridDim.x;
   const int64_t nblk = (M + kNB - 1) / kNB;

@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_qr_kernel(LeafArgs a) {
   double* sW = sout + kSmOut;
   double* sWp = sW + kSmW;
   const TsqrState& s = a.s;
-  if (already_factored(s)) return;
+  if (already_factored(s) || passed_over(s)) return;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int64_t leaf = s.leaf0 + blockIdx.x;
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_qr_kernel(LeafArgs a) {
 __global__ void __launch_bounds__(256) down_pass_kernel(TsqrState s, int64_t step, int64_t r_fixed) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int64_t left = (int64_t)blockIdx.x * 2 * step, right = left + step;
-  if (right >= s.P) return;
+  if (right >= s.P || passed_over(s)) return;
   select_factors(s);
   const int64_t r = (r_fixed >= 0) ? r_fixed : s.hdr->r;
   const int64_t col = (int64_t)blockIdx.y * nwarps + warp;
@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(256) down_pass_kernel(TsqrState s, int64_t ste
 
 // B_root = first r columns of Ur (or the identity when Ur is null).
 __global__ void init_root_kernel(TsqrState s, const double* Ur, int64_t ldur, int64_t r_fixed) {
+  if (passed_over(s)) return;
   const int64_t r = (r_fixed >= 0) ? r_fixed : s.hdr->r;
   const int64_t M = s.M;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * r;
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(kLeafThreads) modes_kernel(TsqrState s, int64_
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  if (passed_over(s)) return;
   select_factors(s);
   const int64_t r = (r_fixed >= 0) ? r_fixed : s.hdr->r;
   if (leaf == 0 && tid == 0 && r_out) *r_out = r;
@@ -395,7 +397,7 @@ void tsqr_state_carve(TsqrState& s, char* base, int64_t N, int64_t M, int64_t P,
   s.Pl = P;
   s.row0 = 0;
   s.ldy = with_y ? y_ld(N) : N;
-  s.gram_y = nullptr;
+  s.gram_y = s.run_if = nullptr;
   s.shift = s.shiftx = 0;
 }
 

@@ -963,7 +963,7 @@ __global__ void __launch_bounds__(kMxThreads) leaf_qr_mixed_kernel(MixedArgs a, 
   __shared__ __align__(8) uint64_t fullbar[2];
   __shared__ uint32_t tmem_base;
   const TsqrState& s = a.s;
-  if (already_factored(s)) return;
+  if (already_factored(s) || passed_over(s)) return;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int64_t leaf = blockIdx.x;
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
@@ -1038,6 +1038,7 @@ __global__ void __launch_bounds__(kMxThreads) modes_mixed_kernel(TsqrState s, co
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  if (passed_over(s)) return;
   if (already_factored(s)) {
     shift_ptr(Yf, s.shiftx);
     shift_ptr(T2, s.shiftx);
@@ -1098,6 +1099,7 @@ __global__ void __launch_bounds__(kMxThreads) leaf_qt_mixed_kernel(TsqrState s, 
   const int64_t r0 = leaf_begin(leaf, s.N, s.P);
   const int64_t h = leaf_begin(leaf + 1, s.N, s.P) - r0;
   const int64_t M = s.M;
+  if (passed_over(s)) return;
   if (already_factored(s)) {
     shift_ptr(Yf, s.shiftx);
     shift_ptr(T2, s.shiftx);
