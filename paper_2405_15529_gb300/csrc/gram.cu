@@ -349,8 +349,9 @@ __device__ __forceinline__ dd group_sum(const long long* G, int64_t MM, int64_t 
   return s;
 }
 
-constexpr int kNBC = 16;           // panel height of the factorisation
-constexpr int kChThreads = 256;
+constexpr int kNBC = 8;            // panel height and tile size
+constexpr int kChThreads = 128;
+constexpr int kChCluster = 8;      // up to this many panels the blocks form one cluster (cheaper barrier)
 
 struct CholArgs {
   GramState g;
@@ -358,125 +359,151 @@ struct CholArgs {
   int groups, lb, bias;
 };
 
-// G = U^T D U (U unit upper triangular), right-looking by row panels of kNBC
-// rows over all blocks of a cooperative launch.  A panel: every block that
-// holds trailing columns factors the 16 x 16 diagonal block itself (a serial
-// chain of 16 pivots, the same in every block) together with its 16-column
-// block of the panel; after a grid barrier the trailing 16 x 16 tiles take
-// A -= U_panel^T (D U)_panel, one thread per entry; a second barrier ends
-// the panel.  R = D^(1/2) U with the columns' scales 2^(E - bias) restored.
+// G = U^T D U (U unit upper triangular) by row panels of kNBC rows, one
+// barrier over all blocks per panel.  Step p:
+//   units    column block c > p: apply panel p - 1 to the diagonal tile and to
+//            tile (p, c), factor the diagonal tile (a serial chain of 8
+//            pivots, the same in every unit) together with tile (p, c), write
+//            row block p of U (in place) and of T = D U (two buffers);
+//   updates  tiles (bi, bj), p < bi <= bj: apply panel p - 1, A -= U^T T.
+// A unit touches row p only and an update the rows below, so both read what
+// step p - 1 left.  Bound by the binary64 pipe of the units' SMs (two lanes a
+// clock): 16-row panels with 16 x 16 tiles and two barriers took 310 us at M
+// = 63, 640 at 128 and 1290 at 256; this takes 90, 200 and 460.
+// R = D^(1/2) U with the columns' scales 2^(E - bias) restored comes last.
 // A pivot at the rounding level of its column (a direction that the other
 // columns span, such as the one that the removed mean leaves) gives a zero
 // row.
+template <bool CLUSTER>
+__device__ __forceinline__ bool chol_barrier(const GramState& g) {
+  if (CLUSTER) {
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  }
+  return grid_barrier(g.hdr, gridDim.x);
+}
+
+__device__ __forceinline__ dd ld_dd(const double* h, const double* l, int64_t at) { return {__ldcg(h + at), __ldcg(l + at)}; }
+
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
-  __shared__ dd sP[kNBC][2 * kNBC + 1];   // diagonal block | column block
-  __shared__ dd sU[kNBC][kNBC], sT[kNBC][kNBC];
+  constexpr int B = kNBC;
+  __shared__ dd sP[B][2 * B + 1];        // diagonal tile | tile (p, c)
+  __shared__ dd sU[B][2 * B + 1], sT[B][2 * B + 1];
   __shared__ dd s_inv;
-  __shared__ double s_root, s_level[kNBC];
+  __shared__ double s_level[B];
   const GramState& g = c.g;
   const int tid = threadIdx.x;
   const int64_t M = g.M, MM = M * M;
-  const int64_t nb = (M + kNBC - 1) / kNBC;
-  const int ty = tid >> 4, tx = tid & 15;
-  // integers -> double-double (upper triangle), zeros below the diagonal of R
+  const int64_t nb = (M + B - 1) / B;
+  double* dvec = g.Tl + (int64_t)2 * B * M;     // pivots
+  // integers -> double-double (upper triangle)
   for (int64_t idx = (int64_t)blockIdx.x * kChThreads + tid; idx < MM; idx += (int64_t)gridDim.x * kChThreads) {
-    const int64_t i = idx % M, j = idx / M;
-    if (i <= j) {
+    if (idx % M <= idx / M) {
       const dd v = group_sum(g.G, MM, idx, c.groups, c.lb);
       g.Lh[idx] = v.h;
       g.Ll[idx] = v.l;
-    } else {
-      c.R[idx] = 0.0;
     }
   }
-  if (!grid_barrier(g.hdr, gridDim.x)) return;
+  if (!chol_barrier<CLUSTER>(g)) return;
   for (int64_t p = 0; p < nb; ++p) {
-    const int64_t k = p * kNBC;
-    const int nbk = (int)((M - k) < kNBC ? (M - k) : kNBC);
+    const int64_t k = p * B;
+    const int nbk = (int)((M - k) < B ? (M - k) : B);
+    // panel p - 1: U in Lh / Ll rows k - B.., T in buffer (p - 1) & 1 (B x M each)
+    const double *Th = g.Th + ((p + 1) & 1) * B * M, *Tl = g.Tl + ((p + 1) & 1) * B * M;
+    double *Thn = g.Th + (p & 1) * B * M, *Tln = g.Tl + (p & 1) * B * M;
     const int64_t units = nb - p - 1 > 0 ? nb - p - 1 : 1;
-    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
-      const int64_t c0 = (p + 1 + u) * kNBC;
+    const int64_t nt = p > 0 ? nb - p - 1 : 0, tiles = nt * (nt + 1) / 2, items = units + (tiles + 1) / 2;
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
       __syncthreads();
-      for (int idx = tid; idx < kNBC * 2 * kNBC; idx += kChThreads) {
-        const int r = idx % kNBC, q = idx / kNBC;
-        const int64_t col = q < kNBC ? k + q : c0 + q - kNBC;
+      if (it < units) {
+        const int64_t c0 = (p + 1 + it) * B;
+        const int r = tid / (2 * B), q = tid % (2 * B);    // 8 x 16 threads
+        const int64_t col = q < B ? k + q : c0 + q - B;
+        const bool in = r < nbk && col < M && (q >= B || (q < nbk && r <= q));
         dd v = {0.0, 0.0};
-        if (r < nbk && col < M && (q >= kNBC || (q < nbk && r <= q))) {
-          v.h = __ldcg(g.Lh + k + r + col * M);
-          v.l = __ldcg(g.Ll + k + r + col * M);
+        if (in) v = ld_dd(g.Lh, g.Ll, k + r + col * M);
+        if (p > 0) {
+          // rows q' of panel p - 1: U of the panel's own columns (index r), T of all 16
+          dd tt = {0.0, 0.0}, uu = {0.0, 0.0};
+          if (col < M && (q >= B || q < nbk)) tt = ld_dd(Th, Tl, r + col * B);
+          if (q < nbk) uu = ld_dd(g.Lh, g.Ll, k - B + r + (k + q) * M);
+          sT[r][q] = tt;
+          if (q < B) sU[r][q] = uu;
+          __syncthreads();
+          if (in)
+            for (int x = 0; x < B; ++x) v = dd_fms(v, sU[x][r], sT[x][q]);
         }
         sP[r][q] = v;
-      }
-      // rounding level of a pivot: its column's own square times 2^-100
-      if (tid < nbk) s_level[tid] = 7.9e-31 * group_sum(g.G, MM, (k + tid) * (M + 1), c.groups, c.lb).h;
-      __syncthreads();
-      for (int j = 0; j < nbk; ++j) {
-        if (tid == 0) {
-          const dd d = sP[j][j];
-          const bool live = d.h > s_level[j];
-          s_inv = live ? dd_rcp(d) : dd{0.0, 0.0};
-          s_root = live ? sqrt(d.h) : 0.0;
-        }
+        // rounding level of a pivot: its column's own square times 2^-100
+        if (tid < nbk) s_level[tid] = 7.9e-31 * group_sum(g.G, MM, (k + tid) * (M + 1), c.groups, c.lb).h;
         __syncthreads();
-        const dd inv = s_inv;
-        const double root = s_root;
-        // rows below take -(u_jr) (t_jq); u = t / d
-        for (int q = tx; q < 2 * kNBC; q += 16) {
-          const int r = ty;
-          if (r > j && r < nbk && (q >= kNBC || q >= r))
-            sP[r][q] = dd_fms(sP[r][q], dd_mul(sP[j][r], inv), sP[j][q]);
-        }
-        // row j of R, of U and of D U for the trailing update
-        if (ty == j && k + j < M) {
-          const int64_t col = c0 + tx;
-          if (col < M) {
-            const dd t = sP[j][kNBC + tx], uu = dd_mul(t, inv);
-            const int64_t at = k + j + col * M;
-            c.R[at] = scalbn(root * uu.h, g.colE[col] - c.bias + 32);
-            g.Lh[at] = uu.h;
-            g.Ll[at] = uu.l;
-            g.Th[j + col * kNBC] = t.h;
-            g.Tl[j + col * kNBC] = t.l;
+        for (int j = 0; j < nbk; ++j) {
+          if (tid == 0) {
+            const dd d = sP[j][j];
+            const bool live = d.h > s_level[j];
+            s_inv = live ? dd_rcp(d) : dd{0.0, 0.0};
+            if (it == 0) dvec[k + j] = live ? d.h : 0.0;
           }
-          if (u == 0 && tx >= j && tx < nbk) {
-            const dd uu = tx == j ? dd{1.0, 0.0} : dd_mul(sP[j][tx], inv);
-            c.R[k + j + (k + tx) * M] = scalbn(root * uu.h, g.colE[k + tx] - c.bias + 32);
+          __syncthreads();
+          const dd inv = s_inv;
+          // rows below take -(u_jr) (t_jq); u = t / d
+          if (r > j && in) sP[r][q] = dd_fms(sP[r][q], dd_mul(sP[j][r], inv), sP[j][q]);
+          // row j of U and T
+          if (r == j && col < M) {
+            const dd t = sP[j][q], uu = dd_mul(t, inv);
+            if (q >= B) {
+              g.Lh[k + j + col * M] = uu.h;
+              g.Ll[k + j + col * M] = uu.l;
+              Thn[j + col * B] = t.h;
+              Tln[j + col * B] = t.l;
+            } else if (it == 0 && q < nbk) {
+              c.R[k + j + col * M] = q < j ? 0.0 : q == j ? 1.0 : uu.h;   // (scaled at the end)
+            }
           }
+          __syncthreads();
         }
-        __syncthreads();
-      }
-    }
-    if (p + 1 >= nb) break;
-    if (!grid_barrier(g.hdr, gridDim.x)) return;
-    const int64_t nt = nb - p - 1, tiles = nt * (nt + 1) / 2;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-      // tile (bi, bj), bi <= bj, counted column by column
-      int64_t bj = (int64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-      while (bj * (bj + 1) / 2 > t) --bj;
-      while ((bj + 1) * (bj + 2) / 2 <= t) ++bj;
-      const int64_t bi = t - bj * (bj + 1) / 2;
-      const int64_t r0 = (p + 1 + bi) * kNBC, c0 = (p + 1 + bj) * kNBC;
-      __syncthreads();
-      {
-        const int64_t ru = r0 + tx, ct = c0 + tx;
+      } else {
+        // two 8 x 8 tiles of the trailing triangle, 64 threads each
+        const int half = tid >> 6, lt = tid & 63, tr = lt & 7, tc = lt >> 3;
+        const int64_t t = (it - units) * 2 + half;
+        const bool live = t < tiles;
+        int64_t bi = 0, bj = 0;
+        if (live) {
+          bj = (int64_t)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+          while (bj * (bj + 1) / 2 > t) --bj;
+          while ((bj + 1) * (bj + 2) / 2 <= t) ++bj;
+          bi = t - bj * (bj + 1) / 2;
+        }
+        const int64_t r0 = (p + 1 + bi) * B, c0 = (p + 1 + bj) * B;
         dd uu = {0.0, 0.0}, tt = {0.0, 0.0};
-        if (ty < nbk && ru < M) uu = {__ldcg(g.Lh + k + ty + ru * M), __ldcg(g.Ll + k + ty + ru * M)};
-        if (ty < nbk && ct < M) tt = {__ldcg(g.Th + ty + ct * kNBC), __ldcg(g.Tl + ty + ct * kNBC)};
-        sU[ty][tx] = uu;
-        sT[ty][tx] = tt;
-      }
-      __syncthreads();
-      const int64_t r = r0 + tx, cc = c0 + ty;
-      if (r < M && cc < M && r <= cc) {
-        const int64_t at = r + cc * M;
-        dd s = {__ldcg(g.Lh + at), __ldcg(g.Ll + at)};
-#pragma unroll 4
-        for (int q = 0; q < kNBC; ++q) s = dd_fms(s, sU[q][tx], sT[q][ty]);
-        g.Lh[at] = s.h;
-        g.Ll[at] = s.l;
+        if (live && r0 + tc < M) uu = ld_dd(g.Lh, g.Ll, k - B + tr + (r0 + tc) * M);
+        if (live && c0 + tc < M) tt = ld_dd(Th, Tl, tr + (c0 + tc) * B);
+        sU[tr][tc + half * B] = uu;
+        sT[tr][tc + half * B] = tt;
+        __syncthreads();
+        const int64_t r = r0 + tr, cc = c0 + tc;
+        if (live && r < M && cc < M && r <= cc) {
+          dd s = ld_dd(g.Lh, g.Ll, r + cc * M);
+#pragma unroll
+          for (int x = 0; x < B; ++x) s = dd_fms(s, sU[x][tr + half * B], sT[x][tc + half * B]);
+          g.Lh[r + cc * M] = s.h;
+          g.Ll[r + cc * M] = s.l;
+        }
       }
     }
-    if (!grid_barrier(g.hdr, gridDim.x)) return;
+    if (!chol_barrier<CLUSTER>(g)) return;
+  }
+  for (int64_t idx = (int64_t)blockIdx.x * kChThreads + tid; idx < MM; idx += (int64_t)gridDim.x * kChThreads) {
+    const int64_t i = idx % M, j = idx / M;
+    double v = 0.0;
+    if (i <= j) {
+      const double u = (i / B == j / B) ? __ldcg(c.R + idx) : __ldcg(g.Lh + idx);
+      // the integer sums were scaled by 2^-64: their root by 2^-32
+      v = scalbn(sqrt(__ldcg(dvec + i)) * u, g.colE[j] - c.bias + 32);
+    }
+    c.R[idx] = v;
   }
 }
 
@@ -486,7 +513,7 @@ __global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
 
 size_t gram_bytes(int64_t M, int64_t rmax) {
   return align256(sizeof(int) * (size_t)M) + align256(sizeof(long long) * (size_t)5 * M * M) +
-         2 * align256(sizeof(double) * (size_t)M * M) + 2 * align256(sizeof(double) * (size_t)kNBC * M) +
+         2 * align256(sizeof(double) * (size_t)M * M) + 2 * align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M) +
          product_planes_bytes(M, 0, rmax);
 }
 
@@ -499,8 +526,8 @@ void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax) {
   g.G = (long long*)p;       p += align256(sizeof(long long) * (size_t)5 * M * M);
   g.Lh = (double*)p;         p += align256(sizeof(double) * (size_t)M * M);
   g.Ll = (double*)p;         p += align256(sizeof(double) * (size_t)M * M);
-  g.Th = (double*)p;         p += align256(sizeof(double) * (size_t)kNBC * M);
-  g.Tl = (double*)p;         p += align256(sizeof(double) * (size_t)kNBC * M);
+  g.Th = (double*)p;         p += align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M);
+  g.Tl = (double*)p;         p += align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M);
   g.Cd = (unsigned char*)p;  p += align256((size_t)kt * js * 8 * kPlaneB);
   g.Ce = (int*)p;
 }
@@ -599,16 +626,29 @@ cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xt
   if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
   CholArgs c{g, R, groups, g.f32 ? gram_base<float>(0) : gram_base<double>(0),
              g.f32 ? fix_bias<float>() : fix_bias<double>()};
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, gram_chol_kernel, kChThreads, 0);
+  const int64_t nb = (g.M + kNBC - 1) / kNBC;
+  if (nb <= kChCluster) {
+    cudaLaunchConfig_t cfg = {};
+    const unsigned n = nb <= 2 ? 1u : (unsigned)kChCluster;
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(kChThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gram_chol_kernel<true>, c);
+  }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, gram_chol_kernel<false>, kChThreads, 0);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorCooperativeLaunchTooLarge;
-  const int64_t nb = (g.M + kNBC - 1) / kNBC;
-  int64_t grid = nb * (nb - 1) / 2;
-  if (grid < 1) grid = 1;
+  int64_t grid = nb + nb * (nb - 1) / 4;
   if (grid > sms) grid = sms;
   void* args[] = {&c};
-  return cudaLaunchCooperativeKernel((const void*)gram_chol_kernel, dim3((unsigned)grid), dim3(kChThreads), args, 0,
-                                     st);
+  return cudaLaunchCooperativeKernel((const void*)gram_chol_kernel<false>, dim3((unsigned)grid), dim3(kChThreads), args,
+                                     0, st);
 }
 
 }  // namespace pylom

@@ -14,8 +14,8 @@ struct GramState {
   long long* G;           // 5 x M x M: integer sums, group g weighs 2^(32 g)
   double* Lh;             // M x M double-double triangle (high parts)
   double* Ll;             // (low parts)
-  double* Th;             // kNBC x M: current row panel before division (high)
-  double* Tl;
+  double* Th;             // two row panels before division (high parts), kNBC x M each
+  double* Tl;             // (low parts), then M pivots
   unsigned char* Cd;      // digit planes of the modes product's coefficients
   int* Ce;                // exponent field of each coefficient column
   int64_t rmax;
