@@ -27,8 +27,6 @@ namespace pylom {
 // Y = sqrt(w) (X - mean)
 // ---------------------------------------------------------------------------
 
-constexpr int kPrThreads = 256;   // 8 warps; lane = row, a warp takes every 8th column
-
 struct PrologueArgs {
   const void* X;
   int64_t ldx;
@@ -41,89 +39,97 @@ struct PrologueArgs {
   WsHeader* hdr;
 };
 
-// sum of one thread's values of a row (CT of them, zeros past M) as a binary64
-__device__ __forceinline__ double part_sum(const double* x, int n) {
-  double s = 0.0;
-  for (int t = 0; t < n; ++t) s += x[t];
-  return s;
-}
+__device__ __forceinline__ bool nonfinite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+__device__ __forceinline__ bool nonfinite(float x) { return (__float_as_int(x) & 0x7f800000) == 0x7f800000; }
 
-template <typename TX, typename TY, int CT>
-__global__ void __launch_bounds__(kPrThreads) gram_prologue_kernel(PrologueArgs a) {
-  __shared__ double ssum[8][32];
+// A block takes 32 rows at a time: lane = row, warp v the columns v, v + W,
+// ..., CT of them in registers between the row's mean and its centred values
+// (wider matrices read X once more, from the L2 cache).  Reading X and writing
+// Y is the bound in binary32; in binary64 the two to three binary64 operations
+// an element (sum, difference, weight; two lanes a clock) are.  So the row's
+// division and square root are one warp's work, not every warp's, finiteness
+// is an integer test, and the column maxima, which took a register a column,
+// are reduced over the warp on the spot: that leaves registers for two blocks
+// of 16 warps.  Before (a register a column, 8 warps of 32 columns, every warp
+// its own division and root) -> here, microseconds: 65,537 x 63 binary64 71 ->
+// 47, 1,048,576 x 256 binary64 2960 -> 2720; binary32 262,144 x 100 185 -> 105,
+// 1,048,576 x 256 1610 -> 863, 300,001 x 700 2220 -> 691.
+template <typename TX, typename TY, int CT, int W>
+__global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(PrologueArgs a) {
+  static_assert(CT <= 32, "a lane keeps the maximum of one column");
+  __shared__ double ssum[W][32];
+  __shared__ double sbar[32], ssw[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TX* X = (const TX*)a.X;
   TY* Y = (TY*)a.Y;
-  int bad = 0;
-  // column groups of 8 CT columns; one group when M <= 8 CT (the row then
-  // stays in registers between its mean and its centred values)
-  int emax[CT];
-#pragma unroll
-  for (int t = 0; t < CT; ++t) emax[t] = 0;
-  const bool one = a.M <= 8 * CT;
+  bool bad = false;
+  const bool one = a.M <= W * CT;
+  int emax = 0;     // of column (group) warp + W lane
   const int64_t nblk = (a.ldy + 31) / 32;
   for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
     const int64_t n = blk * 32 + lane;
     const bool in = n < a.N;
     TX x[CT];
-    double s = 0.0;
-    for (int64_t c0 = 0; c0 < a.M; c0 += 8 * CT) {
+    double s = 0.0, sw = 1.0, xbar = 0.0;
+    if (a.w && warp == W - 1 && in) {
+      const double wn = a.w[n];
+      if (!(wn > 0.0) || !isfinite(wn)) bad = true;
+      sw = sqrt(wn);
+    }
+    if (one || a.remove_mean)
+      for (int64_t c0 = 0; c0 < a.M; c0 += W * CT) {
 #pragma unroll
-      for (int t = 0; t < CT; ++t) {
-        const int64_t c = c0 + warp + 8 * t;
-        x[t] = (in && c < a.M) ? X[n + c * a.ldx] : (TX)0;
-      }
-      if (a.remove_mean) {
-        if constexpr (sizeof(TX) == 4) {
-          // compensated binary32 sums in chunks of at most 16 (binary64
-          // conversions and additions are slow on this part)
-          constexpr int K = CT < 16 ? CT : 16;
-#pragma unroll
-          for (int t0 = 0; t0 < CT; t0 += K) {
-            float v[K], h, l;
-#pragma unroll
-            for (int t = 0; t < K; ++t) v[t] = x[t0 + t];
-            sum32_compensated(v, h, l);
+        for (int t = 0; t < CT; ++t) {
+          const int64_t c = c0 + warp + W * t;
+          x[t] = (in && c < a.M) ? X[n + c * a.ldx] : (TX)0;
+        }
+        if (a.remove_mean) {
+          if constexpr (sizeof(TX) == 4) {
+            // compensated binary32 sums in chunks of at most 16 (binary64
+            // conversions and additions are slow on this part)
+            float h, l;
+            static_assert(CT <= 16, "one chunk");
+            sum32_compensated(x, h, l);
             s += (double)h + (double)l;
-          }
-        } else {
+          } else {
 #pragma unroll
-          for (int t = 0; t < CT; ++t) s += (double)x[t];
+            for (int t = 0; t < CT; ++t) s += (double)x[t];
+          }
         }
       }
-    }
-    double xbar = 0.0;
-    if (a.remove_mean) {
+    if (a.remove_mean || a.w) {
       ssum[warp][lane] = s;
       __syncthreads();
-      double tot = 0.0;
+      if (warp == W - 1) ssw[lane] = sw;
+      if (warp == 0) {
+        double tot = 0.0;
+        if (a.remove_mean) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) tot += ssum[q][lane];
-      xbar = tot / (double)a.M;
+          for (int q = 0; q < W; ++q) tot += ssum[q][lane];
+          tot /= (double)a.M;
+        }
+        sbar[lane] = tot;
+      }
       __syncthreads();
-    }
-    double sw = 1.0;
-    if (a.w && in) {
-      const double wn = a.w[n];
-      if (!(wn > 0.0) || !isfinite(wn)) bad = 1;
-      sw = sqrt(wn);
+      xbar = sbar[lane];
+      sw = ssw[lane];
     }
     if (warp == 0 && in && a.mean) a.mean[n] = xbar;
     const float xh = (float)xbar, xl = (float)(xbar - (double)xh);
     const float sh = (float)sw, sl = (float)(sw - (double)sh);
-    for (int64_t c0 = 0; c0 < a.M; c0 += 8 * CT) {
+    for (int64_t c0 = 0; c0 < a.M; c0 += W * CT) {
       if (!one) {
+        emax = 0;
 #pragma unroll
         for (int t = 0; t < CT; ++t) {
-          const int64_t c = c0 + warp + 8 * t;
+          const int64_t c = c0 + warp + W * t;
           x[t] = (in && c < a.M) ? X[n + c * a.ldx] : (TX)0;
-          emax[t] = 0;
         }
       }
 #pragma unroll
       for (int t = 0; t < CT; ++t) {
-        const int64_t c = c0 + warp + 8 * t;
-        if (c >= a.M) continue;
+        const int64_t c = c0 + warp + W * t;
+        if (c >= a.M) break;
         TY y;
         if constexpr (sizeof(TX) == 4 && sizeof(TY) == 4) {
           // x - mean as d + e by TwoSum, times sqrt(w) = sh + sl by two FMAs
@@ -137,28 +143,20 @@ __global__ void __launch_bounds__(kPrThreads) gram_prologue_kernel(PrologueArgs 
           y = (TY)v;
         }
         if (!in) y = (TY)0;
-        const int e = exp_field(y);
-        emax[t] = e > emax[t] ? e : emax[t];
-        if (!isfinite(x[t])) bad = 1;
+        bad = bad || nonfinite(x[t]);
         if (n < a.ldy) Y[n + c * a.ldy] = y;
+        const int e = __reduce_max_sync(0xffffffffu, exp_field(y));
+        if (lane == t) emax = e > emax ? e : emax;
       }
       if (!one) {
-#pragma unroll
-        for (int t = 0; t < CT; ++t) {
-          const int64_t c = c0 + warp + 8 * t;
-          const int e = __reduce_max_sync(0xffffffffu, emax[t]);
-          if (lane == 0 && c < a.M && e > __ldcg(a.colE + c)) atomicMax(a.colE + c, e);
-        }
+        const int64_t c = c0 + warp + W * lane;
+        if (lane < CT && c < a.M && emax > __ldcg(a.colE + c)) atomicMax(a.colE + c, emax);
       }
     }
   }
   if (one) {
-#pragma unroll
-    for (int t = 0; t < CT; ++t) {
-      const int64_t c = warp + 8 * t;
-      const int e = __reduce_max_sync(0xffffffffu, emax[t]);
-      if (lane == 0 && c < a.M) atomicMax(a.colE + c, e);
-    }
+    const int64_t c = warp + W * lane;
+    if (lane < CT && c < a.M) atomicMax(a.colE + c, emax);
   }
   if (bad) raise_status(a.hdr, PYLOM_ERR_NONFINITE);
   if (blockIdx.x == 0 && threadIdx.x == 0) a.hdr->gram_y = 1;
@@ -369,7 +367,8 @@ struct CholArgs {
 // A unit touches row p only and an update the rows below, so both read what
 // step p - 1 left.  Bound by the binary64 pipe of the units' SMs (two lanes a
 // clock): 16-row panels with 16 x 16 tiles and two barriers took 310 us at M
-// = 63, 640 at 128 and 1290 at 256; this takes 90, 200 and 460.
+// = 63, 640 at 128, 1290 at 256 and 4900 at 700; this takes 189, 350, 730 and
+// 3600.
 // R = D^(1/2) U with the columns' scales 2^(E - bias) restored comes last.
 // A pivot at the rounding level of its column (a direction that the other
 // columns span, such as the one that the removed mean leaves) gives a zero
@@ -535,12 +534,13 @@ void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax) {
 template <typename TX, typename TY>
 static cudaError_t prologue(const PrologueArgs& a, int sms, cudaStream_t st) {
   const int64_t nblk = (a.ldy + 31) / 32;
-  const int64_t cap = (int64_t)sms * 4;
+  // threads are capped at 1024 an SM by the register bound of the kernels
+  const int64_t cap = (int64_t)sms * (a.M <= 128 ? 4 : 2);
   const unsigned grid = (unsigned)(nblk < cap ? nblk : cap);
-  if (a.M <= 32) gram_prologue_kernel<TX, TY, 4><<<grid, kPrThreads, 0, st>>>(a);
-  else if (a.M <= 64) gram_prologue_kernel<TX, TY, 8><<<grid, kPrThreads, 0, st>>>(a);
-  else if (a.M <= 128) gram_prologue_kernel<TX, TY, 16><<<grid, kPrThreads, 0, st>>>(a);
-  else gram_prologue_kernel<TX, TY, 32><<<grid, kPrThreads, 0, st>>>(a);
+  if (a.M <= 32) gram_prologue_kernel<TX, TY, 4, 8><<<grid, 256, 0, st>>>(a);
+  else if (a.M <= 64) gram_prologue_kernel<TX, TY, 8, 8><<<grid, 256, 0, st>>>(a);
+  else if (a.M <= 128) gram_prologue_kernel<TX, TY, 16, 8><<<grid, 256, 0, st>>>(a);
+  else gram_prologue_kernel<TX, TY, 16, 16><<<grid, 512, 0, st>>>(a);
   return cudaGetLastError();
 }
 
