@@ -88,6 +88,7 @@ struct SvdState {
   double* T[5];             // Mp x Mp scratch of the binary64 products
   double* A2;               // M x Mp second copy of A
   int* big;                 // Mp: partner of a column's largest angle
+  double* angle_sum; // Mp: sum of each column's small angles
   unsigned* rot32;          // counters (svd_jacobi32.cu)
 };
 

@@ -14,13 +14,13 @@
 //   2. the same again on fl32(A): each column now has its own binary32
 //      scale, so columns of small singular value, which fl32(R^T) buried
 //      under the rounding of the large ones, become orthogonal too;
-//   3. two to four binary64 steps of simultaneous rotations: with
+//   3. two, four or six binary64 steps of simultaneous rotations: with
 //      G = A^T A, E = V^T V - I and K_ij the Jacobi angle of pair (i, j)
 //      (antisymmetric), Q = I + K + K^2/2 - E/2 and A <- A Q, V <- V Q: all
 //      cosines square (Davies and Modi, "A direct method for completing
 //      eigenproblem solutions on a parallel computer", 1986).  Two columns
 //      whose angle is not small (double singular values) get their exact
-//      rotation instead.
+//      rotation first, and K is formed in the rotated basis.
 // Matrix products run on all SMs.  The binary64 sweeps then start from
 // (A, V); when every pair already meets their stopping test they return at
 // once, else they finish the job: the result is the binary64 SVD either way.
@@ -45,9 +45,9 @@ constexpr int kJ32MaxSweeps = 24;
 constexpr int kJClusterMax = 8;        // up to 8 blocks run as one cluster (cheaper barrier)
 // words of s.rot32: rotations of each sweep of the two stages, then
 constexpr int kJScale = 2 * kJ32MaxSweeps;       // largest exponent field of R
-constexpr int kJSteps = 4;                       // binary64 steps of simultaneous rotations
+constexpr int kJSteps = 6;                       // binary64 steps of simultaneous rotations
 constexpr int kJOpen = kJScale + 1;              // kJSteps + 1 words: pairs not converged at each check; then: entries of V^T V off
-constexpr int kJWords = kJScale + 8;
+constexpr int kJWords = kJOpen + kJSteps + 2;
 
 __global__ void jacobi32_scale_kernel(SvdState s, const double* R, int64_t ldr) {
   int e = 0;
@@ -394,14 +394,12 @@ __device__ __forceinline__ bool pair_open(double al, double be, double ga, doubl
 }
 
 // Check `c` on G: counts the pairs that the binary64 sweeps would rotate
-// (open[c]), and says for each column what the step does with it: big[j] >= 0
-// is the partner of its largest angle if that is not small, -1: its angles
-// are small and sum to at most `limit`, -2: left alone (a crowd of close
-// singular values, where the angles together would not be a small rotation).
+// (open[c]), and leaves for each column the partner of its largest angle if
+// that is not small (big[j], else -1) and the sum of its small ones.
 // With W = V^T V given, entries away from the identity by more than wtol
 // are counted in bad.  A warp per column.
 __global__ void jacobi_check_kernel(SvdState s, const double* G, const double* W, double wtol, unsigned* bad, int c,
-                                    double limit, const unsigned* skip) {
+                                    const unsigned* skip) {
   if (skip && *skip == 0) return;
   const int64_t Mp = s.Mp;
   const int lane = threadIdx.x & 31;
@@ -439,48 +437,73 @@ __global__ void jacobi_check_kernel(SvdState s, const double* G, const double* W
   n = __reduce_add_sync(0xffffffffu, n);
   nw = __reduce_add_sync(0xffffffffu, nw);
   if (lane == 0) {
-    s.big[j] = bi >= 0 ? bi : sum <= limit ? -1 : -2;
+    s.big[j] = bi;
+    s.angle_sum[j] = sum;
     if (n) atomicAdd(s.rot32 + kJOpen + c, n);
     if (nw) atomicAdd(bad, nw);
   }
 }
 
-// K = the antisymmetric small angles, L = K - E and B = I + K - E / 2 with
-// E = W - I, W = V^T V, so that Q = B + L K / 2 = (I - E / 2)(I + K + K^2 / 2)
-// up to E K^2.  B may overwrite W.
 // Two columns that are each other's largest angle get their exact rotation
-// in B (multiple singular values: the angle is anything up to 45 degrees)
-// and no other angle this time.
-__global__ void jacobi_angles_kernel(SvdState s, const double* G, const double* W, double* K, double* L,
-                                     double* B, const unsigned* skip) {
+// (close singular values: the angle is anything up to 45 degrees): P is the
+// product of these disjoint rotations.  In the rotated basis, G' = P^T G P and
+// W' = P^T W P, K = the antisymmetric small angles, L = K - E and B = I + K -
+// E / 2 with E = W' - I, so that B + L K / 2 = (I - E / 2)(I + K + K^2 / 2) up
+// to E K^2; PL = P L and PB = P B go out, and Q = PB + PL K / 2.  A column
+// whose small angles sum to more than `limit` takes none (a crowd of close
+// singular values, where they are no small rotation together).
+__global__ void jacobi_angles_kernel(SvdState s, const double* G, const double* W, double* K, double* PL,
+                                     double* PB, double limit, const unsigned* skip) {
   if (skip && *skip == 0) return;
   const int64_t Mp = s.Mp;
   const double tol = (double)s.M * 1.1102230246251565e-16;
+  struct Col {
+    int64_t at, b;     // itself, its partner (or itself)
+    double c, s, d;    // a' = c a + s a_b; its square
+    bool act;
+  };
+  auto column = [&](int64_t i) {
+    Col r{i, i, 1.0, 0.0, G[i + i * Mp], s.angle_sum[i] <= limit};
+    const int64_t b = s.big[i];
+    if (b >= 0 && s.big[b] == i) {
+      const int64_t lo = i < b ? i : b, hi = i < b ? b : i;
+      const double ga = G[lo + hi * Mp];
+      double t = pair_tangent(G[lo + lo * Mp], G[hi + hi * Mp], ga);
+      if (i == hi) t = -t;
+      r.b = b;
+      r.c = 1.0 / sqrt(1.0 + t * t);
+      r.s = -t * r.c;
+      r.d -= t * ga;
+      r.act = s.angle_sum[i] + s.angle_sum[b] <= limit;
+    }
+    return r;
+  };
+  auto rotated = [&](const double* X, const Col& p, const Col& q) {
+    double x = X[p.at + q.at * Mp];
+    if (p.b != p.at || q.b != q.at)
+      x = p.c * (q.c * x + q.s * X[p.at + q.b * Mp]) +
+          p.s * (q.c * X[p.b + q.at * Mp] + q.s * X[p.b + q.b * Mp]);
+    return x;
+  };
+  auto angle = [&](const Col& p, const Col& q) {
+    if (p.at == q.at || p.b == q.at || !p.act || !q.act) return 0.0;
+    const double ga = rotated(G, p, q), t = pair_tangent(p.d, q.d, ga);
+    return small_angle(pair_open(p.d, q.d, ga, tol), t, (double)s.M) ? t : 0.0;
+  };
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mp * Mp;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = idx % Mp, j = idx / Mp;
-    const int bi = s.big[i], bj = s.big[j];
-    double t = 0.0, x = 0.0;
-    if (i != j) {
-      if (bi == j && bj == i) {
-        const double tt = pair_tangent(G[i + i * Mp], G[j + j * Mp], G[idx]);
-        x = tt / sqrt(1.0 + tt * tt);
-      } else if (bi == -1 && bj == -1) {
-        const double al = G[i + i * Mp], be = G[j + j * Mp], ga = G[idx];
-        t = pair_tangent(al, be, ga);
-        if (!small_angle(pair_open(al, be, ga, tol), t, (double)s.M)) t = 0.0;
-      }
-    } else {
-      x = 1.0;
-      if (bi >= 0 && s.big[bi] == i) {
-        const double tt = pair_tangent(G[i + i * Mp], G[bi + (int64_t)bi * Mp], G[i + bi * Mp]);
-        x = 1.0 / sqrt(1.0 + tt * tt);
-      }
-    }
-    const double E = W[idx] - (i == j ? 1.0 : 0.0);
+    const Col p = column(idx % Mp), q = column(idx / Mp);
+    const double one = p.at == q.at ? 1.0 : 0.0, t = angle(p, q), E = rotated(W, p, q) - one;
+    double l = t - E, b = one + t - 0.5 * E;
     K[idx] = t;
-    L[idx] = t - E;
-    B[idx] = x + t - 0.5 * E;
+    if (p.b != p.at) {
+      const Col p2 = column(p.b);
+      const double one2 = p2.at == q.at ? 1.0 : 0.0, t2 = angle(p2, q), E2 = rotated(W, p2, q) - one2;
+      l = p.c * l - p.s * (t2 - E2);
+      b = p.c * b - p.s * (one2 + t2 - 0.5 * E2);
+    }
+    PL[idx] = l;
+    PB[idx] = b;
   }
 }
 
@@ -504,21 +527,23 @@ size_t jacobi32_extra_bytes(int64_t M) {
   if (M < kJac32MinM) return 0;
   const int64_t Mp = M + (M & 1);
   const int64_t Mb = (M + kJW - 1) / kJW * kJW;
-  return align256(sizeof(float) * (size_t)M * Mb) + align256(sizeof(float) * (size_t)Mb * Mb) +
+  return 2 * align256(sizeof(float) * (size_t)Mb * Mb) +
          5 * align256(sizeof(double) * (size_t)Mp * Mp) + align256(sizeof(unsigned) * kJWords) +
-         align256(sizeof(double) * (size_t)M * Mp) + align256(sizeof(int) * (size_t)Mp);
+         align256(sizeof(double) * (size_t)M * Mp) + align256(sizeof(int) * (size_t)Mp) +
+         align256(sizeof(double) * (size_t)Mp);
 }
 
 void jacobi32_carve(SvdState& s, char* p) {
   const int64_t M = s.M, Mp = s.Mp;
   const size_t sq = align256(sizeof(double) * (size_t)Mp * Mp);
   s.Mb = (M + kJW - 1) / kJW * kJW;
-  s.A32 = (float*)p;    p += align256(sizeof(float) * (size_t)M * s.Mb);
+  s.A32 = (float*)p;    p += align256(sizeof(float) * (size_t)s.Mb * s.Mb);
   s.V32 = (float*)p;    p += align256(sizeof(float) * (size_t)s.Mb * s.Mb);
   for (int i = 0; i < 5; ++i) { s.T[i] = (double*)p; p += sq; }
   s.rot32 = (unsigned*)p; p += align256(sizeof(unsigned) * kJWords);
   s.A2 = (double*)p;    p += align256(sizeof(double) * (size_t)M * Mp);
-  s.big = (int*)p;
+  s.big = (int*)p;      p += align256(sizeof(int) * (size_t)Mp);
+  s.angle_sum = (double*)p;
 }
 
 static cudaError_t stage32(const SvdState& s, int stage, cudaStream_t st) {
@@ -560,7 +585,9 @@ cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int
   cudaError_t e = cudaMemsetAsync(s.rot32, 0, sizeof(unsigned) * kJWords, st);
   if (e != cudaSuccess) return e;
   double *T0 = s.T[0], *T1 = s.T[1], *T2 = s.T[2], *T3 = s.T[3], *T4 = s.T[4];
+  double* T5 = (double*)s.A32;   // (A32 and V32 are done with when the steps begin)
   unsigned* open = s.rot32 + kJOpen;
+  const double wtol = (double)M * 1.1102230246251565e-16 > 1e-14 ? (double)M * 1.1102230246251565e-16 : 1e-14;
   // a product whose left factor op(A) has `m` rows and K = `k` (B then has
   // leading dimension k, C and D m)
   auto mm = [&](int ta, int64_t m, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
@@ -587,32 +614,35 @@ cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int
   jacobi32_widen_kernel<<<gr, 256, 0, st>>>(s, T0);
   e = cudaGetLastError();
   two(mm(0, Mp, Mp, 1.0, T3, Mp, T0, 0.0, nullptr, s.V), mm(0, M, Mp, 1.0, s.A2, M, T0, 0.0, nullptr, s.A));
-  // steps of simultaneous rotations, (A, V) -> (A2, T3) -> (A, V) and, if
-  // pairs are still open, the same again; V's departure from orthogonality
-  // goes 1e-6 -> 1e-12 -> rounding
+  // steps of simultaneous rotations in pairs, (A, V) -> (A2, T3) -> (A, V);
+  // each pair begins with a look at G and, from the second on, ends all if
+  // no pair is open.  V's departure from orthogonality, 1e-6 at first, is
+  // squared by a step, which adds a^4 / 4 for angles that sum to a: the last
+  // steps take small angles only.  The first takes up to 0.3: of 700 columns
+  // whose 300 smallest singular values lie within 20 % of each other most
+  // have angles above 0.05 together, and were left to the sweeps (42 ms).
+  constexpr double kLimit[kJSteps] = {0.3, 0.1, 0.1, 0.02, 0.01, 2e-4};
   const unsigned gc = (unsigned)((Mp * 32 + 255) / 256);
   for (int it = 0; it < kJSteps; ++it) {
     const bool fwd = (it & 1) == 0;
     const double *Ai = fwd ? s.A : s.A2, *Vi = fwd ? s.V : T3;
     double *Ao = fwd ? s.A2 : s.A, *Vo = fwd ? T3 : s.V;
-    const unsigned* skip = it < 2 ? nullptr : open + 2;
-    two(mm(1, Mp, M, 1.0, Ai, M, Ai, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, Vi, Mp, Vi, 0.0, nullptr, T1),
-        it == 2 ? nullptr : skip);
+    // whether this pair of steps runs, and whether the one before did
+    const unsigned* skip = it < 2 ? nullptr : open + (it & ~1);
+    const unsigned* look = fwd ? (it < 4 ? nullptr : open + it - 2) : skip;
+    two(mm(1, Mp, M, 1.0, Ai, M, Ai, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, Vi, Mp, Vi, 0.0, nullptr, T1), look);
     if (e != cudaSuccess) return e;
-    // (a step of angle sum a leaves V off orthogonality by a^4 / 4, which the
-    // next one repairs: the last one takes tiny angles only)
-    jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, it == 2 ? T1 : nullptr, 1e-14, open + 2, it,
-                                            it == kJSteps - 1 ? 2e-4 : 0.05, it == 2 ? nullptr : skip);
-    jacobi_angles_kernel<<<gr, 256, 0, st>>>(s, T0, T1, T2, T4, T1, skip);
+    jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, it >= 2 && fwd ? T1 : nullptr, wtol, open + it, it, look);
+    jacobi_angles_kernel<<<gr, 256, 0, st>>>(s, T0, T1, T2, T4, T5, kLimit[it], skip);
     e = cudaGetLastError();
-    one(mm(0, Mp, Mp, 0.5, T4, Mp, T2, 1.0, T1, T0), skip);                          // Q
+    one(mm(0, Mp, Mp, 0.5, T4, Mp, T2, 1.0, T5, T0), skip);                          // Q
     two(mm(0, M, Mp, 1.0, Ai, M, T0, 0.0, nullptr, Ao), mm(0, Mp, Mp, 1.0, Vi, Mp, T0, 0.0, nullptr, Vo), skip);
   }
-  two(mm(1, Mp, M, 1.0, s.A, M, s.A, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, s.V, Mp, s.V, 0.0, nullptr, T1), open + 2);
+  // (after fewer steps the last look stands)
+  const unsigned* look = open + kJSteps - 2;
+  two(mm(1, Mp, M, 1.0, s.A, M, s.A, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, s.V, Mp, s.V, 0.0, nullptr, T1), look);
   if (e != cudaSuccess) return e;
-  const double wtol = (double)M * 1.1102230246251565e-16;
-  jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, T1, wtol > 1e-14 ? wtol : 1e-14, open + kJSteps + 1, kJSteps, 0.05,
-                                          open + 2);
+  jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, T1, wtol, open + kJSteps + 1, kJSteps, look);
   // a V that is not orthogonal after all: the binary64 sweeps start from R^T
   jacobi_restart_kernel<<<gr, 256, 0, st>>>(s, R, ldr, open + kJSteps + 1, open + kJSteps);
   *open_pairs = open + kJSteps;
