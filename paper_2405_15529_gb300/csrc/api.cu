@@ -422,7 +422,7 @@ extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_byt
     TsqrState os;
     fs.rmax = 0;
     double* UR2 = nullptr;
-    e = launch_refactor(fs, extra, bws, (WsHeader*)ws, mixed, UR, os, &extra,
+    e = launch_refactor(fs, gs, extra, bws, (WsHeader*)ws, mixed, UR, os, &extra,
                         &UR2, st);
     if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward: factorisation");
     fs = os;

@@ -87,12 +87,18 @@ __device__ __forceinline__ uint2 bias_digits(int64_t v) {
   const uint64_t w = (uint64_t)v + kDigitBias64;
   return make_uint2((uint32_t)w, (uint32_t)(w >> 32));
 }
+// the value that a biased word stands for, of a column with exponent field E
+__device__ __forceinline__ double from_fixed(uint2 w, int E) {
+  const int64_t v = (int64_t)((((uint64_t)w.y << 32) | w.x) - kDigitBias64);
+  return scalbn((double)v, E - fix_bias<double>());
+}
 __device__ __forceinline__ int64_t to_fixed(double y, int E) {
   const uint2 w = biased_fixed(y, E);
   return (int64_t)((((uint64_t)w.y << 32) | w.x) - kDigitBias64);
 }
 
-// All digits of eight values, digit s as one 16-byte store at dst + s * plane.
+// All digits of eight values, digit s as one 16-byte store at dst + s * plane
+// (and, dst2 given, at dst2 + s * plane2).
 // A digit of two values becomes a binary16 pair by its bit pattern (1024 +
 // byte: 0x64 above the byte) minus 1152.
 __device__ __forceinline__ uint32_t sub_1152(uint32_t x) {
@@ -101,7 +107,8 @@ __device__ __forceinline__ uint32_t sub_1152(uint32_t x) {
   return r;
 }
 template <int S>
-__device__ __forceinline__ void store_digits(const uint2 (&w)[8], unsigned char* dst, int plane) {
+__device__ __forceinline__ void store_digits(const uint2 (&w)[8], unsigned char* dst, int plane,
+                                             unsigned char* dst2 = nullptr, int plane2 = 0) {
 #pragma unroll
   for (int s = 0; s < S; s += 2) {
     uint32_t d0[4], d1[4];
@@ -114,21 +121,38 @@ __device__ __forceinline__ void store_digits(const uint2 (&w)[8], unsigned char*
     }
     *(uint4*)(dst + s * plane) = make_uint4(d0[0], d0[1], d0[2], d0[3]);
     if (s + 1 < S) *(uint4*)(dst + (s + 1) * plane) = make_uint4(d1[0], d1[1], d1[2], d1[3]);
+    if (dst2) {
+      *(uint4*)(dst2 + s * plane2) = make_uint4(d0[0], d0[1], d0[2], d0[3]);
+      if (s + 1 < S) *(uint4*)(dst2 + (s + 1) * plane2) = make_uint4(d1[0], d1[1], d1[2], d1[3]);
+    }
   }
 }
 
-// Eight elements of one column (scale E) as digits in a stage.
-__device__ __forceinline__ void put_digits(const double (&y)[8], int E, unsigned char* dst, int plane) {
-  uint2 w[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) w[i] = biased_fixed(y[i], E);
+// What Y holds when the products run: binary32 as it is; binary64 as
+// biased fixed-point words (pack_kernel).  A word costs 6 byte selections and
+// 4 subtractions, a binary64 value 18 more operations of the half-rate
+// integer pipe, and the Gram kernel cuts every element about nine times (at
+// 256 columns); one pass over Y in place pays for that.
+template <typename TY> struct Cell { typedef TY type; };
+template <> struct Cell<double> { typedef uint2 type; };
+template <typename C> __device__ __forceinline__ C zero_cell();
+template <> __device__ __forceinline__ float zero_cell<float>() { return 0.f; }
+template <> __device__ __forceinline__ uint2 zero_cell<uint2>() { return make_uint2(kDigitBias, kDigitBias); }
+
+// Eight elements of one column (scale E), or each of its own, as digits in a stage.
+__device__ __forceinline__ void put_digits(const uint2 (&w)[8], int, unsigned char* dst, int plane,
+                                           unsigned char* dst2, int plane2) {
+  store_digits<Dig<double>::S>(w, dst, plane, dst2, plane2);
+}
+__device__ __forceinline__ void put_digits(const uint2 (&w)[8], const int (&)[8], unsigned char* dst, int plane) {
   store_digits<Dig<double>::S>(w, dst, plane);
 }
 // Binary32: digits by rounding, top down, in binary32 itself (d = rint(r),
 // r <- 256 (r - d), every step exact): three operations a digit on the
 // full-rate pipe instead of a 64-bit shift and byte selection on the
 // half-rate one.  The top digit is rint(y 2^(132 - E)), at most 64.
-__device__ __forceinline__ void put_digits(const float (&y)[8], const int (&E)[8], unsigned char* dst, int plane) {
+__device__ __forceinline__ void put_digits(const float (&y)[8], const int (&E)[8], unsigned char* dst, int plane,
+                                           unsigned char* dst2 = nullptr, int plane2 = 0) {
   constexpr int S = Dig<float>::S;
   constexpr float kRound = 12582912.f;   // 1.5 2^23: adding it rounds to an integer
   float r[8];
@@ -147,19 +171,14 @@ __device__ __forceinline__ void put_digits(const float (&y)[8], const int (&E)[8
 #pragma unroll
     for (int i = 0; i < 4; ++i) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(p[i]) : "f"(d[2 * i + 1]), "f"(d[2 * i]));
     *(uint4*)(dst + s * plane) = make_uint4(p[0], p[1], p[2], p[3]);
+    if (dst2) *(uint4*)(dst2 + s * plane2) = make_uint4(p[0], p[1], p[2], p[3]);
   }
 }
-__device__ __forceinline__ void put_digits(const float (&y)[8], int E, unsigned char* dst, int plane) {
+__device__ __forceinline__ void put_digits(const float (&y)[8], int E, unsigned char* dst, int plane,
+                                           unsigned char* dst2, int plane2) {
   const int e[8] = {E, E, E, E, E, E, E, E};
-  put_digits(y, e, dst, plane);
+  put_digits(y, e, dst, plane, dst2, plane2);
 }
-__device__ __forceinline__ void put_digits(const double (&y)[8], const int (&E)[8], unsigned char* dst, int plane) {
-  uint2 w[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) w[i] = biased_fixed(y[i], E[i]);
-  store_digits<Dig<double>::S>(w, dst, plane);
-}
-
 // instruction descriptor of kind::f16: D binary32, A and B binary16, K-major
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -174,22 +193,35 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc05::smem_u32(mbar)) : "memory");
 }
 
-// One thread: the digit products of one stage with level s + t = l into
-// one accumulator of 64 columns; `first`: the stage starts new sums.
-// Descriptors advance 256 bytes per K = 16 step.  The eight accumulators are
-// issued by eight warps: one thread issuing all 72 MMAs of a binary64 stage
-// took longer than the MMAs.
-template <int S>
-__device__ __forceinline__ void issue_level(uint32_t dtmem, uint64_t dA, uint64_t dB, int planeB, int l, bool first) {
-  constexpr uint32_t id = idesc_f16(128, 64);
-  bool acc = !first;
-  const int s0 = l < S ? 0 : l - S + 1, s1 = l < S ? l : S - 1;
-  for (int s = s0; s <= s1; ++s) {
-    const uint64_t a = dA + (uint64_t)((s * kPlaneA) >> 4), b = dB + (uint64_t)(((l - s) * planeB) >> 4);
+// One thread: all digit products of a stage with levels LB .. LB + 7 (s + t,
+// up to S - 1 each).  The right factor's planes follow one another with the
+// stride of their row groups, so planes t .. t + n - 1 are one operand of 64 n
+// rows, and their products with plane s go to the n accumulators of the levels
+// s + t .., which are neighbours too: one MMA of up to 256 columns.  (An MMA
+// reads its left factor from shared memory again: of 64 columns each, the 72
+// of a binary64 stage took 4500 clocks, eight warps issuing; the 28 wide ones
+// do 2300 clocks of multiplications.)  `first`: the stage starts new sums.
+// Descriptors advance 256 bytes per K = 16 step.
+template <int S, int LB>
+__device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t dA, uint64_t dB, bool first) {
+  static_assert(kPlaneB == 8 * kPlaneSbo, "planes of the right factor follow one another");
 #pragma unroll
-    for (int ks = 0; ks < kStK / 16; ++ks) {
-      mma_f16(dtmem, a + (uint64_t)((ks * 256) >> 4), b + (uint64_t)((ks * 256) >> 4), id, acc);
-      acc = true;
+  for (int ks = 0; ks < kStK / 16; ++ks) {
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      // the first products of a sum touch every level once, and overwrite it:
+      // plane 0 (LB = 0) or S - 1 alone, or (S = 5) planes 0 and 4 between them
+      const int s = S == 8 ? (LB == 0 ? i : S - 1 - i) : i == 0 ? 0 : i == 1 ? S - 1 : i - 1;
+      const int ta = LB > s ? LB - s : 0, tb = LB + 7 - s < S - 1 ? LB + 7 - s : S - 1;
+#pragma unroll
+      for (int t = ta; t <= tb;) {
+        const bool lone = S == 5 && i == 1 && t == 0;     // level 4 of plane 4: plane 0 has been there
+        const int n = lone ? 1 : tb - t + 1 < 4 ? tb - t + 1 : 4;
+        const bool fresh = ks == 0 && (i == 0 || (S == 5 && i == 1 && t > 0));
+        mma_f16(tmem + (s + t - LB) * 64, dA + (uint64_t)((s * kPlaneA + ks * 256) >> 4),
+                dB + (uint64_t)((t * kPlaneB + ks * 256) >> 4), idesc_f16(128, 64 * n), !(fresh && first));
+        t += n;
+      }
     }
   }
 }
@@ -236,16 +268,17 @@ constexpr int kDigThreads = 512;   // 128 registers a thread: 64 hold the intege
 
 template <int NST>
 struct DigitBarriers {
-  uint64_t full[NST], empty[NST], dfull, dempty, fin;
+  uint64_t full[NST], empty[NST], dfull, dempty, issued, fin;
   uint32_t tmem;
   // all threads; `extra`: arrivals on a full barrier besides one per warp of a group
   __device__ __forceinline__ void open(int extra) {
     if (threadIdx.x == 0) {
       for (int b = 0; b < NST; ++b) {
         tc05::mbar_init(full + b, kDigThreads / 64 + extra);
-        tc05::mbar_init(empty + b, kSlots);
+        tc05::mbar_init(empty + b, 1);
       }
-      tc05::mbar_init(&dfull, kSlots);
+      tc05::mbar_init(&dfull, 2);
+      tc05::mbar_init(&issued, 1);
       tc05::mbar_init(&dempty, kDigThreads / 32);
       tc05::mbar_init(&fin, kDigThreads / 32);
     }
@@ -266,20 +299,23 @@ struct DigitBarriers {
 };
 
 // Both pipelines: the stages alternate between two groups of eight warps.  A
-// group fills its stage (fills wait on loads and on the integer pipe), waits
-// for its eight warps, and each of them issues one accumulator's MMAs; the
-// other group fills meanwhile.  A stage's MMAs start after those of the stage
-// before are complete, since they go to the same accumulators from other
-// threads.  At the end of a sum all sixteen warps read the accumulators; the
-// group that fills the next sum's first stage does so before it reads.  (All
-// sixteen warps filling every stage together, one thread issuing: 25.8 ms for
-// the Gram matrix of 2,097,152 x 256 binary64; this way 20.)
+// group fills its stage (fills wait on loads and on the integer pipe) and one
+// thread issues the stage's MMAs when its eight warps are through; the other
+// group fills meanwhile.  The MMAs of successive stages go to the same
+// accumulators from two threads: a thread issues after the other has issued
+// (an mbarrier and the fences around it keep the order), not after those MMAs
+// are complete, which left the tensor cores idle for about 1000 clocks a
+// stage.  At the end of a sum all sixteen warps read the accumulators; the
+// group that fills the next sum's first stage does so before it reads.
 //
-// Deadlock freedom: a group waits for (1) the MMAs of an earlier stage,
-// (2) the reads of an earlier sum by the other group, which reads before it
-// fills unless it opens the sum itself, (3) the MMAs of the sum it reads,
-// issued once (2) holds for the sums before.  All are earlier in the order of
-// stages, and every wait is bounded.
+// A commit covers the MMAs of its own thread, so the last two stages of a sum
+// commit to `dfull` (two arrivals; a sum of one stage commits twice).
+//
+// Deadlock freedom: a group waits for (1) the MMAs of an earlier stage to be
+// issued or complete, (2) the reads of an earlier sum by the other group,
+// which reads before it fills unless it opens the sum itself, (3) the MMAs of
+// the sum it reads, issued once (2) holds for the sums before.  All are
+// earlier in the order of stages, and every wait is bounded.
 // (Counters are 32-bit and stage numbers advance without divisions.)
 template <int NST>
 struct StageSlot {      // buffer and phase parity of a stage number
@@ -294,21 +330,25 @@ struct StageSlot {      // buffer and phase parity of a stage number
   }
 };
 
-// One group's part of issuing a stage (every lane calls; lane 0 of each warp
-// issues): `cur` the stage, `prev` the one before it (j: its number).
+// Issuing stage j (buffer and phase `cur`): the first warp of the group that
+// filled it.  `commits`: arrivals on dfull (1 for the last two stages of a
+// sum, 2 for the only one, else 0).
 template <int NST, class Issue>
-__device__ __forceinline__ bool issue_turn(DigitBarriers<NST>& bar, const StageSlot<NST>& cur, const StageSlot<NST>& prev,
-                                           int j, int sum, bool first, bool last, uint32_t sa, Issue issue) {
+__device__ __forceinline__ bool issue_turn(DigitBarriers<NST>& bar, const StageSlot<NST>& cur, int j, int sum, bool first,
+                                           int commits, uint32_t sa, Issue issue) {
+  if ((threadIdx.x & 255) >= 32) return true;
   bool ok = true;
   if ((threadIdx.x & 31) == 0) {
     ok = mbar_wait_fast(bar.full + cur.b, cur.par);
-    if (ok && j > 0) ok = mbar_wait_fast(bar.empty + prev.b, prev.par);
+    if (ok && j > 0) ok = mbar_wait_fast(&bar.issued, (uint32_t)((j - 1) & 1));
     if (ok && first && sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((sum - 1) & 1));
     if (ok) {
       tc05::fence_after();
-      issue(bar.tmem, sa, (int)(threadIdx.x >> 5) & 7, first);
+      issue(bar.tmem, sa, first);
       tc05::commit(bar.empty + cur.b);
-      if (last) tc05::commit(&bar.dfull);
+      for (int c = 0; c < commits; ++c) tc05::commit(&bar.dfull);
+      tc05::fence_before();
+      mbar_arrive(&bar.issued);
     }
   }
   return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
@@ -329,13 +369,13 @@ __device__ __forceinline__ bool drain_turn(DigitBarriers<NST>& bar, int& drained
 }
 
 // Sums over a range of rows: `nstage` stages of kStK rows, read out every
-// kStagesPerSum of them.  fill(j, stage) writes this thread's part of stage
-// j; issue(tensor memory, stage address, slot, first) issues one
-// accumulator's MMAs; flush(acc0, acc1) hands on the 64-bit sums of this
+// kStagesPerSum of them.  fetch(j) loads this thread's part of stage j into
+// registers and fill(stage) writes its digits; issue(tensor memory, stage
+// address, first) issues the MMAs; flush(acc0, acc1) hands on the 64-bit sums of this
 // thread's row and 16 columns.
-template <int NST, class Fill, class Issue, class Flush>
+template <int NST, class Fetch, class Fill, class Issue, class Flush>
 __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int stage_bytes, int nstage,
-                                              int nslots, WsHeader* hdr, Fill fill, Issue issue, Flush flush) {
+                                              int nslots, WsHeader* hdr, Fetch fetch, Fill fill, Issue issue, Flush flush) {
   const int lane = threadIdx.x & 31, group = threadIdx.x >> 8;
   bar.open(0);
   const uint32_t base = tc05::smem_u32(gsm);
@@ -344,18 +384,19 @@ __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned 
 #pragma unroll
   for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
   int drained = 0;
-  StageSlot<NST> cur{group, 0u}, prev{group ? 0 : NST - 1, group ? 0u : 1u};
+  StageSlot<NST> cur{group, 0u};
   for (int j = group; j < nstage; j += 2) {
     const int sum = j / kStagesPerSum, js = j % kStagesPerSum;
     if (js != 0 && drained < sum) {
       ok = drain_turn(bar, drained, nslots, acc0, acc1);
       if (!ok) break;
     }
+    fetch(j);
     if (j >= NST) {
       ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + cur.b, cur.par ^ 1u));
       if (!ok) break;
     }
-    fill(j, gsm + cur.b * stage_bytes);
+    fill(gsm + cur.b * stage_bytes);
     tc05::fence_smem_async();
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.full + cur.b);
@@ -365,10 +406,9 @@ __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned 
     }
     // (64-bit sums of at most 2^20 rows)
     if (drained > 0 && (drained & 8191) == 0 && js < 2) flush(acc0, acc1);
-    ok = issue_turn(bar, cur, prev, j, sum, js == 0, js == kStagesPerSum - 1, base + cur.b * stage_bytes, issue);
+    ok = issue_turn(bar, cur, j, sum, js == 0, js >= kStagesPerSum - 2, base + cur.b * stage_bytes, issue);
     if (!ok) break;
     cur.advance2();
-    prev.advance2();
   }
   while (ok && drained * kStagesPerSum < nstage) ok = drain_turn(bar, drained, nslots, acc0, acc1);
   if (ok) flush(acc0, acc1);
@@ -414,11 +454,10 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
       }
     }
   };
-  auto issue = [&](uint32_t tmem, uint32_t sa, int slot, bool first) {
-    issue_level<S>(tmem + slot * 64, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo),
-                   kPlaneB, LB + slot, first);
+  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+    issue_stage<S, LB>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo), first);
   };
-  StageSlot<NST> cur{group, 0u}, prev{group ? 0 : NST - 1, group ? 0u : 1u};
+  StageSlot<NST> cur{group, 0u};
   int tile = 0, js = group, j = group;
   while (js >= stages) {
     js -= stages;
@@ -441,8 +480,9 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
     if (lane == 0) mbar_arrive(bar.full + cur.b);
     if (first) read_upto(sum);
     if (!ok) break;
-    ok = issue_turn(bar, cur, prev, j, sum, first, js % kStagesPerSum == kStagesPerSum - 1 || js == stages - 1,
-                    base + cur.b * kStage, issue);
+    // stages of this sum from this one on
+    const int in_sum = js % kStagesPerSum, rest = stages - js, left = rest < kStagesPerSum - in_sum ? rest : kStagesPerSum - in_sum;
+    ok = issue_turn(bar, cur, j, sum, first, left > 2 ? 0 : left == 1 && first ? 2 : 1, base + cur.b * kStage, issue);
     if (!ok) break;
     js += 2;
     while (js >= stages) {
@@ -450,7 +490,6 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
       ++tile;
     }
     cur.advance2();
-    prev.advance2();
   }
   read_upto(mine * sums);
   // bulk copies of stages that were never consumed (after a timeout) land

@@ -190,19 +190,15 @@ struct GramArgs {
   const unsigned* unless;
 };
 
-template <typename TY>
-__device__ __forceinline__ void load8(const TY* p, TY (&y)[8]);
-template <>
-__device__ __forceinline__ void load8<double>(const double* p, double (&y)[8]) {
+__device__ __forceinline__ void load8(const uint2* p, uint2 (&y)[8]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const double2 v = __ldg((const double2*)p + i);
-    y[2 * i] = v.x;
-    y[2 * i + 1] = v.y;
+    const uint4 v = __ldg((const uint4*)p + i);
+    y[2 * i] = make_uint2(v.x, v.y);
+    y[2 * i + 1] = make_uint2(v.z, v.w);
   }
 }
-template <>
-__device__ __forceinline__ void load8<float>(const float* p, float (&y)[8]) {
+__device__ __forceinline__ void load8(const float* p, float (&y)[8]) {
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const float4 v = __ldg((const float4*)p + i);
@@ -213,22 +209,65 @@ __device__ __forceinline__ void load8<float>(const float* p, float (&y)[8]) {
   }
 }
 
-// digits of the 8 rows at p of one column into a stage plane (zeros if !in)
-template <typename TY>
-__device__ __forceinline__ void put_column8(const TY* p, bool in, int E, unsigned char* dst, int plane) {
-  TY y[8];
+// the 8 rows at p of one column (zeros if !in)
+template <typename C>
+__device__ __forceinline__ void fetch8(const C* p, bool in, C (&y)[8]) {
   if (in) {
     load8(p, y);
   } else {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = (TY)0;
+    for (int i = 0; i < 8; ++i) y[i] = zero_cell<C>();
   }
-  put_digits(y, E, dst, plane);
+}
+
+// Binary64 columns -> biased fixed-point words in place, two rows a thread and
+// turn.  Bound by memory (16 bytes an element).
+constexpr int kPackThreads = 256, kPackRows = 2048;
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(double* Y, int64_t ldy, int64_t cols, const int* colE,
+                                                            const unsigned* unless) {
+  if (unless && *unless) return;
+  const int64_t r0 = (int64_t)blockIdx.x * kPackRows + 2 * threadIdx.x;
+  for (int64_t c = blockIdx.y; c < cols; c += gridDim.y) {
+    const int E = colE[c];
+    double* q = Y + c * ldy + r0;
+    double2 v[kPackRows / (2 * kPackThreads)];
+#pragma unroll
+    for (int u = 0; u < kPackRows / (2 * kPackThreads); ++u)
+      if (r0 + 2 * u * kPackThreads < ldy) v[u] = *(const double2*)(q + 2 * u * kPackThreads);
+#pragma unroll
+    for (int u = 0; u < kPackRows / (2 * kPackThreads); ++u)
+      if (r0 + 2 * u * kPackThreads < ldy) {
+        const uint2 a = biased_fixed(v[u].x, E), b = biased_fixed(v[u].y, E);
+        *(uint4*)(q + 2 * u * kPackThreads) = make_uint4(a.x, a.y, b.x, b.y);
+      }
+  }
+}
+cudaError_t launch_pack(double* Y, int64_t ldy, int64_t cols, const int* colE, const unsigned* unless, cudaStream_t st) {
+  const dim3 grid((unsigned)((ldy + kPackRows - 1) / kPackRows), (unsigned)(cols < 65535 ? cols : 65535));
+  pack_kernel<<<grid, kPackThreads, 0, st>>>(Y, ldy, cols, colE, unless);
+  return cudaGetLastError();
+}
+
+// Back to binary64 (to another buffer), for a Householder factorisation of
+// this Y; rows past N are not written.
+__global__ void __launch_bounds__(256) unpack_kernel(const double* P, int64_t ldy, int64_t N, int64_t M, const int* colE,
+                                                     double* Y, const unsigned* gram_y, const unsigned* redo) {
+  if (*gram_y == 0 || *redo == 0) return;
+  for (int64_t c = blockIdx.y; c < M; c += gridDim.y)
+    for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
+      Y[n + c * ldy] = from_fixed(*(const uint2*)(P + n + c * ldy), colE[c]);
+}
+cudaError_t launch_unpack(const GramState& g, double* Y, const unsigned* redo, cudaStream_t st) {
+  const int64_t bx = (g.N + 255) / 256;
+  const dim3 grid((unsigned)(bx < 64 ? bx : 64), (unsigned)(g.M < 65535 ? g.M : 65535));
+  unpack_kernel<<<grid, 256, 0, st>>>((const double*)g.Y, g.ldy, g.N, g.M, g.colE, Y, &g.hdr->gram_y, redo);
+  return cudaGetLastError();
 }
 
 template <typename TY>
 __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST;
+  typedef typename Cell<TY>::type C;
   extern __shared__ __align__(1024) unsigned char gsm[];
   __shared__ __align__(8) DigitBarriers<NST> bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -248,11 +287,11 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   }
   const int J = t;
   const bool diag = !a.Z && (J >> 1) == I;       // B's columns are among A's
-  const TY* B = (const TY*)(a.Z ? a.Z : a.Y);
+  const C* B = (const C*)(a.Z ? a.Z : a.Y);
   const int64_t ldb = a.Z ? a.ldz : a.ldy, nB = a.Z ? a.NZ : a.M;
   const int64_t nsum = (a.N + 127) / 128;
   const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
-  const TY* Y = (const TY*)a.Y;
+  const C* Y = (const C*)a.Y;
   const int c8 = lane & 7, kg = lane >> 3;
   const int gw = warp & 7;                       // a stage's eight warps: 16 columns of A and 8 of B each
   const int64_t colA = (int64_t)I * 128 + gw * 16 + c8, colB = (int64_t)J * 64 + gw * 8 + c8;
@@ -262,22 +301,29 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   // this thread's first row of the unit, and how many stages hold rows of Y
   const int64_t row0 = q0 * 128 + kg * 8;
   const int jin = (int)((a.ldy - row0 + kStK - 1) / kStK);
-  const TY* pA = Y + row0 + (colA < a.M ? colA : 0) * a.ldy;
-  const TY* pA8 = Y + row0 + (colA + 8 < a.M ? colA + 8 : 0) * a.ldy;
-  const TY* pB = B + row0 + (colB < nB ? colB : 0) * ldb;
+  const C* pA = Y + row0 + (colA < a.M ? colA : 0) * a.ldy;
+  const C* pA8 = Y + row0 + (colA + 8 < a.M ? colA + 8 : 0) * a.ldy;
+  const C* pB = B + row0 + (colB < nB ? colB : 0) * ldb;
   const int jA = colA < a.M ? jin : 0, jA8 = colA + 8 < a.M ? jin : 0, jB = colB < nB ? jin : 0;
-  auto fill = [&](int j, unsigned char* st) {
-    unsigned char* d = st + off + 2 * gw * kPlaneSbo;
-    put_column8<TY>(pA + j * kStK, j < jA, E0, d, kPlaneA);
-    put_column8<TY>(pA8 + j * kStK, j < jA8, E1, d + kPlaneSbo, kPlaneA);
-    if (!diag) put_column8<TY>(pB + j * kStK, j < jB, EB, st + S * kPlaneA + off + gw * kPlaneSbo, kPlaneB);
+  C yA[8], yA8[8], yB[8];
+  auto fetch = [&](int j) {
+    fetch8(pA + j * kStK, j < jA, yA);
+    fetch8(pA8 + j * kStK, j < jA8, yA8);
+    if (!diag) fetch8(pB + j * kStK, j < jB, yB);
   };
-  auto issue = [&](uint32_t tmem, uint32_t sa, int slot, bool first) {
-    const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
-    const uint64_t dB = diag ? tc05::desc(sa + (J & 1) * 8 * kPlaneSbo, 128, kPlaneSbo)
-                             : tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
-    const int planeB = diag ? kPlaneA : kPlaneB;
-    issue_level<S>(tmem + slot * 64, dA, dB, planeB, gram_base<TY>(half) + slot, first);
+  // on the diagonal four of the warps' columns are B's too
+  const int ob = diag && (gw >> 2) == (J & 1) ? S * kPlaneA + (int)off + 2 * (gw & 3) * kPlaneSbo : 0;
+  auto fill = [&](unsigned char* st) {
+    unsigned char* d = st + off + 2 * gw * kPlaneSbo;
+    unsigned char* db = ob ? st + ob : nullptr;
+    put_digits(yA, E0, d, kPlaneA, db, kPlaneB);
+    put_digits(yA8, E1, d + kPlaneSbo, kPlaneA, ob ? db + kPlaneSbo : nullptr, kPlaneB);
+    if (!diag) put_digits(yB, EB, st + S * kPlaneA + off + gw * kPlaneSbo, kPlaneB, nullptr, 0);
+  };
+  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+    const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo), dB = tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
+    if (half == 0) issue_stage<S, gram_base<TY>(0)>(tmem, dA, dB, first);
+    else issue_stage<S, gram_base<TY>(Dig<TY>::HALVES - 1)>(tmem, dA, dB, first);
   };
   auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
     const int64_t gi = (int64_t)I * 128 + (warp & 3) * 32 + lane;
@@ -292,7 +338,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
     }
   };
   gram_pipeline<NST>(bar, gsm, S * (kPlaneA + kPlaneB), (int)(q1 - q0) * kStagesPerSum,
-                     (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr, fill, issue, flush);
+                     (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr, fetch, fill, issue, flush);
 }
 
 // ---------------------------------------------------------------------------
@@ -620,6 +666,7 @@ cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xt
   if (g.f32) e = xtype == PYLOM_F32 ? prologue<float, float>(pa, sms, st) : prologue<double, float>(pa, sms, st);
   else e = xtype == PYLOM_F32 ? prologue<float, double>(pa, sms, st) : prologue<double, double>(pa, sms, st);
   if (e != cudaSuccess) return e;
+  if (!g.f32 && (e = launch_pack((double*)g.Y, g.ldy, g.M, g.colE, nullptr, st)) != cudaSuccess) return e;
   e = g.f32 ? gram_launch<float>(g, sms, nullptr, 0, 0, nullptr, g.G, nullptr, g.hdr, st)
             : gram_launch<double>(g, sms, nullptr, 0, 0, nullptr, g.G, nullptr, g.hdr, st);
   if (e != cudaSuccess) return e;

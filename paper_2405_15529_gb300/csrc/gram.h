@@ -8,7 +8,7 @@ namespace pylom {
 struct GramState {
   WsHeader* hdr;
   int64_t N, M, ldy;      // ldy: rows of Y rounded up to 8, the padding rows hold zeros
-  void* Y;                // N x M weighted centred matrix, binary64 or binary32
+  void* Y;                // N x M weighted centred matrix: binary32, or binary64 cut to fixed point (pack_kernel)
   bool f32;
   int* colE;              // M: largest exponent field of each column
   long long* G;           // 5 x M x M: integer sums, group g weighs 2^(32 g)
@@ -56,7 +56,11 @@ cudaError_t launch_modes_direct(const GramState& g, const double* C, const doubl
                                 const double* w, int physical, void* U, int64_t ldu, int64_t* r_out,
                                 cudaStream_t st, cudaEvent_t mid);
 
-// W = Y^T Z (M x NZ, ld M) from the same integer products.  G: 5 M NZ integers.
+// Binary64 columns -> fixed-point words in place (rows of zeros up to ldy), and Y
+// of a forward back to binary64 where *redo is set.
+cudaError_t launch_pack(double* Y, int64_t ldy, int64_t cols, const int* colE, const unsigned* unless, cudaStream_t st);
+cudaError_t launch_unpack(const GramState& g, double* Y, const unsigned* redo, cudaStream_t st);
+// W = Y^T Z (M x NZ, ld M) from the same integer products; Z as Y.  G: 5 M NZ integers.
 cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, long long* G,
                          double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st);
 // The product above into U (binary32 if f32, else binary64; ld ldu).

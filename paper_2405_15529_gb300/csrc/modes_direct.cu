@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArg
                                                                      int physical, TY* U, int64_t ldu,
                                                                      int64_t* r_out, WsHeader* hdr) {
   constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST, LB = Dig<TY>::LBM;
+  typedef typename Cell<TY>::type Cl;
   extern __shared__ __align__(1024) unsigned char gsm[];
   __shared__ __align__(8) DigitBarriers<NST> bar;
   if (p.unless && *p.unless) return;
@@ -94,21 +95,21 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArg
     const uint32_t tile = blockIdx.x + t * gridDim.x;
     const int64_t row = (int64_t)(tile / kt32) * 128 + rl;
     const bool rin = row < N, second = js >= s1;
-    const TY* Y = (const TY*)(second ? p.Z : p.Y);
+    const Cl* Y = (const Cl*)(second ? p.Z : p.Y);
     const int64_t ld = second ? p.ldz : p.ldy;
     const int* ex = second ? p.zE : p.colE;
     const int m32 = (int)(second ? p.NZ : p.M), j0 = (second ? js - s1 : js) * kStK;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int kg = 2 * kh + h, c0 = j0 + kg * 8;
-      const TY* q = Y + row + c0 * ld;
-      TY y[8];
+      const Cl* q = Y + row + c0 * ld;
+      Cl y[8];
       int E[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const bool in = c0 + i < m32;
-        y[i] = (in && rin) ? __ldg(q + i * ld) : (TY)0;
-        E[i] = in ? __ldg(ex + c0 + i) : 128;
+        y[i] = (in && rin) ? __ldg(q + i * ld) : zero_cell<Cl>();
+        E[i] = (S == 5 && in) ? __ldg(ex + c0 + i) : 128;   // (words carry their scale)
       }
       put_digits(y, E, st + offA + kg * 128, kPlaneA);
     }

@@ -258,7 +258,7 @@ size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool m
          (mixed ? mixed_extra_bytes(N, M, P) : 0);
 }
 
-cudaError_t launch_refactor(const TsqrState& fs, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
+cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
                             const double* UR, TsqrState& os, char** extra, double** UR_out, cudaStream_t st) {
   const size_t ub = align256(sizeof(double) * (size_t)fs.M * fs.M);
   char* own = base + ub;
@@ -271,8 +271,10 @@ cudaError_t launch_refactor(const TsqrState& fs, const char* fwd_extra, char* ba
   os.shiftx = mixed ? fwd_extra - oextra : 0;
   cudaError_t e = cudaMemsetAsync(os.arrive, 0, sizeof(unsigned) * (size_t)os.P, st);
   if (e != cudaSuccess) return e;
+  // (the leaves' own pass over Y is in place: Y is both source and destination)
+  if (!mixed && (e = launch_unpack(g, os.Y, &hdr->gram_redo, st)) != cudaSuccess) return e;
   e = mixed ? launch_tsqr_mixed(os, oextra, fwd_extra, y_ld(fs.N), PYLOM_F32, nullptr, 0, nullptr, st)
-            : launch_tsqr_fp64(os, fs.Y, fs.ldy, PYLOM_F64, nullptr, 0, nullptr, st);
+            : launch_tsqr_fp64(os, os.Y, os.ldy, PYLOM_F64, nullptr, 0, nullptr, st);
   if (e != cudaSuccess) return e;
   bw_signed_ur_kernel<<<64, 256, 0, st>>>(os, UR, (double*)base);
   *UR_out = (double*)base;

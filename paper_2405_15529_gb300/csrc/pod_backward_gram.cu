@@ -147,6 +147,7 @@ cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const do
     if (f.f32) bg_load_kernel<float><<<grid, 256, 0, st>>>(dU, lddu, w, physical, (float*)L.Z, ldz, N, L.zE, redo);
     else bg_load_kernel<double><<<grid, 256, 0, st>>>(dU, lddu, w, physical, (double*)L.Z, ldz, N, L.zE, redo);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (!f.f32 && (e = launch_pack((double*)L.Z, ldz, r, L.zE, redo, st)) != cudaSuccess) return e;
     if ((e = launch_cross(f, L.Z, ldz, r, L.zE, L.G, L.W, redo, hdr, st)) != cudaSuccess) return e;
     e = launch_bw_gemm(0, 0, M, r, M, 1.0, VT, ldvt, L.W, M, 0.0, L.A1, M, redo, st);            // V^T W
     if (e != cudaSuccess) return e;

@@ -166,10 +166,8 @@ __global__ void __launch_bounds__(256) bg_prologue_kernel(BG a) {
 // right factor is the column block J of 64.
 enum { kPlain = 0, kPacked = 1, kTurned = 2 };
 
-// digits of rows row..row+7 of a column (turned: (-im, re) pairs)
-__device__ __forceinline__ void put_rows8(const GramBin& b, int64_t row, int col, int E, bool turned, unsigned char* dst,
-                                          int plane) {
-  float y[8];
+// rows row..row+7 of a column (turned: (-im, re) pairs)
+__device__ __forceinline__ void fetch_rows8(const GramBin& b, int64_t row, int col, bool turned, float (&y)[8]) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) y[i] = 0.f;
   if (col < b.Nb) {
@@ -197,7 +195,6 @@ __device__ __forceinline__ void put_rows8(const GramBin& b, int64_t row, int col
       y[i + 1] = x;
     }
   }
-  put_digits(y, E, dst, plane);
 }
 
 __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
@@ -217,17 +214,25 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
   const int colB = J * 64 + gw * 8 + c8;
   const int EB = (sepB && colB < b.Nb) ? a.ints[b.colE + colB] : 128;
   const uint32_t off = (uint32_t)(kg * 128 + c8 * 16);
-  auto fill = [&](int j, unsigned char* st) {
+  float yA[8], yA8[8], yB[8];
+  auto fetch = [&](int j) {
     const int64_t row = (u.q0 * kStagesPerSum + j) * kStK + kg * 8;
-    put_rows8(b, row, colA, E0, turned, st + off + 2 * gw * kPlaneSbo, kPlaneA);
-    put_rows8(b, row, colA + 8, E1, turned, st + off + (2 * gw + 1) * kPlaneSbo, kPlaneA);
-    if (sepB) put_rows8(b, row, colB, EB, false, st + kSB * kPlaneA + off + gw * kPlaneSbo, kPlaneB);
+    fetch_rows8(b, row, colA, turned, yA);
+    fetch_rows8(b, row, colA + 8, turned, yA8);
+    if (sepB) fetch_rows8(b, row, colB, false, yB);
   };
-  auto issue = [&](uint32_t tmem, uint32_t sa, int slot, bool first) {
-    const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo);
-    const uint64_t dB = sepB ? tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo)
-                             : tc05::desc(sa + J * 8 * kPlaneSbo, 128, kPlaneSbo);
-    issue_level<kSB>(tmem + slot * 64, dA, dB, sepB ? kPlaneB : kPlaneA, gram_base<float>(0) + slot, first);
+  // the left factor's columns that are the right one's too
+  const int ob = !sepB && (gw >> 2) == J ? kSB * kPlaneA + (int)off + 2 * (gw & 3) * kPlaneSbo : 0;
+  auto fill = [&](unsigned char* st) {
+    unsigned char* d = st + off + 2 * gw * kPlaneSbo;
+    unsigned char* db = ob ? st + ob : nullptr;
+    put_digits(yA, E0, d, kPlaneA, db, kPlaneB);
+    put_digits(yA8, E1, d + kPlaneSbo, kPlaneA, ob ? db + kPlaneSbo : nullptr, kPlaneB);
+    if (sepB) put_digits(yB, EB, st + kSB * kPlaneA + off + gw * kPlaneSbo, kPlaneB, nullptr, 0);
+  };
+  auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
+    issue_stage<kSB, gram_base<float>(0)>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo),
+                                          first);
   };
   auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
     const int row = (warp & 3) * 32 + lane;
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<kNstB>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, fill, issue, flush);
+  gram_pipeline<kNstB>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, fetch, fill, issue, flush);
 }
 
 // ---------------------------------------------------------------------------
