@@ -13,7 +13,7 @@
 //   binary32: 38 bits, 5 digits.
 //
 // Layout of a digit plane in shared memory: K-major, no swizzle, core
-// matrices of 8 rows x 8 binary16 (128 contiguous bytes), kStK = 32 elements
+// matrices of 8 rows x 8 binary16 (128 contiguous bytes), kStK = 16 elements
 // of K per pipeline stage: core (a, b) at a * kPlaneSbo + b * 128.
 #pragma once
 #include "kernels.h"
@@ -21,23 +21,26 @@
 
 namespace pylom {
 
-constexpr int kStK = 32;                     // K elements per stage
+constexpr int kStK = 16;                     // K elements per stage
 constexpr int kPlaneSbo = (kStK / 8) * 128;  // bytes between 8-row groups
-constexpr int kPlaneA = 128 * kStK * 2;      // 8 KB: 128 rows
-constexpr int kPlaneB = 64 * kStK * 2;       // 4 KB: 64 rows
-constexpr int kStagesPerSum = 4;             // stages accumulated before the sums are read: 128 elements of K
+constexpr int kPlaneA = 128 * kStK * 2;      // 4 KB: 128 rows
+constexpr int kPlaneB = 64 * kStK * 2;       // 2 KB: 64 rows
+constexpr int kStagesPerSum = 8;             // stages accumulated before the sums are read: 128 elements of K
 constexpr int kSlots = 8;                    // accumulators (levels) of 64 columns in tensor memory
 
+constexpr int kRaw = 4;                      // stages of Y on their way in the Gram kernel
 template <typename TY> struct Dig;
 template <> struct Dig<double> {
   static constexpr int S = 8;          // digits
-  static constexpr int NST = 2;        // pipeline stages
+  static constexpr int NST = 4;        // pipeline stages of a product
+  static constexpr int GST = 2;        // of the Gram kernel, beside kRaw stages of Y itself
   static constexpr int HALVES = 2;     // level ranges of the Gram kernel: 0..7 and 8..14
   static constexpr int LBM = 7;        // lowest level of the modes kernel
 };
 template <> struct Dig<float> {
   static constexpr int S = 5;
-  static constexpr int NST = 3;
+  static constexpr int NST = 6;
+  static constexpr int GST = 4;
   static constexpr int HALVES = 1;     // levels 1..8 (level 0 lies 2^-60 below the top one)
   static constexpr int LBM = 1;
 };
@@ -332,14 +335,16 @@ struct StageSlot {      // buffer and phase parity of a stage number
 
 // Issuing stage j (buffer and phase `cur`): the first warp of the group that
 // filled it.  `commits`: arrivals on dfull (1 for the last two stages of a
-// sum, 2 for the only one, else 0).
-template <int NST, class Issue>
+// sum, 2 for the only one, else 0); ahead(): what can start once the stage is
+// filled.
+template <int NST, class Ahead, class Issue>
 __device__ __forceinline__ bool issue_turn(DigitBarriers<NST>& bar, const StageSlot<NST>& cur, int j, int sum, bool first,
-                                           int commits, uint32_t sa, Issue issue) {
+                                           int commits, uint32_t sa, Ahead ahead, Issue issue) {
   if ((threadIdx.x & 255) >= 32) return true;
   bool ok = true;
   if ((threadIdx.x & 31) == 0) {
     ok = mbar_wait_fast(bar.full + cur.b, cur.par);
+    if (ok) ahead();
     if (ok && j > 0) ok = mbar_wait_fast(&bar.issued, (uint32_t)((j - 1) & 1));
     if (ok && first && sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((sum - 1) & 1));
     if (ok) {
@@ -369,13 +374,17 @@ __device__ __forceinline__ bool drain_turn(DigitBarriers<NST>& bar, int& drained
 }
 
 // Sums over a range of rows: `nstage` stages of kStK rows, read out every
-// kStagesPerSum of them.  fetch(j) loads this thread's part of stage j into
+// kStagesPerSum of them.  fetch(j) brings this thread's part of stage j into
 // registers and fill(stage) writes its digits; issue(tensor memory, stage
-// address, first) issues the MMAs; flush(acc0, acc1) hands on the 64-bit sums of this
-// thread's row and 16 columns.
-template <int NST, class Fetch, class Fill, class Issue, class Flush>
+// address, first) issues the MMAs; flush(acc0, acc1) hands on the 64-bit sums
+// of this thread's row and 16 columns.  RAW = 0: fetch loads from global
+// memory, a turn ahead.  RAW > 0 (even): it reads a ring of RAW stages in
+// shared memory, which copy(j) (one thread, asynchronous) fills RAW stages
+// ahead; settle(j) waits for the copies up to stage j, after a timeout.
+template <int NST, int RAW, class Copy, class Settle, class Fetch, class Fill, class Issue, class Flush>
 __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int stage_bytes, int nstage,
-                                              int nslots, WsHeader* hdr, Fetch fetch, Fill fill, Issue issue, Flush flush) {
+                                              int nslots, WsHeader* hdr, Copy copy, Settle settle, Fetch fetch, Fill fill,
+                                              Issue issue, Flush flush) {
   const int lane = threadIdx.x & 31, group = threadIdx.x >> 8;
   bar.open(0);
   const uint32_t base = tc05::smem_u32(gsm);
@@ -383,15 +392,27 @@ __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned 
   int64_t acc0[16], acc1[16];
 #pragma unroll
   for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
-  int drained = 0;
+  int drained = 0, copied = group - 2;
+  auto ahead = [&](int j) {
+    if (RAW > 0 && j < nstage) {
+      copy(j);
+      copied = j;
+    }
+  };
+  if ((threadIdx.x & 255) == 0)
+    for (int j = group; j < RAW; j += 2) ahead(j);
   StageSlot<NST> cur{group, 0u};
+  if (RAW == 0 && group < nstage) fetch(group);
   for (int j = group; j < nstage; j += 2) {
     const int sum = j / kStagesPerSum, js = j % kStagesPerSum;
     if (js != 0 && drained < sum) {
       ok = drain_turn(bar, drained, nslots, acc0, acc1);
       if (!ok) break;
     }
-    fetch(j);
+    if (RAW > 0) {
+      ok = fetch(j);
+      if (!ok) break;
+    }
     if (j >= NST) {
       ok = __all_sync(0xffffffffu, mbar_wait_fast(bar.empty + cur.b, cur.par ^ 1u));
       if (!ok) break;
@@ -400,18 +421,21 @@ __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned 
     tc05::fence_smem_async();
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.full + cur.b);
+    if (RAW == 0 && j + 2 < nstage) fetch(j + 2);
     if (js == 0 && drained < sum) {
       ok = drain_turn(bar, drained, nslots, acc0, acc1);
       if (!ok) break;
     }
     // (64-bit sums of at most 2^20 rows)
     if (drained > 0 && (drained & 8191) == 0 && js < 2) flush(acc0, acc1);
-    ok = issue_turn(bar, cur, j, sum, js == 0, js >= kStagesPerSum - 2, base + cur.b * stage_bytes, issue);
+    ok = issue_turn(bar, cur, j, sum, js == 0, js >= kStagesPerSum - 2, base + cur.b * stage_bytes,
+                    [&] { ahead(j + RAW); }, issue);
     if (!ok) break;
     cur.advance2();
   }
   while (ok && drained * kStagesPerSum < nstage) ok = drain_turn(bar, drained, nslots, acc0, acc1);
   if (ok) flush(acc0, acc1);
+  else if (RAW > 0 && (threadIdx.x & 255) == 0) settle(copied);
   bar.close(ok, hdr);
 }
 
@@ -423,14 +447,14 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 }
 
 // Products of `mine` output tiles of 128 rows x 64 columns, K = `stages`
-// stages of kStK elements each, as one sequence of stages: fill(tile, js,
-// stage) writes the left factor's digits, the right factor's planes come by
+// stages of kStK elements each, as one sequence of stages: fetch(tile, js)
+// loads the left factor a turn ahead, fill(tile, js, stage) writes its digits, the right factor's planes come by
 // a bulk copy from bsrc(tile, js), store(tile, acc0, acc1) writes this
 // thread's row and 16 columns.  `tile` counts 0 .. mine - 1.  LB: lowest
 // level that is kept.
-template <int S, int NST, int LB, class Fill, class Src, class Store>
+template <int S, int NST, int LB, class Fetch, class Fill, class Src, class Store>
 __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int mine, int stages,
-                                                 WsHeader* hdr, Fill fill, Src bsrc, Store store) {
+                                                 WsHeader* hdr, Fetch fetch, Fill fill, Src bsrc, Store store) {
   constexpr int kStage = S * (kPlaneA + kPlaneB);
   const int tid = threadIdx.x, lane = tid & 31, group = tid >> 8;
   bar.open(1);
@@ -463,7 +487,13 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
     js -= stages;
     ++tile;
   }
+  if (tile < mine) fetch(tile, js);
   for (; tile < mine; j += 2) {
+    int ntile = tile, njs = js + 2;      // this group's next stage
+    while (njs >= stages) {
+      njs -= stages;
+      ++ntile;
+    }
     const int sum = tile * sums + js / kStagesPerSum;
     const bool first = js % kStagesPerSum == 0;
     if (!first) read_upto(sum);
@@ -478,17 +508,16 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
     tc05::fence_smem_async();
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.full + cur.b);
+    if (ntile < mine) fetch(ntile, njs);
     if (first) read_upto(sum);
     if (!ok) break;
     // stages of this sum from this one on
     const int in_sum = js % kStagesPerSum, rest = stages - js, left = rest < kStagesPerSum - in_sum ? rest : kStagesPerSum - in_sum;
-    ok = issue_turn(bar, cur, j, sum, first, left > 2 ? 0 : left == 1 && first ? 2 : 1, base + cur.b * kStage, issue);
+    ok = issue_turn(bar, cur, j, sum, first, left > 2 ? 0 : left == 1 && first ? 2 : 1, base + cur.b * kStage, [] {},
+                    issue);
     if (!ok) break;
-    js += 2;
-    while (js >= stages) {
-      js -= stages;
-      ++tile;
-    }
+    js = njs;
+    tile = ntile;
     cur.advance2();
   }
   read_upto(mine * sums);

@@ -177,48 +177,18 @@ __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(
 // integer atomics, so the result does not depend on the order.
 
 struct GramArgs {
-  const void* Y;
-  int64_t ldy, N, M;
+  int64_t ldy, N, M;      // ldy: rows that exist (N rounded up to 8)
   const int* colE;
   unsigned long long* G;
   int nJ, items, splits;
   WsHeader* hdr;
   // Y^T Z instead of Y^T Y: Z (N x NZ), its exponents, all tiles
   const void* Z;
-  int64_t ldz, NZ;
+  int64_t NZ;
   const int* zE;
   const unsigned* unless;
+  CUtensorMap mapA, mapB;   // Y in boxes of kStK rows x 128 columns; the right factor, x 64
 };
-
-__device__ __forceinline__ void load8(const uint2* p, uint2 (&y)[8]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint4 v = __ldg((const uint4*)p + i);
-    y[2 * i] = make_uint2(v.x, v.y);
-    y[2 * i + 1] = make_uint2(v.z, v.w);
-  }
-}
-__device__ __forceinline__ void load8(const float* p, float (&y)[8]) {
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float4 v = __ldg((const float4*)p + i);
-    y[4 * i] = v.x;
-    y[4 * i + 1] = v.y;
-    y[4 * i + 2] = v.z;
-    y[4 * i + 3] = v.w;
-  }
-}
-
-// the 8 rows at p of one column (zeros if !in)
-template <typename C>
-__device__ __forceinline__ void fetch8(const C* p, bool in, C (&y)[8]) {
-  if (in) {
-    load8(p, y);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = zero_cell<C>();
-  }
-}
 
 // Binary64 columns -> biased fixed-point words in place, two rows a thread and
 // turn.  Bound by memory (16 bytes an element).
@@ -265,11 +235,13 @@ cudaError_t launch_unpack(const GramState& g, double* Y, const unsigned* redo, c
 }
 
 template <typename TY>
-__global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
-  constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST;
+__global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(const __grid_constant__ GramArgs a) {
+  constexpr int S = Dig<TY>::S, NST = Dig<TY>::GST, kStage = S * (kPlaneA + kPlaneB);
+  constexpr int kPitch = kStK * (int)sizeof(TY), kRawA = 128 * kPitch, kRawStage = kRawA + 64 * kPitch;
   typedef typename Cell<TY>::type C;
   extern __shared__ __align__(1024) unsigned char gsm[];
   __shared__ __align__(8) DigitBarriers<NST> bar;
+  __shared__ __align__(8) uint64_t raw_full[kRaw];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int item = blockIdx.x % a.items, split = blockIdx.x / a.items;
   const int half = item % Dig<TY>::HALVES;
@@ -287,38 +259,60 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
   }
   const int J = t;
   const bool diag = !a.Z && (J >> 1) == I;       // B's columns are among A's
-  const C* B = (const C*)(a.Z ? a.Z : a.Y);
-  const int64_t ldb = a.Z ? a.ldz : a.ldy, nB = a.Z ? a.NZ : a.M;
+  const int64_t nB = a.Z ? a.NZ : a.M;
   const int64_t nsum = (a.N + 127) / 128;
   const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
-  const C* Y = (const C*)a.Y;
-  const int c8 = lane & 7, kg = lane >> 3;
-  const int gw = warp & 7;                       // a stage's eight warps: 16 columns of A and 8 of B each
-  const int64_t colA = (int64_t)I * 128 + gw * 16 + c8, colB = (int64_t)J * 64 + gw * 8 + c8;
-  const int E0 = colA < a.M ? a.colE[colA] : 128, E1 = colA + 8 < a.M ? a.colE[colA + 8] : 128;
+  // a thread of a stage's group: 8 rows of one of A's columns, and threads
+  // 128.. 8 rows of one of B's
+  const int th = tid & 255, ca = th & 127, kg = th >> 7, cb = th & 63, kb = (th >> 6) & 1;
+  const int64_t colA = (int64_t)I * 128 + ca, colB = (int64_t)J * 64 + cb;
+  const int EA = colA < a.M ? a.colE[colA] : 128;
   const int EB = (!diag && colB < nB) ? (a.Z ? a.zE : a.colE)[colB] : 128;
-  const uint32_t off = (uint32_t)(kg * 128 + c8 * 16);
-  // this thread's first row of the unit, and how many stages hold rows of Y
-  const int64_t row0 = q0 * 128 + kg * 8;
-  const int jin = (int)((a.ldy - row0 + kStK - 1) / kStK);
-  const C* pA = Y + row0 + (colA < a.M ? colA : 0) * a.ldy;
-  const C* pA8 = Y + row0 + (colA + 8 < a.M ? colA + 8 : 0) * a.ldy;
-  const C* pB = B + row0 + (colB < nB ? colB : 0) * ldb;
-  const int jA = colA < a.M ? jin : 0, jA8 = colA + 8 < a.M ? jin : 0, jB = colB < nB ? jin : 0;
-  C yA[8], yA8[8], yB[8];
-  auto fetch = [&](int j) {
-    fetch8(pA + j * kStK, j < jA, yA);
-    fetch8(pA8 + j * kStK, j < jA8, yA8);
-    if (!diag) fetch8(pB + j * kStK, j < jB, yB);
+  const int row0 = (int)(q0 * 128);
+  // stages whose rows kg 8.. (kb 8..) are rows of Y (columns past the last: none)
+  const int jA = colA < a.M ? (int)((a.ldy - row0 - kg * 8 + kStK - 1) / kStK) : 0;
+  const int jB = colB < nB ? (int)((a.ldy - row0 - kb * 8 + kStK - 1) / kStK) : 0;
+  unsigned char* raw = gsm + NST * kStage;
+  if (tid == 0)
+    for (int q = 0; q < kRaw; ++q) tc05::mbar_init(raw_full + q, 1);
+  auto copy = [&](int j) {
+    unsigned char* r = raw + (j % kRaw) * kRawStage;
+    uint64_t* m = raw_full + j % kRaw;
+    tc05::mbar_arrive_expect_tx(m, diag ? kRawA : kRawStage);
+    tc05::tma_load_2d(r, &a.mapA, row0 + j * kStK, I * 128, m);
+    if (!diag) tc05::tma_load_2d(r + kRawA, &a.mapB, row0 + j * kStK, J * 64, m);
   };
-  // on the diagonal four of the warps' columns are B's too
-  const int ob = diag && (gw >> 2) == (J & 1) ? S * kPlaneA + (int)off + 2 * (gw & 3) * kPlaneSbo : 0;
+  auto settle = [&](int j) {
+    for (int q = j; q > j - kRaw && q >= 0; q -= 2) tc05::mbar_wait(raw_full + q % kRaw, (uint32_t)((q / kRaw) & 1), 1000000ull);
+  };
+  // eight rows of a column from the swizzled box at p
+  auto read8 = [&](const unsigned char* p, int col, int k8, bool in, C (&y)[8]) {
+    constexpr int kChunks = 8 * (int)sizeof(TY) / 16;
+    const int x = sizeof(TY) == 8 ? col & 7 : (col >> 1) & 3;
+#pragma unroll
+    for (int i = 0; i < kChunks; ++i)
+      ((uint4*)y)[i] = *(const uint4*)(p + col * kPitch + (((k8 * kChunks + i) ^ x) << 4));
+    if (!in) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) y[i] = zero_cell<C>();
+    }
+  };
+  __align__(16) C yA[8], yB[8];
+  auto fetch = [&](int j) {
+    if (!__all_sync(0xffffffffu, mbar_wait_fast(raw_full + j % kRaw, (uint32_t)((j / kRaw) & 1)))) return false;
+    const unsigned char* r = raw + (j % kRaw) * kRawStage;
+    read8(r, ca, kg, j < jA, yA);
+    if (!diag && th >= 128) read8(r + kRawA, cb, kb, j < jB, yB);
+    return true;
+  };
+  const int oa = (ca >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
+  // on the diagonal half of A's columns are B's too
+  const int ob = S * kPlaneA + ((ca & 63) >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
+  const bool both = diag && (ca >> 6) == (J & 1);
   auto fill = [&](unsigned char* st) {
-    unsigned char* d = st + off + 2 * gw * kPlaneSbo;
-    unsigned char* db = ob ? st + ob : nullptr;
-    put_digits(yA, E0, d, kPlaneA, db, kPlaneB);
-    put_digits(yA8, E1, d + kPlaneSbo, kPlaneA, ob ? db + kPlaneSbo : nullptr, kPlaneB);
-    if (!diag) put_digits(yB, EB, st + S * kPlaneA + off + gw * kPlaneSbo, kPlaneB, nullptr, 0);
+    put_digits(yA, EA, st + oa, kPlaneA, both ? st + ob : nullptr, kPlaneB);
+    if (!diag && th >= 128)
+      put_digits(yB, EB, st + S * kPlaneA + (cb >> 3) * kPlaneSbo + (cb & 7) * 16 + kb * 128, kPlaneB, nullptr, 0);
   };
   auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
     const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo), dB = tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
@@ -337,8 +331,8 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(GramArgs a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<NST>(bar, gsm, S * (kPlaneA + kPlaneB), (int)(q1 - q0) * kStagesPerSum,
-                     (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr, fetch, fill, issue, flush);
+  gram_pipeline<NST, kRaw>(bar, gsm, kStage, (int)(q1 - q0) * kStagesPerSum, (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr,
+                           copy, settle, fetch, fill, issue, flush);
 }
 
 // ---------------------------------------------------------------------------
@@ -608,21 +602,48 @@ static int row_splits(int64_t items, int64_t nsum, int sms) {
   return best;
 }
 
+// Row coordinates of the tensor maps are 32-bit: taller matrices go in parts.
+constexpr int64_t kGramRows = 1ll << 30;
+
 template <typename TY>
 static cudaError_t gram_launch(const GramState& g, int sms, const void* Z, int64_t ldz, int64_t NZ, const int* zE,
                                long long* G, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
   constexpr int S = Dig<TY>::S;
-  constexpr size_t smem = (size_t)Dig<TY>::NST * S * (kPlaneA + kPlaneB);
+  constexpr size_t smem = (size_t)Dig<TY>::GST * S * (kPlaneA + kPlaneB) + (size_t)kRaw * 192 * kStK * sizeof(TY);
   cudaError_t e = ensure_dyn_smem((const void*)gram_kernel<TY>, smem);
   if (e != cudaSuccess) return e;
   const int nJ = (int)(((Z ? NZ : g.M) + 63) / 64), nI = (int)((g.M + 127) / 128);
   int tiles = 0;
   for (int I = 0; I < nI; ++I) tiles += Z ? nJ : nJ - 2 * I;
-  GramArgs a{g.Y, g.ldy, g.N, g.M, g.colE, (unsigned long long*)G, nJ, tiles * Dig<TY>::HALVES, 1, hdr, Z, ldz, NZ, zE,
-             unless};
-  a.splits = row_splits(a.items, (g.N + 127) / 128, sms);
-  gram_kernel<TY><<<(unsigned)(a.items * a.splits), kDigThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  for (int64_t r = 0; r < g.N; r += kGramRows) {
+    const int64_t N = g.N - r < kGramRows ? g.N - r : kGramRows;
+    GramArgs a{};
+    a.ldy = g.ldy - r < kGramRows ? g.ldy - r : kGramRows;     // rows of this part
+    a.N = N;
+    a.M = g.M;
+    a.colE = g.colE;
+    a.G = (unsigned long long*)G;
+    a.nJ = nJ;
+    a.items = tiles * Dig<TY>::HALVES;
+    a.hdr = hdr;
+    a.Z = Z;
+    a.NZ = NZ;
+    a.zE = zE;
+    a.unless = unless;
+    a.splits = row_splits(a.items, (N + 127) / 128, sms);
+    // words go as integers; 128 (64) bytes of a column, swizzled so that eight
+    // neighbouring columns lie in different banks
+    const CUtensorMapDataType type = sizeof(TY) == 8 ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const CUtensorMapSwizzle swz = sizeof(TY) == 8 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    const int64_t ldb = Z ? ldz : g.ldy;
+    e = tensor_map_2d(&a.mapA, type, (TY*)g.Y + r, a.ldy, g.M, g.ldy * (int64_t)sizeof(TY), kStK, 128, swz);
+    if (e == cudaSuccess)
+      e = tensor_map_2d(&a.mapB, type, (TY*)(Z ? Z : g.Y) + r, a.ldy, Z ? NZ : g.M, ldb * (int64_t)sizeof(TY), kStK, 64, swz);
+    if (e != cudaSuccess) return e;
+    gram_kernel<TY><<<(unsigned)(a.items * a.splits), kDigThreads, smem, st>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // integers of Y^T Z -> W

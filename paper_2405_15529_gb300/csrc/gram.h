@@ -1,9 +1,15 @@
 // gram.h -- the Gram route of the POD: R from an exact Gram matrix, modes by
 // a direct product (gram.cu, modes_direct.cu).
 #pragma once
+#include <cuda.h>
+
 #include "kernels.h"
 
 namespace pylom {
+
+// tsqr_mixed.cu: tensor map of a column-major matrix in boxes of box_rows x box_cols; what a box has past it reads zeros
+cudaError_t tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, void* base, int64_t rows, int64_t cols,
+                          int64_t ld_bytes, int box_rows, int box_cols, CUtensorMapSwizzle swizzle);
 
 struct GramState {
   WsHeader* hdr;

@@ -91,28 +91,27 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArg
   const int rl = tid & 127, kh = (tid >> 7) & 1; // row of the tile, half of the stage's columns
   const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
   const int mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
-  auto fill = [&](int t, int js, unsigned char* st) {
+  Cl y[8];
+  auto fetch = [&](int t, int js) {
     const uint32_t tile = blockIdx.x + t * gridDim.x;
     const int64_t row = (int64_t)(tile / kt32) * 128 + rl;
     const bool rin = row < N, second = js >= s1;
-    const Cl* Y = (const Cl*)(second ? p.Z : p.Y);
     const int64_t ld = second ? p.ldz : p.ldy;
-    const int* ex = second ? p.zE : p.colE;
-    const int m32 = (int)(second ? p.NZ : p.M), j0 = (second ? js - s1 : js) * kStK;
+    const int c0 = (second ? js - s1 : js) * kStK + kh * 8, m32 = (int)(second ? p.NZ : p.M);
+    const Cl* q = (const Cl*)(second ? p.Z : p.Y) + row + c0 * ld;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int kg = 2 * kh + h, c0 = j0 + kg * 8;
-      const Cl* q = Y + row + c0 * ld;
-      Cl y[8];
-      int E[8];
+    for (int i = 0; i < 8; ++i) y[i] = (c0 + i < m32 && rin) ? __ldg(q + i * ld) : zero_cell<Cl>();
+  };
+  auto fill = [&](int, int js, unsigned char* st) {
+    int E[8];
+    if (S == 5) {       // (words carry their scale)
+      const bool second = js >= s1;
+      const int* ex = second ? p.zE : p.colE;
+      const int c0 = (second ? js - s1 : js) * kStK + kh * 8, m32 = (int)(second ? p.NZ : p.M);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const bool in = c0 + i < m32;
-        y[i] = (in && rin) ? __ldg(q + i * ld) : zero_cell<Cl>();
-        E[i] = (S == 5 && in) ? __ldg(ex + c0 + i) : 128;   // (words carry their scale)
-      }
-      put_digits(y, E, st + offA + kg * 128, kPlaneA);
+      for (int i = 0; i < 8; ++i) E[i] = c0 + i < m32 ? __ldg(ex + c0 + i) : 128;
     }
+    put_digits(y, E, st + offA + kh * 128, kPlaneA);
   };
   auto bsrc = [&](int t, int js) {
     const uint32_t tile = blockIdx.x + t * gridDim.x;
@@ -138,7 +137,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArg
       }
     }
   };
-  product_pipeline<S, NST, LB>(bar, gsm, mine, stages, hdr, fill, bsrc, store);
+  product_pipeline<S, NST, LB>(bar, gsm, mine, stages, hdr, fetch, fill, bsrc, store);
 }
 
 // Smallest kept value, relative to the largest, for which Y V_r S_r^-1 is

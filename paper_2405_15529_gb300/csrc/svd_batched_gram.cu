@@ -204,31 +204,31 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
   const GramUnit u = a.units[blockIdx.x];
   const GramBin b = a.bins[u.bin];
   const int mode = u.mode, J = u.J;
-  // a stage's eight warps: 16 rows of the left factor (columns of Y) and 8 of the right each
-  const int c8 = lane & 7, kg = lane >> 3, gw = warp & 7, ca = gw * 16 + c8;
-  const bool turned = mode == kTurned || (mode == kPacked && gw >= 4);
+  // a thread of a stage's group: 8 rows of one left column, and threads 128..
+  // 8 rows of one right column
+  const int t = threadIdx.x & 255, ca = t & 127, kg = t >> 7, cb = t & 63, kb = (t >> 6) & 1;
+  const bool turned = mode == kTurned || (mode == kPacked && ca >= 64);
   // real items have nothing to turn: their second half is empty
-  const int colA = (mode == kPacked && gw >= 4 && !b.cplx) ? 128 : mode == kPacked ? (ca & 63) : ca;
-  const int E0 = colA < b.Nb ? a.ints[b.colE + colA] : 128, E1 = colA + 8 < b.Nb ? a.ints[b.colE + colA + 8] : 128;
+  const int colA = (mode == kPacked && ca >= 64 && !b.cplx) ? 128 : mode == kPacked ? (ca & 63) : ca;
+  const int EA = colA < b.Nb ? a.ints[b.colE + colA] : 128;
   const bool sepB = mode == kTurned;             // else the right factor's columns are among the left's
-  const int colB = J * 64 + gw * 8 + c8;
+  const int colB = J * 64 + cb;
   const int EB = (sepB && colB < b.Nb) ? a.ints[b.colE + colB] : 128;
-  const uint32_t off = (uint32_t)(kg * 128 + c8 * 16);
-  float yA[8], yA8[8], yB[8];
+  float yA[8], yB[8];
   auto fetch = [&](int j) {
-    const int64_t row = (u.q0 * kStagesPerSum + j) * kStK + kg * 8;
-    fetch_rows8(b, row, colA, turned, yA);
-    fetch_rows8(b, row, colA + 8, turned, yA8);
-    if (sepB) fetch_rows8(b, row, colB, false, yB);
+    const int64_t row = (u.q0 * kStagesPerSum + j) * kStK;
+    fetch_rows8(b, row + kg * 8, colA, turned, yA);
+    if (sepB && t >= 128) fetch_rows8(b, row + kb * 8, colB, false, yB);
+    return true;
   };
+  const int oa = (ca >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
   // the left factor's columns that are the right one's too
-  const int ob = !sepB && (gw >> 2) == J ? kSB * kPlaneA + (int)off + 2 * (gw & 3) * kPlaneSbo : 0;
+  const int ob = kSB * kPlaneA + ((ca & 63) >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
+  const bool both = !sepB && (ca >> 6) == J;
   auto fill = [&](unsigned char* st) {
-    unsigned char* d = st + off + 2 * gw * kPlaneSbo;
-    unsigned char* db = ob ? st + ob : nullptr;
-    put_digits(yA, E0, d, kPlaneA, db, kPlaneB);
-    put_digits(yA8, E1, d + kPlaneSbo, kPlaneA, ob ? db + kPlaneSbo : nullptr, kPlaneB);
-    if (sepB) put_digits(yB, EB, st + kSB * kPlaneA + off + gw * kPlaneSbo, kPlaneB, nullptr, 0);
+    put_digits(yA, EA, st + oa, kPlaneA, both ? st + ob : nullptr, kPlaneB);
+    if (sepB && t >= 128)
+      put_digits(yB, EB, st + kSB * kPlaneA + (cb >> 3) * kPlaneSbo + (cb & 7) * 16 + kb * 128, kPlaneB, nullptr, 0);
   };
   auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
     issue_stage<kSB, gram_base<float>(0)>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo),
@@ -250,7 +250,8 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<kNstB>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, fetch, fill, issue, flush);
+  gram_pipeline<kNstB, 0>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, [](int) {}, [](int) {}, fetch, fill,
+                          issue, flush);
 }
 
 // ---------------------------------------------------------------------------
@@ -866,23 +867,20 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
   const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
   const int* E = a.ints + b.colE;
   const int* Ce = a.ints + b.colE + n;
-  auto fill = [&](int t, int js, unsigned char* st) {
+  float y[8];
+  auto fetch = [&](int t, int js) {
     const int64_t row = (u.q0 + t) * 128 + rl;
-    const bool rin = row < b.rows;
+    const int c0 = js * kStK + kh * 8;
+    const float* p = b.Y + row + c0 * b.ldy;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int kg = 2 * kh + h, c0 = js * kStK + kg * 8;
-      const float* p = b.Y + row + c0 * b.ldy;
-      float y[8];
-      int e[8];
+    for (int i = 0; i < 8; ++i) y[i] = (c0 + i < n && row < b.rows) ? __ldg(p + i * b.ldy) : 0.f;
+  };
+  auto fill = [&](int, int js, unsigned char* st) {
+    const int c0 = js * kStK + kh * 8;
+    int e[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int c = c0 + i;
-        y[i] = (c < n && rin) ? __ldg(p + i * b.ldy) : 0.f;
-        e[i] = c < n ? __ldg(E + c) : 128;
-      }
-      put_digits(y, e, st + offA + kg * 128, kPlaneA);
-    }
+    for (int i = 0; i < 8; ++i) e[i] = c0 + i < n ? __ldg(E + c0 + i) : 128;
+    put_digits(y, e, st + offA + kh * 128, kPlaneA);
   };
   auto bsrc = [&](int, int js) { return a.c + b.c + js * kSB * (int64_t)kPlaneB; };
   auto store = [&](int t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
@@ -911,7 +909,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
         if (k0 + c < b.k && row < b.rows) b.Ur[row + (int64_t)(k0 + c) * b.ldu] = (float)(value(c) * iw);
     }
   };
-  product_pipeline<kSB, kNstB, LB>(bar, gsm, (int)(u.q1 - u.q0), stages, a.hdr, fill, bsrc, store);
+  product_pipeline<kSB, kNstB, LB>(bar, gsm, (int)(u.q1 - u.q0), stages, a.hdr, fetch, fill, bsrc, store);
 }
 
 }  // namespace

@@ -1146,10 +1146,8 @@ size_t mixed_extra_bytes(int64_t N, int64_t M, int64_t P) {
          align256(sizeof(float) * (size_t)(N / kCR + P + 1) * kHrSlot);
 }
 
-// Tensor map of the FP32 working copy (N x M, column-major, leading
-// dimension yf_ld(N)) with boxes of kTmaRows rows x `cols` columns;
-// out-of-range parts of a box read zeros.
-static cudaError_t encode_yf_map(CUtensorMap* map, float* Yf, int64_t N, int64_t M, int cols) {
+cudaError_t tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, void* base, int64_t rows, int64_t cols,
+                          int64_t ld_bytes, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   static std::mutex mu;
   {
@@ -1163,16 +1161,22 @@ static cudaError_t encode_yf_map(CUtensorMap* map, float* Yf, int64_t N, int64_t
       encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     }
   }
-  // rows past N (the padding of the leading dimension) are out of range:
-  // they read as zeros, never as uninitialised memory
-  const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)M};
-  const cuuint64_t strides[1] = {(cuuint64_t)yf_ld(N) * sizeof(float)};
-  const cuuint32_t box[2] = {(cuuint32_t)kTmaRows, (cuuint32_t)cols};
+  const cuuint64_t dims[2] = {(cuuint64_t)rows, (cuuint64_t)cols};
+  const cuuint64_t strides[1] = {(cuuint64_t)ld_bytes};
+  const cuuint32_t box[2] = {(cuuint32_t)box_rows, (cuuint32_t)box_cols};
   const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)Yf, dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+  const CUresult r = encode(map, type, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// Tensor map of the FP32 working copy (N x M, column-major, leading
+// dimension yf_ld(N)) with boxes of kTmaRows rows x `cols` columns;
+// out-of-range parts of a box read zeros: rows past N (the padding of the
+// leading dimension) too, never uninitialised memory.
+static cudaError_t encode_yf_map(CUtensorMap* map, float* Yf, int64_t N, int64_t M, int cols) {
+  return tensor_map_2d(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Yf, N, M, yf_ld(N) * (int64_t)sizeof(float), kTmaRows, cols,
+                       CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 cudaError_t launch_tsqr_mixed(const TsqrState& s, char* extra, const void* X, int64_t ldx, int xtype,
