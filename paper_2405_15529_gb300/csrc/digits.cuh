@@ -24,23 +24,39 @@ namespace pylom {
 constexpr int kStK = 16;                     // K elements per stage
 constexpr int kPlaneSbo = (kStK / 8) * 128;  // bytes between 8-row groups
 constexpr int kPlaneA = 128 * kStK * 2;      // 4 KB: 128 rows
-constexpr int kPlaneB = 64 * kStK * 2;       // 2 KB: 64 rows
 constexpr int kStagesPerSum = 8;             // stages accumulated before the sums are read: 128 elements of K
-constexpr int kSlots = 8;                    // accumulators (levels) of 64 columns in tensor memory
-
+constexpr int kSlots = 8;                    // accumulators (levels) in tensor memory
+// Two shapes of the kernels, by groups of eight warps in a block.
+//   G = 2: one block an SM, output tiles of 128 x 64.  An element of the left
+//          factor is cut for 64 columns; the groups fill alternate stages.
+//   G = 1: two blocks an SM, tiles of 128 x 32, half of the tensor memory each:
+//          while one block's warps read its accumulators or write its tile, the
+//          MMAs of the other run.
+// Long sums want the first (Gram matrix of 1,048,576 x 256: binary64 6.4 ms
+// against 8.9, binary32 3.1 against 4.0), short ones the second (131072 x 1056
+// in SPOD bins of 64 columns: Gram matrices 3.8 against 2.75 ms, modes 2.9
+// against 1.6).
+template <int G>
+struct Shape {
+  static constexpr int THREADS = 256 * G;     // 128 registers a thread: 64 hold the integer sums
+  static constexpr int BLOCKS = 3 - G;        // per SM
+  static constexpr int TILE = 32 * G;         // rows of the right factor, columns of an output tile
+  static constexpr int PLANEB = TILE * kStK * 2;
+  static constexpr int TMEM = kSlots * TILE;  // columns of tensor memory
+};
 constexpr int kRaw = 4;                      // stages of Y on their way in the Gram kernel
 template <typename TY> struct Dig;
 template <> struct Dig<double> {
   static constexpr int S = 8;          // digits
-  static constexpr int NST = 4;        // pipeline stages of a product
-  static constexpr int GST = 2;        // of the Gram kernel, beside kRaw stages of Y itself
+  template <int G> static constexpr int NST = 2;                  // pipeline stages
+  template <int G> static constexpr int AHEAD = G == 1 ? 2 : 3;   // slots of a thread's ring in a product
   static constexpr int HALVES = 2;     // level ranges of the Gram kernel: 0..7 and 8..14
   static constexpr int LBM = 7;        // lowest level of the modes kernel
 };
 template <> struct Dig<float> {
   static constexpr int S = 5;
-  static constexpr int NST = 6;
-  static constexpr int GST = 4;
+  template <int G> static constexpr int NST = G == 1 ? 3 : 4;
+  template <int G> static constexpr int AHEAD = 4;
   static constexpr int HALVES = 1;     // levels 1..8 (level 0 lies 2^-60 below the top one)
   static constexpr int LBM = 1;
 };
@@ -199,60 +215,113 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
 // One thread: all digit products of a stage with levels LB .. LB + 7 (s + t,
 // up to S - 1 each).  The right factor's planes follow one another with the
 // stride of their row groups, so planes t .. t + n - 1 are one operand of 64 n
-// rows, and their products with plane s go to the n accumulators of the levels
+// rows (of 32 n with G = 1), and their products with plane s go to the n accumulators of the levels
 // s + t .., which are neighbours too: one MMA of up to 256 columns.  (An MMA
 // reads its left factor from shared memory again: of 64 columns each, the 72
 // of a binary64 stage took 4500 clocks, eight warps issuing; the 28 wide ones
 // do 2300 clocks of multiplications.)  `first`: the stage starts new sums.
-// Descriptors advance 256 bytes per K = 16 step.
-template <int S, int LB>
+template <int S, int LB, int G>
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint64_t dA, uint64_t dB, bool first) {
-  static_assert(kPlaneB == 8 * kPlaneSbo, "planes of the right factor follow one another");
+  constexpr int T = Shape<G>::TILE, kPlaneB = Shape<G>::PLANEB;
+  static_assert(kPlaneB == T / 8 * kPlaneSbo && kStK == 16, "planes of the right factor follow one another; one K step");
 #pragma unroll
-  for (int ks = 0; ks < kStK / 16; ++ks) {
+  for (int i = 0; i < S; ++i) {
+    // the first products of a sum touch every level once, and overwrite it:
+    // plane 0 (LB = 0) or S - 1 alone, or (S = 5) planes 0 and 4 between them
+    const int s = S == 8 ? (LB == 0 ? i : S - 1 - i) : i == 0 ? 0 : i == 1 ? S - 1 : i - 1;
+    const int ta = LB > s ? LB - s : 0, tb = LB + 7 - s < S - 1 ? LB + 7 - s : S - 1;
 #pragma unroll
-    for (int i = 0; i < S; ++i) {
-      // the first products of a sum touch every level once, and overwrite it:
-      // plane 0 (LB = 0) or S - 1 alone, or (S = 5) planes 0 and 4 between them
-      const int s = S == 8 ? (LB == 0 ? i : S - 1 - i) : i == 0 ? 0 : i == 1 ? S - 1 : i - 1;
-      const int ta = LB > s ? LB - s : 0, tb = LB + 7 - s < S - 1 ? LB + 7 - s : S - 1;
-#pragma unroll
-      for (int t = ta; t <= tb;) {
-        const bool lone = S == 5 && i == 1 && t == 0;     // level 4 of plane 4: plane 0 has been there
-        const int n = lone ? 1 : tb - t + 1 < 4 ? tb - t + 1 : 4;
-        const bool fresh = ks == 0 && (i == 0 || (S == 5 && i == 1 && t > 0));
-        mma_f16(tmem + (s + t - LB) * 64, dA + (uint64_t)((s * kPlaneA + ks * 256) >> 4),
-                dB + (uint64_t)((t * kPlaneB + ks * 256) >> 4), idesc_f16(128, 64 * n), !(fresh && first));
-        t += n;
-      }
+    for (int t = ta; t <= tb;) {
+      const bool lone = S == 5 && i == 1 && t == 0;     // level 4 of plane 4: plane 0 has been there
+      const int n = lone ? 1 : tb - t + 1 < 8 / G ? tb - t + 1 : 8 / G;
+      const bool fresh = i == 0 || (S == 5 && i == 1 && t > 0);
+      mma_f16(tmem + (s + t - LB) * T, dA + (uint64_t)((s * kPlaneA) >> 4), dB + (uint64_t)((t * kPlaneB) >> 4),
+              idesc_f16(128, T * n), !(fresh && first));
+      t += n;
     }
   }
 }
 
-// 16 columns of one accumulator, no wait
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+// 8 columns of one accumulator, no wait
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
 }
 
 // Adds the eight accumulators (exact integers) of this thread's row and 16
-// columns into acc0 (levels 0..3 of the range) and acc1 (levels 4..7).
+// columns into acc0 (levels 0..3 of the range) and acc1 (levels 4..7).  The
+// next eight columns are on their way while eight are added; a value costs a
+// conversion and one 32 x 32 + 64-bit multiply-add (as shift and 64-bit
+// addition it was four operations of the half-rate integer pipe).
+template <int G>
 __device__ __forceinline__ void drain_slots(uint32_t taddr, int nslots, int64_t (&acc0)[16], int64_t (&acc1)[16]) {
+  uint32_t r[2][8];
+  tmem_ld8_nowait(taddr, r[0]);
 #pragma unroll
-  for (int sl = 0; sl < kSlots; ++sl) {
+  for (int q = 0; q < 2 * kSlots; ++q) {
+    const int sl = q >> 1, c0 = (q & 1) * 8;
     if (sl >= nslots) break;
-    uint32_t r[16];
-    tmem_ld16_nowait(taddr + sl * 64, r);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[q & 1][0]), "+r"(r[q & 1][1]), "+r"(r[q & 1][2]), "+r"(r[q & 1][3]), "+r"(r[q & 1][4]),
+                   "+r"(r[q & 1][5]), "+r"(r[q & 1][6]), "+r"(r[q & 1][7])
+                 :
+                 : "memory");
+    if (q + 1 < 2 * kSlots) tmem_ld8_nowait(taddr + ((q + 1) >> 1) * Shape<G>::TILE + ((q + 1) & 1) * 8, r[(q + 1) & 1]);
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int64_t p = (int64_t)__float2int_rn(__uint_as_float(r[c])) * (1 << (8 * (sl & 3)));
-      if (sl < 4) acc0[c] += p;
-      else acc1[c] += p;
+    for (int c = 0; c < 8; ++c) {
+      int64_t& a = sl < 4 ? acc0[c0 + c] : acc1[c0 + c];
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(__float2int_rn(__uint_as_float(r[q & 1][c]))), "r"(1 << (8 * (sl & 3))));
     }
   }
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// (acc1 2^32 + acc0) 2^pk, rounded to nearest, by integer operations: the
+// conversions of 64-bit integers are binary64 operations, of which this part
+// does two a clock.  (Bits below 2^-64 of the value are cut off.)
+struct Normal {
+  uint64_t m;      // leading bit at 63, or 0
+  int ex;          // |value| = m 2^ex
+  bool neg;
+};
+__device__ __forceinline__ Normal normalise(int64_t acc0, int64_t acc1, int pk) {
+  const int64_t hi = acc1 + (acc0 >> 32);
+  const uint32_t lo = (uint32_t)acc0;
+  Normal v;
+  v.neg = hi < 0;
+  const uint64_t h = v.neg ? ~(uint64_t)hi + (lo == 0) : (uint64_t)hi;
+  const uint32_t l = v.neg ? 0u - lo : lo;
+  // the upper 64 of the 96 bits, or all that there is
+  const uint64_t top = h ? h : (uint64_t)l;
+  const int n = __clzll((long long)top);
+  const uint64_t below = h ? (uint64_t)l << 32 : 0;
+  v.m = n ? (n < 64 ? (top << n) | (below >> (64 - n)) : 0) : top;
+  v.ex = pk - n + (h ? 32 : 0);
+  return v;
+}
+__device__ __forceinline__ double from_sums(int64_t acc0, int64_t acc1, int pk, double) {
+  const Normal v = normalise(acc0, acc1, pk);
+  if (v.m == 0) return 0.0;
+  const uint64_t r = (v.m >> 11) + ((v.m >> 10) & 1);        // 53 bits, or 2^53
+  const uint64_t sign = (uint64_t)v.neg << 63;
+  const int e = v.ex + 11 + 52 + 1023;
+  if (e >= 1 && e <= 2045) return __longlong_as_double((long long)(sign | (((uint64_t)(e - 1) << 52) + r)));
+  return scalbn(__longlong_as_double((long long)(sign | (((uint64_t)(1023 + 52 - 1) << 52) + r))), v.ex + 11);
+}
+__device__ __forceinline__ float from_sums(int64_t acc0, int64_t acc1, int pk, float) {
+  const Normal v = normalise(acc0, acc1, pk);
+  if (v.m == 0) return 0.f;
+  const uint32_t r = (uint32_t)(v.m >> 40) + ((uint32_t)(v.m >> 39) & 1u);
+  const uint32_t sign = (uint32_t)v.neg << 31;
+  const int e = v.ex + 40 + 23 + 127;
+  if (e >= 1 && e <= 253) return __uint_as_float(sign | (((uint32_t)(e - 1) << 23) + r));
+  return scalbnf(__uint_as_float(sign | (((uint32_t)(127 + 23 - 1) << 23) + r)), v.ex + 40);
+}
+
+template <int BYTES>
+__device__ __forceinline__ void async_copy(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" :: "r"(tc05::smem_u32(dst)), "l"(src), "n"(BYTES) : "memory");
 }
 
 // waits that first look once, without reading the clock
@@ -265,11 +334,9 @@ __device__ __forceinline__ bool mbar_wait_fast(uint64_t* mbar, uint32_t parity) 
 }
 
 // ---------------------------------------------------------------------------
-// the two pipelines (512 threads, one block per SM)
+// the two pipelines
 // ---------------------------------------------------------------------------
-constexpr int kDigThreads = 512;   // 128 registers a thread: 64 hold the integer sums
-
-template <int NST>
+template <int NST, int G>
 struct DigitBarriers {
   uint64_t full[NST], empty[NST], dfull, dempty, issued, fin;
   uint32_t tmem;
@@ -277,15 +344,15 @@ struct DigitBarriers {
   __device__ __forceinline__ void open(int extra) {
     if (threadIdx.x == 0) {
       for (int b = 0; b < NST; ++b) {
-        tc05::mbar_init(full + b, kDigThreads / 64 + extra);
+        tc05::mbar_init(full + b, 8 + extra);
         tc05::mbar_init(empty + b, 1);
       }
-      tc05::mbar_init(&dfull, 2);
+      tc05::mbar_init(&dfull, G);
       tc05::mbar_init(&issued, 1);
-      tc05::mbar_init(&dempty, kDigThreads / 32);
-      tc05::mbar_init(&fin, kDigThreads / 32);
+      tc05::mbar_init(&dempty, 8 * G);
+      tc05::mbar_init(&fin, 8 * G);
     }
-    if (threadIdx.x < 32) tc05::tmem_alloc(&tmem, 512);
+    if (threadIdx.x < 32) tc05::tmem_alloc(&tmem, Shape<G>::TMEM);
     tc05::fence_before();
     __syncthreads();
     tc05::fence_after();
@@ -297,7 +364,7 @@ struct DigitBarriers {
     if (!ok) raise_status(hdr, PYLOM_ERR_TIMEOUT);
     tc05::fence_before();
     __syncthreads();
-    if (threadIdx.x < 32) tc05::tmem_dealloc(tmem, 512);
+    if (threadIdx.x < 32) tc05::tmem_dealloc(tmem, Shape<G>::TMEM);
   }
 };
 
@@ -311,8 +378,9 @@ struct DigitBarriers {
 // stage.  At the end of a sum all sixteen warps read the accumulators; the
 // group that fills the next sum's first stage does so before it reads.
 //
-// A commit covers the MMAs of its own thread, so the last two stages of a sum
-// commit to `dfull` (two arrivals; a sum of one stage commits twice).
+// A commit covers the MMAs of its own thread, so with two groups the last two
+// stages of a sum commit to `dfull` (two arrivals; a sum of one stage commits
+// twice).
 //
 // Deadlock freedom: a group waits for (1) the MMAs of an earlier stage to be
 // issued or complete, (2) the reads of an earlier sum by the other group,
@@ -324,8 +392,8 @@ template <int NST>
 struct StageSlot {      // buffer and phase parity of a stage number
   int b;
   uint32_t par;
-  __device__ __forceinline__ void advance2() {
-    b += 2;
+  __device__ __forceinline__ void advance(int n) {
+    b += n;
     if (b >= NST) {
       b -= NST;
       par ^= 1u;
@@ -337,35 +405,37 @@ struct StageSlot {      // buffer and phase parity of a stage number
 // filled it.  `commits`: arrivals on dfull (1 for the last two stages of a
 // sum, 2 for the only one, else 0); ahead(): what can start once the stage is
 // filled.
-template <int NST, class Ahead, class Issue>
-__device__ __forceinline__ bool issue_turn(DigitBarriers<NST>& bar, const StageSlot<NST>& cur, int j, int sum, bool first,
+template <int NST, int G, class Ahead, class Issue>
+__device__ __forceinline__ bool issue_turn(DigitBarriers<NST, G>& bar, const StageSlot<NST>& cur, int j, int sum, bool first,
                                            int commits, uint32_t sa, Ahead ahead, Issue issue) {
   if ((threadIdx.x & 255) >= 32) return true;
   bool ok = true;
   if ((threadIdx.x & 31) == 0) {
     ok = mbar_wait_fast(bar.full + cur.b, cur.par);
     if (ok) ahead();
-    if (ok && j > 0) ok = mbar_wait_fast(&bar.issued, (uint32_t)((j - 1) & 1));
+    if (G > 1 && ok && j > 0) ok = mbar_wait_fast(&bar.issued, (uint32_t)((j - 1) & 1));
     if (ok && first && sum > 0) ok = mbar_wait_fast(&bar.dempty, (uint32_t)((sum - 1) & 1));
     if (ok) {
       tc05::fence_after();
       issue(bar.tmem, sa, first);
       tc05::commit(bar.empty + cur.b);
       for (int c = 0; c < commits; ++c) tc05::commit(&bar.dfull);
-      tc05::fence_before();
-      mbar_arrive(&bar.issued);
+      if (G > 1) {
+        tc05::fence_before();
+        mbar_arrive(&bar.issued);
+      }
     }
   }
   return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
 }
 
-template <int NST>
-__device__ __forceinline__ bool drain_turn(DigitBarriers<NST>& bar, int& drained, int nslots, int64_t (&acc0)[16],
+template <int NST, int G>
+__device__ __forceinline__ bool drain_turn(DigitBarriers<NST, G>& bar, int& drained, int nslots, int64_t (&acc0)[16],
                                            int64_t (&acc1)[16]) {
   const int warp = threadIdx.x >> 5;
   if (!__all_sync(0xffffffffu, mbar_wait_fast(&bar.dfull, (uint32_t)(drained & 1)))) return false;
   tc05::fence_after();
-  drain_slots(bar.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16, nslots, acc0, acc1);
+  drain_slots<G>(bar.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 16, nslots, acc0, acc1);
   tc05::fence_before();
   __syncwarp();
   if ((threadIdx.x & 31) == 0) mbar_arrive(&bar.dempty);
@@ -381,18 +451,18 @@ __device__ __forceinline__ bool drain_turn(DigitBarriers<NST>& bar, int& drained
 // memory, a turn ahead.  RAW > 0 (even): it reads a ring of RAW stages in
 // shared memory, which copy(j) (one thread, asynchronous) fills RAW stages
 // ahead; settle(j) waits for the copies up to stage j, after a timeout.
-template <int NST, int RAW, class Copy, class Settle, class Fetch, class Fill, class Issue, class Flush>
-__device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int stage_bytes, int nstage,
+template <int NST, int RAW, int G, class Copy, class Settle, class Fetch, class Fill, class Issue, class Flush>
+__device__ __forceinline__ void gram_pipeline(DigitBarriers<NST, G>& bar, unsigned char* gsm, int stage_bytes, int nstage,
                                               int nslots, WsHeader* hdr, Copy copy, Settle settle, Fetch fetch, Fill fill,
                                               Issue issue, Flush flush) {
-  const int lane = threadIdx.x & 31, group = threadIdx.x >> 8;
+  const int lane = threadIdx.x & 31, group = G == 1 ? 0 : threadIdx.x >> 8;
   bar.open(0);
   const uint32_t base = tc05::smem_u32(gsm);
   bool ok = true;
   int64_t acc0[16], acc1[16];
 #pragma unroll
   for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
-  int drained = 0, copied = group - 2;
+  int drained = 0, copied = group - G;
   auto ahead = [&](int j) {
     if (RAW > 0 && j < nstage) {
       copy(j);
@@ -400,10 +470,10 @@ __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned 
     }
   };
   if ((threadIdx.x & 255) == 0)
-    for (int j = group; j < RAW; j += 2) ahead(j);
+    for (int j = group; j < RAW; j += G) ahead(j);
   StageSlot<NST> cur{group, 0u};
   if (RAW == 0 && group < nstage) fetch(group);
-  for (int j = group; j < nstage; j += 2) {
+  for (int j = group; j < nstage; j += G) {
     const int sum = j / kStagesPerSum, js = j % kStagesPerSum;
     if (js != 0 && drained < sum) {
       ok = drain_turn(bar, drained, nslots, acc0, acc1);
@@ -421,17 +491,17 @@ __device__ __forceinline__ void gram_pipeline(DigitBarriers<NST>& bar, unsigned 
     tc05::fence_smem_async();
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.full + cur.b);
-    if (RAW == 0 && j + 2 < nstage) fetch(j + 2);
+    if (RAW == 0 && j + G < nstage) fetch(j + G);
     if (js == 0 && drained < sum) {
       ok = drain_turn(bar, drained, nslots, acc0, acc1);
       if (!ok) break;
     }
     // (64-bit sums of at most 2^20 rows)
-    if (drained > 0 && (drained & 8191) == 0 && js < 2) flush(acc0, acc1);
-    ok = issue_turn(bar, cur, j, sum, js == 0, js >= kStagesPerSum - 2, base + cur.b * stage_bytes,
+    if (drained > 0 && (drained & 8191) == 0 && js < G) flush(acc0, acc1);
+    ok = issue_turn(bar, cur, j, sum, js == 0, js >= kStagesPerSum - G, base + cur.b * stage_bytes,
                     [&] { ahead(j + RAW); }, issue);
     if (!ok) break;
-    cur.advance2();
+    cur.advance(G);
   }
   while (ok && drained * kStagesPerSum < nstage) ok = drain_turn(bar, drained, nslots, acc0, acc1);
   if (ok) flush(acc0, acc1);
@@ -446,17 +516,20 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
-// Products of `mine` output tiles of 128 rows x 64 columns, K = `stages`
-// stages of kStK elements each, as one sequence of stages: fetch(tile, js)
-// loads the left factor a turn ahead, fill(tile, js, stage) writes its digits, the right factor's planes come by
+// Products of `mine` output tiles of 128 rows x 32 G columns, K = `stages`
+// stages of kStK elements each, as one sequence of stages: load(tile, js,
+// slot) starts copies of this thread's part of the left factor into its slot
+// of a ring of AHEAD (cp.async: the latency of memory spans several stages, and
+// a thread that reads what it copied itself needs no barrier), fill(tile, js,
+// slot, stage) writes its digits, the right factor's planes come by
 // a bulk copy from bsrc(tile, js), store(tile, acc0, acc1) writes this
 // thread's row and 16 columns.  `tile` counts 0 .. mine - 1.  LB: lowest
 // level that is kept.
-template <int S, int NST, int LB, class Fetch, class Fill, class Src, class Store>
-__device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsigned char* gsm, int mine, int stages,
-                                                 WsHeader* hdr, Fetch fetch, Fill fill, Src bsrc, Store store) {
-  constexpr int kStage = S * (kPlaneA + kPlaneB);
-  const int tid = threadIdx.x, lane = tid & 31, group = tid >> 8;
+template <int S, int NST, int LB, int AHEAD, int G, class Load, class Fill, class Src, class Store>
+__device__ __forceinline__ void product_pipeline(DigitBarriers<NST, G>& bar, unsigned char* gsm, int mine, int stages,
+                                                 WsHeader* hdr, Load load, Fill fill, Src bsrc, Store store) {
+  constexpr int kPlaneB = Shape<G>::PLANEB, kStage = S * (kPlaneA + kPlaneB);
+  const int tid = threadIdx.x, lane = tid & 31, group = G == 1 ? 0 : tid >> 8;
   bar.open(1);
   const uint32_t base = tc05::smem_u32(gsm);
   const int sums = (stages + kStagesPerSum - 1) / kStagesPerSum;
@@ -465,35 +538,57 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
 #pragma unroll
   for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
   int drained = 0, dr_tile = 0, dr_sum = 0;
+  // reads the sums before `upto`; the tile that the last of them completes is
+  // written out by write_tile once the next MMAs are on their way
+  bool whole = false;
+  auto write_tile = [&] {
+    if (!whole) return;
+    store(dr_tile, acc0, acc1);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
+    ++dr_tile;
+    whole = false;
+  };
   auto read_upto = [&](int upto) {
     while (ok && drained < upto) {
+      write_tile();
       ok = drain_turn(bar, drained, kSlots, acc0, acc1);
-      if (!ok) return;
-      if (++dr_sum == sums) {
-        store(dr_tile, acc0, acc1);
-#pragma unroll
-        for (int c = 0; c < 16; ++c) acc0[c] = acc1[c] = 0;
+      if (ok && ++dr_sum == sums) {
+        whole = true;
         dr_sum = 0;
-        ++dr_tile;
       }
     }
   };
   auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
-    issue_stage<S, LB>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo), first);
+    issue_stage<S, LB, G>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo), first);
   };
   StageSlot<NST> cur{group, 0u};
   int tile = 0, js = group, j = group;
-  while (js >= stages) {
-    js -= stages;
-    ++tile;
-  }
-  if (tile < mine) fetch(tile, js);
-  for (; tile < mine; j += 2) {
-    int ntile = tile, njs = js + 2;      // this group's next stage
-    while (njs >= stages) {
-      njs -= stages;
-      ++ntile;
+  auto next = [&](int& t, int& q) {       // wraps the stage number
+    if (G == 1) {
+      if (q == stages) {
+        q = 0;
+        ++t;
+      }
+      return;
     }
+    while (q >= stages) {
+      q -= stages;
+      ++t;
+    }
+  };
+  next(tile, js);
+  int ltile = tile, ljs = js, slot = 0;
+  auto start = [&](int at) {
+    if (ltile < mine) load(ltile, ljs, at);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    ljs += G;
+    next(ltile, ljs);
+  };
+#pragma unroll
+  for (int q = 0; q < AHEAD - 1; ++q) start(q);
+  for (; tile < mine; j += G) {
+    asm volatile("cp.async.wait_group %0;" :: "n"(AHEAD - 2) : "memory");
     const int sum = tile * sums + js / kStagesPerSum;
     const bool first = js % kStagesPerSum == 0;
     if (!first) read_upto(sum);
@@ -504,23 +599,27 @@ __device__ __forceinline__ void product_pipeline(DigitBarriers<NST>& bar, unsign
       tc05::mbar_arrive_expect_tx(bar.full + cur.b, S * kPlaneB);
       bulk_load(st + S * kPlaneA, bsrc(tile, js), S * kPlaneB, bar.full + cur.b);
     }
-    fill(tile, js, st);
+    fill(tile, js, slot, st);
     tc05::fence_smem_async();
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.full + cur.b);
-    if (ntile < mine) fetch(ntile, njs);
+    start(slot == 0 ? AHEAD - 1 : slot - 1);
+    slot = slot == AHEAD - 1 ? 0 : slot + 1;
     if (first) read_upto(sum);
     if (!ok) break;
     // stages of this sum from this one on
     const int in_sum = js % kStagesPerSum, rest = stages - js, left = rest < kStagesPerSum - in_sum ? rest : kStagesPerSum - in_sum;
-    ok = issue_turn(bar, cur, j, sum, first, left > 2 ? 0 : left == 1 && first ? 2 : 1, base + cur.b * kStage, [] {},
-                    issue);
+    const int commits = left > G ? 0 : G == 2 && left == 1 && first ? 2 : 1;
+    ok = issue_turn(bar, cur, j, sum, first, commits, base + cur.b * kStage, [] {}, issue);
     if (!ok) break;
-    js = njs;
-    tile = ntile;
-    cur.advance2();
+    write_tile();
+    js += G;
+    next(tile, js);
+    cur.advance(G);
   }
   read_upto(mine * sums);
+  if (ok) write_tile();
+  asm volatile("cp.async.wait_all;" ::: "memory");
   // bulk copies of stages that were never consumed (after a timeout) land
   // before the block ends
   if (!ok && tid == 0)

@@ -13,9 +13,10 @@
 // does at 1/60 of its binary32 rate.
 //
 // Measured (4,194,304 x 256, binary64): Householder leaves + tree 554 + 13
-// ms; here Y 8.2, Gram matrix 40, Cholesky factor 1.3 ms.  1,048,576 x 128
-// leaves + tree 39 + 3.8 ms.  Binary32 leaves (mixed, 4,194,304 x 256) 57.7 +
-// 8.8 ms; here 6.4, 16.7 and 1.3 ms.
+// ms; here Y 8.6, cutting it 2.4, Gram matrix 25.8, Cholesky factor 0.74 ms.
+// 1,048,576 x 128: leaves + tree 39 + 3.8 ms; here 1.4, 0.3, 2.1 and 0.35.
+// Binary32 (mixed, 4,194,304 x 256): leaves + tree 57.7 + 8.8 ms; here 3.4,
+// 12.5 and 0.71 ms.
 #include <atomic>
 
 #include "digits.cuh"
@@ -167,14 +168,20 @@ __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(
 // ---------------------------------------------------------------------------
 // A unit is an output tile of 128 x 64 columns of Y on or above the
 // diagonal, a range of digit levels (two for binary64: eight accumulators of
-// 64 columns fill the tensor memory) and a range of rows.  16 warps cut rows
-// of Y into digit planes in shared memory (a thread takes 8 rows of one
-// column: 64 contiguous bytes in, one conflict-free 16-byte store per digit
-// out) and one thread issues a stage's MMAs once all warps have written it;
-// every 128 rows the accumulators are added to 64-bit integers in registers
-// (after the next stages have been filled, so the warps work while the last
-// MMAs of the sum run), and at the end those go to the global sums by
-// integer atomics, so the result does not depend on the order.
+// 64 columns fill the tensor memory) and a range of rows.  TMA boxes of 16 rows
+// x 128 (64) columns bring Y into a ring in shared memory, swizzled so that
+// neighbouring columns lie in different banks; 16 warps in two groups cut
+// them into digit planes (a thread takes 8 rows of one column: one
+// conflict-free 16-byte store per digit out); one thread a group issues a
+// stage's MMAs; every 128 rows the accumulators are added to 64-bit integers
+// in registers, and at the end those go to the global sums by integer
+// atomics, so the result does not depend on the order.
+//
+// Bound by the tensor pipe (1540 clocks a stage of 16 rows, 12300 a sum of 128)
+// and the reads of the accumulators between sums, which the MMAs wait for
+// (about 6000).  1,048,576 x 256: binary64 9.5 ms with Y loaded by the warps
+// themselves (the latency of their loads was the bound), 6.4 here; binary32
+// 3.45 and 3.1.
 
 struct GramArgs {
   int64_t ldy, N, M;      // ldy: rows that exist (N rounded up to 8)
@@ -235,12 +242,13 @@ cudaError_t launch_unpack(const GramState& g, double* Y, const unsigned* redo, c
 }
 
 template <typename TY>
-__global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(const __grid_constant__ GramArgs a) {
-  constexpr int S = Dig<TY>::S, NST = Dig<TY>::GST, kStage = S * (kPlaneA + kPlaneB);
+__global__ void __launch_bounds__(Shape<2>::THREADS, 1) gram_kernel(const __grid_constant__ GramArgs a) {
+  constexpr int S = Dig<TY>::S, NST = Dig<TY>::template NST<2>, kPlaneB = Shape<2>::PLANEB;
+  constexpr int kStage = S * (kPlaneA + kPlaneB);
   constexpr int kPitch = kStK * (int)sizeof(TY), kRawA = 128 * kPitch, kRawStage = kRawA + 64 * kPitch;
   typedef typename Cell<TY>::type C;
   extern __shared__ __align__(1024) unsigned char gsm[];
-  __shared__ __align__(8) DigitBarriers<NST> bar;
+  __shared__ __align__(8) DigitBarriers<NST, 2> bar;
   __shared__ __align__(8) uint64_t raw_full[kRaw];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int item = blockIdx.x % a.items, split = blockIdx.x / a.items;
@@ -262,9 +270,9 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(const __grid_const
   const int64_t nB = a.Z ? a.NZ : a.M;
   const int64_t nsum = (a.N + 127) / 128;
   const int64_t q0 = nsum * split / a.splits, q1 = nsum * (split + 1) / a.splits;
-  // a thread of a stage's group: 8 rows of one of A's columns, and threads
-  // 128.. 8 rows of one of B's
-  const int th = tid & 255, ca = th & 127, kg = th >> 7, cb = th & 63, kb = (th >> 6) & 1;
+  // a thread of a stage's group: 8 rows of one of A's columns, and four of the
+  // eight warps, in turn, 8 rows of one of B's
+  const int th = tid & 255, ca = th & 127, kg = th >> 7, cb = th & 63, kb = (th >> 6) & 1, quad = th >> 7;
   const int64_t colA = (int64_t)I * 128 + ca, colB = (int64_t)J * 64 + cb;
   const int EA = colA < a.M ? a.colE[colA] : 128;
   const int EB = (!diag && colB < nB) ? (a.Z ? a.zE : a.colE)[colB] : 128;
@@ -298,11 +306,13 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(const __grid_const
     }
   };
   __align__(16) C yA[8], yB[8];
+  bool withB = false;
   auto fetch = [&](int j) {
     if (!__all_sync(0xffffffffu, mbar_wait_fast(raw_full + j % kRaw, (uint32_t)((j / kRaw) & 1)))) return false;
     const unsigned char* r = raw + (j % kRaw) * kRawStage;
     read8(r, ca, kg, j < jA, yA);
-    if (!diag && th >= 128) read8(r + kRawA, cb, kb, j < jB, yB);
+    withB = !diag && ((j >> 1) & 1) == quad;
+    if (withB) read8(r + kRawA, cb, kb, j < jB, yB);
     return true;
   };
   const int oa = (ca >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
@@ -311,13 +321,13 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(const __grid_const
   const bool both = diag && (ca >> 6) == (J & 1);
   auto fill = [&](unsigned char* st) {
     put_digits(yA, EA, st + oa, kPlaneA, both ? st + ob : nullptr, kPlaneB);
-    if (!diag && th >= 128)
+    if (withB)
       put_digits(yB, EB, st + S * kPlaneA + (cb >> 3) * kPlaneSbo + (cb & 7) * 16 + kb * 128, kPlaneB, nullptr, 0);
   };
   auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
     const uint64_t dA = tc05::desc(sa, 128, kPlaneSbo), dB = tc05::desc(sa + S * kPlaneA, 128, kPlaneSbo);
-    if (half == 0) issue_stage<S, gram_base<TY>(0)>(tmem, dA, dB, first);
-    else issue_stage<S, gram_base<TY>(Dig<TY>::HALVES - 1)>(tmem, dA, dB, first);
+    if (half == 0) issue_stage<S, gram_base<TY>(0), 2>(tmem, dA, dB, first);
+    else issue_stage<S, gram_base<TY>(Dig<TY>::HALVES - 1), 2>(tmem, dA, dB, first);
   };
   auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
     const int64_t gi = (int64_t)I * 128 + (warp & 3) * 32 + lane;
@@ -331,7 +341,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) gram_kernel(const __grid_const
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<NST, kRaw>(bar, gsm, kStage, (int)(q1 - q0) * kStagesPerSum, (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr,
+  gram_pipeline<NST, kRaw, 2>(bar, gsm, kStage, (int)(q1 - q0) * kStagesPerSum, (sizeof(TY) == 8 && half == 1) ? 7 : 8, a.hdr,
                            copy, settle, fetch, fill, issue, flush);
 }
 
@@ -567,7 +577,7 @@ void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax) {
   g.Ll = (double*)p;         p += align256(sizeof(double) * (size_t)M * M);
   g.Th = (double*)p;         p += align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M);
   g.Tl = (double*)p;         p += align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M);
-  g.Cd = (unsigned char*)p;  p += align256((size_t)kt * js * 8 * kPlaneB);
+  g.Cd = (unsigned char*)p;  p += align256((size_t)kt * js * 8 * Shape<2>::PLANEB);
   g.Ce = (int*)p;
 }
 
@@ -609,7 +619,7 @@ template <typename TY>
 static cudaError_t gram_launch(const GramState& g, int sms, const void* Z, int64_t ldz, int64_t NZ, const int* zE,
                                long long* G, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
   constexpr int S = Dig<TY>::S;
-  constexpr size_t smem = (size_t)Dig<TY>::GST * S * (kPlaneA + kPlaneB) + (size_t)kRaw * 192 * kStK * sizeof(TY);
+  constexpr size_t smem = (size_t)Dig<TY>::template NST<2> * S * (kPlaneA + Shape<2>::PLANEB) + (size_t)kRaw * 192 * kStK * sizeof(TY);
   cudaError_t e = ensure_dyn_smem((const void*)gram_kernel<TY>, smem);
   if (e != cudaSuccess) return e;
   const int nJ = (int)(((Z ? NZ : g.M) + 63) / 64), nI = (int)((g.M + 127) / 128);
@@ -640,7 +650,7 @@ static cudaError_t gram_launch(const GramState& g, int sms, const void* Z, int64
     if (e == cudaSuccess)
       e = tensor_map_2d(&a.mapB, type, (TY*)(Z ? Z : g.Y) + r, a.ldy, Z ? NZ : g.M, ldb * (int64_t)sizeof(TY), kStK, 64, swz);
     if (e != cudaSuccess) return e;
-    gram_kernel<TY><<<(unsigned)(a.items * a.splits), kDigThreads, smem, st>>>(a);
+    gram_kernel<TY><<<(unsigned)(a.items * a.splits), Shape<2>::THREADS, smem, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -5,15 +5,18 @@
 // multiplied without rounding on the tcgen05 tensor cores; digit products
 // below the level of a binary64 (binary32) rounding of the sum are left out.
 // Measured (4,194,304 x 256, r = 43): top-down pass + reflectors 7.3 + 209 ms
-// in binary64, 5.2 + 16.7 ms mixed; here 8.4 and 7.5 ms.
+// in binary64, 5.2 + 16.7 ms mixed; here 7.6 and 6.2 ms.
 //
-// A block takes tiles of 128 rows x 64 columns of U.  16 warps cut 32
-// columns of the tile's rows of Y into digit planes per stage (a thread
-// takes 8 columns of one row: coalesced loads, one conflict-free 16-byte
-// store per digit), a bulk copy brings the stage's planes of C, which a
-// small kernel has laid out in shared-memory order, and one thread issues
-// the MMAs; every 128 columns of Y the accumulators go to 64-bit integers in
-// registers, and at the tile's end those become U.
+// A block takes tiles of 128 rows x 64 (32) columns of U (digits.cuh: two
+// shapes).  The warps cut 16 columns of the tile's rows of Y into digit planes
+// per stage (a thread takes 8 columns of one row: coalesced copies into its own
+// ring in shared memory, one conflict-free 16-byte store per digit), a bulk
+// copy brings the stage's planes of C, which a small kernel has laid out in
+// shared-memory order, and one thread issues the MMAs; every 128 columns of Y
+// the accumulators go to 64-bit integers in registers, and at the tile's end
+// those become U, after the next tile's first MMAs have been issued.  The sums
+// are made binary64 (binary32) by integer operations: 262,144 x 100 mixed 287
+// us with binary64 ones, 234 with both changes.
 #include "digits.cuh"
 #include "gram.h"
 
@@ -26,13 +29,13 @@ __host__ __device__ __forceinline__ int product_stages(int64_t n) { return (int)
 // Digit planes of the coefficients times their rows' scales 2^(E - bias),
 // one block per column; planes of column tile kt and stage js at
 // ((kt * stages + js) * S) kPlaneB bytes.
-template <typename TY>
+template <typename TY, int G>
 __global__ void __launch_bounds__(128) coef_digits_kernel(ProductArgs p) {
-  constexpr int SD = Dig<TY>::S;
+  constexpr int SD = Dig<TY>::S, T = Shape<G>::TILE, kPlaneB = Shape<G>::PLANEB;
   __shared__ int s_e;
   if (p.unless && *p.unless) return;
   const int64_t k = blockIdx.x, r = product_cols(p);
-  if (k >= (r + 63) / 64 * 64) return;
+  if (k >= (r + T - 1) / T * T) return;
   const int s1 = product_stages(p.M), stages = s1 + product_stages(p.NZ);
   if (threadIdx.x == 0) s_e = kMinField64;
   __syncthreads();
@@ -65,51 +68,60 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(ProductArgs p) {
       if (SD == 5) v = (v + (1ll << 23)) >> 24;
       w[i] = bias_digits(v);
     }
-    unsigned char* dst = p.Cd + (((k / 64) * stages + j0 / kStK) * SD) * (int64_t)kPlaneB + ((k & 63) >> 3) * kPlaneSbo +
+    unsigned char* dst = p.Cd + (((k / T) * stages + j0 / kStK) * SD) * (int64_t)kPlaneB + ((k % T) >> 3) * kPlaneSbo +
                          ((j0 % kStK) >> 3) * 128 + (k & 7) * 16;
     store_digits<SD>(w, dst, kPlaneB);
   }
 }
 
-template <typename TY>
-__global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArgs p, const double* S0, const double* w,
+template <typename TY, int G>
+__global__ void __launch_bounds__(Shape<G>::THREADS, Shape<G>::BLOCKS) modes_direct_kernel(ProductArgs p, const double* S0, const double* w,
                                                                      int physical, TY* U, int64_t ldu,
                                                                      int64_t* r_out, WsHeader* hdr) {
-  constexpr int S = Dig<TY>::S, NST = Dig<TY>::NST, LB = Dig<TY>::LBM;
+  constexpr int S = Dig<TY>::S, NST = Dig<TY>::template NST<G>, LB = Dig<TY>::LBM, AHEAD = Dig<TY>::template AHEAD<G>;
+  constexpr int T = Shape<G>::TILE, kPlaneB = Shape<G>::PLANEB;
   typedef typename Cell<TY>::type Cl;
   extern __shared__ __align__(1024) unsigned char gsm[];
-  __shared__ __align__(8) DigitBarriers<NST> bar;
+  __shared__ __align__(8) DigitBarriers<NST, G> bar;
   if (p.unless && *p.unless) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t N = p.N, r = product_cols(p);
   // a zero matrix keeps all modes (there is no energy to share): unit vectors
   const bool zero = S0 && S0[0] == 0.0;
   if (blockIdx.x == 0 && tid == 0 && r_out) *r_out = r;
-  const int64_t ktiles = (r + 63) / 64, tiles = (N + 127) / 128 * ktiles;
+  const int64_t ktiles = (r + T - 1) / T, tiles = (N + 127) / 128 * ktiles;
   const int s1 = product_stages(p.M), stages = s1 + product_stages(p.NZ);
   const uint32_t kt32 = (uint32_t)ktiles;
   const int rl = tid & 127, kh = (tid >> 7) & 1; // row of the tile, half of the stage's columns
   const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
   const int mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
-  Cl y[8];
-  auto fetch = [&](int t, int js) {
+  // element i of this thread in slot q of its ring: ring[(q 8 + i) 256]
+  Cl* ring = (Cl*)(gsm + NST * S * (kPlaneA + kPlaneB)) + (tid >> 8) * (AHEAD * 8 * 256) + (tid & 255);
+  auto load = [&](int t, int js, int q) {
     const uint32_t tile = blockIdx.x + t * gridDim.x;
     const int64_t row = (int64_t)(tile / kt32) * 128 + rl;
-    const bool rin = row < N, second = js >= s1;
+    const bool second = js >= s1;
     const int64_t ld = second ? p.ldz : p.ldy;
     const int c0 = (second ? js - s1 : js) * kStK + kh * 8, m32 = (int)(second ? p.NZ : p.M);
-    const Cl* q = (const Cl*)(second ? p.Z : p.Y) + row + c0 * ld;
+    const Cl* src = (const Cl*)(second ? p.Z : p.Y) + row + c0 * ld;
+    if (row < N) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = (c0 + i < m32 && rin) ? __ldg(q + i * ld) : zero_cell<Cl>();
+      for (int i = 0; i < 8; ++i)
+        if (c0 + i < m32) async_copy<(int)sizeof(Cl)>(ring + (q * 8 + i) * 256, src + i * ld);
+    }
   };
-  auto fill = [&](int, int js, unsigned char* st) {
+  auto fill = [&](int t, int js, int q, unsigned char* st) {
+    const uint32_t tile = blockIdx.x + t * gridDim.x;
+    const bool rin = (int64_t)(tile / kt32) * 128 + rl < N, second = js >= s1;
+    const int* ex = second ? p.zE : p.colE;
+    const int c0 = (second ? js - s1 : js) * kStK + kh * 8, m32 = (int)(second ? p.NZ : p.M);
+    Cl y[8];
     int E[8];
-    if (S == 5) {       // (words carry their scale)
-      const bool second = js >= s1;
-      const int* ex = second ? p.zE : p.colE;
-      const int c0 = (second ? js - s1 : js) * kStK + kh * 8, m32 = (int)(second ? p.NZ : p.M);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) E[i] = c0 + i < m32 ? __ldg(ex + c0 + i) : 128;
+    for (int i = 0; i < 8; ++i) {
+      const bool in = c0 + i < m32;
+      y[i] = in && rin ? ring[(q * 8 + i) * 256] : zero_cell<Cl>();
+      E[i] = (S == 5 && in) ? __ldg(ex + c0 + i) : 128;     // (words carry their scale)
     }
     put_digits(y, E, st + offA + kh * 128, kPlaneA);
   };
@@ -121,23 +133,24 @@ __global__ void __launch_bounds__(kDigThreads, 1) modes_direct_kernel(ProductArg
     // the tile's rows of U: lanes hold consecutive rows
     const uint32_t tile = blockIdx.x + t * gridDim.x;
     const int64_t row = (int64_t)(tile / kt32) * 128 + (warp & 3) * 32 + lane;
-    const int k0 = (int)(tile % kt32) * 64 + (warp >> 2) * 16;
+    const int k0 = (int)(tile % kt32) * T + (warp >> 2) * 16;
     const double iw = (physical && w && row < N) ? 1.0 / sqrt(w[row]) : 1.0;
+    if (k0 >= r) return;
+    const int ce = lane < 16 && k0 + lane < r ? __ldg(p.Ce + k0 + lane) : 0;
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
       const int k = k0 + c;
-      if (k >= r) break;     // uniform over the warp
-      if (row < N) {
-        const int pk = 8 * LB + __ldg(p.Ce + k) - fix_bias<double>() + (S == 5 ? 24 : 0);
-        double v = __fma_rn((double)acc1[c], 4294967296.0, (double)acc0[c]);
-        v = (pk > -900 && pk < 900) ? v * __hiloint2double((pk + 1023) << 20, 0) : scalbn(v, pk);
-        if (zero) v = row == k ? 1.0 : 0.0;
-        if (physical && w) v *= iw;
-        U[row + k * ldu] = (TY)v;
+      const int pk = 8 * LB + __shfl_sync(0xffffffffu, ce, c) - fix_bias<double>() + (S == 5 ? 24 : 0);
+      if (k < r && row < N) {
+        TY v;
+        if (zero) v = (TY)(row == k ? iw : 0.0);
+        else if (physical && w) v = (TY)(from_sums(acc0[c], acc1[c], pk, 0.0) * iw);
+        else v = from_sums(acc0[c], acc1[c], pk, (TY)0);
+        U[row + k * ldu] = v;
       }
     }
   };
-  product_pipeline<S, NST, LB>(bar, gsm, mine, stages, hdr, fetch, fill, bsrc, store);
+  product_pipeline<S, NST, LB, AHEAD, G>(bar, gsm, mine, stages, hdr, load, fill, bsrc, store);
 }
 
 // Smallest kept value, relative to the largest, for which Y V_r S_r^-1 is
@@ -172,28 +185,40 @@ cudaError_t launch_sign_ur(const TsqrState& ts, double* UR, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <typename TY>
-static cudaError_t run(const ProductArgs& p, const double* S0, const double* w, int physical, void* U, int64_t ldu,
-                       int64_t* r_out, WsHeader* hdr, cudaStream_t st, cudaEvent_t mid) {
-  constexpr size_t smem = (size_t)Dig<TY>::NST * Dig<TY>::S * (kPlaneA + kPlaneB);
+template <typename TY, int G>
+static cudaError_t run_shape(const ProductArgs& p, const double* S0, const double* w, int physical, void* U, int64_t ldu,
+                             int64_t* r_out, WsHeader* hdr, cudaStream_t st, cudaEvent_t mid) {
+  constexpr int T = Shape<G>::TILE, threads = Shape<G>::THREADS;
+  constexpr size_t smem = (size_t)Dig<TY>::template NST<G> * Dig<TY>::S * (kPlaneA + Shape<G>::PLANEB) +
+                          (size_t)Dig<TY>::template AHEAD<G> * 8 * threads * sizeof(TY);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = ensure_dyn_smem((const void*)modes_direct_kernel<TY>, smem)) != cudaSuccess) return e;
-  const int64_t kt = (p.cols_max + 63) / 64;
-  coef_digits_kernel<TY><<<(unsigned)(kt * 64), 128, 0, st>>>(p);
+  if ((e = ensure_dyn_smem((const void*)modes_direct_kernel<TY, G>, smem)) != cudaSuccess) return e;
+  const int64_t kt = (p.cols_max + T - 1) / T;
+  coef_digits_kernel<TY, G><<<(unsigned)(kt * T), 128, 0, st>>>(p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
   int64_t grid = (p.N + 127) / 128 * kt;
-  if (grid > sms) grid = sms;
-  modes_direct_kernel<TY><<<(unsigned)grid, kDigThreads, smem, st>>>(p, S0, w, physical, (TY*)U, ldu, r_out, hdr);
+  if (grid > Shape<G>::BLOCKS * sms) grid = Shape<G>::BLOCKS * sms;
+  modes_direct_kernel<TY, G><<<(unsigned)grid, threads, smem, st>>>(p, S0, w, physical, (TY*)U, ldu, r_out, hdr);
   return cudaGetLastError();
 }
 
+// Short sums (up to 64 columns of Y) in two blocks an SM: 65,537 x 63, r = 42
+// 40 us against 70; 262,144 x 100 mixed 336 against 234, 1,048,576 x 128
+// 1360 against 1040.
+template <typename TY>
+static cudaError_t run(const ProductArgs& p, const double* S0, const double* w, int physical, void* U, int64_t ldu,
+                       int64_t* r_out, WsHeader* hdr, cudaStream_t st, cudaEvent_t mid) {
+  return p.M + p.NZ <= 64 ? run_shape<TY, 1>(p, S0, w, physical, U, ldu, r_out, hdr, st, mid)
+                          : run_shape<TY, 2>(p, S0, w, physical, U, ldu, r_out, hdr, st, mid);
+}
+
 size_t product_planes_bytes(int64_t M, int64_t NZ, int64_t cols) {
-  const int64_t kt = (cols + 63) / 64;
-  return align256((size_t)kt * (product_stages(M) + product_stages(NZ)) * 8 * kPlaneB) +
+  const int64_t kt = (cols + 63) / 64;       // (64 columns hold two tiles of the narrower shape)
+  return align256((size_t)kt * (product_stages(M) + product_stages(NZ)) * 8 * Shape<2>::PLANEB) +
          align256(sizeof(int) * (size_t)kt * 64);
 }
 

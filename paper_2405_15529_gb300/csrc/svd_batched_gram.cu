@@ -33,7 +33,9 @@ namespace pylom {
 namespace {
 
 constexpr int kSB = Dig<float>::S;                 // 5 digits
-constexpr int kNstB = Dig<float>::NST;
+constexpr int kG = 1;                              // two blocks an SM: the sums of a bin are short
+constexpr int kTile = Shape<kG>::TILE, kPlaneB = Shape<kG>::PLANEB, kThreads = Shape<kG>::THREADS;
+constexpr int kNstB = Dig<float>::NST<kG>, kAhead = Dig<float>::AHEAD<kG>;
 constexpr int kStageB = kSB * (kPlaneA + kPlaneB);
 constexpr double kKeptLevel = 1e-4;
 constexpr double kOpenCos = 1e-6;                  // kept columns: largest cosine before the last step
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(256) bg_prologue_kernel(BG a) {
 // Unit modes: the 128 rows of the left factor are columns 0..127 (kPlain),
 // columns 0..63 and the same turned by 90 degrees (kPacked: Re and Im in one
 // pass, for the first 64 columns), or columns 0..127 turned (kTurned).  The
-// right factor is the column block J of 64.
+// right factor is the column block J of 32.
 enum { kPlain = 0, kPacked = 1, kTurned = 2 };
 
 // rows row..row+7 of a column (turned: (-im, re) pairs)
@@ -197,41 +199,43 @@ __device__ __forceinline__ void fetch_rows8(const GramBin& b, int64_t row, int c
   }
 }
 
-__global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
+__global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_gram_kernel(BG a) {
   extern __shared__ __align__(1024) unsigned char gsm[];
-  __shared__ __align__(8) DigitBarriers<kNstB> bar;
+  __shared__ __align__(8) DigitBarriers<kNstB, kG> bar;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const GramUnit u = a.units[blockIdx.x];
   const GramBin b = a.bins[u.bin];
   const int mode = u.mode, J = u.J;
-  // a thread of a stage's group: 8 rows of one left column, and threads 128..
-  // 8 rows of one right column
-  const int t = threadIdx.x & 255, ca = t & 127, kg = t >> 7, cb = t & 63, kb = (t >> 6) & 1;
+  // a thread: 8 rows of one left column, and in two of the eight warps, in turn
+  // from stage to stage, 8 rows of one right column
+  const int t = threadIdx.x, ca = t & 127, kg = t >> 7, cb = lane;
   const bool turned = mode == kTurned || (mode == kPacked && ca >= 64);
   // real items have nothing to turn: their second half is empty
   const int colA = (mode == kPacked && ca >= 64 && !b.cplx) ? 128 : mode == kPacked ? (ca & 63) : ca;
   const int EA = colA < b.Nb ? a.ints[b.colE + colA] : 128;
   const bool sepB = mode == kTurned;             // else the right factor's columns are among the left's
-  const int colB = J * 64 + cb;
+  const int colB = J * kTile + cb;
   const int EB = (sepB && colB < b.Nb) ? a.ints[b.colE + colB] : 128;
   float yA[8], yB[8];
+  int turn = 7;
   auto fetch = [&](int j) {
     const int64_t row = (u.q0 * kStagesPerSum + j) * kStK;
     fetch_rows8(b, row + kg * 8, colA, turned, yA);
-    if (sepB && t >= 128) fetch_rows8(b, row + kb * 8, colB, false, yB);
+    turn = (warp + 2 * j) & 7;
+    if (sepB && turn < 2) fetch_rows8(b, row + turn * 8, colB, false, yB);
     return true;
   };
   const int oa = (ca >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
   // the left factor's columns that are the right one's too
-  const int ob = kSB * kPlaneA + ((ca & 63) >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
-  const bool both = !sepB && (ca >> 6) == J;
+  const int ob = kSB * kPlaneA + ((ca & 31) >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
+  const bool both = !sepB && (ca >> 5) == J;
   auto fill = [&](unsigned char* st) {
     put_digits(yA, EA, st + oa, kPlaneA, both ? st + ob : nullptr, kPlaneB);
-    if (sepB && t >= 128)
-      put_digits(yB, EB, st + kSB * kPlaneA + (cb >> 3) * kPlaneSbo + (cb & 7) * 16 + kb * 128, kPlaneB, nullptr, 0);
+    if (sepB && turn < 2)
+      put_digits(yB, EB, st + kSB * kPlaneA + (cb >> 3) * kPlaneSbo + (cb & 7) * 16 + turn * 128, kPlaneB, nullptr, 0);
   };
   auto issue = [&](uint32_t tmem, uint32_t sa, bool first) {
-    issue_stage<kSB, gram_base<float>(0)>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo),
+    issue_stage<kSB, gram_base<float>(0), kG>(tmem, tc05::desc(sa, 128, kPlaneSbo), tc05::desc(sa + kSB * kPlaneA, 128, kPlaneSbo),
                                           first);
   };
   auto flush = [&](int64_t (&acc0)[16], int64_t (&acc1)[16]) {
@@ -242,7 +246,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
     unsigned long long* G = a.g + b.g + (im ? 3 * MM : 0);
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-      const int j = J * 64 + (warp >> 2) * 16 + c;
+      const int j = J * kTile + (warp >> 2) * 16 + c;
       if (i < b.Nb && j < b.Nb && (im ? (i < j && b.cplx) : i <= j)) {
         add_group(G, MM, i + (int64_t)j * b.Nb, 0, acc0[c]);
         add_group(G, MM, i + (int64_t)j * b.Nb, 1, acc1[c]);
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_gram_kernel(BG a) {
       acc0[c] = acc1[c] = 0;
     }
   };
-  gram_pipeline<kNstB, 0>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, [](int) {}, [](int) {}, fetch, fill,
+  gram_pipeline<kNstB, 0, kG>(bar, gsm, kStageB, (int)(u.q1 - u.q0) * kStagesPerSum, 8, a.hdr, [](int) {}, [](int) {}, fetch, fill,
                           issue, flush);
 }
 
@@ -848,49 +852,58 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
     uint2 w[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = bias_digits((to_fixed(value(j0 + i, col), s_ce[col]) + (1ll << 23)) >> 24);
-    unsigned char* dst = a.c + b.c + (int64_t)(j0 / kStK) * kSB * kPlaneB + (col >> 3) * kPlaneSbo + ((j0 % kStK) >> 3) * 128 +
+    unsigned char* dst = a.c + b.c + ((int64_t)(col / kTile) * stages + j0 / kStK) * kSB * kPlaneB +
+                         ((col % kTile) >> 3) * kPlaneSbo + ((j0 % kStK) >> 3) * 128 +
                          (col & 7) * 16;
     store_digits<kSB>(w, dst, kPlaneB);
   }
 }
 
 // U = Y C
-__global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
+__global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_modes_kernel(BG a) {
   constexpr int LB = Dig<float>::LBM;
   extern __shared__ __align__(1024) unsigned char gsm[];
-  __shared__ __align__(8) DigitBarriers<kNstB> bar;
+  __shared__ __align__(8) DigitBarriers<kNstB, kG> bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const GramUnit u = a.units[blockIdx.x];
   const GramBin b = a.bins[u.bin];
   const int n = b.Nb, stages = (n + kStK - 1) / kStK;
-  const int rl = tid & 127, kh = (tid >> 7) & 1;
+  const int rl = tid & 127, kh = tid >> 7;
   const uint32_t offA = (uint32_t)((rl >> 3) * kPlaneSbo + (rl & 7) * 16);
   const int* E = a.ints + b.colE;
   const int* Ce = a.ints + b.colE + n;
-  float y[8];
-  auto fetch = [&](int t, int js) {
+  float* ring = (float*)(gsm + kNstB * kStageB) + tid;
+  auto load = [&](int t, int js, int q) {
     const int64_t row = (u.q0 + t) * 128 + rl;
     const int c0 = js * kStK + kh * 8;
     const float* p = b.Y + row + c0 * b.ldy;
+    if (row < b.rows) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = (c0 + i < n && row < b.rows) ? __ldg(p + i * b.ldy) : 0.f;
+      for (int i = 0; i < 8; ++i)
+        if (c0 + i < n) async_copy<4>(ring + (q * 8 + i) * kThreads, p + i * b.ldy);
+    }
   };
-  auto fill = [&](int, int js, unsigned char* st) {
+  auto fill = [&](int t, int js, int q, unsigned char* st) {
+    const bool rin = (u.q0 + t) * 128 + rl < b.rows;
     const int c0 = js * kStK + kh * 8;
+    float y[8];
     int e[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) e[i] = c0 + i < n ? __ldg(E + c0 + i) : 128;
+    for (int i = 0; i < 8; ++i) {
+      const bool in = c0 + i < n;
+      y[i] = in && rin ? ring[(q * 8 + i) * kThreads] : 0.f;
+      e[i] = in ? __ldg(E + c0 + i) : 128;
+    }
     put_digits(y, e, st + offA + kh * 128, kPlaneA);
   };
-  auto bsrc = [&](int, int js) { return a.c + b.c + js * kSB * (int64_t)kPlaneB; };
+  auto bsrc = [&](int, int js) { return a.c + b.c + (u.J * stages + js) * kSB * (int64_t)kPlaneB; };
   auto store = [&](int t, const int64_t (&acc0)[16], const int64_t (&acc1)[16]) {
     const int64_t row = (u.q0 + t) * 128 + (warp & 3) * 32 + lane;
-    const int k0 = (warp >> 2) * 16;
+    const int k0 = u.J * kTile + (warp >> 2) * 16;
     const double iw = (b.physical && b.w && row < b.rows) ? 1.0 / sqrt(b.w[row]) : 1.0;
     auto value = [&](int c) {
       const int pk = 8 * LB + __ldg(Ce + k0 + c) - fix_bias<double>() + 24;
-      const double x = __fma_rn((double)acc1[c], 4294967296.0, (double)acc0[c]);
-      return (pk > -900 && pk < 900) ? x * __hiloint2double((pk + 1023) << 20, 0) : scalbn(x, pk);
+      return from_sums(acc0[c], acc1[c], pk, 0.0);
     };
     if (b.cplx) {
       // rows 2m, 2m + 1 hold re, im of point m times the coefficients' parts
@@ -909,7 +922,7 @@ __global__ void __launch_bounds__(kDigThreads, 1) bg_modes_kernel(BG a) {
         if (k0 + c < b.k && row < b.rows) b.Ur[row + (int64_t)(k0 + c) * b.ldu] = (float)(value(c) * iw);
     }
   };
-  product_pipeline<kSB, kNstB, LB>(bar, gsm, (int)(u.q1 - u.q0), stages, a.hdr, fetch, fill, bsrc, store);
+  product_pipeline<kSB, kNstB, LB, kAhead, kG>(bar, gsm, (int)(u.q1 - u.q0), stages, a.hdr, load, fill, bsrc, store);
 }
 
 }  // namespace
@@ -928,7 +941,7 @@ void batched_gram_add(BatchedGramPlan& p, int item, int64_t N, int64_t Nb, int64
   b.g = p.n_g;                      p.n_g += 6 * Nb * Nb;
   b.z = p.n_z;                      p.n_z += (int64_t)kBinMats * Nb * Nb;
   b.f = p.n_f;                      p.n_f += Nb * b.Mb + (int64_t)b.Mb * b.Mb;
-  b.c = p.n_c;                      p.n_c += (Nb + kStK - 1) / kStK * kSB * (int64_t)kPlaneB;
+  b.c = p.n_c;                      p.n_c += (Nb + kStK - 1) / kStK * kSB * (int64_t)kPlaneB * (64 / kTile);
   b.d = p.n_d;                      p.n_d += 1 + 2 * Nb;
   b.s_off = s_off;
   b.flag = item;
@@ -966,15 +979,19 @@ void batched_gram_units(BatchedGramPlan& p, int sms) {
   p.gram.clear();
   p.mod.clear();
   double total = 0.0, mtotal = 0.0, ptotal = 0.0;
-  auto passes = [](const GramBin& b) { return b.Nb <= 64 ? 1 : b.cplx ? 3 : 2; };
+  auto blocks = [](int n) { return (n + kTile - 1) / kTile; };      // column blocks
+  auto passes = [&](const GramBin& b) {
+    return b.Nb <= 64 ? blocks(b.Nb) : 2 + (blocks(b.Nb) - 2) * (b.cplx ? 2 : 1);
+  };
+  auto mtiles = [&](const GramBin& b) { return blocks(b.cplx ? 2 * b.k : b.k); };
   auto mcost = [](const GramBin& b) { return (double)((b.Nb + kStK - 1) / kStK); };
   for (const GramBin& b : p.bins) {
     total += (double)b.rows * passes(b);
-    if (b.k > 0) mtotal += (double)b.rows * mcost(b);
+    if (b.k > 0) mtotal += (double)b.rows * mcost(b) * mtiles(b);
     ptotal += (double)b.rows * b.Nb;
   }
-  const int64_t cap = max_units((int64_t)p.bins.size()) - 4 * (int64_t)p.bins.size();
-  const double want = (double)std::min<int64_t>(4 * (int64_t)sms, cap / 2);
+  const int64_t cap = max_units((int64_t)p.bins.size()) - 8 * (int64_t)p.bins.size();
+  const double want = (double)std::min<int64_t>(8 * (int64_t)sms, cap / 2);
   for (size_t f = 0; f < p.bins.size(); ++f) {
     const GramBin& b = p.bins[f];
     const int64_t sums = (b.rows + 127) / 128;
@@ -984,12 +1001,11 @@ void batched_gram_units(BatchedGramPlan& p, int sms) {
       for (int64_t i = 0; i < s; ++i) v.push_back(GramUnit{(int)f, mode, J, 0, n * i / s, n * (i + 1) / s});
     };
     const double share = want * (double)b.rows / total;
-    cut(p.gram, share, kPacked, 0, sums);
-    if (b.Nb > 64) {
-      cut(p.gram, share, kPlain, 1, sums);
-      if (b.cplx) cut(p.gram, share, kTurned, 1, sums);
+    for (int J = 0; J < blocks(b.Nb); ++J) {
+      cut(p.gram, share, J < 2 ? kPacked : kPlain, J, sums);
+      if (J >= 2 && b.cplx) cut(p.gram, share, kTurned, J, sums);
     }
-    if (b.k > 0) cut(p.mod, want * (double)b.rows * mcost(b) / mtotal, 0, 0, sums);
+    for (int J = 0; J < mtiles(b); ++J) cut(p.mod, want * (double)b.rows * mcost(b) / mtotal, 0, J, sums);
     // prologue: points (bins) or rows rounded to 32 (windows)
     const int64_t pts = b.cplx ? b.rows / 2 : b.ldy;
     const int64_t blk = (pts + 31) / 32;
@@ -1048,11 +1064,11 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   a.S = S;
   a.hdr = hdr;
   const unsigned nb = (unsigned)p.bins.size();
-  const size_t smem = (size_t)kNstB * kStageB;
+  const size_t smem = (size_t)kNstB * kStageB, msmem = smem + (size_t)kAhead * 8 * kThreads * sizeof(float);
   const size_t csmem = sizeof(double2) * ((size_t)p.maxNb * (p.maxNb + 1) / 2);
   const size_t jsmem = sizeof(float2) * ((size_t)kZW * kZW + 2 * kZW * (kZW + 1) + kZW * (kZW + 2) + 64);
   if ((e = ensure_dyn_smem((const void*)bg_gram_kernel, smem)) != cudaSuccess) return e;
-  if ((e = ensure_dyn_smem((const void*)bg_modes_kernel, smem)) != cudaSuccess) return e;
+  if ((e = ensure_dyn_smem((const void*)bg_modes_kernel, msmem)) != cudaSuccess) return e;
   if ((e = ensure_dyn_smem((const void*)bg_chol_kernel, sizeof(double2) * 128 * 129 / 2)) != cudaSuccess) return e;
   if ((e = ensure_dyn_smem((const void*)bg_jacobi32_kernel, jsmem)) != cudaSuccess) return e;
   const size_t nfl = (size_t)p.nitems + 1;
@@ -1065,7 +1081,7 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   au.units = units;
   bg_prologue_kernel<<<(unsigned)p.pro.size(), 256, 0, st>>>(au);
   au.units = units + m;
-  bg_gram_kernel<<<(unsigned)p.gram.size(), kDigThreads, smem, st>>>(au);
+  bg_gram_kernel<<<(unsigned)p.gram.size(), kThreads, smem, st>>>(au);
   bg_chol_kernel<<<nb, kCholThreads, csmem, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned tiles = (unsigned)((p.maxNb + 7) / 8), el = (unsigned)std::max(1, p.maxNb * p.maxNb / 2048);
@@ -1110,7 +1126,7 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   bg_finalize_kernel<<<nb, 256, 0, st>>>(a);
   if (!p.mod.empty()) {
     au.units = units + 2 * m;
-    bg_modes_kernel<<<(unsigned)p.mod.size(), kDigThreads, smem, st>>>(au);
+    bg_modes_kernel<<<(unsigned)p.mod.size(), kThreads, msmem, st>>>(au);
   }
   return cudaGetLastError();
 }
