@@ -57,17 +57,29 @@ __device__ __forceinline__ bool nonfinite(float x) { return (__float_as_int(x) &
 // 1,048,576 x 256 1610 -> 863, 300,001 x 700 2220 -> 691.
 template <typename TX, typename TY, int CT, int W>
 __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(PrologueArgs a) {
-  static_assert(CT <= 32, "a lane keeps the maximum of one column");
+  static_assert(CT % 2 == 0, "maxima in pairs");
   __shared__ double ssum[W][32];
-  __shared__ double sbar[32], ssw[32];
+  __shared__ double sbar[32], ssw[2][32];   // (a warp may be an iteration ahead of the reads of ssw)
+  __shared__ float4 sf[32];      // mean and root of the weight as binary32 pairs
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TX* X = (const TX*)a.X;
   TY* Y = (TY*)a.Y;
   bool bad = false;
   const bool one = a.M <= W * CT;
-  int emax = 0;     // of column (group) warp + W lane
+  uint32_t emax[CT / 2] = {};     // of columns 2 u, 2 u + 1 of this warp, 16 bits each
+  auto flush = [&](int64_t c0) {
+#pragma unroll
+    for (int t = 0; t < CT; ++t) {
+      const int64_t c = c0 + warp + W * t;
+      const int e = __reduce_max_sync(0xffffffffu, (emax[t / 2] >> (16 * (t & 1))) & 0xffffu);
+      if (lane == 0 && c < a.M && e > __ldcg(a.colE + c)) atomicMax(a.colE + c, e);
+    }
+#pragma unroll
+    for (int u = 0; u < CT / 2; ++u) emax[u] = 0;
+  };
   const int64_t nblk = (a.ldy + 31) / 32;
-  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+  int turn = 0;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x, turn ^= 1) {
     const int64_t n = blk * 32 + lane;
     const bool in = n < a.N;
     TX x[CT];
@@ -98,10 +110,11 @@ __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(
           }
         }
       }
+    float4 f = {0.f, 0.f, 1.f, 0.f};
     if (a.remove_mean || a.w) {
       ssum[warp][lane] = s;
+      if (warp == W - 1) ssw[turn][lane] = sw;
       __syncthreads();
-      if (warp == W - 1) ssw[lane] = sw;
       if (warp == 0) {
         double tot = 0.0;
         if (a.remove_mean) {
@@ -109,18 +122,22 @@ __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(
           for (int q = 0; q < W; ++q) tot += ssum[q][lane];
           tot /= (double)a.M;
         }
+        const double root = ssw[turn][lane];
         sbar[lane] = tot;
+        if (sizeof(TX) == 4 && sizeof(TY) == 4) {
+          const float xh = (float)tot, sh = (float)root;
+          sf[lane] = make_float4(xh, (float)(tot - (double)xh), sh, (float)(root - (double)sh));
+        }
       }
       __syncthreads();
       xbar = sbar[lane];
-      sw = ssw[lane];
+      sw = ssw[turn][lane];
+      f = sf[lane];
     }
     if (warp == 0 && in && a.mean) a.mean[n] = xbar;
-    const float xh = (float)xbar, xl = (float)(xbar - (double)xh);
-    const float sh = (float)sw, sl = (float)(sw - (double)sh);
+    const float xh = f.x, xl = f.y, sh = f.z, sl = f.w;
     for (int64_t c0 = 0; c0 < a.M; c0 += W * CT) {
       if (!one) {
-        emax = 0;
 #pragma unroll
         for (int t = 0; t < CT; ++t) {
           const int64_t c = c0 + warp + W * t;
@@ -146,19 +163,12 @@ __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(
         if (!in) y = (TY)0;
         bad = bad || nonfinite(x[t]);
         if (n < a.ldy) Y[n + c * a.ldy] = y;
-        const int e = __reduce_max_sync(0xffffffffu, exp_field(y));
-        if (lane == t) emax = e > emax ? e : emax;
+        emax[t / 2] = __vmaxu2(emax[t / 2], (uint32_t)exp_field(y) << (16 * (t & 1)));
       }
-      if (!one) {
-        const int64_t c = c0 + warp + W * lane;
-        if (lane < CT && c < a.M && emax > __ldcg(a.colE + c)) atomicMax(a.colE + c, emax);
-      }
+      if (!one) flush(c0);
     }
   }
-  if (one) {
-    const int64_t c = warp + W * lane;
-    if (lane < CT && c < a.M) atomicMax(a.colE + c, emax);
-  }
+  if (one) flush(0);
   if (bad) raise_status(a.hdr, PYLOM_ERR_NONFINITE);
   if (blockIdx.x == 0 && threadIdx.x == 0) a.hdr->gram_y = 1;
 }
