@@ -142,15 +142,23 @@ __global__ void __launch_bounds__(kJ32Threads) jacobi32_block_kernel(SvdState s,
         for (int a = 0; a < 4; ++a)
 #pragma unroll
           for (int b = 0; b < 4; ++b) g[a][b] = 0.f;
+        // (the next row tile is on its way while this one is multiplied)
+        constexpr int kLoads = kJRows * kJW / kJ32Threads;
+        const int lr = tid % kJRows, lc = tid / kJRows;
+        const float* src[kLoads];
+        float nx[kLoads];
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+          src[u] = s.A32 + lr + column(lc + u * (kJ32Threads / kJRows)) * M;
+          nx[u] = lr < M ? __ldcg(src[u]) : 0.f;
+        }
         for (int64_t r0 = 0; r0 < M; r0 += kJRows) {
           __syncthreads();
 #pragma unroll
-          for (int u = 0; u < kJRows * kJW / kJ32Threads; ++u) {
-            const int idx = tid + u * kJ32Threads;
-            const int r = idx % kJRows, l = idx / kJRows;
-            sA[r * LD + l] = (r0 + r < M) ? __ldcg(s.A32 + r0 + r + column(l) * M) : 0.f;
-          }
+          for (int u = 0; u < kLoads; ++u) sA[lr * LD + lc + u * (kJ32Threads / kJRows)] = nx[u];
           __syncthreads();
+#pragma unroll
+          for (int u = 0; u < kLoads; ++u) nx[u] = r0 + kJRows + lr < M ? __ldcg(src[u] + r0 + kJRows) : 0.f;
 #pragma unroll 4
           for (int r = sl; r < kJRows; r += 4) {
             const float4 x = *(const float4*)(sA + r * LD + ti), y = *(const float4*)(sA + r * LD + tj);
@@ -242,12 +250,23 @@ __global__ void __launch_bounds__(kJ32Threads) jacobi32_block_kernel(SvdState s,
           __syncthreads();
         }
         // A32 and V32 columns <- columns J (a thread per row)
+        float nv[kJW];
+        auto fetch = [&](int64_t row) {
+          const float* base = row < M ? s.A32 + row : s.V32 + (row - M);
+          const int64_t ld = row < M ? M : Mb;
+          if (row < M + Mb) {
+#pragma unroll
+            for (int l = 0; l < kJW; ++l) nv[l] = __ldcg(base + column(l) * ld);
+          }
+        };
+        fetch(tid);
         for (int64_t row = tid; row < M + Mb; row += kJ32Threads) {
           float* base = row < M ? s.A32 + row : s.V32 + (row - M);
           const int64_t ld = row < M ? M : Mb;
           float v[kJW];
 #pragma unroll
-          for (int l = 0; l < kJW; ++l) v[l] = __ldcg(base + column(l) * ld);
+          for (int l = 0; l < kJW; ++l) v[l] = nv[l];
+          fetch(row + kJ32Threads);
 #pragma unroll 1
           for (int l = 0; l < kJW; l += 4) {
             float o[4] = {0.f, 0.f, 0.f, 0.f};
@@ -304,6 +323,7 @@ struct SmallGemm {
   double alpha, beta;
   const double* D;   // ld m
   double* C;         // ld m
+  int sym;           // op(A) B is symmetric: tiles on and above the diagonal, and their mirror images
 };
 struct SmallGemms {
   SmallGemm g[2];
@@ -318,7 +338,7 @@ __global__ void __launch_bounds__(128) small_gemm_kernel(SmallGemms gs) {
   const SmallGemm& p = gs.g[blockIdx.z];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const int64_t i0 = (int64_t)blockIdx.x * T, j0 = (int64_t)blockIdx.y * T;
-  if (i0 >= p.m || j0 >= p.n) return;
+  if (i0 >= p.m || j0 >= p.n || (p.sym && i0 > j0)) return;
   double acc[U][U][2];
 #pragma unroll
   for (int a = 0; a < U; ++a)
@@ -353,7 +373,9 @@ __global__ void __launch_bounds__(128) small_gemm_kernel(SmallGemms gs) {
     const int64_t i = i0 + r, j = j0 + c;
     if (i < p.m && j < p.n) {
       const double v = (part[0][r][c] + part[1][r][c]) + (part[2][r][c] + part[3][r][c]);
-      p.C[i + j * p.m] = p.alpha * v + (p.D ? p.beta * p.D[i + j * p.m] : 0.0);
+      const double x = p.alpha * v + (p.D ? p.beta * p.D[i + j * p.m] : 0.0);
+      p.C[i + j * p.m] = x;
+      if (p.sym && i0 != j0) p.C[j + i * p.m] = x;
     }
   }
 }
@@ -592,7 +614,7 @@ cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int
   // leading dimension k, C and D m)
   auto mm = [&](int ta, int64_t m, int64_t k, double alpha, const double* A, int64_t lda, const double* B,
                 double beta, const double* D, double* C) {
-    return SmallGemm{ta, m, Mp, k, A, lda, B, k, alpha, beta, D, C};
+    return SmallGemm{ta, m, Mp, k, A, lda, B, k, alpha, beta, D, C, ta && A == B};
   };
   auto one = [&](const SmallGemm& g, const unsigned* skip = nullptr) {
     if (e == cudaSuccess) e = small_gemms(SmallGemms{{g, g}, skip}, 1, st);
