@@ -260,11 +260,20 @@ def gpu_numa_info(local_rank):
     return info
 
 
+def digit_flops(N, M, pairs):
+    """Operations of the exact Gram matrix: `pairs` digit products an element
+    pair (64 in binary64, 24 in binary32) on the 128 x 64 tiles on and above the
+    diagonal."""
+    nJ, nI = (M + 63) // 64, (M + 127) // 128
+    tiles = sum(nJ - 2 * i for i in range(nI))
+    return 2.0 * N * 128 * 64 * tiles * pairs
+
+
 def bench_adjoint(args, dev):
     """Forward + hand-written backward of the truncated-POD reconstruction
     loss on the 4,194,304 x 256 float32 known-spectrum matrix, r = 20: timed
-    on the mixed-precision path (FP32 modes, 3xTF32 products on tcgen05,
-    binary64 tree passes and square SVD adjoint) and, for comparison, on the
+    on the mixed-precision path (binary32 Y, digit products on tcgen05,
+    binary64 square SVD adjoint) and, for comparison, on the
     binary64 path."""
     import torch
     import paper_2405_15529_gb300 as pg
@@ -308,7 +317,7 @@ def bench_adjoint(args, dev):
     ms64, rel64 = run(pg.PREC_FP64, 1, 1)
     out = {"workload": "known_spectrum_4194304x256_f32_weighted_r20_loss_grad", "ms_per_step": ms,
            "value": N * M * 4 / (ms * 1e-3) / 1e9, "unit": "GB/s of X (forward + backward)",
-           "steps": args.adj_steps, "precision": "mixed (3xTF32 tcgen05; binary64 tree and square SVD adjoint)",
+           "steps": args.adj_steps, "precision": "mixed (binary32 Y, digit products on tcgen05; binary64 square SVD adjoint)",
            "grad_rel_err_vs_closed_form": rel,
            "fp64_path_ms_same_x": ms64, "fp64_path_grad_rel_err_vs_closed_form": rel64,
            "speedup_vs_fp64_path": ms64 / ms,
@@ -320,8 +329,8 @@ def bench_adjoint(args, dev):
 
 def bench_mixed(args, dev):
     """The 4,194,304 x 256 float32 known-spectrum matrix through the mixed
-    path (FP32 leaves, 3xTF32 block reflectors on tcgen05, FP64 tree and
-    SVD) and, once, through the FP64 path on the same X."""
+    path (binary32 Y, exact digit products on tcgen05, binary64 SVD) and,
+    once, through the FP64 path on the same X."""
     import numpy as np
     import torch
     import paper_2405_15529_gb300 as pg
@@ -330,10 +339,7 @@ def bench_mixed(args, dev):
     XT, w, s = synth.known_spectrum_torch(N, M, device=dev, dtype=torch.float32)
     X = XT.t()
     prec = pg.PREC_MIXED_3XTF32
-    leaf = 0
-    if args.tune:
-        from paper_2405_15529_gb300 import tune
-        leaf = tune.pod_leaf_rows_for(N, M, prec, tune=True)
+    leaf = 0          # automatic: R from the exact Gram matrix
     ws = torch.empty(pg.pod_workspace_size(N, M, leaf, M, pg.F32, prec), dtype=torch.uint8, device=dev)
     U = pg.empty_colmajor(N, M, torch.float32, dev)
     S = torch.empty(M, dtype=torch.float64, device=dev)
@@ -368,15 +374,14 @@ def bench_mixed(args, dev):
     S64 = ref.S.cpu().numpy()
     leaf_ms = phases["leaf_qr"] / max(n, 1)
     out = {"workload": f"known_spectrum_{N}x{M}_f32_weighted_energy0.99", "status": st, "r": r,
-           "leaf_rows": leaf, "leaves": pg.leaf_count(N, M, leaf) if leaf else min(152, pg.leaf_count(N, M, 0)),
+           "leaf_rows": leaf, "route": "gram",
            "ms_per_step": ms, "value": N * M * 4 / (ms * 1e-3) / 1e9, "unit": "GB/s of X (float32)",
            "phases_ms_per_step": {k: v / max(n, 1) for k, v in phases.items()},
            "fp64_path_ms_same_x": ms64, "speedup_vs_fp64_path": ms64 / ms,
            "sigma_max_abs_diff_vs_fp64_path_over_smax": float(np.max(np.abs(S_mix - S64)) / S64[0]),
            "sigma_max_abs_err_vs_closed_form_over_smax": float(np.max(np.abs(S_mix - s)) / s[0]),
-           "leaf_kernel": {"kernel": "leaf_qr_mixed_kernel (FP32 panels + 3xTF32 tcgen05 trailing updates)",
-                           "ms_per_launch": leaf_ms,
-                           "useful_tflops": 2.0 * N * M * M / (leaf_ms * 1e-3) / 1e12}}
+           "gram_phase": {"kernels": "gram_prologue_kernel, gram_kernel<float>", "ms": leaf_ms,
+                          "digit_product_tflops": digit_flops(N, M, 24) / (leaf_ms * 1e-3) / 1e12}}
     del X, XT, w, ws, U, S, VT, r_dev, ref
     torch.cuda.empty_cache()
     return out
@@ -672,29 +677,22 @@ def bench_waves_1808(args, dev):
     except (OSError, ValueError):
         pass
     hbm = peaks.get("hbm_gbs", 6800.0)
-    tf32_3x = peaks.get("bf16_tflops", 1900.0) * 0.5 / 3.0     # nominal tf32/bf16 = 1/2; three MMAs per product
-    t_roof = max(bytes_x / (hbm * 1e9), 2.0 * N * M * M / (tf32_3x * 1e12))
+    bf16 = peaks.get("bf16_tflops", 1900.0)
+    t_roof = max(bytes_x / (hbm * 1e9), digit_flops(N, M, 24) / (bf16 * 1e12))
     leaf_ms = mix["phases_ms"]["leaf_qr"]
     tree_ms = mix["phases_ms"]["tree"]
-    # dominant kernel of the mixed step: the leaves (FP32 panels + 3xTF32
-    # trailing updates, 2NM^2 - (2/3)PM^3 flops as three TF32 products); the
-    # binary64 cooperative tree that follows is reported beside it
-    P = pg.leaf_count(N, M, 0)
-    P = min(P, 152) if P > 152 else P
-    leaf_flops = 2.0 * N * M * M - (2.0 / 3.0) * P * M ** 3
-    tree_flops = (P - 1) * (2.0 / 3.0) * M ** 3
-    fp64_peak = probe_peak("mma")
-    leaf_bytes = N * M * 4 + N * M * 4      # read X (FP32), write the FP32 reflectors
-    t_leaf_roof = max(leaf_flops / (tf32_3x * 1e12), leaf_bytes / (hbm * 1e9))
-    roofline = {"bound": "tensor", "achieved": leaf_flops / (leaf_ms * 1e-3) / 1e12, "peak": tf32_3x,
+    # dominant kernels of the mixed step: the centring and the digit products of the Gram
+    # matrix; its double-double Cholesky factor is reported beside them
+    leaf_flops = digit_flops(N, M, 24)
+    leaf_bytes = N * M * 4 + N * M * 4      # read X, write the binary32 Y
+    t_leaf_roof = max(leaf_flops / (bf16 * 1e12), leaf_bytes / (hbm * 1e9))
+    roofline = {"bound": "tensor", "achieved": leaf_flops / (leaf_ms * 1e-3) / 1e12, "peak": bf16,
                 "unit": "TFLOP/s", "frac": t_leaf_roof / (leaf_ms * 1e-3), "traffic": None,
-                "kernel": "leaf_qr_mixed_kernel",
-                "peak_source": "3xTF32 = measured bf16 burst x nominal tf32/bf16 (1/2) / 3",
+                "kernel": "gram_prologue_kernel + gram_kernel<float>",
+                "peak_source": "measured cuBLAS bf16 burst",
                 "algorithmic_flops_per_launch": leaf_flops, "algorithmic_bytes_per_launch": leaf_bytes,
-                "ms_per_launch": leaf_ms, "leaves": P,
-                "tree": {"kernel": "tree_coop_kernel (binary64)", "ms_per_launch": tree_ms,
-                         "algorithmic_flops_per_launch": tree_flops, "peak_fp64_tflops": fp64_peak,
-                         "frac": tree_flops / (fp64_peak * 1e12) / (tree_ms * 1e-3) if tree_ms > 0 else None}}
+                "ms_per_launch": leaf_ms,
+                "tree": {"kernel": "gram_chol_kernel", "ms_per_launch": tree_ms}}
     cpu = {"skipped": "the oracle's unblocked QR and cyclic Jacobi at 1808 columns take minutes even on a "
                       "row sample; run bench.py --c3-cpu for the extrapolated figure"}
     if args.c3_cpu:
@@ -713,11 +711,10 @@ def bench_waves_1808(args, dev):
             "noise_weyl_bound_over_smax": noise_bound / s_cf[0],
             "min_mode_overlap_vs_fp64_path": worst, "mixed_U_orthonormality_fro": orth_mix,
             "pct_roofline": {"value": t_roof / (mix["ms"] * 1e-3),
-                             "formula": "max(bytes_X/HBM_peak, 2NM^2/(tf32_peak/3)) / step time",
-                             "tf32_peak_tflops": peaks.get("bf16_tflops", 1900.0) * 0.5,
+                             "formula": "max(bytes_X/HBM_peak, digit flops/bf16_peak) / step time",
+                             "bf16_peak_tflops": bf16,
                              "hbm_peak_gbs": hbm},
-            "leaf_kernel": {"kernel": "leaf_qr_mixed_kernel", "ms_per_step": leaf_ms,
-                            "useful_tflops": 2.0 * N * M * M / (leaf_ms * 1e-3) / 1e12}}
+            "gram_phase_ms": leaf_ms}
 
 
 def bench_spod(args, dev):
@@ -888,14 +885,8 @@ def run_ours(args, rank, world, local_rank):
     XT, w, s = synth.known_spectrum_torch(N, M, device=dev)
     X = XT.t()
     torch.cuda.synchronize()
-    # leaf height: given, or the autotuner's (timed outside the timed region, cached)
-    tuned_leaf = None
-    if args.leaf_rows == 0 and args.tune:
-        from paper_2405_15529_gb300 import tune
-        t_tune = time.perf_counter()
-        tuned_leaf = tune.pod_leaf_rows_for(N, M, pg.PREC_FP64, tune=True)
-        t_tune = time.perf_counter() - t_tune
-        args.leaf_rows = tuned_leaf
+    # leaf height: given (Householder leaves and tree), or automatic (R from the exact Gram matrix)
+    gram = args.leaf_rows == 0 and not os.environ.get("PYLOM_TREE")
     P = pg.leaf_count(N, M, args.leaf_rows)
     ws_bytes = pg.pod_workspace_size(N, M, args.leaf_rows, M, pg.F64, pg.PREC_FP64)
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
@@ -977,24 +968,31 @@ def run_ours(args, rank, world, local_rank):
     bytes_x = N * M * 8
     value = job_gbs(bytes_x, ms, world)
 
-    # dominant kernel: the leaf QR kernel (one launch per step).  When the
-    # tree runs as its own cooperative kernel (from 64 leaves) the leaf
-    # kernel's work is the leaves' 2NM^2 - (2/3)PM^3; when the leaves merge
-    # as they finish, the tree's (P - 1)(2/3)M^3 is in the same launch.
+    # dominant kernels: on the Gram route the digit products (phase: Y, its
+    # fixed-point form, the Gram matrix); on the Householder route the leaf QR
+    # kernel (one launch per step).  When the tree runs as its own cooperative
+    # kernel (from 64 leaves) the leaf kernel's work is the leaves' 2NM^2 -
+    # (2/3)PM^3; when the leaves merge as they finish, the tree's (P -
+    # 1)(2/3)M^3 is in the same launch.
     leaf_ms = phases["leaf_qr"] / max(ncalls, 1)
     tree_ms = phases["tree"] / max(ncalls, 1)
     coop_tree = tree_ms > 0.0
     flops_tree = (P - 1) * (2.0 / 3.0) * M ** 3
     flops_leaf = 2.0 * N * M * M - (2.0 / 3.0) * P * M ** 3 + (0.0 if coop_tree else flops_tree)
+    if gram:
+        flops_leaf = digit_flops(N, M, 64)
     achieved = flops_leaf / (leaf_ms * 1e-3) / 1e12
-    hbm_peak = None
+    hbm_peak = bf16_peak = None
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            hbm_peak = json.load(f).get("hbm_gbs")
+            peaks = json.load(f)
+            hbm_peak, bf16_peak = peaks.get("hbm_gbs"), peaks.get("bf16_tflops")
     except (OSError, ValueError):
         pass
     hbm_peak = hbm_peak or 6800.0
-    t_roof = max(bytes_x / (hbm_peak * 1e9), 2.0 * N * M * M / (peak_mma * 1e12))
+    bf16_peak = bf16_peak or 1900.0
+    t_roof = max(bytes_x / (hbm_peak * 1e9),
+                 digit_flops(N, M, 64) / (bf16_peak * 1e12) if gram else 2.0 * N * M * M / (peak_mma * 1e12))
     pct_roof = t_roof / (ms * 1e-3)
 
     # end to end through the public API from pinned host memory: pylom_pod
@@ -1140,6 +1138,12 @@ def run_ours(args, rank, world, local_rank):
     # one top-down launch per tree level, the modes
     svd_launches = (3 + 5 + 2 if M >= 256 else 1) + 2
     launches_per_step = 1 + (1 if P >= 64 or M >= 384 else 0) + svd_launches + 1 + levels + 1
+    if gram:
+        # centring, cutting (binary64), Gram matrix, Cholesky factor; small SVD: 49 (scale, two
+        # binary32 stages with their init and widen, four products, six steps of check, angles and
+        # three products, the last look, restart, sweeps, norms, order, output, completion);
+        # coefficients, modes
+        launches_per_step = 4 + 49 + 2
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": "GB/s", "n_gpus": world, "steps": args.steps,
@@ -1147,28 +1151,32 @@ def run_ours(args, rank, world, local_rank):
             "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": WORKLOAD, "N": N, "M": M, "leaves": P, "r": r,
                        "leaf_rows": args.leaf_rows,
-                       "leaf_rows_source": ("autotuned (tune.pod_leaf_rows_for, %.0f s outside the timed region)"
-                                            % t_tune) if tuned_leaf else (
-                           "given" if args.leaf_rows else "automatic"),
+                       "leaf_rows_source": "given" if args.leaf_rows else "automatic",
+                       "route": "gram" if gram else "householder",
                        "l2": "inputs (8.6 GB per rank) larger than L2 (129 MB); no flush",
                        "parallelism": f"independent problems x{world}"},
-            "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak_mma, "unit": "TFLOP/s",
-                         "frac": achieved / peak_mma, "traffic": LEAF_FP64_TRAFFIC_BYTES if (
+            "roofline": {"bound": "tensor", "achieved": achieved, "peak": bf16_peak if gram else peak_mma, "unit": "TFLOP/s",
+                         "frac": achieved / (bf16_peak if gram else peak_mma),
+                         "traffic": None if gram else LEAF_FP64_TRAFFIC_BYTES if (
                              N == N_FULL and M == M_FULL and P == 304) else None,
-                         "traffic_source": LEAF_FP64_TRAFFIC_SOURCE,
+                         "traffic_source": None if gram else LEAF_FP64_TRAFFIC_SOURCE,
                          "algorithmic_bytes_per_launch": (8 + 8) * N * M,
-                         "kernel": "leaf_qr_kernel (leaf Householder QR%s)" % (
+                         "kernel": "gram_prologue_kernel + pack_kernel + gram_kernel (64 digit products of an "
+                                   "element pair, binary16 operands)" if gram else
+                                   "leaf_qr_kernel (leaf Householder QR%s)" % (
                              "; the tree is its own kernel" if coop_tree else " + tree merges"),
-                         "peak_source": "measured live: FP64 mma.sync.m8n8k4 throughput probe with "
+                         "peak_source": "measured cuBLAS bf16 burst" if gram else "measured live: FP64 mma.sync.m8n8k4 throughput probe with "
                                         "independent chains (bench_probe.cu; MEASURED_PEAKS.json has no "
                                         "FP64 figure); cross-checked by the FP64 4096^3 product",
                          "algorithmic_flops_per_launch": flops_leaf, "ms_per_launch": leaf_ms,
-                         "tree": {"kernel": tree_kernel, "ms_per_launch": tree_ms,
+                         "tree": {"kernel": "gram_chol_kernel", "ms_per_launch": tree_ms} if gram else
+                                 {"kernel": tree_kernel, "ms_per_launch": tree_ms,
                                   "algorithmic_flops_per_launch": flops_tree,
                                   "achieved_tflops": flops_tree / (tree_ms * 1e-3) / 1e12 if coop_tree else None}},
             "pct_roofline_pod": {"value": pct_roof,
-                                 "formula": "max(bytes_X/HBM_peak, 2NM^2/FP64_mma_peak) / step time",
-                                 "hbm_peak_gbs": hbm_peak, "fp64_mma_tflops": peak_mma,
+                                 "formula": ("max(bytes_X/HBM_peak, digit flops/bf16_peak) / step time" if gram else
+                                             "max(bytes_X/HBM_peak, 2NM^2/FP64_mma_peak) / step time"),
+                                 "bf16_peak_tflops": bf16_peak, "hbm_peak_gbs": hbm_peak, "fp64_mma_tflops": peak_mma,
                                  "fp64_fma_tflops": peak_fma,
                                  "fp64_matmul_4096cubed_tflops": mm_tflops},
             "phases_ms_per_step": {k: v / max(ncalls, 1) for k, v in phases.items()},
