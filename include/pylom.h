@@ -132,7 +132,13 @@ pylom_status pylom_workspace_status(const void* ws, void* stream, int64_t* r, in
  *               capped at r_max; energy <= 0 keeps r = r_max.
  *  r_max        1 <= r_max <= M: the columns U has room for.
  *  mode_kind    pylom_mode_kind (see above).
- *  leaf_rows    TSQR leaf height hint b (0 = automatic; else b >= M).
+ *  leaf_rows    TSQR leaf height hint b >= M: Householder leaves and tree.  0 =
+ *              automatic: where energy > 0 (at most 1 - 1e-4) or r_max < M, R
+ *              is the Cholesky factor of the exact Gram matrix of the weighted
+ *              centred data (its diagonal is non-negative) and the modes are Y
+ *              V_r S_r^-1; with r_max < M and no such energy share the device
+ *              takes leaves and tree instead when S_r < 1e-4 S_1 (1e-5 mixed).
+ *              The environment variable PYLOM_TREE asks for leaves and tree too.
  *  U      out  N x r_max, ldu >= N: the first r columns receive the
  *              modes, the rest are left untouched.  Element type: binary64
  *              for PYLOM_PREC_FP64, binary32 for PYLOM_PREC_MIXED_3XTF32.
@@ -284,7 +290,10 @@ pylom_status pylom_pod_shard_modes(const double* Bg, const int64_t* r, int64_t N
  * pylom_pod_backward -- hand-written adjoint of pylom_pod (no counterpart in
  * the paper; it differentiates the composition of Alg. 2, Alg. 1 and Eqs.
  * svdqr1-svdqr3).  Given cotangents dU (of the r returned modes), dS and
- * dVT, writes dX, the cotangent of X.  Q is recomputed from the leaf and
+ * dVT, writes dX, the cotangent of X.  With leaf_rows = 0 and a forward that
+ * did not factor Y: two products with Y (W = Y^T dU; dY = Y C + dU D) where
+ * the singular values to invert are large enough (1e-4 S_1, 1e-5 mixed);
+ * else, decided on the device, Q is recomputed from the leaf and
  * tree reflectors that the forward call left in its workspace (Q^T dU by
  * the leaf reflectors and a bottom-up tree pass; Q [B; 0] by the top-down
  * pass); the square SVD adjoint of R runs in binary64 on M x M matrices.
@@ -331,7 +340,9 @@ pylom_status pylom_tsqr(const void* A, int64_t N, int64_t M, int64_t lda, int xt
 
 /* ------------------------------------------------------------------------
  * pylom_svd_small -- SVD of the small M x M factor, R = U S V^T
- * (Eq. svdqr2), by parallel one-sided Jacobi in binary64 across thread
+ * (Eq. svdqr2), by one-sided Jacobi: from M = 12 (max_sweeps >= 8) two binary32
+ * stages and binary64 steps of simultaneous rotations first; then parallel
+ * sweeps in binary64 across thread
  * blocks (round-robin pair ordering; a pair rotates while
  * |a_i.a_j| > M 2^-53 |a_i| |a_j|).  Sorted descending, same sign rule as
  * pylom_pod.  R is any M x M matrix (triangular or not), not modified.
@@ -476,7 +487,7 @@ pylom_status pylom_matmul(int transA, const double* A, const double* B, double* 
  * the scratch is a fixed array inside the library (about 1 MiB per device
  * that loads it, held until the process exits).  The binary64 sweeps start
  * from R^T: this entry point skips the binary32 preconditioning that
- * pylom_svd_small runs from M = 256 on (same SVD, more sweeps).
+ * pylom_svd_small runs from M = 12 on (same SVD, more sweeps).
  *  R, U, S, VT, ldr, ldu, ldvt, max_sweeps   as pylom_svd_small.
  *  M      1 <= M <= 256; larger M returns PYLOM_ERR_SHAPE (use
  *         pylom_svd_small with a workspace).

@@ -49,12 +49,12 @@ __device__ __forceinline__ bool nonfinite(float x) { return (__float_as_int(x) &
 // Y is the bound in binary32; in binary64 the two to three binary64 operations
 // an element (sum, difference, weight; two lanes a clock) are.  So the row's
 // division and square root are one warp's work, not every warp's, finiteness
-// is an integer test, and the column maxima, which took a register a column,
-// are reduced over the warp on the spot: that leaves registers for two blocks
-// of 16 warps.  Before (a register a column, 8 warps of 32 columns, every warp
-// its own division and root) -> here, microseconds: 65,537 x 63 binary64 71 ->
-// 47, 1,048,576 x 256 binary64 2960 -> 2720; binary32 262,144 x 100 185 -> 105,
-// 1,048,576 x 256 1610 -> 863, 300,001 x 700 2220 -> 691.
+// is an integer test, and the column maxima take half a register a column: that
+// leaves registers for two blocks of 16 warps.  Before (a register a column, 8
+// warps of 32 columns, every warp its own division and root) -> here,
+// microseconds: 65,537 x 63 binary64 71 -> 41, 1,048,576 x 256 binary64 2960 ->
+// 2720; binary32 262,144 x 100 146 -> 80, 4,194,304 x 256 6400 -> 3020,
+// 300,001 x 700 2150 -> 690.
 template <typename TX, typename TY, int CT, int W>
 __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(PrologueArgs a) {
   static_assert(CT % 2 == 0, "maxima in pairs");
@@ -67,13 +67,15 @@ __global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) gram_prologue_kernel(
   bool bad = false;
   const bool one = a.M <= W * CT;
   uint32_t emax[CT / 2] = {};     // of columns 2 u, 2 u + 1 of this warp, 16 bits each
-  auto flush = [&](int64_t c0) {
+  auto flush = [&](int64_t c0) {      // lane t: column t of this warp
+    int mine = 0;
 #pragma unroll
     for (int t = 0; t < CT; ++t) {
-      const int64_t c = c0 + warp + W * t;
       const int e = __reduce_max_sync(0xffffffffu, (emax[t / 2] >> (16 * (t & 1))) & 0xffffu);
-      if (lane == 0 && c < a.M && e > __ldcg(a.colE + c)) atomicMax(a.colE + c, e);
+      mine = lane == t ? e : mine;
     }
+    const int64_t c = c0 + warp + W * lane;
+    if (lane < CT && c < a.M && mine > __ldcg(a.colE + c)) atomicMax(a.colE + c, mine);
 #pragma unroll
     for (int u = 0; u < CT / 2; ++u) emax[u] = 0;
   };

@@ -31,8 +31,10 @@
 // SVD of a field with a decaying spectrum on a floor, ten binary64 sweeps ->
 // here: M = 32 2.1 -> 0.25 ms, 64 4.2 -> 0.45, 128 9.6 -> 1.0; with the
 // earlier preconditioning (8-column blocks, three binary64 sweeps after it)
-// M = 256 13.3 -> 4.0, 700 114 -> 40 ms; singular values within 1.5e-15
-// S_max (2e-14 before: fewer rotations).
+// M = 256 13.3 -> 3.5, 700 114 -> 36 ms; singular values within 1.5e-15
+// S_max (2e-14 before: fewer rotations).  At M = 700 the binary32 stages take
+// 21 ms (23.8 before the next row tile was fetched during the products) and
+// the products 14.5 (17.8 before symmetric ones computed half their tiles).
 #include "kernels.h"
 
 namespace pylom {
