@@ -48,6 +48,7 @@ constexpr int kJClusterMax = 8;        // up to 8 blocks run as one cluster (che
 // words of s.rot32: rotations of each sweep of the two stages, then
 constexpr int kJScale = 2 * kJ32MaxSweeps;       // largest exponent field of R
 constexpr int kJSteps = 6;                       // binary64 steps of simultaneous rotations
+constexpr int kJManyColumns = 128;               // from here on all of them
 constexpr int kJOpen = kJScale + 1;              // kJSteps + 1 words: pairs not converged at each check; then: entries of V^T V off
 constexpr int kJWords = kJOpen + kJSteps + 2;
 
@@ -646,8 +647,11 @@ cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int
   // whose 300 smallest singular values lie within 20 % of each other most
   // have angles above 0.05 together, and were left to the sweeps (42 ms).
   constexpr double kLimit[kJSteps] = {0.3, 0.1, 0.1, 0.02, 0.01, 2e-4};
+  // (fewer columns hold no such crowd: the last two steps' ten empty launches
+  // cost 65,537 x 63 25 of 1,100 us)
+  const int steps = M >= kJManyColumns ? kJSteps : 4;
   const unsigned gc = (unsigned)((Mp * 32 + 255) / 256);
-  for (int it = 0; it < kJSteps; ++it) {
+  for (int it = 0; it < steps; ++it) {
     const bool fwd = (it & 1) == 0;
     const double *Ai = fwd ? s.A : s.A2, *Vi = fwd ? s.V : T3;
     double *Ao = fwd ? s.A2 : s.A, *Vo = fwd ? T3 : s.V;
@@ -657,19 +661,19 @@ cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int
     two(mm(1, Mp, M, 1.0, Ai, M, Ai, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, Vi, Mp, Vi, 0.0, nullptr, T1), look);
     if (e != cudaSuccess) return e;
     jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, it >= 2 && fwd ? T1 : nullptr, wtol, open + it, it, look);
-    jacobi_angles_kernel<<<gr, 256, 0, st>>>(s, T0, T1, T2, T4, T5, kLimit[it], skip);
+    jacobi_angles_kernel<<<gr, 256, 0, st>>>(s, T0, T1, T2, T4, T5, kLimit[it < 2 ? it : it + kJSteps - steps], skip);
     e = cudaGetLastError();
     one(mm(0, Mp, Mp, 0.5, T4, Mp, T2, 1.0, T5, T0), skip);                          // Q
     two(mm(0, M, Mp, 1.0, Ai, M, T0, 0.0, nullptr, Ao), mm(0, Mp, Mp, 1.0, Vi, Mp, T0, 0.0, nullptr, Vo), skip);
   }
   // (after fewer steps the last look stands)
-  const unsigned* look = open + kJSteps - 2;
+  const unsigned* look = open + steps - 2;
   two(mm(1, Mp, M, 1.0, s.A, M, s.A, 0.0, nullptr, T0), mm(1, Mp, Mp, 1.0, s.V, Mp, s.V, 0.0, nullptr, T1), look);
   if (e != cudaSuccess) return e;
-  jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, T1, wtol, open + kJSteps + 1, kJSteps, look);
+  jacobi_check_kernel<<<gc, 256, 0, st>>>(s, T0, T1, wtol, open + kJSteps + 1, steps, look);
   // a V that is not orthogonal after all: the binary64 sweeps start from R^T
-  jacobi_restart_kernel<<<gr, 256, 0, st>>>(s, R, ldr, open + kJSteps + 1, open + kJSteps);
-  *open_pairs = open + kJSteps;
+  jacobi_restart_kernel<<<gr, 256, 0, st>>>(s, R, ldr, open + kJSteps + 1, open + steps);
+  *open_pairs = open + steps;
   return cudaGetLastError();
 }
 
