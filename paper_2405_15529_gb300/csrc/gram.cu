@@ -15,7 +15,7 @@
 // Measured (4,194,304 x 256, binary64): Householder leaves + tree 554 + 13
 // ms; here Y 8.6, cutting it 2.4, Gram matrix 25.8, Cholesky factor 0.74 ms.
 // 1,048,576 x 128: leaves + tree 39 + 3.8 ms; here 1.4, 0.3, 2.1 and 0.35.
-// Binary32 (mixed, 4,194,304 x 256): leaves + tree 57.7 + 8.8 ms; here 3.4,
+// Binary32 (mixed, 4,194,304 x 256): leaves + tree 57.7 + 8.8 ms; here 3.0,
 // 12.5 and 0.71 ms.
 #include <atomic>
 

@@ -21,8 +21,8 @@
 // zero matrix) are flagged on the device and left to that kernel.
 //
 // Persistent kernel -> here: 24 bins (N 16k..262k, Nb 16..128, 1.3 GB) 374 ->
-// 14.5 ms, 12 windows (N 16k..262k, M 16..96) 115 -> 4.9 ms, SPOD of 131072 x
-// 1056 25.6 -> 9.7 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
+// 13.6 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.6 ms, SPOD of 131072 x
+// 1056 25.6 -> 7.3 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
 #include <algorithm>
 
 #include "digits.cuh"
