@@ -19,6 +19,7 @@
 // Precision: the leaf working copy is complex64 (TC = float, the "mixed"
 // path: FP32 storage and updates, compensated FP32 sums reduced in FP64) or
 // complex128 (TC = double); tree, Jacobi and all reflector scalars are FP64.
+#include <new>
 #include <type_traits>
 
 #include "kernels.h"
@@ -1273,9 +1274,15 @@ static pylom_status batched_upload_tables(pylom_batched_plan* plan, void* ws, vo
     int dev = 0, sms = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) batched_gram_units(plan->gram, sms);
-    if (e == cudaSuccess)
-      e = batched_gram_upload(plan->gram, base, plan->forced.data(), (int)plan->forced.size(), st);
+    // (the lists of units are host memory: an allocation that fails must not
+    // leave this C entry as an exception)
+    try {
+      if (e == cudaSuccess) batched_gram_units(plan->gram, sms);
+      if (e == cudaSuccess)
+        e = batched_gram_upload(plan->gram, base, plan->forced.data(), (int)plan->forced.size(), st);
+    } catch (const std::bad_alloc&) {
+      e = cudaErrorMemoryAllocation;
+    }
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
