@@ -261,20 +261,19 @@ __device__ void hessenberg_reduce(double* H, int64_t ldh, double* Z, int64_t ldz
   }
 }
 
-// P = I - tau v v^T with v = [1, v1, v2] mapping (x, y, z) to (beta, 0, 0)
-__device__ __forceinline__ void reflector3(double x, double y, double z, double& tau, double& v1, double& v2) {
+// P = I - tau v v^T with v = [1, v1, v2] mapping (x, y, z) to (beta, 0, 0).
+// Called by lanes 0..2 with the same arguments: they leave tau, v1 and v2 in
+// sc[3..5], each by its own quotient of the one division.
+__device__ __forceinline__ void reflector3(double x, double y, double z, double* sc) {
+  const int lane = threadIdx.x & 31;
   const double sigma = fma(y, y, z * z);
-  tau = 0.0;
-  v1 = 0.0;
-  v2 = 0.0;
+  double q = 0.0;
   if (sigma > 0.0) {
     const double nrm = sqrt(fma(x, x, sigma));
     const double beta = x >= 0.0 ? -nrm : nrm;
-    tau = (beta - x) / beta;
-    const double inv = 1.0 / (x - beta);
-    v1 = y * inv;
-    v2 = z * inv;
+    q = (lane == 0 ? beta - x : lane == 1 ? y : z) / (lane == 0 ? beta : x - beta);
   }
+  sc[3 + lane] = q;
 }
 
 // One implicit double-shift (Francis) QR step on the active window [l, hi]
@@ -284,10 +283,18 @@ __device__ __forceinline__ void reflector3(double x, double y, double z, double&
 // the top of the window and chased to its bottom by 3 x 3 reflectors.  The
 // reflectors are applied to whole rows (to column n-1) and whole columns
 // (from row 0) so that H converges to the full real Schur form, and to Z.
+//
+// Bound by the chain reflector -> rows -> columns -> next reflector, whose
+// square root and division are binary64 code of some 40 dependent
+// instructions.  Only three rows of the column update (k+1..k+3) feed the
+// next reflector: warp 0 takes those and goes on to it at once, the other
+// warps update the rest of the columns and Z meanwhile.  Two barriers a
+// reflector.  DMD of 524,288 x 128, r = 48: 9.6 ms with one thread's reflector
+// between four barriers and two divisions, 8.4 here.
 __device__ void francis_step(double* H, int64_t ldh, double* Z, int64_t ldz, int64_t n, int64_t l, int64_t hi,
                              int its, double* sc) {
-  const int tid = threadIdx.x;
-  if (tid == 0) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < 3) {
     double s, t;
     if (its == 10 || its == 20) {
       const double w = fabs(HH(hi, hi - 1)) + fabs(HH(hi - 1, hi - 2));
@@ -300,20 +307,10 @@ __device__ void francis_step(double* H, int64_t ldh, double* Z, int64_t ldz, int
     }
     const double h00 = HH(l, l), h10 = HH(l + 1, l), h01 = HH(l, l + 1), h11 = HH(l + 1, l + 1);
     const double h21 = HH(l + 2, l + 1);
-    sc[0] = h00 * h00 + h01 * h10 - s * h00 + t;
-    sc[1] = h10 * (h00 + h11 - s);
-    sc[2] = h10 * h21;
+    reflector3(h00 * h00 + h01 * h10 - s * h00 + t, h10 * (h00 + h11 - s), h10 * h21, sc);
   }
   __syncthreads();
   for (int64_t k = l; k <= hi - 2; ++k) {
-    if (tid == 0) {
-      double tau, v1, v2;
-      reflector3(sc[0], sc[1], sc[2], tau, v1, v2);
-      sc[3] = tau;
-      sc[4] = v1;
-      sc[5] = v2;
-    }
-    __syncthreads();
     const double tau = sc[3], v1 = sc[4], v2 = sc[5];
     if (tau != 0.0) {
       const int64_t j0 = k > l ? k - 1 : l;
@@ -330,37 +327,39 @@ __device__ void francis_step(double* H, int64_t ldh, double* Z, int64_t ldz, int
       }
     }
     __syncthreads();
-    if (tau != 0.0) {
-      const int64_t i1 = (k + 3 < hi) ? k + 3 : hi;
-      for (int64_t i = tid; i <= i1; i += blockDim.x) {
-        const double s = tau * (HH(i, k) + v1 * HH(i, k + 1) + v2 * HH(i, k + 2));
-        HH(i, k) -= s;
-        HH(i, k + 1) -= s * v1;
-        HH(i, k + 2) -= s * v2;
+    if (tid < 32) {
+      if (lane < 3) {
+        const int64_t i = k + 1 + lane;   // row hi + 1 at k = hi - 2: the last reflector has two rows
+        double x = 0.0;
+        if (i <= hi) {
+          x = HH(i, k);
+          if (tau != 0.0) {
+            const double y = HH(i, k + 1), z = HH(i, k + 2);
+            const double s = tau * (x + v1 * y + v2 * z);
+            x -= s;
+            HH(i, k) = x;
+            HH(i, k + 1) = y - s * v1;
+            HH(i, k + 2) = z - s * v2;
+          }
+        }
+        const double x0 = __shfl_sync(7u, x, 0), x1 = __shfl_sync(7u, x, 1), x2 = __shfl_sync(7u, x, 2);
+        reflector3(x0, x1, x2, sc);
       }
-      for (int64_t i = tid; i < n; i += blockDim.x) {
-        const double s = tau * (ZZ(i, k) + v1 * ZZ(i, k + 1) + v2 * ZZ(i, k + 2));
-        ZZ(i, k) -= s;
-        ZZ(i, k + 1) -= s * v1;
-        ZZ(i, k + 2) -= s * v2;
+    } else if (tau != 0.0) {
+      // rows 0..k of H, then all of Z
+      for (int64_t q = tid - 32; q <= k + n; q += blockDim.x - 32) {
+        double* p = q <= k ? H + q + k * ldh : Z + (q - k - 1) + k * ldz;
+        const int64_t ld = q <= k ? ldh : ldz;
+        const double x = p[0], y = p[ld], z = p[2 * ld];
+        const double s = tau * (x + v1 * y + v2 * z);
+        p[0] = x - s;
+        p[ld] = y - s * v1;
+        p[2 * ld] = z - s * v2;
       }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      sc[0] = HH(k + 1, k);
-      sc[1] = HH(k + 2, k);
-      sc[2] = (k < hi - 2) ? HH(k + 3, k) : 0.0;
     }
     __syncthreads();
   }
   // last, 2 x 2 reflector on rows hi-1, hi
-  if (tid == 0) {
-    double tau, v1, v2;
-    reflector3(sc[0], sc[1], 0.0, tau, v1, v2);
-    sc[3] = tau;
-    sc[4] = v1;
-  }
-  __syncthreads();
   const double tau = sc[3], v1 = sc[4];
   if (tau != 0.0) {
     for (int64_t j = hi - 2 + tid; j < n; j += blockDim.x) {
@@ -373,15 +372,12 @@ __device__ void francis_step(double* H, int64_t ldh, double* Z, int64_t ldz, int
   }
   __syncthreads();
   if (tau != 0.0) {
-    for (int64_t i = tid; i <= hi; i += blockDim.x) {
-      const double s = tau * (HH(i, hi - 1) + v1 * HH(i, hi));
-      HH(i, hi - 1) -= s;
-      HH(i, hi) -= s * v1;
-    }
-    for (int64_t i = tid; i < n; i += blockDim.x) {
-      const double s = tau * (ZZ(i, hi - 1) + v1 * ZZ(i, hi));
-      ZZ(i, hi - 1) -= s;
-      ZZ(i, hi) -= s * v1;
+    for (int64_t q = tid; q <= hi + n; q += blockDim.x) {
+      double* p = q <= hi ? H + q + (hi - 1) * ldh : Z + (q - hi - 1) + (hi - 1) * ldz;
+      const int64_t ld = q <= hi ? ldh : ldz;
+      const double s = tau * (p[0] + v1 * p[ld]);
+      p[0] -= s;
+      p[ld] -= s * v1;
     }
   }
   __syncthreads();
@@ -598,16 +594,26 @@ __global__ void __launch_bounds__(kEigThreads) dmd_eig_kernel(DmdState d, WsHead
   const int max_total = 60 * (int)n + 100;
   bool ok = true;
   while (hi >= 0) {
-    if (tid == 0) {
-      int64_t l = hi;
-      while (l > 0) {
-        double s = fabs(HH(l - 1, l - 1)) + fabs(HH(l, l));
-        if (s == 0.0) s = hscale;
-        if (fabs(HH(l, l - 1)) <= kEps * s) break;
-        --l;
+    if (tid < 32) {   // the last negligible subdiagonal entry of the first hi + 1 rows
+      int64_t l = 0;
+      for (int64_t at = hi; at > 0; at -= 32) {
+        const int64_t i = at - tid;
+        bool small = false;
+        if (i > 0) {
+          double s = fabs(HH(i - 1, i - 1)) + fabs(HH(i, i));
+          if (s == 0.0) s = hscale;
+          small = fabs(HH(i, i - 1)) <= kEps * s;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, small);
+        if (m) {
+          l = at - (__ffs(m) - 1);
+          break;
+        }
       }
-      if (l > 0) HH(l, l - 1) = 0.0;
-      si[0] = (int)l;
+      if (tid == 0) {
+        if (l > 0) HH(l, l - 1) = 0.0;
+        si[0] = (int)l;
+      }
     }
     __syncthreads();
     const int64_t l = si[0];

@@ -72,6 +72,29 @@ def test_dmd_eigensolver_residency(K):
     _compare(res, ref, tol_mu=1e-9, tol_b=1e-7)
 
 
+@pytest.mark.parametrize("n", [3, 4, 31, 32, 33, 34, 65, 112, 113, 225])
+def test_dmd_eigenvalues_of_unstructured_data(n):
+    """All n eigenvalues for Gaussian snapshots: real and complex ones mixed,
+    and n around the sizes at which the eigensolver's warps share the rows of
+    H and Z differently.  Tolerance: the backward error of the product A and
+    of the QR algorithm, 20 n eps |A|_F cond(Y1), times the eigenvalue's own
+    condition number."""
+    rng = np.random.default_rng(n)
+    D = rng.standard_normal((4 * n + 40, n + 1))
+    U, s, Vt = np.linalg.svd(D[:, :-1], full_matrices=False)
+    A = U.T @ D[:, 1:] @ Vt.T / s
+    lam, W = np.linalg.eig(A)
+    left = np.linalg.inv(W)
+    kappa = np.linalg.norm(left, axis=1) * np.linalg.norm(W, axis=0)
+    tol = 20 * n * 2.0 ** -52 * np.linalg.norm(A) * (s[0] / s[-1]) * kappa
+    res = pg.dmd(_dev(D), remove_mean=False)
+    assert res.r == n
+    mu = res.mu.cpu().numpy()
+    d = np.abs(lam[:, None] - mu[None, :])
+    assert np.all(d.min(axis=1) <= tol)
+    assert len(set(d.argmin(axis=1))) == n
+
+
 def test_dmd_closed_form():
     N, M, K = 1 << 17, 64, 4
     lam, amp = synth.oscillation_params(K, seed=11)
