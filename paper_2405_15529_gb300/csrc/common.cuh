@@ -22,7 +22,8 @@ struct WsHeader {
   unsigned gram_y;          // pylom_pod: 1 when Y was left unfactored (the Gram route)
   unsigned rot[64];         // Jacobi: rotations performed in each sweep
   unsigned gram_redo;       // 1: the Gram route leaves this problem to the Householder route
-  unsigned char pad0[384 - 24 - 64 * 4 - 4];
+  unsigned svd_e;           // small SVD: largest exponent field of its matrix
+  unsigned char pad0[384 - 24 - 64 * 4 - 8];
   unsigned barrier_gen;     // grid barrier: generation (own line)
   unsigned char pad1[512 - 384 - 4];
 };

@@ -102,6 +102,23 @@ void jacobi32_carve(SvdState& s, char* p);
 cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int64_t ldr, const unsigned** open_pairs,
                                          cudaStream_t st);
 
+#ifdef __CUDACC__
+// The small SVD works on its matrix times the power of two that brings the
+// largest entry next to one (hdr->svd_e): squares stay in range at any scale.
+__device__ __forceinline__ int unit_field(int largest) { return 2046 - largest > 1 ? 2046 - largest : 1; }
+__device__ __forceinline__ int svd_scale_field(const SvdState& s) { return unit_field((int)s.hdr->svd_e); }
+__device__ __forceinline__ double svd_scale(const SvdState& s) { return __hiloint2double(svd_scale_field(s) << 20, 0); }
+
+// Whether one-sided Jacobi rotates a pair of columns with squared norms al, be
+// and dot product ga.  A direction that the other columns span (a matrix with
+// a zero row) shrinks by 2^-53 a sweep and would go on rotating as subnormals:
+// below kNullSquare, where squares are still exact, it counts as zero.
+constexpr double kNullSquare = 1e-250;
+__device__ __forceinline__ bool jacobi_open(double al, double be, double ga, double tol) {
+  return ga != 0.0 && fmin(al, be) >= kNullSquare && fabs(ga) > tol * sqrt(al) * sqrt(be);
+}
+#endif
+
 // with_y: include the N x M FP64 working copy (the FP64 path; the mixed
 // path keeps an FP32 copy in its own extra region instead)
 size_t tsqr_state_bytes(int64_t N, int64_t M, int64_t P, int64_t rmax, bool with_y = true);

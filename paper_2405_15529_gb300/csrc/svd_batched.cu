@@ -595,10 +595,24 @@ __device__ void bin_jacobi(const BatchArgs& a, const BinDesc& b, double2* sd, in
   double2* A = a.zbase + b.jac_off;        // Nb x Np
   double2* Vm = A + Nb * Np;               // Np x Np
   double2* UR = a.zbase + b.ur_off;        // Nb x Nb
+  // the power of two that brings R's largest entry next to one
+  int e = 0;
+  if (tid == 0) si[1] = 0;
+  __syncthreads();
+  for (int64_t idx = tid; idx < Nb * Nb; idx += blockDim.x) {
+    if (idx % Nb > idx / Nb) continue;
+    const double2 v = __ldcg(R + idx);
+    const int ex = (__double2hiint(v.x) >> 20) & 0x7ff, ey = (__double2hiint(v.y) >> 20) & 0x7ff;
+    e = max(e, max(ex == 0x7ff ? 0 : ex, ey == 0x7ff ? 0 : ey));
+  }
+  atomicMax(si + 1, e);
+  __syncthreads();
+  const int field = unit_field(si[1]);
+  const double sc = __hiloint2double(field << 20, 0);
   for (int64_t idx = tid; idx < Nb * Np; idx += blockDim.x) {
     const int64_t i = idx % Nb, j = idx / Nb;
     // A = R^H: A(i, j) = conj(R(j, i)); R is upper triangular; column Nb pads odd Nb
-    A[idx] = (j < Nb && j <= i) ? cconj(__ldcg(R + j + i * Nb)) : make_double2(0.0, 0.0);
+    A[idx] = (j < Nb && j <= i) ? cscale(cconj(__ldcg(R + j + i * Nb)), sc) : make_double2(0.0, 0.0);
   }
   for (int64_t idx = tid; idx < Np * Np; idx += blockDim.x)
     Vm[idx] = (idx % Np == idx / Np) ? make_double2(1.0, 0.0) : make_double2(0.0, 0.0);
@@ -632,7 +646,7 @@ __device__ void bin_jacobi(const BatchArgs& a, const BinDesc& b, double2* sd, in
         double2 eph = make_double2(0.0, 0.0);   // e^{-i phi}
         if (lane == 0) {
           const double g = sqrt(cabs2(ga));
-          if (g != 0.0 && g > tol * sqrt(al * be)) {
+          if (jacobi_open(al, be, g, tol)) {
             eph = cscale(cconj(ga), 1.0 / g);
             const double zeta = (be - al) / (2.0 * g);
             const double t = ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
@@ -675,7 +689,7 @@ __device__ void bin_jacobi(const BatchArgs& a, const BinDesc& b, double2* sd, in
     double s2 = 0.0;
     for (int64_t r = lane; r < Nb; r += 32) s2 += cabs2(A[r + j * Nb]);
     s2 = warp_sum(s2);
-    if (lane == 0) sig[j] = sqrt(s2);
+    if (lane == 0) sig[j] = s2 < kNullSquare ? 0.0 : sqrt(s2);
   }
   __syncthreads();
   for (int64_t j = tid; j < Nb; j += blockDim.x) {
@@ -706,7 +720,7 @@ __device__ void bin_jacobi(const BatchArgs& a, const BinDesc& b, double2* sd, in
     const double mag = sqrt(cabs2(vk));
     const double2 ph = (mag > 0.0) ? cscale(cconj(vk), 1.0 / mag) : make_double2(1.0, 0.0);
     for (int64_t r = lane; r < Nb; r += 32) UR[r + c * Nb] = cmul(Vm[r + j * Np], ph);
-    if (lane == 0) a.S[b.s_off + c] = sig[j];
+    if (lane == 0) a.S[b.s_off + c] = scalbn(sig[j], 1023 - field);
     if (b.kind != 0 && b.VT) {
       // real window: v_c = a_j ph / sigma_j is real (its largest entry is
       // real and positive); rows of exactly zero sigma are left zero

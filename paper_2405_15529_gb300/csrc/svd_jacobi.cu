@@ -41,12 +41,25 @@ void svd_state_carve(SvdState& s, char* base, int64_t M, bool precond) {
     jacobi32_carve(s, (char*)s.V + align256(sizeof(double) * (size_t)s.Mp * s.Mp));
 }
 
+__global__ void jacobi_scale_kernel(SvdState s, const double* R, int64_t ldr) {
+  int e = 0;
+  const int64_t M = s.M;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int f = (__double2hiint(R[idx % M + (idx / M) * ldr]) >> 20) & 0x7ff;
+    e = (f != 0x7ff && f > e) ? f : e;
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0 && e > 0) atomicMax(&s.hdr->svd_e, (unsigned)e);
+}
+
 __global__ void jacobi_init_kernel(SvdState s, const double* R, int64_t ldr) {
   const int64_t M = s.M, Mp = s.Mp;
+  const double sc = svd_scale(s);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * Mp; idx += stride) {
     const int64_t i = idx % M, j = idx / M;
-    s.A[idx] = (j < M) ? R[j + i * ldr] : 0.0;   // A = R^T
+    s.A[idx] = (j < M) ? sc * R[j + i * ldr] : 0.0;   // A = R^T
   }
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mp * Mp; idx += stride)
     s.V[idx] = (idx % Mp == idx / Mp) ? 1.0 : 0.0;
@@ -114,7 +127,7 @@ __global__ void __launch_bounds__(kJacThreads) jacobi_kernel(SvdState s, int max
           }
           const double alpha = tot[0], beta = tot[1], gamma = tot[2];
           sout[2] = 0.0;
-          if (gamma != 0.0 && fabs(gamma) > tol * sqrt(alpha * beta)) {
+          if (jacobi_open(alpha, beta, gamma, tol)) {
             const double zeta = (beta - alpha) / (2.0 * gamma);
             const double t = ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
             const double c = 1.0 / sqrt(1.0 + t * t);
@@ -246,7 +259,7 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
       a += x * x;
     }
     a = warp_sum(a);
-    if (lane == 0) sig[j] = sqrt(a);
+    if (lane == 0) sig[j] = a < kNullSquare ? 0.0 : sqrt(a);
   }
   __syncthreads();
   // NaN (from non-finite input) sorts last as key -1, so ranks stay a
@@ -268,7 +281,8 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
     U[i + c * ldu] = s.V[i + j * Mp];
     VT[c + i * ldvt] = (sj > 0.0) ? s.A[i + j * M] / sj : 0.0;
   }
-  for (int64_t c = tid; c < M; c += nthr) S[c] = sig[perm[c]];
+  const int up = 1023 - svd_scale_field(s);
+  for (int64_t c = tid; c < M; c += nthr) S[c] = scalbn(sig[perm[c]], up);
   __syncthreads();
   complete_right_vectors(S, M, VT, ldvt, sred, sout);
   __syncthreads();
@@ -295,7 +309,10 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
       VT[c + i * ldvt] = -VT[c + i * ldvt];
     }
   }
-  if (tid == 0) s.hdr->r = energy_rank(S, M, energy, r_max);
+  __syncthreads();
+  for (int64_t c = tid; c < M; c += nthr) sgn[c] = sig[perm[c]];   // (the signs are applied)
+  __syncthreads();
+  if (tid == 0) s.hdr->r = energy_rank(sgn, M, energy, r_max);
 }
 
 // The same outputs over the whole chip, when the preconditioning's scratch is
@@ -326,7 +343,7 @@ __global__ void svd_norms_kernel(SvdState s) {
     }
   }
   if (lane == 0) {
-    s.T[0][j] = sqrt(a);
+    s.T[0][j] = a < kNullSquare ? 0.0 : sqrt(a);
     s.T[0][M + j] = s.A[kb + j * M] < 0.0 ? -1.0 : 1.0;
   }
 }
@@ -335,6 +352,7 @@ __global__ void __launch_bounds__(kFinThreads) svd_order_kernel(SvdState s, doub
   __shared__ double sS[4096];   // M <= 4096 at every entry point
   const int64_t M = s.M;
   const double* sig = s.T[0];
+  const int up = 1023 - svd_scale_field(s);
   for (int64_t j = threadIdx.x; j < M; j += blockDim.x) {
     const double sj = (sig[j] == sig[j]) ? sig[j] : -1.0;   // NaN last
     int rank = 0;
@@ -343,7 +361,7 @@ __global__ void __launch_bounds__(kFinThreads) svd_order_kernel(SvdState s, doub
       rank += (sq > sj) || (sq == sj && q < j);
     }
     s.big[rank] = (int)j;
-    S[rank] = sig[j];
+    S[rank] = scalbn(sig[j], up);
     sS[rank] = sig[j];
   }
   __syncthreads();
@@ -399,6 +417,8 @@ cudaError_t launch_svd_fp64(const SvdState& s, const double* R, int64_t ldr, dou
   cudaError_t e;
   // a caller who allows only a few sweeps sees whether those converge
   const unsigned* open_pairs = nullptr;
+  jacobi_scale_kernel<<<s.M <= 64 ? 16 : s.M <= 256 ? 128 : 304, 256, 0, st>>>(s, R, ldr);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (s.A32 && max_sweeps >= 8) {
     e = launch_jacobi32_precondition(s, R, ldr, &open_pairs, st);
   } else {

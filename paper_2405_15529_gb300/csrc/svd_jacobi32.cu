@@ -46,33 +46,25 @@ constexpr int kJRows = 64;             // rows of the staged tile
 constexpr int kJ32MaxSweeps = 24;
 constexpr int kJClusterMax = 8;        // up to 8 blocks run as one cluster (cheaper barrier)
 // words of s.rot32: rotations of each sweep of the two stages, then
-constexpr int kJScale = 2 * kJ32MaxSweeps;       // largest exponent field of R
 constexpr int kJSteps = 6;                       // binary64 steps of simultaneous rotations
 constexpr int kJManyColumns = 128;               // from here on all of them
-constexpr int kJOpen = kJScale + 1;              // kJSteps + 1 words: pairs not converged at each check; then: entries of V^T V off
+constexpr int kJOpen = 2 * kJ32MaxSweeps;        // kJSteps + 1 words: pairs not converged at each check; then: entries of V^T V off
 constexpr int kJWords = kJOpen + kJSteps + 2;
 
-__global__ void jacobi32_scale_kernel(SvdState s, const double* R, int64_t ldr) {
-  int e = 0;
-  const int64_t M = s.M;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int f = (__double2hiint(R[idx % M + (idx / M) * ldr]) >> 20) & 0x7ff;
-    e = (f != 0x7ff && f > e) ? f : e;
-  }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0 && e > 0) atomicMax(s.rot32 + kJScale, (unsigned)e);
-}
-
-// A32 = 2^-e src^T or 2^-e src (binary32, zero padding columns), V32 = I
-__global__ void jacobi32_init_kernel(SvdState s, const double* src, int64_t ld, int trans) {
+// A32 = A (M x Mp), binary32, zero padding columns; V32 = I.  First A = R^T,
+// scaled (R given).
+__global__ void jacobi32_init_kernel(SvdState s, double* A, const double* R, int64_t ldr) {
   const int64_t M = s.M, Mb = s.Mb;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int e = 1023 - (int)s.rot32[kJScale];
-  const double sc = __hiloint2double((e < -1021 ? 1 : e > 1023 ? 2046 : e + 1023) << 20, 0);
+  const double sc = svd_scale(s);
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * Mb; idx += stride) {
     const int64_t i = idx % M, j = idx / M;
-    s.A32[idx] = (j < M) ? (float)(sc * (trans ? src[j + i * ld] : src[i + j * ld])) : 0.f;
+    double x = 0.0;
+    if (j < M) {
+      if (R) A[idx] = sc * R[j + i * ldr];
+      x = A[idx];
+    }
+    s.A32[idx] = (float)x;
   }
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mb * Mb; idx += stride)
     s.V32[idx] = (idx % Mb == idx / Mb) ? 1.f : 0.f;
@@ -414,9 +406,6 @@ constexpr double kSmallAngle = 0.02;
 __device__ __forceinline__ bool small_angle(bool open, double t, double M) {
   return open ? fabs(t) <= kSmallAngle : fabs(t) * M <= 1e-3;
 }
-__device__ __forceinline__ bool pair_open(double al, double be, double ga, double tol) {
-  return ga != 0.0 && fabs(ga) > tol * sqrt(al * be);
-}
 
 // Check `c` on G: counts the pairs that the binary64 sweeps would rotate
 // (open[c]), and leaves for each column the partner of its largest angle if
@@ -439,7 +428,7 @@ __global__ void jacobi_check_kernel(SvdState s, const double* G, const double* W
     if (W) nw += !(fabs(W[i + j * Mp] - (i == j ? 1.0 : 0.0)) <= wtol);
     if (i == j) continue;
     const double al = G[i + i * Mp], ga = G[i + j * Mp];
-    const bool open = pair_open(al, be, ga, tol);
+    const bool open = jacobi_open(al, be, ga, tol);
     n += open && i < j;
     const double t = fabs(pair_tangent(al, be, ga));
     if (open && t > best) {
@@ -513,7 +502,7 @@ __global__ void jacobi_angles_kernel(SvdState s, const double* G, const double* 
   auto angle = [&](const Col& p, const Col& q) {
     if (p.at == q.at || p.b == q.at || !p.act || !q.act) return 0.0;
     const double ga = rotated(G, p, q), t = pair_tangent(p.d, q.d, ga);
-    return small_angle(pair_open(p.d, q.d, ga, tol), t, (double)s.M) ? t : 0.0;
+    return small_angle(jacobi_open(p.d, q.d, ga, tol), t, (double)s.M) ? t : 0.0;
   };
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < Mp * Mp;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -535,11 +524,12 @@ __global__ void jacobi_angles_kernel(SvdState s, const double* G, const double* 
 __global__ void jacobi_restart_kernel(SvdState s, const double* R, int64_t ldr, const unsigned* bad, unsigned* open) {
   if (*bad == 0) return;
   const int64_t M = s.M, Mp = s.Mp, na = M * Mp, nv = Mp * Mp;
+  const double sc = svd_scale(s);
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < na + nv;
        idx += (int64_t)gridDim.x * blockDim.x) {
     if (idx < na) {
       const int64_t i = idx % M, j = idx / M;
-      s.A[idx] = (j < M) ? R[j + i * ldr] : 0.0;
+      s.A[idx] = (j < M) ? sc * R[j + i * ldr] : 0.0;
     } else {
       const int64_t v = idx - na;
       s.V[v] = (v % Mp == v / Mp) ? 1.0 : 0.0;
@@ -625,16 +615,15 @@ cudaError_t launch_jacobi32_precondition(const SvdState& s, const double* R, int
   auto two = [&](const SmallGemm& g, const SmallGemm& h, const unsigned* skip = nullptr) {
     if (e == cudaSuccess) e = small_gemms(SmallGemms{{g, h}, skip}, 2, st);
   };
-  jacobi32_scale_kernel<<<gr, 256, 0, st>>>(s, R, ldr);
-  jacobi32_init_kernel<<<gr, 256, 0, st>>>(s, R, ldr, 1);
+  jacobi32_init_kernel<<<gr, 256, 0, st>>>(s, s.A, R, ldr);
   if ((e = cudaGetLastError()) != cudaSuccess || (e = stage32(s, 0, st)) != cudaSuccess) return e;
   jacobi32_widen_kernel<<<gr, 256, 0, st>>>(s, T0);
   e = cudaGetLastError();
   one(mm(1, Mp, Mp, 1.0, T0, Mp, T0, 0.0, nullptr, T1));                             // V^T V
   one(mm(0, Mp, Mp, -0.5, T0, Mp, T1, 1.5, T0, T3));                                 // V <- 1.5 V - 0.5 V V^T V
-  one(SmallGemm{1, M, Mp, M, R, ldr, T3, Mp, 1.0, 0.0, nullptr, s.A2});              // A = R^T V (rows of V past M meet no row of R)
+  one(SmallGemm{0, M, Mp, M, s.A, M, T3, Mp, 1.0, 0.0, nullptr, s.A2});              // A = R^T V (rows of V past M meet no row of R)
   if (e != cudaSuccess) return e;
-  jacobi32_init_kernel<<<gr, 256, 0, st>>>(s, s.A2, M, 0);
+  jacobi32_init_kernel<<<gr, 256, 0, st>>>(s, s.A2, nullptr, 0);
   if ((e = cudaGetLastError()) != cudaSuccess || (e = stage32(s, 1, st)) != cudaSuccess) return e;
   jacobi32_widen_kernel<<<gr, 256, 0, st>>>(s, T0);
   e = cudaGetLastError();
