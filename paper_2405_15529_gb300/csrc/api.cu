@@ -276,14 +276,16 @@ extern "C" pylom_status pylom_pod(const void* X, int64_t N, int64_t M, int64_t l
   if (gram) {
     if (route == kGramChecked && (e = launch_gram_check(gs, S, st)) != cudaSuccess)
       return cuda_fail(e, "pylom_pod: modes");
-    e = launch_modes_direct(gs, nullptr, S, VT, ldvt, w, mode_kind == PYLOM_MODES_PHYSICAL, U, ldu, r_out, st,
-                            prof ? g_prof.at(call, 4) : nullptr);
+    e = launch_modes_direct(gs, nullptr, S, VT, ldvt, w, mode_kind == PYLOM_MODES_PHYSICAL, U, ldu, r_out,
+                            route == kGramChecked ? &hdr->gram_redo : nullptr, st, prof ? g_prof.at(call, 4) : nullptr);
     if (route == kGramChecked) {
       ts.run_if = &hdr->gram_redo;
       if (e == cudaSuccess)
         e = mixed ? launch_tsqr_mixed(ts, extra, X, ldx, xtype, w, remove_mean, mean, st)
                   : launch_tsqr_fp64(ts, X, ldx, xtype, w, remove_mean, mean, st);
-      if (e == cudaSuccess) e = launch_sign_ur(ts, UR, st);
+      // U_R for that Q, which is not the Cholesky factor's; the integer sums are done with
+      static_assert(sizeof(long long) == sizeof(double), "frame_doubles fit in the Gram sums");
+      if (e == cudaSuccess) e = launch_frame(ts, S, VT, ldvt, nullptr, (double*)gs.G, UR, st);
       if (e == cudaSuccess)
         e = mixed ? launch_modes_mixed(ts, extra, UR, M, -1, w, mode_kind == PYLOM_MODES_PHYSICAL, (float*)U, ldu,
                                        r_out, st, nullptr)

@@ -1061,7 +1061,7 @@ extern "C" pylom_status pylom_dmd(const void* X, int64_t N, int64_t M, int64_t l
   dmd_pack_kernel<<<grid_for(M * r_max, kSmallThreads), kSmallThreads, 0, st>>>(d, hdr);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail("small DMD kernels");
   if (gram) {
-    if ((e = launch_modes_direct(gs, d.Bp, nullptr, nullptr, 0, nullptr, 0, Phi, ldphi, r_out, st, nullptr)) !=
+    if ((e = launch_modes_direct(gs, d.Bp, nullptr, nullptr, 0, nullptr, 0, Phi, ldphi, r_out, nullptr, st, nullptr)) !=
         cudaSuccess)
       return fail("modes");
     return PYLOM_OK;

@@ -57,10 +57,11 @@ cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xt
                           int remove_mean, double* mean, double* R, cudaStream_t st, cudaEvent_t mid);
 
 // U (N x r) = Y C: C (M x rmax, ld M) given, or (C null) V_r S_r^-1 from VT and S.
-// r is read from hdr->r.  U is binary64, or binary32 for a binary32 Y.
+// r is read from hdr->r.  U is binary64, or binary32 for a binary32 Y.  unless
+// (nullable): nothing is done when *unless is not 0.
 cudaError_t launch_modes_direct(const GramState& g, const double* C, const double* S, const double* VT, int64_t ldvt,
                                 const double* w, int physical, void* U, int64_t ldu, int64_t* r_out,
-                                cudaStream_t st, cudaEvent_t mid);
+                                const unsigned* unless, cudaStream_t st, cudaEvent_t mid);
 
 // Binary64 columns -> fixed-point words in place (rows of zeros up to ldy), and Y
 // of a forward back to binary64 where *redo is set.
@@ -94,8 +95,5 @@ cudaError_t launch_bw_finalize_gram(const void* dY, bool f32, const double* w, i
 // S known): else hdr->gram_redo = 1 and hdr->gram_y = 0, and the Householder
 // route on `ts` (ts.run_if = &hdr->gram_redo) gives the modes.
 cudaError_t launch_gram_check(const GramState& g, const double* S, cudaStream_t st);
-// The rows of U_R with the signs of the Householder R's diagonal (the Gram
-// route's R has a non-negative one), for the Householder route after a redo.
-cudaError_t launch_sign_ur(const TsqrState& ts, double* UR, cudaStream_t st);
 
 }  // namespace pylom

@@ -161,6 +161,12 @@ cudaError_t launch_modes_fp64(const TsqrState& s, const double* Ur, int64_t ldur
                               const double* w, int physical, double* U, int64_t ldu,
                               int64_t* r_out, cudaStream_t st, cudaEvent_t mid = nullptr);
 
+// U_R for the Q and R of `s` from a call's S and V (frame.cu); where *s.gram_y is
+// 0, UR itself.  scratch: frame_doubles(M) doubles; Q: M x M.  Obeys s.run_if.
+size_t frame_doubles(int64_t M);
+cudaError_t launch_frame(const TsqrState& s, const double* S, const double* VT, int64_t ldvt, const double* UR,
+                         double* scratch, double* Q, cudaStream_t st);
+
 // Adjoint of the POD path (pod_backward.cu).  fs: the forward's TSQR state
 // (reflectors, T, tree); UR/S/VT: the forward's small-SVD factors.
 size_t pod_backward_bytes(int64_t N, int64_t M, int64_t P, int64_t r);

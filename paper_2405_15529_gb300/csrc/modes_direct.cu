@@ -170,21 +170,6 @@ cudaError_t launch_gram_check(const GramState& g, const double* S, cudaStream_t 
   return cudaGetLastError();
 }
 
-__global__ void sign_ur_kernel(TsqrState s, double* UR) {
-  if (passed_over(s)) return;
-  const int64_t M = s.M;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = idx % M;
-    if (s.Rs[i + i * M] < 0.0) UR[idx] = -UR[idx];
-  }
-}
-
-cudaError_t launch_sign_ur(const TsqrState& ts, double* UR, cudaStream_t st) {
-  sign_ur_kernel<<<64, 256, 0, st>>>(ts, UR);
-  return cudaGetLastError();
-}
-
 template <typename TY, int G>
 static cudaError_t run_shape(const ProductArgs& p, const double* S0, const double* w, int physical, void* U, int64_t ldu,
                              int64_t* r_out, WsHeader* hdr, cudaStream_t st, cudaEvent_t mid) {
@@ -229,8 +214,9 @@ cudaError_t launch_product(const ProductArgs& p, bool f32, void* U, int64_t ldu,
 
 cudaError_t launch_modes_direct(const GramState& g, const double* C, const double* S, const double* VT, int64_t ldvt,
                                 const double* w, int physical, void* U, int64_t ldu, int64_t* r_out,
-                                cudaStream_t st, cudaEvent_t mid) {
+                                const unsigned* unless, cudaStream_t st, cudaEvent_t mid) {
   ProductArgs p{};
+  p.unless = unless;
   p.Y = g.Y;
   p.ldy = g.ldy;
   p.N = g.N;
