@@ -179,8 +179,10 @@ static size_t pod_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, int prec
 // that by sqrt(M / 1e-4) (the share left out is at least that, so the last
 // kept value is no smaller than its mean).  With r_max < M columns asked for
 // instead, the device looks at sigma_r and has the Householder route done
-// behind it where it is too small (about 15 launches that return at once
-// otherwise, 25 us).  All modes, where sigma_M is usually at the rounding
+// behind it where it is too small (about 17 launches that return at once
+// otherwise, 35 us; a call that falls back pays for the Gram route too, and
+// still takes no longer than leaves, tree and a plain Jacobi did: 4096 x 32
+// 2.9 ms against 3.7, 1048576 x 128, r_max 127, 112 against 116).  All modes, where sigma_M is usually at the rounding
 // level, a leaf height or a tree that the caller asks for take the
 // Householder TSQR directly.  Whole calls, Householder / Gram: 4096 x 32
 // 3.8 / 0.6 ms, 65537 x 63 10.0 / 1.1 ms, 1048576 x 128 (r_max 40) 79 / 6.5
@@ -424,8 +426,7 @@ extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_byt
     TsqrState os;
     fs.rmax = 0;
     double* UR2 = nullptr;
-    e = launch_refactor(fs, gs, extra, bws, (WsHeader*)ws, mixed, UR, os, &extra,
-                        &UR2, st);
+    e = launch_refactor(fs, gs, extra, bws, (WsHeader*)ws, mixed, UR, S, VT, ldvt, os, &extra, &UR2, st);
     if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward: factorisation");
     fs = os;
     UR = UR2;

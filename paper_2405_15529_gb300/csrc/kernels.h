@@ -182,7 +182,8 @@ void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r);
 size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed);
 struct GramState;
 cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
-                            const double* UR, TsqrState& os, char** extra, double** UR_out, cudaStream_t st);
+                            const double* UR, const double* S, const double* VT, int64_t ldvt, TsqrState& os,
+                            char** extra, double** UR_out, cudaStream_t st);
 // Mixed-precision adjoint support (tsqr_mixed.cu): per leaf C := Q_leaf^T C
 // (FP32, ld N) on tcgen05, top M rows into the binary64 slots Z.
 cudaError_t launch_leaf_qt_mixed(const TsqrState& s, char* extra, float* C, int64_t r, double* Z, cudaStream_t st);

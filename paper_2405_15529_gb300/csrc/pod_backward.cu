@@ -240,28 +240,16 @@ __global__ void __launch_bounds__(256) bw_add_du_c_f32_kernel(const float* C, co
   }
 }
 
-// U_R for the factorisation that the adjoint applies: the forward's own when
-// it factored Y, else its rows with the signs of the Householder R (R is
-// unique up to row signs; the Gram route's has a non-negative diagonal).
-__global__ void bw_signed_ur_kernel(TsqrState s, const double* UR, double* out) {
-  const int64_t M = s.M;
-  const bool same = already_factored(s);
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < M * M;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = idx % M;
-    out[idx] = (!same && s.Rs[i + i * M] < 0.0) ? -UR[idx] : UR[idx];
-  }
-}
-
 size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed) {
-  return align256(sizeof(double) * (size_t)M * M) + tsqr_state_bytes(N, M, P, r_max, !mixed) +
-         (mixed ? mixed_extra_bytes(N, M, P) : 0);
+  return align256(sizeof(double) * (size_t)M * M) + align256(sizeof(double) * frame_doubles(M)) +
+         tsqr_state_bytes(N, M, P, r_max, !mixed) + (mixed ? mixed_extra_bytes(N, M, P) : 0);
 }
 
 cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
-                            const double* UR, TsqrState& os, char** extra, double** UR_out, cudaStream_t st) {
-  const size_t ub = align256(sizeof(double) * (size_t)fs.M * fs.M);
-  char* own = base + ub;
+                            const double* UR, const double* S, const double* VT, int64_t ldvt, TsqrState& os,
+                            char** extra, double** UR_out, cudaStream_t st) {
+  double* scratch = (double*)(base + align256(sizeof(double) * (size_t)fs.M * fs.M));
+  char* own = (char*)scratch + align256(sizeof(double) * frame_doubles(fs.M));
   char* oextra = mixed ? own + tsqr_state_bytes(fs.N, fs.M, fs.P, fs.rmax, false) : nullptr;
   tsqr_state_carve(os, own, fs.N, fs.M, fs.P, fs.rmax, !mixed);
   os.hdr = hdr;
@@ -276,10 +264,9 @@ cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char*
   e = mixed ? launch_tsqr_mixed(os, oextra, fwd_extra, y_ld(fs.N), PYLOM_F32, nullptr, 0, nullptr, st)
             : launch_tsqr_fp64(os, os.Y, os.ldy, PYLOM_F64, nullptr, 0, nullptr, st);
   if (e != cudaSuccess) return e;
-  bw_signed_ur_kernel<<<64, 256, 0, st>>>(os, UR, (double*)base);
   *UR_out = (double*)base;
   *extra = oextra;
-  return cudaGetLastError();
+  return launch_frame(os, S, VT, ldvt, UR, scratch, *UR_out, st);
 }
 
 struct BwLayout {

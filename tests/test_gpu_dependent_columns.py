@@ -2,7 +2,8 @@
 twice, a run of nearly parallel ones) before independent ones, in calls that
 the device takes from the Gram route to the Householder route: the Cholesky
 factor and the Householder R of such a matrix differ by more than row signs.
-Modes against LAPACK column by column."""
+Modes against LAPACK column by column, the adjoint against the one of an
+explicit leaf height."""
 import numpy as np
 import pytest
 
@@ -67,3 +68,27 @@ def test_modes_after_the_fallback(N, M, kind, prec):
         assert np.linalg.norm(Ug[:, i] - U[:, i]) <= back / gap[i], i
     assert np.linalg.norm(Ug.T @ Ug - np.eye(M - 1), 2) <= M * eps
 
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("N,M", [(4096, 24), (6000, 150)])
+def test_adjoint_after_the_fallback(N, M, kind, prec):
+    """A cotangent on a small singular value sends the adjoint of a Gram
+    forward to a factorisation of its own."""
+    s = np.concatenate([2.0 ** -np.arange(8.0), 1e-6 * 0.9 ** np.arange(M - 9)])
+    X = _dev(_field(N, M, kind, 7 + M, s), torch.float32 if prec else torch.float64)
+    g = torch.Generator(device="cuda")
+    out = []
+    for b in (0, 1000):
+        f = pg.pod(X, remove_mean=False, energy=0.999, prec=prec, leaf_rows=b)
+        dU = torch.randn((f.r, N), dtype=torch.float64, device="cuda", generator=g.manual_seed(1)).t() / N ** 0.5
+        dS = torch.randn(M, dtype=torch.float64, device="cuda", generator=g.manual_seed(2))
+        dS[f.r:] = 0.0
+        dS[10] = 1e-6
+        out.append(pg.pod_backward(f, (N, M), None, False, 0, b, M, dU=dU, dS=dS))
+    # kept values are at least a factor of two apart (1/16 of the largest or
+    # more), so the cotangent moves by at most some 1e2 M eps; u_10 itself,
+    # uncertain in binary32, enters with 1e-6
+    eps = 2.0 ** -24 if prec else 2.0 ** -53
+    tol = 1e2 * M * eps + (1e-6 if prec else 1e-6 * M * eps / 1e-7)
+    assert torch.norm(out[0] - out[1]) <= tol * torch.norm(out[1])
