@@ -170,7 +170,7 @@ extern "C" pylom_status pylom_workspace_status(const void* ws, void* stream, int
 static size_t pod_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, int prec = PYLOM_PREC_FP64) {
   const bool mixed = prec == PYLOM_PREC_MIXED_3XTF32;
   return sizeof(WsHeader) + tsqr_state_bytes(N, M, P, r_max, !mixed) + svd_state_bytes(M) +
-         align256(sizeof(double) * (size_t)M * M) + (mixed ? mixed_extra_bytes(N, M, P) : 0) + gram_bytes(M, r_max);
+         align256(sizeof(double) * (size_t)M * M) + (mixed ? mixed_extra_bytes(N, M, P) : 0) + gram_bytes(N, M, r_max);
 }
 
 // Which route gives R and the modes.  The Gram route (gram.cu) needs no

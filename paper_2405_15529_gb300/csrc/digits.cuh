@@ -11,6 +11,10 @@
 //   binary64: 62 bits below the column's largest power of two, 8 digits;
 //             elements within 2^9 of the column maximum are exact.
 //   binary32: 38 bits, 5 digits.
+// Rows that are small in every column would keep few of those bits, so a row
+// has a shift (row_scale_kernel, gram.cu): how far its largest element lies
+// below its column's power of two.  The product Y C takes rows times 2^shift;
+// a sum over rows takes every row at its columns' scale.
 //
 // Layout of a digit plane in shared memory: K-major, no swizzle, core
 // matrices of 8 rows x 8 binary16 (128 contiguous bytes), kStK = 16 elements
@@ -68,6 +72,8 @@ template <typename TY> __host__ __device__ constexpr int fix_bias() { return siz
 // Exponent field that a column's scale is taken from, of one element: the
 // biased exponent, from a floor on (elements below it count as zero in
 // binary64; in binary32 the floor keeps the scale finite and loses nothing).
+// (A row's shift can take the scale of a column that lies below 2^-100
+// further down; what such a column has in that row counts for less.)
 constexpr int kMinField64 = 64, kMinField32 = 8;
 __device__ __forceinline__ int exp_field(double y) {
   const int e = (__double2hiint(y) >> 20) & 0x7ff;
@@ -111,6 +117,14 @@ __device__ __forceinline__ double from_fixed(uint2 w, int E) {
   const int64_t v = (int64_t)((((uint64_t)w.y << 32) | w.x) - kDigitBias64);
   return scalbn((double)v, E - fix_bias<double>());
 }
+// the word of the same value with its last `s` bits shifted out (rounded down)
+__device__ __forceinline__ uint2 shift_word(uint2 w, uint32_t s) {
+  return bias_digits((int64_t)((((uint64_t)w.y << 32) | w.x) - kDigitBias64) >> (s < 63u ? s : 63u));
+}
+// shift i of eight packed ones
+__device__ __forceinline__ uint32_t packed_shift(const uint4& s, int i) {
+  return (((const uint32_t*)&s)[i >> 1] >> (16 * (i & 1))) & 0xffffu;
+}
 __device__ __forceinline__ int64_t to_fixed(double y, int E) {
   const uint2 w = biased_fixed(y, E);
   return (int64_t)((((uint64_t)w.y << 32) | w.x) - kDigitBias64);
@@ -148,7 +162,7 @@ __device__ __forceinline__ void store_digits(const uint2 (&w)[8], unsigned char*
 }
 
 // What Y holds when the products run: binary32 as it is; binary64 as
-// biased fixed-point words (pack_kernel).  A word costs 6 byte selections and
+// biased fixed-point words (row_scale_kernel).  A word costs 6 byte selections and
 // 4 subtractions, a binary64 value 18 more operations of the half-rate
 // integer pipe, and the Gram kernel cuts every element about nine times (at
 // 256 columns); one pass over Y in place pays for that.
@@ -176,7 +190,7 @@ __device__ __forceinline__ void put_digits(const float (&y)[8], const int (&E)[8
   constexpr float kRound = 12582912.f;   // 1.5 2^23: adding it rounds to an integer
   float r[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) r[i] = y[i] * __int_as_float((132 - E[i] + 127) << 23);
+  for (int i = 0; i < 8; ++i) r[i] = y[i] * __int_as_float(min(132 - E[i] + 127, 254) << 23);   // (see kMinField32)
 #pragma unroll
   for (int s = S - 1; s >= 0; --s) {
     float d[8];

@@ -949,7 +949,7 @@ int grid_for(int64_t work, int threads) {
 
 size_t dmd_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max) {
   return sizeof(WsHeader) + tsqr_state_bytes(N, M, P, r_max, true) + svd_state_bytes(M - 1) +
-         dmd_small_bytes(M, r_max) + gram_bytes(M, r_max);
+         dmd_small_bytes(M, r_max) + gram_bytes(N, M, r_max);
 }
 
 }  // namespace

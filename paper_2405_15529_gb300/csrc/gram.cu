@@ -13,10 +13,10 @@
 // does at 1/60 of its binary32 rate.
 //
 // Measured (4,194,304 x 256, binary64): Householder leaves + tree 554 + 13
-// ms; here Y 8.6, cutting it 2.4, Gram matrix 25.8, Cholesky factor 0.74 ms.
-// 1,048,576 x 128: leaves + tree 39 + 3.8 ms; here 1.4, 0.3, 2.1 and 0.35.
-// Binary32 (mixed, 4,194,304 x 256): leaves + tree 57.7 + 8.8 ms; here 3.0,
-// 12.5 and 0.71 ms.
+// ms; here Y 8.6, cutting it 3.0, Gram matrix 26.3, Cholesky factor 0.74 ms.
+// 1,048,576 x 128: leaves + tree 39 + 3.8 ms; here 1.4, 0.4, 2.1 and 0.35.
+// Binary32 (mixed, 4,194,304 x 256): leaves + tree 57.7 + 8.8 ms; here Y 3.0,
+// row shifts 0.7, Gram matrix 12.5 and Cholesky factor 0.71 ms.
 #include <atomic>
 
 #include "digits.cuh"
@@ -205,51 +205,144 @@ struct GramArgs {
   const void* Z;
   int64_t NZ;
   const int* zE;
+  const uint16_t *rowS, *zS;
   const unsigned* unless;
   CUtensorMap mapA, mapB;   // Y in boxes of kStK rows x 128 columns; the right factor, x 64
 };
 
-// Binary64 columns -> biased fixed-point words in place, two rows a thread and
-// turn.  Bound by memory (16 bytes an element).
-constexpr int kPackThreads = 256, kPackRows = 2048;
-__global__ void __launch_bounds__(kPackThreads) pack_kernel(double* Y, int64_t ldy, int64_t cols, const int* colE,
-                                                            const unsigned* unless) {
+// Shift of each row: how many binary places its elements all lie below their
+// columns' largest exponents (0 for a row of zeros).  In sums over rows small
+// rows hardly count, but the modes of a row are made of that row alone, and a
+// reflector would keep them to its own rounding.
+//   binary32: the product Y C scales a row's elements by its shift.
+//   binary64: the elements become biased fixed-point words, in place.  Up to
+//     kRowShift places the words are at their columns' scale (still exact: they
+//     have 9 bits to spare) and the shift reads 0; rows further down are
+//     stored times 2^shift, and the Gram kernel shifts them back.
+// A block takes 32 V rows at a time, V = 16 bytes of a column a lane, warp v the
+// columns v, v + W, ..; the warps' maxima meet in shared memory.  Bound by
+// memory (4 and 16 bytes an element).  For the words binary64 elements are read
+// again, from the L2 cache, but for a warp's last eight columns, which are
+// still in registers.  4,194,304 x 256: binary64 3.0 ms (2.4 at one scale a
+// column, without shifts), binary32 0.68; the Gram kernel's look at the shifts
+// 0.5 of 26.3.
+constexpr int kRowShift = 3;
+template <typename T> struct RowVec;
+template <> struct RowVec<float> { typedef float4 type; };
+template <> struct RowVec<double> { typedef double2 type; };
+template <typename T, int W>
+__global__ void __launch_bounds__(32 * W, 1024 / (32 * W)) row_scale_kernel(T* Y, int64_t ldy, int M, const int* colE,
+                                                                             uint16_t* rowS, const unsigned* unless) {
+  typedef typename RowVec<T>::type Vec;
+  constexpr int V = 16 / sizeof(T), R = 32 * V, U = 8, kBits = sizeof(T) == 8 ? 20 : 23;   // mantissa bits of the upper word
+  constexpr int kFloor = sizeof(T) == 8 ? kMinField64 : kMinField32, kNone = -2147483647;
+  __shared__ int stop[2][W][R];      // (a warp may be an iteration ahead of the reads)
+  __shared__ int sshift[2][R];
   if (unless && *unless) return;
-  const int64_t r0 = (int64_t)blockIdx.x * kPackRows + 2 * threadIdx.x;
-  for (int64_t c = blockIdx.y; c < cols; c += gridDim.y) {
-    const int E = colE[c];
-    double* q = Y + c * ldy + r0;
-    double2 v[kPackRows / (2 * kPackThreads)];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t nblk = (ldy + R - 1) / R, step = (int64_t)W * ldy;
+  // first column of this warp's last chunk
+  const int last = warp < M ? warp + (M - 1 - warp) / (U * W) * (U * W) : warp;
+  int turn = 0;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x, turn ^= 1) {
+    const int64_t n0 = blk * R + lane * V;         // (ldy is a multiple of 8: a lane's rows exist together)
+    const int lim = n0 < ldy ? M : 0;
+    Vec x[U];
+    auto read = [&](int c0) {
+      const T* p = Y + n0 + c0 * ldy;
 #pragma unroll
-    for (int u = 0; u < kPackRows / (2 * kPackThreads); ++u)
-      if (r0 + 2 * u * kPackThreads < ldy) v[u] = *(const double2*)(q + 2 * u * kPackThreads);
+      for (int u = 0; u < U; ++u, p += step) x[u] = c0 + u * W < lim ? *(const Vec*)p : Vec{};
+    };
+    int top[V];
 #pragma unroll
-    for (int u = 0; u < kPackRows / (2 * kPackThreads); ++u)
-      if (r0 + 2 * u * kPackThreads < ldy) {
-        const uint2 a = biased_fixed(v[u].x, E), b = biased_fixed(v[u].y, E);
-        *(uint4*)(q + 2 * u * kPackThreads) = make_uint4(a.x, a.y, b.x, b.y);
+    for (int v = 0; v < V; ++v) top[v] = kNone;
+    for (int c0 = warp; c0 <= last; c0 += U * W) {
+      read(c0);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int E = c0 + u * W < M ? __ldg(colE + c0 + u * W) << kBits : 0;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          int hi;
+          if constexpr (sizeof(T) == 8) hi = __double2hiint(((const double*)&x[u])[v]);
+          else hi = __float_as_int(((const float*)&x[u])[v]);
+          hi &= sizeof(T) == 8 ? 0x7ff00000 : 0x7f800000;
+          if (hi > (kFloor << kBits)) top[v] = max(top[v], hi - E);
+        }
       }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) stop[turn][warp][lane * V + v] = top[v];
+    __syncthreads();
+    if (threadIdx.x < R) {
+      int t = kNone;
+#pragma unroll
+      for (int q = 0; q < W; ++q) t = max(t, stop[turn][q][threadIdx.x]);
+      int s = t == kNone ? 0 : -(t >> kBits);
+      if (sizeof(T) == 8 && s <= kRowShift) s = 0;
+      if (blk * R + threadIdx.x < ldy) rowS[blk * R + threadIdx.x] = (uint16_t)s;
+      sshift[turn][threadIdx.x] = s;
+    }
+    if constexpr (sizeof(T) == 8) {
+      __syncthreads();
+      int s[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) s[v] = sshift[turn][lane * V + v];
+      for (int c0 = last; c0 >= 0; c0 -= U * W) {
+        if (c0 != last) read(c0);
+        T* p = Y + n0 + c0 * ldy;
+#pragma unroll
+        for (int u = 0; u < U; ++u, p += step) {
+          if (c0 + u * W >= lim) break;
+          const int E = __ldg(colE + c0 + u * W);
+          uint2 w[V];
+          // (a column that lies lower still has only elements below the floor here)
+#pragma unroll
+          for (int v = 0; v < V; ++v)
+            w[v] = E - s[v] >= kFloor ? biased_fixed(((const double*)&x[u])[v], E - s[v]) : zero_cell<uint2>();
+          *(uint4*)p = make_uint4(w[0].x, w[0].y, w[V - 1].x, w[V - 1].y);
+        }
+      }
+    }
   }
 }
-cudaError_t launch_pack(double* Y, int64_t ldy, int64_t cols, const int* colE, const unsigned* unless, cudaStream_t st) {
-  const dim3 grid((unsigned)((ldy + kPackRows - 1) / kPackRows), (unsigned)(cols < 65535 ? cols : 65535));
-  pack_kernel<<<grid, kPackThreads, 0, st>>>(Y, ldy, cols, colE, unless);
+
+template <typename T>
+static cudaError_t row_scale(T* Y, int64_t ldy, int64_t M, const int* colE, uint16_t* rowS, const unsigned* unless, int sms,
+                             cudaStream_t st) {
+  constexpr int R = 32 * 16 / (int)sizeof(T);
+  const int64_t nblk = (ldy + R - 1) / R;
+  // eight warps up to 64 columns (eight columns in flight a warp), else sixteen
+  const int64_t cap = (int64_t)sms * (M <= 64 ? 4 : 2);
+  const unsigned grid = (unsigned)(nblk < cap ? nblk : cap);
+  if (M <= 64) row_scale_kernel<T, 8><<<grid, 256, 0, st>>>(Y, ldy, (int)M, colE, rowS, unless);
+  else row_scale_kernel<T, 16><<<grid, 512, 0, st>>>(Y, ldy, (int)M, colE, rowS, unless);
   return cudaGetLastError();
+}
+cudaError_t launch_row_scale(void* Y, bool f32, int64_t ldy, int64_t cols, const int* colE, uint16_t* rowS,
+                             const unsigned* unless, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  return f32 ? row_scale<float>((float*)Y, ldy, cols, colE, rowS, unless, sms, st)
+             : row_scale<double>((double*)Y, ldy, cols, colE, rowS, unless, sms, st);
 }
 
 // Back to binary64 (to another buffer), for a Householder factorisation of
 // this Y; rows past N are not written.
 __global__ void __launch_bounds__(256) unpack_kernel(const double* P, int64_t ldy, int64_t N, int64_t M, const int* colE,
-                                                     double* Y, const unsigned* gram_y, const unsigned* redo) {
+                                                     const uint16_t* rowS, double* Y, const unsigned* gram_y, const unsigned* redo) {
   if (*gram_y == 0 || *redo == 0) return;
   for (int64_t c = blockIdx.y; c < M; c += gridDim.y)
     for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
-      Y[n + c * ldy] = from_fixed(*(const uint2*)(P + n + c * ldy), colE[c]);
+      Y[n + c * ldy] = from_fixed(*(const uint2*)(P + n + c * ldy), colE[c] - rowS[n]);
 }
 cudaError_t launch_unpack(const GramState& g, double* Y, const unsigned* redo, cudaStream_t st) {
   const int64_t bx = (g.N + 255) / 256;
   const dim3 grid((unsigned)(bx < 64 ? bx : 64), (unsigned)(g.M < 65535 ? g.M : 65535));
-  unpack_kernel<<<grid, 256, 0, st>>>((const double*)g.Y, g.ldy, g.N, g.M, g.colE, Y, &g.hdr->gram_y, redo);
+  unpack_kernel<<<grid, 256, 0, st>>>((const double*)g.Y, g.ldy, g.N, g.M, g.colE, g.rowS, Y, &g.hdr->gram_y,
+                                      redo);
   return cudaGetLastError();
 }
 
@@ -293,12 +386,19 @@ __global__ void __launch_bounds__(Shape<2>::THREADS, 1) gram_kernel(const __grid
   const int jA = colA < a.M ? (int)((a.ldy - row0 - kg * 8 + kStK - 1) / kStK) : 0;
   const int jB = colB < nB ? (int)((a.ldy - row0 - kb * 8 + kStK - 1) / kStK) : 0;
   unsigned char* raw = gsm + NST * kStage;
+  // binary64: behind the ring, the shifts of a stage's rows of Y, then of Z
+  uint16_t* shifts = (uint16_t*)(raw + kRaw * kRawStage);
   if (tid == 0)
     for (int q = 0; q < kRaw; ++q) tc05::mbar_init(raw_full + q, 1);
   auto copy = [&](int j) {
     unsigned char* r = raw + (j % kRaw) * kRawStage;
     uint64_t* m = raw_full + j % kRaw;
-    tc05::mbar_arrive_expect_tx(m, diag ? kRawA : kRawStage);
+    constexpr int kShift = sizeof(TY) == 8 ? 2 * kStK : 0;     // bytes
+    tc05::mbar_arrive_expect_tx(m, (diag ? kRawA : kRawStage) + (a.Z ? 2 : 1) * kShift);
+    if constexpr (sizeof(TY) == 8) {
+      bulk_load(shifts + (j % kRaw) * 2 * kStK, a.rowS + row0 + j * kStK, kShift, m);
+      if (a.Z) bulk_load(shifts + ((j % kRaw) * 2 + 1) * kStK, a.zS + row0 + j * kStK, kShift, m);
+    }
     tc05::tma_load_2d(r, &a.mapA, row0 + j * kStK, I * 128, m);
     if (!diag) tc05::tma_load_2d(r + kRawA, &a.mapB, row0 + j * kStK, J * 64, m);
   };
@@ -317,14 +417,28 @@ __global__ void __launch_bounds__(Shape<2>::THREADS, 1) gram_kernel(const __grid
       for (int i = 0; i < 8; ++i) y[i] = zero_cell<C>();
     }
   };
+  // small rows at their columns' scale (eight rows, the same for a whole warp)
+  auto unshift8 = [&](int j, int z, int k8, C (&y)[8]) {
+    if constexpr (sizeof(TY) == 8) {
+      const uint4 s = *(const uint4*)(shifts + ((j % kRaw) * 2 + z) * kStK + k8 * 8);
+      if (s.x | s.y | s.z | s.w) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = shift_word(y[i], packed_shift(s, i));
+      }
+    }
+  };
   __align__(16) C yA[8], yB[8];
   bool withB = false;
   auto fetch = [&](int j) {
     if (!__all_sync(0xffffffffu, mbar_wait_fast(raw_full + j % kRaw, (uint32_t)((j / kRaw) & 1)))) return false;
     const unsigned char* r = raw + (j % kRaw) * kRawStage;
     read8(r, ca, kg, j < jA, yA);
+    unshift8(j, 0, kg, yA);
     withB = !diag && ((j >> 1) & 1) == quad;
-    if (withB) read8(r + kRawA, cb, kb, j < jB, yB);
+    if (withB) {
+      read8(r + kRawA, cb, kb, j < jB, yB);
+      unshift8(j, a.Z ? 1 : 0, kb, yB);
+    }
     return true;
   };
   const int oa = (ca >> 3) * kPlaneSbo + (ca & 7) * 16 + kg * 128;
@@ -572,8 +686,11 @@ __global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
 // host side
 // ---------------------------------------------------------------------------
 
-size_t gram_bytes(int64_t M, int64_t rmax) {
-  return align256(sizeof(int) * (size_t)M) + align256(sizeof(long long) * (size_t)5 * M * M) +
+// (rows past N are read, and belong to no element)
+size_t row_shift_bytes(int64_t N) { return align256(sizeof(uint16_t) * (size_t)((N + 127) / 128 * 128)); }
+
+size_t gram_bytes(int64_t N, int64_t M, int64_t rmax) {
+  return row_shift_bytes(N) + align256(sizeof(int) * (size_t)M) + align256(sizeof(long long) * (size_t)5 * M * M) +
          2 * align256(sizeof(double) * (size_t)M * M) + 2 * align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M) +
          product_planes_bytes(M, 0, rmax);
 }
@@ -590,7 +707,8 @@ void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax) {
   g.Th = (double*)p;         p += align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M);
   g.Tl = (double*)p;         p += align256(sizeof(double) * (size_t)(2 * kNBC + 1) * M);
   g.Cd = (unsigned char*)p;  p += align256((size_t)kt * js * 8 * Shape<2>::PLANEB);
-  g.Ce = (int*)p;
+  g.Ce = (int*)p;            p += align256(sizeof(int) * (size_t)kt * 64);
+  g.rowS = (uint16_t*)p;
 }
 
 template <typename TX, typename TY>
@@ -629,9 +747,10 @@ constexpr int64_t kGramRows = 1ll << 30;
 
 template <typename TY>
 static cudaError_t gram_launch(const GramState& g, int sms, const void* Z, int64_t ldz, int64_t NZ, const int* zE,
-                               long long* G, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
+                               const uint16_t* zS, long long* G, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
   constexpr int S = Dig<TY>::S;
-  constexpr size_t smem = (size_t)Dig<TY>::template NST<2> * S * (kPlaneA + Shape<2>::PLANEB) + (size_t)kRaw * 192 * kStK * sizeof(TY);
+  constexpr size_t smem = (size_t)Dig<TY>::template NST<2> * S * (kPlaneA + Shape<2>::PLANEB) + (size_t)kRaw * 192 * kStK * sizeof(TY) +
+                          (sizeof(TY) == 8 ? kRaw * 4 * kStK : 0);
   cudaError_t e = ensure_dyn_smem((const void*)gram_kernel<TY>, smem);
   if (e != cudaSuccess) return e;
   const int nJ = (int)(((Z ? NZ : g.M) + 63) / 64), nI = (int)((g.M + 127) / 128);
@@ -651,6 +770,8 @@ static cudaError_t gram_launch(const GramState& g, int sms, const void* Z, int64
     a.Z = Z;
     a.NZ = NZ;
     a.zE = zE;
+    a.rowS = g.rowS + r;
+    a.zS = Z ? zS + r : nullptr;
     a.unless = unless;
     a.splits = row_splits(a.items, (N + 127) / 128, sms);
     // words go as integers; 128 (64) bytes of a column, swizzled so that eight
@@ -678,8 +799,8 @@ __global__ void cross_sum_kernel(GramState g, int64_t NZ, const int* zE, const l
   }
 }
 
-cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, long long* G,
-                         double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
+cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, const uint16_t* zS,
+                         long long* G, double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st) {
   cudaError_t e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -687,8 +808,8 @@ cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t
   const int groups = g.f32 ? 3 : 5;
   e = cudaMemsetAsync(G, 0, sizeof(long long) * (size_t)groups * g.M * NZ, st);
   if (e != cudaSuccess) return e;
-  e = g.f32 ? gram_launch<float>(g, sms, Z, ldz, NZ, zE, G, unless, hdr, st)
-            : gram_launch<double>(g, sms, Z, ldz, NZ, zE, G, unless, hdr, st);
+  e = g.f32 ? gram_launch<float>(g, sms, Z, ldz, NZ, zE, zS, G, unless, hdr, st)
+            : gram_launch<double>(g, sms, Z, ldz, NZ, zE, zS, G, unless, hdr, st);
   if (e != cudaSuccess) return e;
   cross_sum_kernel<<<64, 256, 0, st>>>(g, NZ, zE, G, W, groups, g.f32 ? gram_base<float>(0) : 0,
                                        g.f32 ? fix_bias<float>() : fix_bias<double>());
@@ -709,9 +830,9 @@ cudaError_t launch_gram_r(const GramState& g, const void* X, int64_t ldx, int xt
   if (g.f32) e = xtype == PYLOM_F32 ? prologue<float, float>(pa, sms, st) : prologue<double, float>(pa, sms, st);
   else e = xtype == PYLOM_F32 ? prologue<float, double>(pa, sms, st) : prologue<double, double>(pa, sms, st);
   if (e != cudaSuccess) return e;
-  if (!g.f32 && (e = launch_pack((double*)g.Y, g.ldy, g.M, g.colE, nullptr, st)) != cudaSuccess) return e;
-  e = g.f32 ? gram_launch<float>(g, sms, nullptr, 0, 0, nullptr, g.G, nullptr, g.hdr, st)
-            : gram_launch<double>(g, sms, nullptr, 0, 0, nullptr, g.G, nullptr, g.hdr, st);
+  if ((e = launch_row_scale(g.Y, g.f32, g.ldy, g.M, g.colE, g.rowS, nullptr, st)) != cudaSuccess) return e;
+  e = g.f32 ? gram_launch<float>(g, sms, nullptr, 0, 0, nullptr, nullptr, g.G, nullptr, g.hdr, st)
+            : gram_launch<double>(g, sms, nullptr, 0, 0, nullptr, nullptr, g.G, nullptr, g.hdr, st);
   if (e != cudaSuccess) return e;
   if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
   CholArgs c{g, R, groups, g.f32 ? gram_base<float>(0) : gram_base<double>(0),

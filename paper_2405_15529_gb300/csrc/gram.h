@@ -14,9 +14,10 @@ cudaError_t tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, void* base
 struct GramState {
   WsHeader* hdr;
   int64_t N, M, ldy;      // ldy: rows of Y rounded up to 8, the padding rows hold zeros
-  void* Y;                // N x M weighted centred matrix: binary32, or binary64 cut to fixed point (pack_kernel)
+  void* Y;                // N x M weighted centred matrix: binary32, or binary64 cut to fixed point (row_scale_kernel)
   bool f32;
   int* colE;              // M: largest exponent field of each column
+  uint16_t* rowS;         // N, rounded up to 128: shift of each row (row_scale_kernel)
   long long* G;           // 5 x M x M: integer sums, group g weighs 2^(32 g)
   double* Lh;             // M x M double-double triangle (high parts)
   double* Ll;             // (low parts)
@@ -35,9 +36,11 @@ struct ProductArgs {
   const void* Y;
   int64_t ldy, N, M;
   const int* colE;
+  const uint16_t* rowS;
   const void* Z;
   int64_t ldz, NZ;
   const int* zE;
+  const uint16_t* zS;
   const double *C, *D, *S, *VT;
   int64_t ldc, ldd, ldvt;
   int64_t cols, cols_max;
@@ -47,7 +50,8 @@ struct ProductArgs {
   const WsHeader* hdr;
 };
 
-size_t gram_bytes(int64_t M, int64_t rmax);
+size_t row_shift_bytes(int64_t N);
+size_t gram_bytes(int64_t N, int64_t M, int64_t rmax);
 void gram_carve(GramState& g, char* base, int64_t M, int64_t rmax);
 
 // Y = sqrt(w) (X - mean), the column exponents and the means; then the exact
@@ -63,13 +67,14 @@ cudaError_t launch_modes_direct(const GramState& g, const double* C, const doubl
                                 const double* w, int physical, void* U, int64_t ldu, int64_t* r_out,
                                 const unsigned* unless, cudaStream_t st, cudaEvent_t mid);
 
-// Binary64 columns -> fixed-point words in place (rows of zeros up to ldy), and Y
-// of a forward back to binary64 where *redo is set.
-cudaError_t launch_pack(double* Y, int64_t ldy, int64_t cols, const int* colE, const unsigned* unless, cudaStream_t st);
+// Shifts of the rows of Y (rows of zeros up to ldy); binary64 columns -> fixed-point
+// words in place.  And Y of a forward back to binary64 where *redo is set.
+cudaError_t launch_row_scale(void* Y, bool f32, int64_t ldy, int64_t cols, const int* colE, uint16_t* rowS,
+                             const unsigned* unless, cudaStream_t st);
 cudaError_t launch_unpack(const GramState& g, double* Y, const unsigned* redo, cudaStream_t st);
 // W = Y^T Z (M x NZ, ld M) from the same integer products; Z as Y.  G: 5 M NZ integers.
-cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, long long* G,
-                         double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st);
+cudaError_t launch_cross(const GramState& g, const void* Z, int64_t ldz, int64_t NZ, const int* zE, const uint16_t* zS,
+                         long long* G, double* W, const unsigned* unless, WsHeader* hdr, cudaStream_t st);
 // The product above into U (binary32 if f32, else binary64; ld ldu).
 size_t product_planes_bytes(int64_t M, int64_t NZ, int64_t cols);
 cudaError_t launch_product(const ProductArgs& p, bool f32, void* U, int64_t ldu, WsHeader* hdr, cudaStream_t st);

@@ -5,7 +5,7 @@
 // multiplied without rounding on the tcgen05 tensor cores; digit products
 // below the level of a binary64 (binary32) rounding of the sum are left out.
 // Measured (4,194,304 x 256, r = 43): top-down pass + reflectors 7.3 + 209 ms
-// in binary64, 5.2 + 16.7 ms mixed; here 7.6 and 6.2 ms.
+// in binary64, 5.2 + 16.7 ms mixed; here 7.4 and 5.9 ms.
 //
 // A block takes tiles of 128 rows x 64 (32) columns of U (digits.cuh: two
 // shapes).  The warps cut 16 columns of the tile's rows of Y into digit planes
@@ -97,6 +97,16 @@ __global__ void __launch_bounds__(Shape<G>::THREADS, Shape<G>::BLOCKS) modes_dir
   const int mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
   // element i of this thread in slot q of its ring: ring[(q 8 + i) 256]
   Cl* ring = (Cl*)(gsm + NST * S * (kPlaneA + kPlaneB)) + (tid >> 8) * (AHEAD * 8 * 256) + (tid & 255);
+  // shift of this thread's row of tile t: of Y, and of Z in the upper half
+  auto shifts = [&](int t) {
+    const int64_t row = (int64_t)((blockIdx.x + t * gridDim.x) / kt32) * 128 + rl;
+    if (row >= N) return 0u;
+    const uint32_t a = __ldg(p.rowS + row);
+    return p.Z ? a | (uint32_t)__ldg(p.zS + row) << 16 : a | a << 16;
+  };
+  auto joint = [&](uint32_t s) { return (int)min(s & 0xffffu, s >> 16); };
+  uint32_t s_now = 0, s_next = 0;
+  int s_tile = -2;
   auto load = [&](int t, int js, int q) {
     const uint32_t tile = blockIdx.x + t * gridDim.x;
     const int64_t row = (int64_t)(tile / kt32) * 128 + rl;
@@ -115,13 +125,27 @@ __global__ void __launch_bounds__(Shape<G>::THREADS, Shape<G>::BLOCKS) modes_dir
     const bool rin = (int64_t)(tile / kt32) * 128 + rl < N, second = js >= s1;
     const int* ex = second ? p.zE : p.colE;
     const int c0 = (second ? js - s1 : js) * kStK + kh * 8, m32 = (int)(second ? p.NZ : p.M);
+    // the shifts of the next tile's row are on their way while this one is done
+    if ((S == 5 || p.Z) && t != s_tile) {
+      s_now = t == s_tile + 1 ? s_next : shifts(t);
+      s_tile = t;
+      if (t + 1 < mine) s_next = shifts(t + 1);
+    }
     Cl y[8];
     int E[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const bool in = c0 + i < m32;
       y[i] = in && rin ? ring[(q * 8 + i) * 256] : zero_cell<Cl>();
-      E[i] = (S == 5 && in) ? __ldg(ex + c0 + i) : 128;     // (words carry their scale)
+      E[i] = (S == 5 && in) ? __ldg(ex + c0 + i) - joint(s_now) : 128;     // (words carry their scale)
+    }
+    if constexpr (S == 8) {
+      // words of Y and of Z at the scale that both have room for
+      const uint32_t d = (second ? s_now >> 16 : s_now & 0xffffu) - joint(s_now);
+      if (__any_sync(0xffffffffu, d != 0)) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = shift_word(y[i], d);
+      }
     }
     put_digits(y, E, st + offA + kh * 128, kPlaneA);
   };
@@ -136,11 +160,12 @@ __global__ void __launch_bounds__(Shape<G>::THREADS, Shape<G>::BLOCKS) modes_dir
     const int k0 = (int)(tile % kt32) * T + (warp >> 2) * 16;
     const double iw = (physical && w && row < N) ? 1.0 / sqrt(w[row]) : 1.0;
     if (k0 >= r) return;
+    const int rs = joint(shifts(t));
     const int ce = lane < 16 && k0 + lane < r ? __ldg(p.Ce + k0 + lane) : 0;
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
       const int k = k0 + c;
-      const int pk = 8 * LB + __shfl_sync(0xffffffffu, ce, c) - fix_bias<double>() + (S == 5 ? 24 : 0);
+      const int pk = 8 * LB + __shfl_sync(0xffffffffu, ce, c) - fix_bias<double>() + (S == 5 ? 24 : 0) - rs;
       if (k < r && row < N) {
         TY v;
         if (zero) v = (TY)(row == k ? iw : 0.0);
@@ -222,6 +247,7 @@ cudaError_t launch_modes_direct(const GramState& g, const double* C, const doubl
   p.N = g.N;
   p.M = g.M;
   p.colE = g.colE;
+  p.rowS = g.rowS;
   p.C = C;
   p.ldc = g.M;
   p.S = S;

@@ -91,6 +91,7 @@ __global__ void bg_core_kernel(const double* A1, const double* A2, const double*
 struct BgLayout {
   void* Z;         // N x r (ld y_ld(N)), the working type
   int* zE;         // r
+  uint16_t* zS;    // N: shifts of the rows of Z
   long long* G;    // 5 M r
   double *W, *A1, *A2, *K, *T, *C, *D;
   unsigned char* Cd;
@@ -103,7 +104,7 @@ static size_t planes_only(int64_t M, int64_t r) {
 
 size_t pod_backward_gram_bytes(int64_t N, int64_t M, int64_t r) {
   const int64_t r1 = r > 0 ? r : 1;
-  return align256(sizeof(double) * (size_t)y_ld(N) * r1) + align256(sizeof(int) * (size_t)r1) +
+  return align256(sizeof(double) * (size_t)y_ld(N) * r1) + align256(sizeof(int) * (size_t)r1) + row_shift_bytes(N) +
          align256(sizeof(long long) * (size_t)5 * M * r1) + 3 * align256(sizeof(double) * (size_t)M * r1) +
          4 * align256(sizeof(double) * (size_t)M * M) + product_planes_bytes(M, r, M);
 }
@@ -114,6 +115,7 @@ static BgLayout carve(char* p, int64_t N, int64_t M, int64_t r) {
   const size_t mr = align256(sizeof(double) * (size_t)M * r1), mm = align256(sizeof(double) * (size_t)M * M);
   L.Z = p;                 p += align256(sizeof(double) * (size_t)y_ld(N) * r1);
   L.zE = (int*)p;          p += align256(sizeof(int) * (size_t)r1);
+  L.zS = (uint16_t*)p;     p += row_shift_bytes(N);
   L.G = (long long*)p;     p += align256(sizeof(long long) * (size_t)5 * M * r1);
   L.W = (double*)p;        p += mr;
   L.A1 = (double*)p;       p += mr;
@@ -147,8 +149,8 @@ cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const do
     if (f.f32) bg_load_kernel<float><<<grid, 256, 0, st>>>(dU, lddu, w, physical, (float*)L.Z, ldz, N, L.zE, redo);
     else bg_load_kernel<double><<<grid, 256, 0, st>>>(dU, lddu, w, physical, (double*)L.Z, ldz, N, L.zE, redo);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (!f.f32 && (e = launch_pack((double*)L.Z, ldz, r, L.zE, redo, st)) != cudaSuccess) return e;
-    if ((e = launch_cross(f, L.Z, ldz, r, L.zE, L.G, L.W, redo, hdr, st)) != cudaSuccess) return e;
+    if ((e = launch_row_scale(L.Z, f.f32, ldz, r, L.zE, L.zS, redo, st)) != cudaSuccess) return e;
+    if ((e = launch_cross(f, L.Z, ldz, r, L.zE, L.zS, L.G, L.W, redo, hdr, st)) != cudaSuccess) return e;
     e = launch_bw_gemm(0, 0, M, r, M, 1.0, VT, ldvt, L.W, M, 0.0, L.A1, M, redo, st);            // V^T W
     if (e != cudaSuccess) return e;
     if ((e = launch_bw_scale_rows(VT, ldvt, S, L.D, r, M, redo, st)) != cudaSuccess) return e;    // S_r^-1 V_r^T
@@ -156,6 +158,7 @@ cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const do
     p.ldz = ldz;
     p.NZ = r;
     p.zE = L.zE;
+    p.zS = L.zS;
     p.D = L.D;
     p.ldd = r;
   }
@@ -171,6 +174,7 @@ cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const do
   p.N = N;
   p.M = M;
   p.colE = f.colE;
+  p.rowS = f.rowS;
   p.C = L.C;
   p.ldc = M;
   p.cols = p.cols_max = M;
