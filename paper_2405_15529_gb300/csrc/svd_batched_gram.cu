@@ -21,8 +21,8 @@
 // zero matrix) are flagged on the device and left to that kernel.
 //
 // Persistent kernel -> here: 24 bins (N 16k..262k, Nb 16..128, 1.3 GB) 374 ->
-// 13.6 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.6 ms, SPOD of 131072 x
-// 1056 25.6 -> 7.3 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
+// 13.5 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.7 ms, SPOD of 131072 x
+// 1056 25.6 -> 7.4 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
 #include <algorithm>
 
 #include "digits.cuh"
@@ -49,6 +49,7 @@ struct BG {
   float2* f;
   unsigned char* c;
   double* d;
+  uint16_t* rows;
   int* flags;
   double* S;
   WsHeader* hdr;
@@ -61,15 +62,34 @@ __device__ __forceinline__ double2* mat(const BG& a, const GramBin& b, int i) {
 // ---------------------------------------------------------------------------
 // 1. column exponents; windows: Y = sqrt(w) (x - mean) in binary32
 // ---------------------------------------------------------------------------
+// Rows' largest exponent fields: lanes hold (pairs of) consecutive rows, warps
+// take columns in turn; the eight warps' maxima meet in shared memory.
+constexpr int kTopRows = 256;
+struct RowTops {
+  int t[2][8][kTopRows];       // (a warp may be an iteration ahead of the reads)
+};
+// all threads: `n` rows (a warp's maxima are in its line), the first `live` of them to `out`
+__device__ __forceinline__ void store_tops(const RowTops& s, int turn, int n, int64_t live, uint16_t* out) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < n && i < live; i += 256) {
+    int t = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t = max(t, s.t[turn][q][i]);
+    out[i] = (uint16_t)t;
+  }
+}
+
 template <typename TX>
-__device__ void window_rows(const GramBin& b, float* Y, int64_t r0, int64_t r1, int* sE, int& bad) {
+__device__ void window_rows(const GramBin& b, float* Y, uint16_t* rows, int64_t r0, int64_t r1, int* sE, RowTops& tops,
+                            int& bad) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ double ssum[8][32];
   const TX* X = (const TX*)b.Xr;
   int em[16];
 #pragma unroll
   for (int t = 0; t < 16; ++t) em[t] = 0;
-  for (int64_t blk = r0; blk < r1; blk += 32) {
+  int turn = 0;
+  for (int64_t blk = r0; blk < r1; blk += 32, turn ^= 1) {
     const int64_t n = blk + lane;
     const bool in = n < b.rows;
     TX x[16];
@@ -106,6 +126,7 @@ __device__ void window_rows(const GramBin& b, float* Y, int64_t r0, int64_t r1, 
     if (warp == 0 && in && b.mean) b.mean[n] = xbar;
     const float xh = (float)xbar, xl = (float)(xbar - (double)xh);
     const float sh = (float)sw, sl = (float)(sw - (double)sh);
+    int top = 0;
 #pragma unroll
     for (int t = 0; t < 16; ++t) {
       const int c = warp + 8 * t;
@@ -120,9 +141,13 @@ __device__ void window_rows(const GramBin& b, float* Y, int64_t r0, int64_t r1, 
       }
       if (!in) y = 0.f;
       if (!isfinite(x[t])) bad = 1;
-      em[t] = max(em[t], exp_field(y));
+      const int e = exp_field(y);
+      em[t] = max(em[t], e);
+      top = max(top, e);
       if (n < b.ldy) Y[n + (int64_t)c * b.ldy] = y;
     }
+    tops.t[turn][warp][lane] = top;
+    store_tops(tops, turn, 32, b.ldy - blk, rows + blk);
   }
 #pragma unroll
   for (int t = 0; t < 16; ++t) {
@@ -131,32 +156,136 @@ __device__ void window_rows(const GramBin& b, float* Y, int64_t r0, int64_t r1, 
   }
 }
 
+// A bin: NC columns a warp, 16 / NC groups of 32 points a turn (16 loads in flight).
+template <int NC>
+__device__ void bin_rows(const GramBin& b, uint16_t* rows, int64_t p0, int64_t p1, int* sE, RowTops& tops, int& bad) {
+  constexpr int G = 64 / NC < 4 ? 64 / NC : 4;
+  static_assert(G * NC <= 64 && 64 * G <= kTopRows, "loads a turn; room for the maxima");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float2* col = (const float2*)b.Y + (int64_t)warp * (b.ldy / 2) + lane;
+  int em[NC];
+#pragma unroll
+  for (int t = 0; t < NC; ++t) em[t] = 0;
+  int turn = 0;
+  for (int64_t pr = p0; pr < p1; pr += 32 * G, turn ^= 1) {
+    float2 x[G][NC];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int t = 0; t < NC; ++t)
+        x[g][t] = pr + 32 * g + lane < p1 && warp + 8 * t < b.Nb ? __ldg(col + pr + 32 * g + t * 4 * b.ldy) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      int tx = 0, ty = 0;
+#pragma unroll
+      for (int t = 0; t < NC; ++t) {
+        const int ex = (__float_as_int(x[g][t].x) >> 23) & 0xff, ey = (__float_as_int(x[g][t].y) >> 23) & 0xff;
+        em[t] = max(em[t], max(ex, ey));
+        tx = max(tx, ex);
+        ty = max(ty, ey);
+      }
+      *(int2*)&tops.t[turn][warp][64 * g + 2 * lane] = make_int2(tx, ty);
+    }
+    store_tops(tops, turn, 64 * G, 2 * (p1 - pr), rows + 2 * pr);
+  }
+#pragma unroll
+  for (int t = 0; t < NC; ++t) {
+    const int e = __reduce_max_sync(0xffffffffu, em[t]);
+    if (e == 0xff) bad = 1;
+    if (lane == 0 && warp + 8 * t < b.Nb) sE[warp + 8 * t] = max(e, kMinField32);
+  }
+}
+
+// Besides the columns' exponents every row's largest one goes to a.rows; up
+// to 16 loads a lane hide the latency of memory (a warp per column took 0.52
+// ms for the 1.1 GB of 131072 x 1056 in bins of 32 columns, this 0.29).
 __global__ void __launch_bounds__(256) bg_prologue_kernel(BG a) {
   __shared__ int sE[128];
+  __shared__ RowTops tops;
   const GramUnit u = a.units[blockIdx.x];
   const GramBin b = a.bins[u.bin];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int bad = 0;
   if (b.kind == 0) {
-    for (int c = warp; c < b.Nb; c += 8) {
-      const float2* col = (const float2*)(b.Y + (int64_t)c * b.ldy);
-      int e = 0;
-      for (int64_t n = u.q0 + lane; n < u.q1; n += 32) {
-        const float2 x = __ldg(col + n);
-        if (!isfinite(x.x) || !isfinite(x.y)) bad = 1;
-        e = max(e, max(exp_field(x.x), exp_field(x.y)));
-      }
-      e = __reduce_max_sync(0xffffffffu, e);
-      if (lane == 0) sE[c] = e;
-    }
+    if (b.Nb <= 32) bin_rows<4>(b, a.rows + b.r, u.q0, u.q1, sE, tops, bad);
+    else if (b.Nb <= 64) bin_rows<8>(b, a.rows + b.r, u.q0, u.q1, sE, tops, bad);
+    else bin_rows<16>(b, a.rows + b.r, u.q0, u.q1, sE, tops, bad);
   } else if (b.kind == 1) {
-    window_rows<float>(b, (float*)b.Y, u.q0, u.q1, sE, bad);
+    window_rows<float>(b, (float*)b.Y, a.rows + b.r, u.q0, u.q1, sE, tops, bad);
   } else {
-    window_rows<double>(b, (float*)b.Y, u.q0, u.q1, sE, bad);
+    window_rows<double>(b, (float*)b.Y, a.rows + b.r, u.q0, u.q1, sE, tops, bad);
   }
   __syncthreads();
   for (int c = threadIdx.x; c < b.Nb; c += 256) atomicMax(a.ints + b.colE + c, sE[c]);
   if (bad) raise_status(a.hdr, PYLOM_ERR_NONFINITE);
+}
+
+// Shift of each row, as in the single POD (row_scale_kernel, gram.cu): how far
+// its elements all lie below their columns' largest exponents.  Where these
+// differ by at most kSpread, how far the row's largest exponent lies below the
+// smallest of them is near enough (38 bits are 14 more than the modes hold),
+// and nothing is read again.  Else a lane takes a pair of rows (a point of a
+// bin: its real and imaginary parts), bound by memory.
+constexpr int kSpread = 8;
+__global__ void __launch_bounds__(256) bg_rows_kernel(BG a) {
+  __shared__ int sE[128];
+  __shared__ int stop[2][8][64];     // (a warp may be an iteration ahead of the reads)
+  constexpr int kNone = -2147483647;
+  __shared__ int s_lo, s_hi;
+  const GramUnit u = a.units[blockIdx.x];
+  const GramBin b = a.bins[u.bin];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    s_lo = 0x100;
+    s_hi = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x < b.Nb) {
+    const int E = a.ints[b.colE + threadIdx.x];
+    sE[threadIdx.x] = E << 23;
+    if (E > kMinField32) {           // (columns of zeros apart)
+      atomicMin(&s_lo, E);
+      atomicMax(&s_hi, E);
+    }
+  }
+  __syncthreads();
+  if (s_hi - s_lo <= kSpread) {
+    const int64_t f = b.cplx ? 2 : 1;
+    for (int64_t n = f * u.q0 + threadIdx.x; n < f * u.q1; n += 256) {
+      uint16_t& r = a.rows[b.r + n];
+      r = r > kMinField32 && r < s_lo ? (uint16_t)(s_lo - r) : 0;
+    }
+    return;
+  }
+  const int64_t p0 = b.cplx ? u.q0 : u.q0 / 2, p1 = b.cplx ? u.q1 : u.q1 / 2;
+  int turn = 0;
+  for (int64_t pr = p0; pr < p1; pr += 32, turn ^= 1) {
+    const bool in = pr + lane < p1;
+    const float* p = b.Y + 2 * (pr + lane);
+    float2 x[16];
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int c = warp + 8 * t;
+      x[t] = in && c < b.Nb ? __ldg((const float2*)(p + c * b.ldy)) : make_float2(0.f, 0.f);
+    }
+    int t0 = kNone, t1 = kNone;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      const int c = warp + 8 * t;
+      const int E = c < b.Nb ? sE[c] : 0;
+      const int hx = __float_as_int(x[t].x) & 0x7f800000, hy = __float_as_int(x[t].y) & 0x7f800000;
+      if (hx > (kMinField32 << 23)) t0 = max(t0, hx - E);
+      if (hy > (kMinField32 << 23)) t1 = max(t1, hy - E);
+    }
+    stop[turn][warp][2 * lane] = t0;
+    stop[turn][warp][2 * lane + 1] = t1;
+    __syncthreads();
+    if (threadIdx.x < 64 && pr + threadIdx.x / 2 < p1) {
+      int t = kNone;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t = max(t, stop[turn][q][threadIdx.x]);
+      a.rows[b.r + 2 * pr + threadIdx.x] = (uint16_t)(t == kNone ? 0 : -(t >> 23));
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -873,6 +1002,12 @@ __global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_modes_kernel(B
   const int* E = a.ints + b.colE;
   const int* Ce = a.ints + b.colE + n;
   float* ring = (float*)(gsm + kNstB * kStageB) + tid;
+  // shift of row rl of a tile; the next tile's is on its way while one is done
+  auto shift = [&](int t) {
+    const int64_t row = (u.q0 + t) * 128 + rl;
+    return row < b.rows ? (int)__ldg(a.rows + b.r + row) : 0;
+  };
+  int s_now = 0, s_next = 0, s_tile = -2;
   auto load = [&](int t, int js, int q) {
     const int64_t row = (u.q0 + t) * 128 + rl;
     const int c0 = js * kStK + kh * 8;
@@ -886,13 +1021,18 @@ __global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_modes_kernel(B
   auto fill = [&](int t, int js, int q, unsigned char* st) {
     const bool rin = (u.q0 + t) * 128 + rl < b.rows;
     const int c0 = js * kStK + kh * 8;
+    if (t != s_tile) {
+      s_now = t == s_tile + 1 ? s_next : shift(t);
+      s_tile = t;
+      s_next = shift(t + 1);
+    }
     float y[8];
     int e[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const bool in = c0 + i < n;
       y[i] = in && rin ? ring[(q * 8 + i) * kThreads] : 0.f;
-      e[i] = in ? __ldg(E + c0 + i) : 128;
+      e[i] = in ? __ldg(E + c0 + i) - s_now : 128;
     }
     put_digits(y, e, st + offA + kh * 128, kPlaneA);
   };
@@ -901,8 +1041,9 @@ __global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_modes_kernel(B
     const int64_t row = (u.q0 + t) * 128 + (warp & 3) * 32 + lane;
     const int k0 = u.J * kTile + (warp >> 2) * 16;
     const double iw = (b.physical && b.w && row < b.rows) ? 1.0 / sqrt(b.w[row]) : 1.0;
+    const int rs = shift(t);
     auto value = [&](int c) {
-      const int pk = 8 * LB + __ldg(Ce + k0 + c) - fix_bias<double>() + 24;
+      const int pk = 8 * LB + __ldg(Ce + k0 + c) - fix_bias<double>() + 24 - rs;
       return from_sums(acc0[c], acc1[c], pk, 0.0);
     };
     if (b.cplx) {
@@ -943,13 +1084,13 @@ void batched_gram_add(BatchedGramPlan& p, int item, int64_t N, int64_t Nb, int64
   b.f = p.n_f;                      p.n_f += Nb * b.Mb + (int64_t)b.Mb * b.Mb;
   b.c = p.n_c;                      p.n_c += (Nb + kStK - 1) / kStK * kSB * (int64_t)kPlaneB * (64 / kTile);
   b.d = p.n_d;                      p.n_d += 1 + 2 * Nb;
+  b.r = p.n_r;                      p.n_r += 2 * ((N + 7) & ~int64_t(7));     // real or complex: bind tells
   b.s_off = s_off;
   b.flag = item;
   p.items.push_back(item);
   p.bins.push_back(b);
   p.maxNb = std::max(p.maxNb, b.Nb);
   p.maxpairs = std::max(p.maxpairs, b.Mb / kZW);
-  p.kmax = std::max(p.kmax, b.k);
 }
 
 // Units hold at most this many per item: the tables' sizes must not depend on
@@ -969,6 +1110,7 @@ size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems) {
   p.off_f = off;     off += align256(sizeof(float2) * (size_t)p.n_f);
   p.off_c = off;     off += align256((size_t)p.n_c);
   p.off_d = off;     off += align256(sizeof(double) * (size_t)p.n_d);
+  p.off_r = off;     off += align256(sizeof(uint16_t) * (size_t)p.n_r);
   return off;
 }
 
@@ -1060,6 +1202,7 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   a.f = (float2*)(ws + p.off_f);
   a.c = (unsigned char*)(ws + p.off_c);
   a.d = (double*)(ws + p.off_d);
+  a.rows = (uint16_t*)(ws + p.off_r);
   a.flags = (int*)(ws + p.off_flags) + 1;
   a.S = S;
   a.hdr = hdr;
@@ -1080,6 +1223,7 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   BG au = a;
   au.units = units;
   bg_prologue_kernel<<<(unsigned)p.pro.size(), 256, 0, st>>>(au);
+  if (!p.mod.empty()) bg_rows_kernel<<<(unsigned)p.pro.size(), 256, 0, st>>>(au);
   au.units = units + m;
   bg_gram_kernel<<<(unsigned)p.gram.size(), kThreads, smem, st>>>(au);
   bg_chol_kernel<<<nb, kCholThreads, csmem, st>>>(a);

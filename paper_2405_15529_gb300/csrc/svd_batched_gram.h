@@ -17,6 +17,7 @@ struct GramBin {
   int64_t z;             // double2: kBinMats matrices Nb x Nb
   int64_t f;             // float2: A32 (Nb x Mb), V32 (Mb x Mb)
   int64_t c;             // bytes: digit planes of the coefficients
+  int64_t r;             // uint16: shifts of the rows (twice the points)
   int64_t d;             // doubles: Nb (norms) + Nb (angle flags)
   int64_t s_off;         // offset in the packed S
   int flag;              // index in the flag array (the item's number in the plan)
@@ -45,9 +46,9 @@ struct BatchedGramPlan {
   std::vector<int> items;          // item numbers of the plan that take this route
   std::vector<GramBin> bins;       // offsets by the plan, pointers by bind
   std::vector<GramUnit> pro, gram, mod;   // prologue, Gram and modes units
-  int nitems = 0, maxNb = 0, maxpairs = 0, kmax = 0;
-  size_t off_bins = 0, off_units = 0, off_i = 0, off_g = 0, off_z = 0, off_f = 0, off_c = 0, off_d = 0, off_flags = 0;
-  int64_t n_i = 0, n_g = 0, n_z = 0, n_f = 0, n_c = 0, n_d = 0;
+  int nitems = 0, maxNb = 0, maxpairs = 0;
+  size_t off_bins = 0, off_units = 0, off_i = 0, off_g = 0, off_z = 0, off_f = 0, off_c = 0, off_d = 0, off_r = 0, off_flags = 0;
+  int64_t n_i = 0, n_g = 0, n_z = 0, n_f = 0, n_c = 0, n_d = 0, n_r = 0;
 };
 
 // Adds an item (N x Nb, kmodes modes) and, at the end, the sections to the workspace.

@@ -138,3 +138,50 @@ def test_rows_of_the_adjoint(N, M, small_du, prec):
     for q in (rows, ~rows):
         assert np.linalg.norm(out[0][q] - ref[q]) <= 1e2 * M * eps * np.linalg.norm(ref[q])
     assert np.linalg.norm((out[0] - out[1])[~rows]) <= 1e2 * M * eps * np.linalg.norm(out[1][~rows])
+
+
+@pytest.mark.parametrize("small", [0.05, 1e-3, 1e-5, 1e-8, 1e-30])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_rows_of_batched_modes(small, shift):
+    """Windows and bins of one plan, mixed precision; bins off a 16-byte boundary too."""
+    wins = [_field(N, M, N, small, np.float32, zc) for N, M, zc in ((1500, 12, False), (801, 63, True), (2100, 96, False))]
+    bins = []
+    for N, M in ((1400, 20), (901, 70)):
+        re, im = _field(N, M, N, small, np.float32), _field(N, M, N + 1, small, np.float32)
+        im[2::3] *= small                                   # rows whose imaginary part is small
+        bins.append(re + 1j * im.astype(np.float32))
+    dev = []
+    for Q in bins:
+        big = torch.zeros((Q.shape[1], Q.shape[0] + shift), dtype=torch.complex64, device="cuda")
+        big[:, shift:] = torch.from_numpy(np.ascontiguousarray(Q.T)).cuda()
+        dev.append(big[:, shift:].t())
+    b = pg.BatchedPOD([_dev(X, torch.float32) for X in wins], remove_mean=False, kmodes=3, prec=pg.PREC_MIXED_3XTF32,
+                      bins=dev)
+    b.run()
+    assert b.status() == pg.OK
+    eps = 2.0 ** -24
+    for i, X in enumerate(wins):
+        _rows_agree(b.modes[i].double().cpu().numpy(), X, eps, 3)
+    for i, Q in enumerate(bins):
+        U, S, VH = np.linalg.svd(Q, full_matrices=False)
+        top = VH[np.arange(len(S)), np.argmax(np.abs(VH), axis=1)]
+        V = (VH * (np.conj(top) / np.abs(top))[:, None]).conj().T
+        gap = np.minimum(np.abs(np.diff(S, prepend=np.inf)), np.abs(np.diff(S, append=-np.inf)))
+        got = b.modes[len(wins) + i].to(torch.complex128).cpu().numpy()
+        rho = np.linalg.norm(Q, axis=1)
+        for k in range(3):
+            err = np.abs(got[:, k] - Q @ V[:, k] / S[k])[rho > 0] / (rho[rho > 0] / S[k])
+            assert err.max() <= Q.shape[1] * eps * S[0] / gap[k], (i, k, err.max())
+
+
+@pytest.mark.parametrize("spread", [2.0 ** -7, 2.0 ** -12, 2.0 ** -16])
+def test_rows_of_batched_modes_with_uneven_columns(spread):
+    """Columns within the spread that the shifts' short cut takes, and past it
+    (further down the item is left to the Householder kernel)."""
+    X = _field(1700, 24, 3, 1e-5, np.float32)
+    X[:, ::2] *= spread
+    X = X.astype(np.float32).astype(np.float64)
+    b = pg.BatchedPOD([_dev(X, torch.float32)], remove_mean=False, kmodes=3, prec=pg.PREC_MIXED_3XTF32)
+    b.run()
+    assert b.status() == pg.OK
+    _rows_agree(b.modes[0].double().cpu().numpy(), X, 2.0 ** -24, 3)
