@@ -75,6 +75,10 @@ template <typename TY> __host__ __device__ constexpr int fix_bias() { return siz
 // (A row's shift can take the scale of a column that lies below 2^-100
 // further down; what such a column has in that row counts for less.)
 constexpr int kMinField64 = 64, kMinField32 = 8;
+// That of infinities and NaN: such a column has no scale, and what is made of it is NaN.
+constexpr int kMaxField64 = 2047, kMaxField32 = 255;
+template <typename T> __host__ __device__ constexpr int max_field() { return sizeof(T) == 8 ? kMaxField64 : kMaxField32; }
+__device__ __forceinline__ double quiet_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
 __device__ __forceinline__ int exp_field(double y) {
   const int e = (__double2hiint(y) >> 20) & 0x7ff;
   return e > kMinField64 ? e : kMinField64;

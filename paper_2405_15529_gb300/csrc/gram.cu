@@ -677,6 +677,7 @@ __global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
       const double u = (i / B == j / B) ? __ldcg(c.R + idx) : __ldcg(g.Lh + idx);
       // the integer sums were scaled by 2^-64: their root by 2^-32
       v = scalbn(sqrt(__ldcg(dvec + i)) * u, g.colE[j] - c.bias + 32);
+      if (g.colE[j] == (g.f32 ? kMaxField32 : kMaxField64)) v = quiet_nan();
     }
     c.R[idx] = v;
   }

@@ -44,10 +44,13 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(ProductArgs p) {
     if (k >= r) return 0.0;
     if (j < (int64_t)s1 * kStK) {
       if (j >= p.M) return 0.0;
+      if (p.colE[j] == max_field<TY>()) return quiet_nan();
       return scalbn(p.C ? p.C[j + k * p.ldc] : p.VT[k + j * p.ldvt] / sk, p.colE[j] - fix_bias<TY>());
     }
     j -= (int64_t)s1 * kStK;
-    return j < p.NZ ? scalbn(p.D[j + k * p.ldd], p.zE[j] - fix_bias<TY>()) : 0.0;
+    if (j >= p.NZ) return 0.0;
+    if (p.zE[j] == max_field<TY>()) return quiet_nan();
+    return scalbn(p.D[j + k * p.ldd], p.zE[j] - fix_bias<TY>());
   };
   int e = kMinField64;
   for (int64_t j = threadIdx.x; j < (int64_t)stages * kStK; j += blockDim.x) {
@@ -165,10 +168,12 @@ __global__ void __launch_bounds__(Shape<G>::THREADS, Shape<G>::BLOCKS) modes_dir
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
       const int k = k0 + c;
-      const int pk = 8 * LB + __shfl_sync(0xffffffffu, ce, c) - fix_bias<double>() + (S == 5 ? 24 : 0) - rs;
+      const int cc = __shfl_sync(0xffffffffu, ce, c);
+      const int pk = 8 * LB + cc - fix_bias<double>() + (S == 5 ? 24 : 0) - rs;
       if (k < r && row < N) {
         TY v;
         if (zero) v = (TY)(row == k ? iw : 0.0);
+        else if (cc == kMaxField64) v = (TY)quiet_nan();      // a coefficient, or a column of Y, is not finite
         else if (physical && w) v = (TY)(from_sums(acc0[c], acc1[c], pk, 0.0) * iw);
         else v = from_sums(acc0[c], acc1[c], pk, (TY)0);
         U[row + k * ldu] = v;

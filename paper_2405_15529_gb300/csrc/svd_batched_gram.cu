@@ -473,6 +473,7 @@ __global__ void __launch_bounds__(kCholThreads) bg_chol_kernel(BG a) {
       // the sums count from level 1 (2^8)
       const double s = scalbn(16.0, E[j] - fix_bias<float>());
       v = make_double2(r.x * s, -r.y * s);
+      if (E[j] == kMaxField32) v.x = quiet_nan();      // (the item is left to the Householder kernel)
     }
     A[idx] = v;
     em = max(em, (unsigned)max(exp_field(v.x), exp_field(v.y)));
