@@ -19,6 +19,15 @@ of a seeded known-spectrum matrix of that shape at each candidate leaf count
 (whole multiples of the SM count, so every wave of leaves fills the GPU)
 and keeps the fastest leaf height.
 
+A leaf height is a choice among Householder leaves.  Where the library's
+automatic choice (0) takes the Gram route instead -- pylom_pod with an energy
+share or r_max < M, mixed-precision batches -- any height is slower: 799
+against 50 ms for 4194304 x 256, 374 against 13.5 ms for 24 SPOD bins.  So
+`pod_leaf_rows_for` gives 0 for calls that it is told about,
+`tune_batched_workload` times the built-in choice too, and heights serve the
+calls that use leaves in any case: all modes, pylom_tsqr, the streamed and
+sharded POD, binary64 batches.
+
 Results are cached in JSON, keyed by GPU name, precision and class; the cache
 file is a runtime artifact (PYLOM_TUNE_CACHE overrides its path).
 """
@@ -120,7 +129,9 @@ def gpu_name() -> str:
 
 def leaf_rows_for(Ns, Nbs, prec: int, tune: bool = False):
     """Leaf heights for a batch (from the cache; missing classes are tuned
-    when `tune`, else left to the library's built-in choice, 0)."""
+    when `tune`, else left to the library's built-in choice, 0).  The fastest
+    heights, not the fastest choice: a mixed-precision batch runs faster
+    without any (`tune_batched_workload` compares)."""
     gpu = gpu_name()
     cache = _load()
     out = []
@@ -236,9 +247,21 @@ def tune_pod(N: int, M: int, prec: int, sms: int = None):
     return best, times
 
 
-def pod_leaf_rows_for(N: int, M: int, prec: int, tune: bool = False) -> int:
+def automatic_takes_gram_route(M: int, energy: float = 0.0, r_max: int = None) -> bool:
+    """Whether pylom_pod with leaf_rows = 0 leaves Y unfactored for these
+    arguments (the rule of pod_route, api.cu)."""
+    if os.environ.get("PYLOM_TREE") is not None:
+        return False
+    return 0.0 < energy <= 1.0 - 1e-4 or (r_max is not None and r_max < M)
+
+
+def pod_leaf_rows_for(N: int, M: int, prec: int, tune: bool = False, energy: float = 0.0, r_max: int = None) -> int:
     """The cached leaf height for this (N, M, precision) -- tuned first when
-    `tune` and not cached -- or 0 (the library's automatic choice)."""
+    `tune` and not cached -- or 0 (the library's automatic choice): always 0
+    where energy and r_max of the call have that choice take the Gram route,
+    which is faster than any height."""
+    if automatic_takes_gram_route(M, energy, r_max):
+        return 0
     key = f"{gpu_name()}|pod|prec{prec}|N{N}|M{M}"
     cache = _load()
     if key not in cache and tune:
