@@ -1230,43 +1230,50 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   bg_chol_kernel<<<nb, kCholThreads, csmem, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned tiles = (unsigned)((p.maxNb + 7) / 8), el = (unsigned)std::max(1, p.maxNb * p.maxNb / 2048);
-  auto stage = [&]() {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.maxpairs, nb);
-    cfg.blockDim = dim3(kZThreads);
-    cfg.dynamicSmemBytes = jsmem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)p.maxpairs;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, bg_jacobi32_kernel, a);
-  };
-  auto gemm = [&](const ZGemm& x) {
-    bg_gemm_kernel<<<dim3(tiles, tiles, nb), 128, 0, st>>>(a, ZGemms{{x, x}, 1});
-  };
-  auto gemm2 = [&](const ZGemm& x, const ZGemm& y) {
-    bg_gemm_kernel<<<dim3(tiles, tiles, 2 * nb), 128, 0, st>>>(a, ZGemms{{x, y}, 2});
-  };
   enum { A = 0, V = 1, A2 = 2, T0 = 3, T1 = 4, T2 = 5, T3 = 6, T4 = 7 };
-  if ((e = stage()) != cudaSuccess) return e;
-  bg_widen_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
-  gemm(ZGemm{1, T0, T0, -1, T1, 1.0, 0.0});                 // V^H V
-  gemm(ZGemm{0, T0, T1, T0, T3, -0.5, 1.5});                // V <- 1.5 V - 0.5 V V^H V
-  gemm(ZGemm{0, A, T3, -1, A2, 1.0, 0.0});                  // A = R^H V
-  bg_init_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess || (e = stage()) != cudaSuccess) return e;
-  bg_widen_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
-  gemm2(ZGemm{0, T3, T0, -1, V, 1.0, 0.0}, ZGemm{0, A2, T0, -1, A, 1.0, 0.0});
-  for (int it = 0; it < 2; ++it) {
-    const int Ai = it ? A2 : A, Vi = it ? T3 : V, Ao = it ? A : A2, Vo = it ? V : T3;
-    gemm2(ZGemm{1, Ai, Ai, -1, T0, 1.0, 0.0}, ZGemm{1, Vi, Vi, -1, T1, 1.0, 0.0});
-    bg_check_kernel<<<dim3((unsigned)((p.maxNb + 7) / 8), nb), 256, 0, st>>>(a, it);
-    bg_angles_kernel<<<dim3(el, nb), 256, 0, st>>>(a);
-    gemm(ZGemm{0, T4, T2, T1, T0, 0.5, 1.0});               // Q
-    gemm2(ZGemm{0, Ai, T0, -1, Ao, 1.0, 0.0}, ZGemm{0, Vi, T0, -1, Vo, 1.0, 0.0});
+  // items count in the grid's y, or twice in its z, which end at 65,535
+  constexpr unsigned kItems = 32767;
+  for (unsigned f0 = 0; f0 < nb; f0 += kItems) {
+    const unsigned ni = std::min(kItems, nb - f0);
+    BG ac = a;
+    ac.bins += f0;
+    auto stage = [&]() {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)p.maxpairs, ni);
+      cfg.blockDim = dim3(kZThreads);
+      cfg.dynamicSmemBytes = jsmem;
+      cfg.stream = st;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)p.maxpairs;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      return cudaLaunchKernelEx(&cfg, bg_jacobi32_kernel, ac);
+    };
+    auto gemm = [&](const ZGemm& x) {
+      bg_gemm_kernel<<<dim3(tiles, tiles, ni), 128, 0, st>>>(ac, ZGemms{{x, x}, 1});
+    };
+    auto gemm2 = [&](const ZGemm& x, const ZGemm& y) {
+      bg_gemm_kernel<<<dim3(tiles, tiles, 2 * ni), 128, 0, st>>>(ac, ZGemms{{x, y}, 2});
+    };
+    if ((e = stage()) != cudaSuccess) return e;
+    bg_widen_kernel<<<dim3(el, ni), 256, 0, st>>>(ac);
+    gemm(ZGemm{1, T0, T0, -1, T1, 1.0, 0.0});                 // V^H V
+    gemm(ZGemm{0, T0, T1, T0, T3, -0.5, 1.5});                // V <- 1.5 V - 0.5 V V^H V
+    gemm(ZGemm{0, A, T3, -1, A2, 1.0, 0.0});                  // A = R^H V
+    bg_init_kernel<<<dim3(el, ni), 256, 0, st>>>(ac);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = stage()) != cudaSuccess) return e;
+    bg_widen_kernel<<<dim3(el, ni), 256, 0, st>>>(ac);
+    gemm2(ZGemm{0, T3, T0, -1, V, 1.0, 0.0}, ZGemm{0, A2, T0, -1, A, 1.0, 0.0});
+    for (int it = 0; it < 2; ++it) {
+      const int Ai = it ? A2 : A, Vi = it ? T3 : V, Ao = it ? A : A2, Vo = it ? V : T3;
+      gemm2(ZGemm{1, Ai, Ai, -1, T0, 1.0, 0.0}, ZGemm{1, Vi, Vi, -1, T1, 1.0, 0.0});
+      bg_check_kernel<<<dim3((unsigned)((p.maxNb + 7) / 8), ni), 256, 0, st>>>(ac, it);
+      bg_angles_kernel<<<dim3(el, ni), 256, 0, st>>>(ac);
+      gemm(ZGemm{0, T4, T2, T1, T0, 0.5, 1.0});               // Q
+      gemm2(ZGemm{0, Ai, T0, -1, Ao, 1.0, 0.0}, ZGemm{0, Vi, T0, -1, Vo, 1.0, 0.0});
+    }
   }
   bg_finalize_kernel<<<nb, 256, 0, st>>>(a);
   if (!p.mod.empty()) {
