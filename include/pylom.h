@@ -453,7 +453,10 @@ typedef struct {
                          binary64 with complex128 leaves (PYLOM_PREC_FP64) */
   int64_t ldu;
   double* VT;         /* real windows: device Nb x Nb right vectors out (row i = v_i^T, the sign rule
-                         of pylom_pod; rows of an exactly zero singular value are zero), or NULL */
+                         of pylom_pod; rows of an exactly zero singular value are zero, the others
+                         orthonormal to binary64 rounding; on the Gram route those past the kept modes
+                         may mix within a crowd of values closer than 2^-22 sqrt(Nb) of each other),
+                         or NULL */
   int64_t ldvt;
 } pylom_batched_item;
 pylom_status pylom_svd_batched_bind_items(pylom_batched_plan* plan, const pylom_batched_item* items, void* ws,

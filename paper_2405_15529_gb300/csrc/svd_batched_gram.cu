@@ -17,11 +17,11 @@
 //   5. U = Y W_k S_k^-1 (W the right vectors) by digit products.
 // Items whose result would be less accurate than the Householder route's
 // (a kept mode below 1e-4 of the largest singular value, where squaring
-// costs binary32 digits; kept values too close to separate in two steps; a
-// zero matrix) are flagged on the device and left to that kernel.
+// costs binary32 digits; kept values too close to separate in two steps; any
+// sound column that the binary32 stages left open; a zero matrix) are flagged on the device and left to that kernel.
 //
 // Persistent kernel -> here: 24 bins (N 16k..262k, Nb 16..128, 1.3 GB) 374 ->
-// 13.5 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.7 ms, SPOD of 131072 x
+// 13.5 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.9 ms, SPOD of 131072 x
 // 1056 25.6 -> 7.4 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
 #include <algorithm>
 
@@ -39,6 +39,9 @@ constexpr int kNstB = Dig<float>::NST<kG>, kAhead = Dig<float>::AHEAD<kG>;
 constexpr int kStageB = kSB * (kPlaneA + kPlaneB);
 constexpr double kKeptLevel = 1e-4;
 constexpr double kOpenCos = 1e-6;                  // kept columns: largest cosine before the last step
+// Singular values below this share of the first are rounding (the square root
+// of the pivots that the Cholesky factor drops, and some room)
+constexpr double kSoundLevel = 1e-7;
 
 struct BG {
   const GramBin* bins;
@@ -54,6 +57,9 @@ struct BG {
   double* S;
   WsHeader* hdr;
 };
+
+// a window whose right vectors are asked for
+__device__ __forceinline__ bool has_vt(const GramBin& b) { return b.kind != 0 && b.VT; }
 
 __device__ __forceinline__ double2* mat(const BG& a, const GramBin& b, int i) {
   return a.z + b.z + (int64_t)i * b.Nb * b.Nb;
@@ -763,6 +769,7 @@ struct ZGemm {
 struct ZGemms {
   ZGemm g[2];
   int count;
+  bool vt_only;             // only items with has_vt
 };
 
 __global__ void __launch_bounds__(128) bg_gemm_kernel(BG a, ZGemms gs) {
@@ -770,7 +777,7 @@ __global__ void __launch_bounds__(128) bg_gemm_kernel(BG a, ZGemms gs) {
   const GramBin b = a.bins[blockIdx.z / gs.count];
   const ZGemm& p = gs.g[blockIdx.z % gs.count];
   const int n = b.Nb, i0 = blockIdx.x * 8, j0 = blockIdx.y * 8;
-  if (i0 >= n || j0 >= n) return;
+  if (i0 >= n || j0 >= n || (gs.vt_only && !has_vt(b))) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const double2* A = mat(a, b, p.A);
   const double2* B = mat(a, b, p.B);
@@ -848,8 +855,8 @@ __global__ void __launch_bounds__(256) bg_check_kernel(BG a, int last) {
   }
   if (lane == 0) {
     const bool moves = big <= 0.02 && sum <= 0.05;
-    // a column that keeps a cosine it cannot shed counts with it in full
-    a.d[b.d + 1 + j] = last ? (moves ? cosm : cosm + 1.0) : 0.0;
+    // 2 more for a column that keeps the cosine
+    a.d[b.d + 1 + j] = last ? (moves ? cosm : cosm + 2.0) : 0.0;
     a.d[b.d + 1 + n + j] = moves ? 1.0 : 0.0;
   }
 }
@@ -938,20 +945,32 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
   if (tid == 0) {
     const double s1 = sig[perm[0]];
     bool bad = !(s1 > 0.0);
-    for (int c = 0; c < b.k; ++c) {
+    // the other sound columns: what the binary32 stages leave (their limit is 4
+    // sqrt(n) 2^-24), else they ran out of sweeps
+    const double left = 16.0 * sqrt((double)n) * 5.9604644775390625e-8;
+    for (int c = 0; c < n; ++c) {
       const int j = perm[c];
-      bad = bad || !(sig[j] >= kKeptLevel * s1) || !(a.d[b.d + 1 + j] <= kOpenCos);
+      const double cs = a.d[b.d + 1 + j];
+      if (c < b.k) bad = bad || !(sig[j] >= kKeptLevel * s1) || !(cs <= kOpenCos);
+      else if (sig[j] >= kSoundLevel * s1) bad = bad || !((cs >= 2.0 ? cs - 2.0 : cs) <= left);
     }
     if (bad) {
       a.flags[b.flag] = 1;
       atomicAdd(a.flags - 1, 1);
     }
   }
-  if (b.VT && b.kind != 0) {
+  if (has_vt(b)) {
+    // matrix 3: the right vectors in its columns; which of them are sound
+    double2* W = mat(a, b, 3);
     for (int64_t idx = tid; idx < (int64_t)n * n; idx += 256) {
-      const int c = (int)(idx % n), r = (int)(idx / n), j = perm[c];
+      const int c = (int)(idx / n), r = (int)(idx % n), j = perm[c];
       const double2 v = A[r + (int64_t)j * n], p = phs[j];
-      b.VT[c + r * b.ldvt] = sig[j] > 0.0 ? (v.x * p.x - v.y * p.y) / sig[j] : 0.0;
+      W[idx] = make_double2(sig[j] > 0.0 ? (v.x * p.x - v.y * p.y) / sig[j] : 0.0, 0.0);
+    }
+    __syncthreads();                 // (the cosines have been read)
+    if (tid < n) {
+      const double s = sig[perm[tid]];
+      a.d[b.d + 1 + tid] = s >= kSoundLevel * sig[perm[0]] && s > 0.0 ? 1.0 : s > 0.0 ? 0.5 : 0.0;
     }
   }
   if (b.k == 0) return;
@@ -986,6 +1005,81 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
                          ((col % kTile) >> 3) * kPlaneSbo + ((j0 % kStK) >> 3) * 128 +
                          (col & 7) * 16;
     store_digits<kSB>(w, dst, kPlaneB);
+  }
+}
+
+// Windows: all right vectors orthonormal to binary64 rounding, although only
+// the kept columns are diagonalised to that.  Sound ones by two Newton-Schulz
+// steps, W <- W (I - E / 2) with E = W^T W - I among them (cosines of binary32
+// rounding square in each); then those of rounding-level values, one after the
+// other, against all before them.
+__global__ void __launch_bounds__(256) bg_ortho_kernel(BG a) {
+  const GramBin b = a.bins[blockIdx.y];
+  if (!has_vt(b)) return;
+  const int n = b.Nb;
+  const double2* G = mat(a, b, 4);
+  double2* B = mat(a, b, 5);
+  const double* sound = a.d + b.d + 1;
+  for (int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x; idx < (int64_t)n * n; idx += (int64_t)gridDim.x * 256) {
+    const int i = (int)(idx % n), j = (int)(idx / n);
+    const double one = i == j ? 1.0 : 0.0;
+    B[idx] = make_double2(sound[i] == 1.0 && sound[j] == 1.0 ? one - 0.5 * (G[idx].x - one) : one, 0.0);
+  }
+}
+
+__global__ void __launch_bounds__(256) bg_vt_kernel(BG a) {
+  __shared__ double v[128], cf[128], s_norm;
+  const GramBin b = a.bins[blockIdx.x];
+  if (!has_vt(b)) return;
+  const int n = b.Nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double2* W = mat(a, b, 3);
+  const double* sound = a.d + b.d + 1;
+  int unit = 0;                            // next unit vector to try
+  for (int c = 0; c < n; ++c) {
+    if (sound[c] != 0.5) continue;         // (rows of exactly zero values stay zero)
+    if (tid < n) v[tid] = W[tid + (int64_t)c * n].x;
+    __syncthreads();
+    for (;;) {
+      for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 4
+        for (int q = warp; q < c; q += 8) {
+          double d = 0.0;
+          for (int i = lane; i < n; i += 32) d = fma(W[i + (int64_t)q * n].x, v[i], d);
+          d = warp_sum(d);
+          if (lane == 0) cf[q] = d;
+        }
+        __syncthreads();
+        if (tid < n) {
+          double x = v[tid];
+#pragma unroll 8
+          for (int q = 0; q < c; ++q) x = fma(-cf[q], W[tid + (int64_t)q * n].x, x);
+          v[tid] = x;
+        }
+        __syncthreads();
+      }
+      if (warp == 0) {
+        double s = 0.0;
+        for (int i = lane; i < n; i += 32) s = fma(v[i], v[i], s);
+        s = warp_sum(s);
+        if (lane == 0) s_norm = sqrt(s);
+      }
+      __syncthreads();
+      const double nn = s_norm;
+      if (nn > 0.5 / sqrt((double)n) || unit >= n) {
+        if (tid < n) W[tid + (int64_t)c * n].x = nn > 0.0 ? v[tid] / nn : 0.0;
+        break;
+      }
+      // it lay among those before it (of n unit vectors one is left with 1 / sqrt(n) or more)
+      __syncthreads();
+      if (tid < n) v[tid] = tid == unit ? 1.0 : 0.0;
+      ++unit;
+      __syncthreads();
+    }
+    __syncthreads();
+  }
+  for (int64_t idx = tid; idx < (int64_t)n * n; idx += 256) {
+    const int c = (int)(idx % n), r = (int)(idx / n);
+    b.VT[c + r * b.ldvt] = W[r + (int64_t)c * n].x;
   }
 }
 
@@ -1118,6 +1212,8 @@ size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems) {
 // Units of about equal cost, about four waves of them: an item's tiles (cost
 // tiles x rows) are cut into row ranges.
 void batched_gram_units(BatchedGramPlan& p, int sms) {
+  p.any_vt = false;
+  for (const GramBin& b : p.bins) p.any_vt = p.any_vt || (b.kind != 0 && b.VT);
   p.pro.clear();
   p.gram.clear();
   p.mod.clear();
@@ -1251,11 +1347,11 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
       cfg.numAttrs = 1;
       return cudaLaunchKernelEx(&cfg, bg_jacobi32_kernel, ac);
     };
-    auto gemm = [&](const ZGemm& x) {
-      bg_gemm_kernel<<<dim3(tiles, tiles, ni), 128, 0, st>>>(ac, ZGemms{{x, x}, 1});
+    auto gemm = [&](const ZGemm& x, bool vt_only = false) {
+      bg_gemm_kernel<<<dim3(tiles, tiles, ni), 128, 0, st>>>(ac, ZGemms{{x, x}, 1, vt_only});
     };
     auto gemm2 = [&](const ZGemm& x, const ZGemm& y) {
-      bg_gemm_kernel<<<dim3(tiles, tiles, 2 * ni), 128, 0, st>>>(ac, ZGemms{{x, y}, 2});
+      bg_gemm_kernel<<<dim3(tiles, tiles, 2 * ni), 128, 0, st>>>(ac, ZGemms{{x, y}, 2, false});
     };
     if ((e = stage()) != cudaSuccess) return e;
     bg_widen_kernel<<<dim3(el, ni), 256, 0, st>>>(ac);
@@ -1274,8 +1370,16 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
       gemm(ZGemm{0, T4, T2, T1, T0, 0.5, 1.0});               // Q
       gemm2(ZGemm{0, Ai, T0, -1, Ao, 1.0, 0.0}, ZGemm{0, Vi, T0, -1, Vo, 1.0, 0.0});
     }
+    bg_finalize_kernel<<<ni, 256, 0, st>>>(ac);
+    if (p.any_vt) {
+      for (int it = 0; it < 2; ++it) {
+        gemm(ZGemm{1, it ? T3 : T0, it ? T3 : T0, -1, T1, 1.0, 0.0}, true);      // W^T W
+        bg_ortho_kernel<<<dim3(el, ni), 256, 0, st>>>(ac);
+        gemm(ZGemm{0, it ? T3 : T0, T2, -1, it ? T0 : T3, 1.0, 0.0}, true);
+      }
+      bg_vt_kernel<<<ni, 256, 0, st>>>(ac);
+    }
   }
-  bg_finalize_kernel<<<nb, 256, 0, st>>>(a);
   if (!p.mod.empty()) {
     au.units = units + 2 * m;
     bg_modes_kernel<<<(unsigned)p.mod.size(), kThreads, msmem, st>>>(au);

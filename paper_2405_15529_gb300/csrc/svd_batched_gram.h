@@ -47,6 +47,7 @@ struct BatchedGramPlan {
   std::vector<GramBin> bins;       // offsets by the plan, pointers by bind
   std::vector<GramUnit> pro, gram, mod;   // prologue, Gram and modes units
   int nitems = 0, maxNb = 0, maxpairs = 0;
+  bool any_vt = false;             // right vectors of some window are asked for
   size_t off_bins = 0, off_units = 0, off_i = 0, off_g = 0, off_z = 0, off_f = 0, off_c = 0, off_d = 0, off_r = 0, off_flags = 0;
   int64_t n_i = 0, n_g = 0, n_z = 0, n_f = 0, n_c = 0, n_d = 0, n_r = 0;
 };
