@@ -1118,6 +1118,9 @@ extern "C" pylom_status pylom_svd_batched_plan(int nbins, const int64_t* N, cons
   p->nA = (int)p->itemsA.size();
   p->total_y = y; p->total_z = z; p->total_u = u; p->total_s = sacc;
   cudaError_t e = (prec == PYLOM_PREC_FP64) ? batched_grid<double>(&p->grid) : batched_grid<float>(&p->grid);
+  int dev = 0, sms = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) {
     set_error_message("pylom_svd_batched_plan: %s", cudaGetErrorString(e));
     delete p;
@@ -1133,7 +1136,7 @@ extern "C" pylom_status pylom_svd_batched_plan(int nbins, const int64_t* N, cons
   p->off_f = off;     off += align256(sizeof(float2) * (size_t)(fz > 0 ? fz : 1));
   p->off_y = off;     off += align256(ye * (size_t)y);
   p->off_scr = off;   off += align256(sizeof(double2) * (size_t)p->grid * 2 * kMaxNb * kMaxK);
-  off = batched_gram_layout(p->gram, off, nbins);
+  off = batched_gram_layout(p->gram, off, nbins, sms);
   p->bytes = off;
   *plan_out = p;
   *ws_bytes = off;
@@ -1285,13 +1288,10 @@ static pylom_status batched_upload_tables(pylom_batched_plan* plan, void* ws, vo
     g.mean = b.mean;
   }
   if (e == cudaSuccess) {
-    int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // (the lists of units are host memory: an allocation that fails must not
     // leave this C entry as an exception)
     try {
-      if (e == cudaSuccess) batched_gram_units(plan->gram, sms);
+      if (e == cudaSuccess) batched_gram_units(plan->gram);
       if (e == cudaSuccess)
         e = batched_gram_upload(plan->gram, base, plan->forced.data(), (int)plan->forced.size(), st);
     } catch (const std::bad_alloc&) {

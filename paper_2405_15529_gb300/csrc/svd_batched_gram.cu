@@ -21,8 +21,8 @@
 // sound column that the binary32 stages left open; a zero matrix) are flagged on the device and left to that kernel.
 //
 // Persistent kernel -> here: 24 bins (N 16k..262k, Nb 16..128, 1.3 GB) 374 ->
-// 13.5 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.9 ms, SPOD of 131072 x
-// 1056 25.6 -> 7.4 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
+// 13.1 ms, 12 windows (N 16k..262k, M 16..96) 119 -> 4.8 ms, SPOD of 131072 x
+// 1056 25.6 -> 7.3 ms; modes within 2.5e-8 of binary64 (2.4e-7 before).
 #include <algorithm>
 
 #include "digits.cuh"
@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(256) bg_prologue_kernel(BG a) {
   __shared__ int sE[128];
   __shared__ RowTops tops;
   const GramUnit u = a.units[blockIdx.x];
+  if (u.bin < 0) return;
   const GramBin b = a.bins[u.bin];
   int bad = 0;
   if (b.kind == 0) {
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(256) bg_rows_kernel(BG a) {
   constexpr int kNone = -2147483647;
   __shared__ int s_lo, s_hi;
   const GramUnit u = a.units[blockIdx.x];
+  if (u.bin < 0) return;
   const GramBin b = a.bins[u.bin];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
@@ -339,6 +341,7 @@ __global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_gram_kernel(BG
   __shared__ __align__(8) DigitBarriers<kNstB, kG> bar;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const GramUnit u = a.units[blockIdx.x];
+  if (u.bin < 0) return;
   const GramBin b = a.bins[u.bin];
   const int mode = u.mode, J = u.J;
   // a thread: 8 rows of one left column, and in two of the eight warps, in turn
@@ -1012,7 +1015,7 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
 // the kept columns are diagonalised to that.  Sound ones by two Newton-Schulz
 // steps, W <- W (I - E / 2) with E = W^T W - I among them (cosines of binary32
 // rounding square in each); then those of rounding-level values, one after the
-// other, against all before them.
+// other, against all before them.  0.18 of 4.8 ms for 12 windows.
 __global__ void __launch_bounds__(256) bg_ortho_kernel(BG a) {
   const GramBin b = a.bins[blockIdx.y];
   if (!has_vt(b)) return;
@@ -1090,6 +1093,7 @@ __global__ void __launch_bounds__(kThreads, Shape<kG>::BLOCKS) bg_modes_kernel(B
   __shared__ __align__(8) DigitBarriers<kNstB, kG> bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const GramUnit u = a.units[blockIdx.x];
+  if (u.bin < 0) return;
   const GramBin b = a.bins[u.bin];
   const int n = b.Nb, stages = (n + kStK - 1) / kStK;
   const int rl = tid & 127, kh = tid >> 7;
@@ -1188,17 +1192,25 @@ void batched_gram_add(BatchedGramPlan& p, int item, int64_t N, int64_t Nb, int64
   p.maxpairs = std::max(p.maxpairs, b.Mb / kZW);
 }
 
-// Units hold at most this many per item: the tables' sizes must not depend on
-// what bind learns (real or complex items).
-static int64_t max_units(int64_t nitems) { return 16 * nitems + 2048; }
+static int column_blocks(int n) { return (n + kTile - 1) / kTile; }
 
-size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems) {
+size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems, int sms) {
   const int64_t nb = (int64_t)p.bins.size();
   p.nitems = nitems;
+  // about four waves of units, and a tile's share rounded up (complex items have the most tiles)
+  p.want = 8 * (int64_t)sms;
+  p.n_pro = p.n_gram = p.n_mod = p.want;
+  for (const GramBin& b : p.bins) {
+    const int n = column_blocks(b.Nb);
+    p.n_pro += 1;
+    p.n_gram += n + (n > 2 ? n - 2 : 0);
+    p.n_mod += column_blocks(2 * b.k);
+  }
+  if (p.n_mod == p.want) p.n_mod = 0;      // no modes
   p.off_flags = off; off += align256(sizeof(int) * ((size_t)nitems + 1) * 2);
   if (nb == 0) return off;
   p.off_bins = off;  off += align256(sizeof(GramBin) * (size_t)nb);
-  p.off_units = off; off += align256(sizeof(GramUnit) * 3 * (size_t)max_units(nb));
+  p.off_units = off; off += align256(sizeof(GramUnit) * (size_t)(p.n_pro + p.n_gram + p.n_mod));
   p.off_i = off;     off += align256(sizeof(int) * (size_t)p.n_i);
   p.off_g = off;     off += align256(sizeof(long long) * (size_t)p.n_g);
   p.off_z = off;     off += align256(sizeof(double2) * (size_t)p.n_z);
@@ -1211,36 +1223,33 @@ size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems) {
 
 // Units of about equal cost, about four waves of them: an item's tiles (cost
 // tiles x rows) are cut into row ranges.
-void batched_gram_units(BatchedGramPlan& p, int sms) {
-  p.any_vt = false;
+void batched_gram_units(BatchedGramPlan& p) {
   for (const GramBin& b : p.bins) p.any_vt = p.any_vt || (b.kind != 0 && b.VT);
   p.pro.clear();
   p.gram.clear();
   p.mod.clear();
   double total = 0.0, mtotal = 0.0, ptotal = 0.0;
-  auto blocks = [](int n) { return (n + kTile - 1) / kTile; };      // column blocks
   auto passes = [&](const GramBin& b) {
-    return b.Nb <= 64 ? blocks(b.Nb) : 2 + (blocks(b.Nb) - 2) * (b.cplx ? 2 : 1);
+    return b.Nb <= 64 ? column_blocks(b.Nb) : 2 + (column_blocks(b.Nb) - 2) * (b.cplx ? 2 : 1);
   };
-  auto mtiles = [&](const GramBin& b) { return blocks(b.cplx ? 2 * b.k : b.k); };
+  auto mtiles = [&](const GramBin& b) { return column_blocks(b.cplx ? 2 * b.k : b.k); };
   auto mcost = [](const GramBin& b) { return (double)((b.Nb + kStK - 1) / kStK); };
   for (const GramBin& b : p.bins) {
     total += (double)b.rows * passes(b);
     if (b.k > 0) mtotal += (double)b.rows * mcost(b) * mtiles(b);
     ptotal += (double)b.rows * b.Nb;
   }
-  const int64_t cap = max_units((int64_t)p.bins.size()) - 8 * (int64_t)p.bins.size();
-  const double want = (double)std::min<int64_t>(8 * (int64_t)sms, cap / 2);
+  const double want = (double)p.want;
   for (size_t f = 0; f < p.bins.size(); ++f) {
     const GramBin& b = p.bins[f];
     const int64_t sums = (b.rows + 127) / 128;
     auto cut = [&](std::vector<GramUnit>& v, double share, int mode, int J, int64_t n) {
-      int64_t s = (int64_t)(share + 0.5);
+      int64_t s = (int64_t)share;          // (rounded down: no fifth wave of a few blocks)
       s = std::max<int64_t>(1, std::min(s, n));
       for (int64_t i = 0; i < s; ++i) v.push_back(GramUnit{(int)f, mode, J, 0, n * i / s, n * (i + 1) / s});
     };
     const double share = want * (double)b.rows / total;
-    for (int J = 0; J < blocks(b.Nb); ++J) {
+    for (int J = 0; J < column_blocks(b.Nb); ++J) {
       cut(p.gram, share, J < 2 ? kPacked : kPlain, J, sums);
       if (J >= 2 && b.cplx) cut(p.gram, share, kTurned, J, sums);
     }
@@ -1273,15 +1282,18 @@ cudaError_t batched_gram_upload(const BatchedGramPlan& p, char* ws, const int* f
                                   sizeof(int) * fl.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess || p.bins.empty()) return e;
-  const size_t m = (size_t)max_units((int64_t)p.bins.size());
   e = cudaMemcpyAsync(ws + p.off_bins, p.bins.data(), sizeof(GramBin) * p.bins.size(), cudaMemcpyHostToDevice, st);
+  // (a few rounded shares may leave fewer units than there is room for)
+  std::vector<GramUnit> all;
   const std::vector<GramUnit>* lists[3] = {&p.pro, &p.gram, &p.mod};
-  for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
-    if (lists[i]->size() > m) return cudaErrorInvalidValue;
-    if (!lists[i]->empty())
-      e = cudaMemcpyAsync(ws + p.off_units + sizeof(GramUnit) * m * i, lists[i]->data(),
-                          sizeof(GramUnit) * lists[i]->size(), cudaMemcpyHostToDevice, st);
+  const int64_t room[3] = {p.n_pro, p.n_gram, p.n_mod};
+  for (int i = 0; i < 3; ++i) {
+    if ((int64_t)lists[i]->size() > room[i]) return cudaErrorInvalidValue;
+    all.insert(all.end(), lists[i]->begin(), lists[i]->end());
+    all.resize(all.size() + (size_t)(room[i] - (int64_t)lists[i]->size()), GramUnit{-1, 0, 0, 0, 0, 0});
   }
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ws + p.off_units, all.data(), sizeof(GramUnit) * all.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e;
 }
@@ -1289,7 +1301,6 @@ cudaError_t batched_gram_upload(const BatchedGramPlan& p, char* ws, const int* f
 cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, double* S, cudaStream_t st) {
   if (p.bins.empty()) return cudaSuccess;
   cudaError_t e;
-  const size_t m = (size_t)max_units((int64_t)p.bins.size());
   BG a{};
   a.bins = (const GramBin*)(ws + p.off_bins);
   const GramUnit* units = (const GramUnit*)(ws + p.off_units);
@@ -1319,10 +1330,10 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
   if (e != cudaSuccess) return e;
   BG au = a;
   au.units = units;
-  bg_prologue_kernel<<<(unsigned)p.pro.size(), 256, 0, st>>>(au);
-  if (!p.mod.empty()) bg_rows_kernel<<<(unsigned)p.pro.size(), 256, 0, st>>>(au);
-  au.units = units + m;
-  bg_gram_kernel<<<(unsigned)p.gram.size(), kThreads, smem, st>>>(au);
+  bg_prologue_kernel<<<(unsigned)p.n_pro, 256, 0, st>>>(au);
+  if (p.n_mod) bg_rows_kernel<<<(unsigned)p.n_pro, 256, 0, st>>>(au);
+  au.units = units + p.n_pro;
+  bg_gram_kernel<<<(unsigned)p.n_gram, kThreads, smem, st>>>(au);
   bg_chol_kernel<<<nb, kCholThreads, csmem, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned tiles = (unsigned)((p.maxNb + 7) / 8), el = (unsigned)std::max(1, p.maxNb * p.maxNb / 2048);
@@ -1380,9 +1391,9 @@ cudaError_t batched_gram_run(const BatchedGramPlan& p, char* ws, WsHeader* hdr, 
       bg_vt_kernel<<<ni, 256, 0, st>>>(ac);
     }
   }
-  if (!p.mod.empty()) {
-    au.units = units + 2 * m;
-    bg_modes_kernel<<<(unsigned)p.mod.size(), kThreads, msmem, st>>>(au);
+  if (p.n_mod) {
+    au.units = units + p.n_pro + p.n_gram;
+    bg_modes_kernel<<<(unsigned)p.n_mod, kThreads, msmem, st>>>(au);
   }
   return cudaGetLastError();
 }

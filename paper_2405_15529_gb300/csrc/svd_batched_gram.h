@@ -36,7 +36,7 @@ struct GramBin {
 };
 constexpr int kBinMats = 8;   // A, V, A2, T0, T1, T2, T3, T4
 
-// A piece of an item's work: kind of tile, its column block, a row range.
+// A piece of an item's work: kind of tile, its column block, a row range (bin < 0: none).
 struct GramUnit {
   int bin, mode, J, pad_;
   int64_t q0, q1;
@@ -47,16 +47,20 @@ struct BatchedGramPlan {
   std::vector<GramBin> bins;       // offsets by the plan, pointers by bind
   std::vector<GramUnit> pro, gram, mod;   // prologue, Gram and modes units
   int nitems = 0, maxNb = 0, maxpairs = 0;
-  bool any_vt = false;             // right vectors of some window are asked for
+  bool any_vt = false;             // some bind has asked for a window's right vectors
+  // A plan may be bound to several workspaces, to bins in one and windows in
+  // another: run launches what holds for all of them.  Units wanted, and the
+  // lengths of the three lists (filled up with empty units).
+  int64_t want = 0, n_pro = 0, n_gram = 0, n_mod = 0;
   size_t off_bins = 0, off_units = 0, off_i = 0, off_g = 0, off_z = 0, off_f = 0, off_c = 0, off_d = 0, off_r = 0, off_flags = 0;
   int64_t n_i = 0, n_g = 0, n_z = 0, n_f = 0, n_c = 0, n_d = 0, n_r = 0;
 };
 
 // Adds an item (N x Nb, kmodes modes) and, at the end, the sections to the workspace.
 void batched_gram_add(BatchedGramPlan& p, int item, int64_t N, int64_t Nb, int64_t k, int64_t s_off);
-size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems);
+size_t batched_gram_layout(BatchedGramPlan& p, size_t off, int nitems, int sms);
 // Row units once the items' row counts are known (after bind).
-void batched_gram_units(BatchedGramPlan& p, int sms);
+void batched_gram_units(BatchedGramPlan& p);
 cudaError_t batched_gram_upload(const BatchedGramPlan& p, char* ws, const int* forced, int nitems, cudaStream_t st);
 // Runs the route; afterwards flags[i] != 0 marks the items that the
 // Householder route has to do (given at upload, or found to need it).
