@@ -356,12 +356,9 @@ extern "C" size_t pylom_pod_backward_workspace_size(int64_t N, int64_t M, int64_
   if (!tall_shape_ok(N, M, leaf_rows) || r < 0 || r > M) return 0;
   if (prec != PYLOM_PREC_FP64 && prec != PYLOM_PREC_MIXED_3XTF32) return 0;
   const int64_t P = leaves_of(N, M, leaf_rows, prec);
-  // the forward's r_max enters the layout last, so any value gives the same
-  // offsets of what is refactored: r is at most r_max
-  return pod_backward_bytes(N, M, P, r) +
-         (leaf_rows == 0 ? pod_refactor_bytes(N, M, P, 0, prec == PYLOM_PREC_MIXED_3XTF32) +
-                               pod_backward_gram_bytes(N, M, r)
-                         : 0);
+  const bool mixed = prec == PYLOM_PREC_MIXED_3XTF32;
+  return pod_backward_bytes(N, M, P, r, leaf_rows == 0, mixed) +
+         (leaf_rows == 0 ? pod_refactor_bytes(N, M, P, mixed) + pod_backward_gram_bytes(N, M, r) : 0);
 }
 
 extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_bytes, int64_t N, int64_t M,
@@ -403,6 +400,7 @@ extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_byt
   char* extra = mixed ? p2 + svd_state_bytes(M) + align256(sizeof(double) * (size_t)M * M) : nullptr;
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(WsHeader), st);
   if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward: header clear");
+  double* chunk = nullptr;
   if (leaf_rows == 0) {
     // the forward may have left Y unfactored (its header says so): then the
     // form with two products of Y does the call, where the singular values
@@ -415,24 +413,23 @@ extern "C" pylom_status pylom_pod_backward(const void* fwd_ws, size_t fwd_ws_byt
     gs.f32 = mixed;
     gram_carve(gs, p2 + svd_state_bytes(M) + align256(sizeof(double) * (size_t)M * M) +
                        (mixed ? mixed_extra_bytes(N, M, P) : 0), M, r_max);
-    char* bws = (char*)ws + pod_backward_bytes(N, M, P, r);
-    void* dY = pod_backward_dy((char*)ws, N, M, P, r);
+    char* bws = (char*)ws + pod_backward_bytes(N, M, P, r, true, mixed);
+    void* dY = pod_backward_dy((char*)ws, N, M, P, r, true);
     e = launch_pod_backward_gram(gs, (WsHeader*)ws, S, VT, ldvt, dU, lddu, dS, dVT, lddvt, w,
-                                 mode_kind == PYLOM_MODES_PHYSICAL, r, dY, bws + pod_refactor_bytes(N, M, P, 0, mixed),
-                                 st);
+                                 mode_kind == PYLOM_MODES_PHYSICAL, r, pod_backward_du((char*)ws), dY,
+                                 bws + pod_refactor_bytes(N, M, P, mixed), st);
     if (e == cudaSuccess)
       e = launch_bw_finalize_gram(dY, mixed, w, remove_mean, dX, lddx, dxtype, N, M, &((WsHeader*)ws)->gram_redo, st);
     if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward");
     TsqrState os;
-    fs.rmax = 0;
     double* UR2 = nullptr;
-    e = launch_refactor(fs, gs, extra, bws, (WsHeader*)ws, mixed, UR, S, VT, ldvt, os, &extra, &UR2, st);
+    e = launch_refactor(fs, gs, extra, bws, dY, (WsHeader*)ws, mixed, UR, S, VT, ldvt, os, &extra, &UR2, &chunk, st);
     if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward: factorisation");
     fs = os;
     UR = UR2;
   }
   e = launch_pod_backward(fs, UR, S, VT, ldvt, dU, lddu, dS, dVT, lddvt, w, remove_mean,
-                          mode_kind == PYLOM_MODES_PHYSICAL, r, dX, lddx, dxtype, (char*)ws, extra, st);
+                          mode_kind == PYLOM_MODES_PHYSICAL, r, dX, lddx, dxtype, (char*)ws, extra, chunk, st);
   if (e != cudaSuccess) return cuda_fail(e, "pylom_pod_backward");
   return PYLOM_OK;
 }

@@ -82,9 +82,10 @@ cudaError_t launch_product(const ProductArgs& p, bool f32, void* U, int64_t ldu,
 // The adjoint without reflectors (pod_backward_gram.cu); `f` the forward's
 // state.  hdr->gram_redo = 1 afterwards: nothing was done.
 size_t pod_backward_gram_bytes(int64_t N, int64_t M, int64_t r);
+// Z: room for y_ld(N) max(r, 1) doubles.
 cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const double* S, const double* VT, int64_t ldvt,
                                      const double* dU, int64_t lddu, const double* dS, const double* dVT,
-                                     int64_t lddvt, const double* w, int physical, int64_t r, void* dY, char* base,
+                                     int64_t lddvt, const double* w, int physical, int64_t r, void* Z, void* dY, char* base,
                                      cudaStream_t st);
 // pod_backward.cu: C = alpha op(A) op(B) + beta C, and C = diag(1 / S) VT (rows of them), unless *unless
 cudaError_t launch_bw_gemm(int ta, int tb, int64_t m, int64_t n, int64_t k, double alpha, const double* A, int64_t lda,

@@ -47,7 +47,7 @@ struct TsqrState {
   // given and *gram_y is 0, the factorisation is the forward's, `shift`
   // (mixed extra region: `shiftx`) bytes away from these pointers
   const unsigned* gram_y;
-  int64_t shift, shiftx;
+  int64_t shift, shiftx, shifty;   // (Y lies apart: shifty)
   // if given, the kernels on this state do nothing while *run_if is 0 (the
   // Householder route behind the Gram route of the same call)
   const unsigned* run_if;
@@ -68,7 +68,7 @@ __device__ __forceinline__ void shift_ptr(T*& p, int64_t bytes) {
 }
 __device__ __forceinline__ void select_factors(TsqrState& s) {
   if (!already_factored(s)) return;
-  shift_ptr(s.Y, s.shift);
+  shift_ptr(s.Y, s.shifty);
   shift_ptr(s.tau, s.shift);
   shift_ptr(s.T, s.shift);
   shift_ptr(s.Rs, s.shift);
@@ -169,21 +169,26 @@ cudaError_t launch_frame(const TsqrState& s, const double* S, const double* VT, 
 
 // Adjoint of the POD path (pod_backward.cu).  fs: the forward's TSQR state
 // (reflectors, T, tree); UR/S/VT: the forward's small-SVD factors.
-size_t pod_backward_bytes(int64_t N, int64_t M, int64_t P, int64_t r);
+// `unfactored`: the forward may have left Y so (automatic leaf height); the
+// region of dY then also has room for a factorisation of Y.
+size_t pod_backward_bytes(int64_t N, int64_t M, int64_t P, int64_t r, bool unfactored, bool mixed);
 cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const double* S, const double* VT,
                                 int64_t ldvt, const double* dU, int64_t lddu, const double* dS,
                                 const double* dVT, int64_t lddvt, const double* w, int remove_mean,
                                 int physical, int64_t r, void* dX, int64_t lddx, int dxtype,
-                                char* bw_base, char* mixed_extra, cudaStream_t st);
-// Room in the backward's workspace for a factorisation of the forward's Y
-// (forwards with the automatic leaf height may have left Y unfactored), and
-// its state: os (and *extra, mixed path) in the backward's workspace.
-void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r);
-size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed);
+                                char* bw_base, char* mixed_extra, double* chunk, cudaStream_t st);
+// The factorisation of a Y that the forward left unfactored: besides the
+// reflectors, in the region of dY, its state os (and *extra, mixed path) and
+// *chunk (binary64): room for kBwChunk columns of dY, since dY has to be
+// formed beside the reflectors.
+constexpr int64_t kBwChunk = 16;
+void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r, bool unfactored);
+void* pod_backward_du(char* base);
+size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, bool mixed);
 struct GramState;
-cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
-                            const double* UR, const double* S, const double* VT, int64_t ldvt, TsqrState& os,
-                            char** extra, double** UR_out, cudaStream_t st);
+cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, void* dY,
+                            WsHeader* hdr, bool mixed, const double* UR, const double* S, const double* VT, int64_t ldvt,
+                            TsqrState& os, char** extra, double** UR_out, double** chunk, cudaStream_t st);
 // Mixed-precision adjoint support (tsqr_mixed.cu): per leaf C := Q_leaf^T C
 // (FP32, ld N) on tcgen05, top M rows into the binary64 slots Z.
 cudaError_t launch_leaf_qt_mixed(const TsqrState& s, char* extra, float* C, int64_t r, double* Z, cudaStream_t st);

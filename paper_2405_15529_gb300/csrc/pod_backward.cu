@@ -240,23 +240,37 @@ __global__ void __launch_bounds__(256) bw_add_du_c_f32_kernel(const float* C, co
   }
 }
 
-size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, bool mixed) {
-  return align256(sizeof(double) * (size_t)M * M) + align256(sizeof(double) * frame_doubles(M)) +
-         tsqr_state_bytes(N, M, P, r_max, !mixed) + (mixed ? mixed_extra_bytes(N, M, P) : 0);
+static size_t refactor_state(int64_t M) {
+  return align256(sizeof(double) * (size_t)M * M) + align256(sizeof(double) * frame_doubles(M));
 }
 
-cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, WsHeader* hdr, bool mixed,
-                            const double* UR, const double* S, const double* VT, int64_t ldvt, TsqrState& os,
-                            char** extra, double** UR_out, cudaStream_t st) {
+size_t pod_refactor_bytes(int64_t N, int64_t M, int64_t P, bool mixed) {
+  return refactor_state(M) + tsqr_state_bytes(N, M, P, 0, false) +
+         (mixed ? 0 : align256(sizeof(double) * (size_t)N * (M < kBwChunk ? M : kBwChunk)));
+}
+
+// (mixed: the binary32 dY fills half of its region, the copy of Y the rest)
+static size_t mixed_dy_bytes(int64_t N, int64_t M) { return align256(sizeof(float) * (size_t)N * M); }
+
+cudaError_t launch_refactor(const TsqrState& fs, const GramState& g, const char* fwd_extra, char* base, void* dY,
+                            WsHeader* hdr, bool mixed, const double* UR, const double* S, const double* VT, int64_t ldvt,
+                            TsqrState& os, char** extra, double** UR_out, double** chunk, cudaStream_t st) {
   double* scratch = (double*)(base + align256(sizeof(double) * (size_t)fs.M * fs.M));
-  char* own = (char*)scratch + align256(sizeof(double) * frame_doubles(fs.M));
-  char* oextra = mixed ? own + tsqr_state_bytes(fs.N, fs.M, fs.P, fs.rmax, false) : nullptr;
-  tsqr_state_carve(os, own, fs.N, fs.M, fs.P, fs.rmax, !mixed);
+  char* own = base + refactor_state(fs.M);
+  char* oextra = mixed ? (char*)dY + mixed_dy_bytes(fs.N, fs.M) : nullptr;
+  tsqr_state_carve(os, own, fs.N, fs.M, fs.P, 0, false);
   os.hdr = hdr;
   os.run_if = &hdr->gram_redo;
   os.gram_y = &fs.hdr->gram_y;
   os.shift = (const char*)fs.tau - (const char*)os.tau;
   os.shiftx = mixed ? fwd_extra - oextra : 0;
+  *chunk = nullptr;
+  if (!mixed) {
+    os.Y = (double*)dY;
+    os.ldy = fs.ldy;
+    os.shifty = (const char*)fs.Y - (const char*)os.Y;
+    *chunk = (double*)(own + tsqr_state_bytes(fs.N, fs.M, fs.P, 0, false));
+  }
   cudaError_t e = cudaMemsetAsync(os.arrive, 0, sizeof(unsigned) * (size_t)os.P, st);
   if (e != cudaSuccess) return e;
   // (the leaves' own pass over Y is in place: Y is both source and destination)
@@ -282,21 +296,31 @@ struct BwLayout {
   double* dY;     // N x M
 };
 
-size_t pod_backward_bytes(int64_t N, int64_t M, int64_t P, int64_t r) {
+// Bytes of the regions of dU (its padded copy on the Gram route) and of dY
+static size_t du_bytes(int64_t N, int64_t r, bool unfactored) {
+  return align256(sizeof(double) * (size_t)(unfactored ? y_ld(N) * (r > 0 ? r : 1) : N * r));
+}
+static size_t dy_bytes(int64_t N, int64_t M, int64_t P, bool unfactored, bool mixed) {
+  const size_t b = align256(sizeof(double) * (size_t)(unfactored ? y_ld(N) : N) * M);
+  const size_t c = unfactored && mixed ? mixed_dy_bytes(N, M) + mixed_extra_bytes(N, M, P) : 0;
+  return b > c ? b : c;
+}
+
+size_t pod_backward_bytes(int64_t N, int64_t M, int64_t P, int64_t r, bool unfactored, bool mixed) {
   size_t b = sizeof(WsHeader);
-  b += align256(sizeof(double) * (size_t)N * r);
+  b += du_bytes(N, r, unfactored);
   b += align256(sizeof(double) * (size_t)P * M * r);
   b += align256(sizeof(double) * (size_t)P * M * M);
   b += 5 * align256(sizeof(double) * (size_t)M * M);
   b += align256(sizeof(double) * (size_t)r * M);
-  b += align256(sizeof(double) * (size_t)N * M);
+  b += dy_bytes(N, M, P, unfactored, mixed);
   return b;
 }
 
-static BwLayout carve_backward(char* base, int64_t N, int64_t M, int64_t P, int64_t r) {
+static BwLayout carve_backward(char* base, int64_t N, int64_t M, int64_t P, int64_t r, bool unfactored) {
   BwLayout L;
   char* p = base + sizeof(WsHeader);
-  L.C = (double*)p;  p += align256(sizeof(double) * (size_t)N * r);
+  L.C = (double*)p;  p += du_bytes(N, r, unfactored);
   L.Z = (double*)p;  p += align256(sizeof(double) * (size_t)P * M * r);
   L.B = (double*)p;  p += align256(sizeof(double) * (size_t)P * M * M);
   L.A1 = (double*)p; p += align256(sizeof(double) * (size_t)M * M);
@@ -309,9 +333,22 @@ static BwLayout carve_backward(char* base, int64_t N, int64_t M, int64_t P, int6
   return L;
 }
 
-// where the adjoint's dY (N x M) lies in the workspace
-void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r) {
-  return carve_backward(base, N, M, P, r).dY;
+// where the adjoint's dY (N x M) and its copy of dU lie in the workspace
+void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r, bool unfactored) {
+  return carve_backward(base, N, M, P, r, unfactored).dY;
+}
+void* pod_backward_du(char* base) { return base + sizeof(WsHeader); }
+
+// every row of C (rows x cols) minus its mean: the adjoint of the mean removal
+// on the coefficients of dY
+__global__ void __launch_bounds__(256) bw_center_kernel(double* C, int64_t rows, int64_t cols, const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int64_t j = 0; j < cols; ++j) s += C[i + j * rows];
+    s /= (double)cols;
+    for (int64_t j = 0; j < cols; ++j) C[i + j * rows] -= s;
+  }
 }
 
 static cudaError_t gemm(int ta, int tb, int64_t m, int64_t n, int64_t k, double alpha, const double* A,
@@ -353,10 +390,10 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
                                 int64_t ldvt, const double* dU, int64_t lddu, const double* dS,
                                 const double* dVT, int64_t lddvt, const double* w, int remove_mean,
                                 int physical, int64_t r, void* dX, int64_t lddx, int dxtype,
-                                char* bw_base, char* mixed_extra, cudaStream_t st) {
+                                char* bw_base, char* mixed_extra, double* chunk, cudaStream_t st) {
   const int64_t N = fs.N, M = fs.M, P = fs.P;
   const unsigned* run_if = fs.run_if;   // null: always
-  BwLayout L = carve_backward(bw_base, N, M, P, r);
+  BwLayout L = carve_backward(bw_base, N, M, P, r, fs.gram_y != nullptr);
   const bool mixed = mixed_extra != nullptr;   // FP32 reflectors of a mixed-precision forward
   float* C32 = (float*)L.C;
   float* dY32 = (float*)L.dY;
@@ -426,6 +463,31 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
     else
       bw_finalize_kernel<double, float><<<1024, 256, 0, st>>>(dY32, w, remove_mean, (double*)dX, lddx, N, M, run_if, 1u);
     return cudaGetLastError();
+  }
+  if (chunk) {
+    // the region of dY holds the reflectors: a few columns of dY at a time,
+    // their row means taken off the coefficients
+    if (remove_mean) {
+      bw_center_kernel<<<16, 256, 0, st>>>(L.Bm, M, M, run_if);
+      if (r > 0) bw_center_kernel<<<16, 256, 0, st>>>(L.Cm, r, M, run_if);
+    }
+    const bool add = dU && r > 0;
+    if (add) bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r, run_if);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_down_pass_fp64(ds, L.Bm, M, M, st)) != cudaSuccess) return e;
+    for (int64_t c = 0; c < M; c += kBwChunk) {
+      const int64_t n = M - c < kBwChunk ? M - c : kBwChunk;
+      TsqrState cs = ds;
+      cs.B = ds.B + c * M;
+      if ((e = launch_leaf_modes_fp64(cs, n, nullptr, 0, chunk, N, nullptr, st)) != cudaSuccess) return e;
+      if (add) bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm + c * r, r, chunk, N, n, r, run_if);
+      if (dxtype == PYLOM_F32)
+        bw_finalize_kernel<float, double><<<1024, 256, 0, st>>>(chunk, w, 0, (float*)dX + c * lddx, lddx, N, n, run_if, 1u);
+      else
+        bw_finalize_kernel<double, double><<<1024, 256, 0, st>>>(chunk, w, 0, (double*)dX + c * lddx, lddx, N, n, run_if, 1u);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
   }
   if ((e = launch_modes_fp64(ds, L.Bm, M, M, nullptr, 0, L.dY, N, nullptr, st)) != cudaSuccess) return e;
   // ... + dU_w C (dU reloaded: step 1 transformed its copy in place)

@@ -104,16 +104,16 @@ static size_t planes_only(int64_t M, int64_t r) {
 
 size_t pod_backward_gram_bytes(int64_t N, int64_t M, int64_t r) {
   const int64_t r1 = r > 0 ? r : 1;
-  return align256(sizeof(double) * (size_t)y_ld(N) * r1) + align256(sizeof(int) * (size_t)r1) + row_shift_bytes(N) +
+  return align256(sizeof(int) * (size_t)r1) + row_shift_bytes(N) +
          align256(sizeof(long long) * (size_t)5 * M * r1) + 3 * align256(sizeof(double) * (size_t)M * r1) +
          4 * align256(sizeof(double) * (size_t)M * M) + product_planes_bytes(M, r, M);
 }
 
-static BgLayout carve(char* p, int64_t N, int64_t M, int64_t r) {
+static BgLayout carve(char* p, void* Z, int64_t N, int64_t M, int64_t r) {
   const int64_t r1 = r > 0 ? r : 1;
   BgLayout L;
   const size_t mr = align256(sizeof(double) * (size_t)M * r1), mm = align256(sizeof(double) * (size_t)M * M);
-  L.Z = p;                 p += align256(sizeof(double) * (size_t)y_ld(N) * r1);
+  L.Z = Z;
   L.zE = (int*)p;          p += align256(sizeof(int) * (size_t)r1);
   L.zS = (uint16_t*)p;     p += row_shift_bytes(N);
   L.G = (long long*)p;     p += align256(sizeof(long long) * (size_t)5 * M * r1);
@@ -132,10 +132,10 @@ static BgLayout carve(char* p, int64_t N, int64_t M, int64_t r) {
 // dY (N x M, ld N, binary64 or binary32 as the forward's Y) where hdr->gram_redo stays 0.
 cudaError_t launch_pod_backward_gram(const GramState& f, WsHeader* hdr, const double* S, const double* VT, int64_t ldvt,
                                      const double* dU, int64_t lddu, const double* dS, const double* dVT,
-                                     int64_t lddvt, const double* w, int physical, int64_t r, void* dY, char* base,
+                                     int64_t lddvt, const double* w, int physical, int64_t r, void* Z, void* dY, char* base,
                                      cudaStream_t st) {
   const int64_t N = f.N, M = f.M;
-  BgLayout L = carve(base, N, M, r);
+  BgLayout L = carve(base, Z, N, M, r);
   const unsigned* redo = &hdr->gram_redo;
   if (!dU) r = 0;
   bg_route_kernel<<<1, 256, 0, st>>>(f.hdr, hdr, S, dS, M, r, f.f32 ? 0.1 * kInvertLevel : kInvertLevel);

@@ -398,7 +398,7 @@ void tsqr_state_carve(TsqrState& s, char* base, int64_t N, int64_t M, int64_t P,
   s.row0 = 0;
   s.ldy = with_y ? y_ld(N) : N;
   s.gram_y = s.run_if = nullptr;
-  s.shift = s.shiftx = 0;
+  s.shift = s.shiftx = s.shifty = 0;
 }
 
 cudaError_t launch_tsqr_fp64(const TsqrState& s, const void* X, int64_t ldx, int xtype,
