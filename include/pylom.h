@@ -138,6 +138,10 @@ pylom_status pylom_workspace_status(const void* ws, void* stream, int64_t* r, in
  *              centred data (its diagonal is non-negative) and the modes are Y
  *              V_r S_r^-1; with r_max < M and no such energy share the device
  *              takes leaves and tree instead when S_r < 1e-4 S_1 (1e-5 mixed).
+ *              Each row of such modes is accurate relative to its own norm.
+ *              They are orthonormal to the cosines at which the small SVD
+ *              stops, M 2^-53 a pair (binary64; r M 2^-53 in the norm of U^T U
+ *              - I), or to binary32 rounding, 2^-38 S_1 / S_r where that is larger (mixed).
  *              The environment variable PYLOM_TREE asks for leaves and tree too.
  *  U      out  N x r_max, ldu >= N: the first r columns receive the
  *              modes, the rest are left untouched.  Element type: binary64

@@ -684,6 +684,111 @@ __global__ void __launch_bounds__(kChThreads) gram_chol_kernel(CholArgs c) {
 }
 
 // ---------------------------------------------------------------------------
+// orthonormal modes
+// ---------------------------------------------------------------------------
+// The rounding of V, and of C = V_r S_r^-1 itself, grows by s_1 / s_r in the
+// modes Y C: U^T U = I + F with F up to eps s_1 / s_r.  F = C^T G C - I comes
+// from the exact integers in double-double; with T its strict upper triangle
+// and half its diagonal, the modes Y (C - C T) are orthonormal to F^2.  (As in
+// Gram-Schmidt each mode sheds its part along the larger ones, which moves it
+// by its own uncertainty; a symmetric correction would move the large modes by
+// that of the small ones.)  The product takes C - C T in 62 bits
+// (coef_digits_kernel).  Where s_r is at least s_1 / kOrthoRatio, F is no larger
+// than what the small SVD's stopping test leaves (cosines of M eps), and the
+// two kernels return at once, 9 us.
+// Bound by the binary64 pipe: a product in double-double is 14 of its
+// operations.  W, T and the coefficients' share: 21 + 15 + 17 us at M = 32, r =
+// 27, 71 + 46 + 25 at M = 128, r = 40, 365 + 88 + 25 at M = 256, r = 43.
+struct OrthoArgs {
+  const long long* G;
+  const int* colE;
+  const double *S, *VT;
+  int64_t ldvt, M;
+  double *Wh, *Wl, *T;          // M x r (ld M); r x r (ld rmax): T, its rows over S
+  int64_t rmax;
+  const WsHeader* hdr;
+  const unsigned* unless;
+  int groups, lb, bias;
+};
+
+// kept columns, or 0: nothing to correct
+__device__ __forceinline__ int64_t ortho_cols(const OrthoArgs& a) {
+  return a.unless && *a.unless ? 0 : ortho_rank(a.hdr, a.S);
+}
+__device__ __forceinline__ double ortho_c(const OrthoArgs& a, int64_t j, int64_t k) { return a.VT[k + j * a.ldvt] / a.S[k]; }
+// C at the scale of the integer sums (their 2^-64 is 2^32 twice)
+__device__ __forceinline__ double ortho_cs(const OrthoArgs& a, int64_t j, int64_t k) {
+  return scalbn(ortho_c(a, j, k), a.colE[j] - a.bias + 32);
+}
+__device__ __forceinline__ dd dd_fma1(dd s, dd a, double b) {   // s + a b
+  const double p = __dmul_rn(a.h, b);
+  const double e = __fma_rn(a.l, b, __fma_rn(a.h, b, -p));
+  const dd t = dd_two_sum(s.h, p);
+  return dd_quick(t.h, __dadd_rn(t.l, __dadd_rn(s.l, e)));
+}
+
+// 8 x 8 tiles, K in chunks of 32 of which each of four groups of 64 threads
+// takes eight.  WHICH 0: W = G C; 1: T from F = C^T W - I.
+template <int WHICH>
+__global__ void __launch_bounds__(256) ortho_product_kernel(OrthoArgs a) {
+  __shared__ dd sL[8][33], sum[3][64];
+  __shared__ double sC[32][9];
+  const int64_t r = ortho_cols(a), M = a.M, i0 = (int64_t)blockIdx.x * 8, k0 = (int64_t)blockIdx.y * 8;
+  if (k0 >= r || (WHICH == 1 && i0 > k0)) return;
+  const int tid = threadIdx.x, i = tid & 7, k = (tid >> 3) & 7, sl = tid >> 6;
+  dd acc = {0.0, 0.0};
+  for (int64_t j0 = 0; j0 < M; j0 += 32) {
+    __syncthreads();
+    {
+      // left tile (row x of the 8, chunk element y): G, or W transposed
+      const int x = tid & 7, y = tid >> 3;
+      dd v = {0.0, 0.0};
+      if (j0 + y < M) {
+        if (WHICH == 0) {
+          const int64_t p = i0 + x, q = j0 + y;
+          if (p < M) v = group_sum(a.G, M * M, p < q ? p + q * M : q + p * M, a.groups, a.lb);
+        } else if (i0 + x < r) {
+          v = dd{a.Wh[j0 + y + (i0 + x) * M], a.Wl[j0 + y + (i0 + x) * M]};
+        }
+      }
+      sL[x][y] = v;
+      const int kc = tid & 7;
+      sC[y][kc] = j0 + y < M && k0 + kc < r ? ortho_cs(a, j0 + y, k0 + kc) : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc = dd_fma1(acc, sL[i][sl * 8 + q], sC[sl * 8 + q][k]);
+  }
+  if (sl > 0) sum[sl - 1][tid & 63] = acc;
+  __syncthreads();
+  if (sl > 0) return;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) acc = dd_add(acc, sum[q][tid]);
+  if (WHICH == 0) {
+    if (i0 + i < M && k0 + k < r) {
+      a.Wh[i0 + i + (k0 + k) * M] = acc.h;
+      a.Wl[i0 + i + (k0 + k) * M] = acc.l;
+    }
+  } else if (i0 + i <= k0 + k && k0 + k < r) {
+    const bool diag = i0 + i == k0 + k;
+    const dd t = dd_two_sum(acc.h, diag ? -1.0 : 0.0);
+    a.T[i0 + i + (k0 + k) * a.rmax] = (t.h + (t.l + acc.l)) * (diag ? 0.5 : 1.0) / a.S[i0 + i];
+  }
+}
+
+// W into the scratch of the Cholesky factor, T over the sums that W is made of.
+cudaError_t launch_ortho(const GramState& g, const double* S, const double* VT, int64_t ldvt, const unsigned* unless,
+                         const double** T, cudaStream_t st) {
+  OrthoArgs a{g.G, g.colE, S, VT, ldvt, g.M, g.Lh, g.Ll, (double*)g.G, g.rmax, g.hdr, unless, 5, gram_base<double>(0),
+              fix_bias<double>()};
+  const unsigned m8 = (unsigned)((g.M + 7) / 8), r8 = (unsigned)((g.rmax + 7) / 8);
+  ortho_product_kernel<0><<<dim3(m8, r8), 256, 0, st>>>(a);
+  ortho_product_kernel<1><<<dim3(r8, r8), 256, 0, st>>>(a);
+  *T = a.T;
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 

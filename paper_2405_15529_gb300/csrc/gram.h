@@ -42,6 +42,7 @@ struct ProductArgs {
   const int* zE;
   const uint16_t* zS;
   const double *C, *D, *S, *VT;
+  const double* T;          // nullable: C - V T instead of C where ortho_rank is not 0 (cols x cols, upper, ld cols_max)
   int64_t ldc, ldd, ldvt;
   int64_t cols, cols_max;
   unsigned char* Cd;
@@ -49,6 +50,20 @@ struct ProductArgs {
   const unsigned* unless;   // nullable: nothing to do when *unless is not 0
   const WsHeader* hdr;
 };
+
+#ifdef __CUDACC__
+// Kept modes whose coefficients are corrected (launch_ortho): all or, where the
+// smallest kept value is near the largest, none.
+constexpr double kOrthoRatio = 16.0;
+__device__ __forceinline__ int64_t ortho_rank(const WsHeader* hdr, const double* S) {
+  const int64_t r = hdr->r;
+  return r > 0 && S[r - 1] > 0.0 && !(S[r - 1] * kOrthoRatio >= S[0]) ? r : 0;
+}
+#endif
+// The triangle T with which the modes Y (C - V T), C = V_r S_r^-1, are
+// orthonormal to binary64 rounding (binary64 Y); uses the integer sums up.
+cudaError_t launch_ortho(const GramState& g, const double* S, const double* VT, int64_t ldvt, const unsigned* unless,
+                         const double** T, cudaStream_t st);
 
 size_t row_shift_bytes(int64_t N);
 size_t gram_bytes(int64_t N, int64_t M, int64_t rmax);

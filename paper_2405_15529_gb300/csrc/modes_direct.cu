@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(ProductArgs p) {
   if (threadIdx.x == 0) s_e = kMinField64;
   __syncthreads();
   const double sk = (!p.C && k < r) ? p.S[k] : 1.0;
+  const double* tri = p.T && k < r && ortho_rank(p.hdr, p.S) ? p.T + k * p.cols_max : nullptr;
   auto value = [&](int64_t j) {
     if (k >= r) return 0.0;
     if (j < (int64_t)s1 * kStK) {
@@ -67,6 +68,12 @@ __global__ void __launch_bounds__(128) coef_digits_kernel(ProductArgs p) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       int64_t v = to_fixed(value(j0 + i), e);
+      const int64_t j = j0 + i;
+      if (tri && j < p.M) {
+        double d = 0.0;
+        for (int64_t c = 0; c <= k; ++c) d = fma(-p.VT[c + j * p.ldvt], tri[c], d);
+        v += to_fixed(scalbn(d, p.colE[j] - fix_bias<TY>()), e);
+      }
       // binary32 left factors: the coefficients keep 38 of the 62 bits (rounded)
       if (SD == 5) v = (v + (1ll << 23)) >> 24;
       w[i] = bias_digits(v);
@@ -264,6 +271,10 @@ cudaError_t launch_modes_direct(const GramState& g, const double* C, const doubl
   p.Ce = g.Ce;
   p.hdr = g.hdr;
   const double* S0 = C ? nullptr : S;
+  if (!C && !g.f32) {
+    const cudaError_t e = launch_ortho(g, S, VT, ldvt, unless, &p.T, st);
+    if (e != cudaSuccess) return e;
+  }
   return g.f32 ? run<float>(p, S0, w, physical, U, ldu, r_out, g.hdr, st, mid)
                : run<double>(p, S0, w, physical, U, ldu, r_out, g.hdr, st, mid);
 }
