@@ -179,8 +179,8 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
                                 char* bw_base, char* mixed_extra, double* chunk, cudaStream_t st);
 // The factorisation of a Y that the forward left unfactored: besides the
 // reflectors, in the region of dY, its state os (and *extra, mixed path) and
-// *chunk (binary64): room for kBwChunk columns of dY, since dY has to be
-// formed beside the reflectors.
+// *chunk (binary64): room for kBwChunk columns of dY, which has to be formed
+// beside the reflectors (a binary64 dX takes all of it).
 constexpr int64_t kBwChunk = 16;
 void* pod_backward_dy(char* base, int64_t N, int64_t M, int64_t P, int64_t r, bool unfactored);
 void* pod_backward_du(char* base);

@@ -155,10 +155,10 @@ __global__ void bw_scale_rows_kernel(const double* VT, int64_t ldvt, const doubl
   }
 }
 
-// dY += dU C (N x r times r x M) on the FP64 tensor pipe: each warp owns
-// 8-row tiles and sweeps all 8-column tiles; k = r in steps of 4.
+// dY (ld ldy) += dU C (N x r times r x M) on the FP64 tensor pipe: each warp
+// owns 8-row tiles and sweeps all 8-column tiles; k = r in steps of 4.
 __global__ void __launch_bounds__(256) bw_add_du_c_kernel(const double* dU, const double* Cm,
-                                                          int64_t ldcm, double* dY, int64_t N,
+                                                          int64_t ldcm, double* dY, int64_t ldy, int64_t N,
                                                           int64_t M, int64_t r, const unsigned* run_if) {
   if (run_if && *run_if == 0) return;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -169,17 +169,27 @@ __global__ void __launch_bounds__(256) bw_add_du_c_kernel(const double* dU, cons
     const int64_t row = rt * 8 + g;
     for (int64_t c0 = 0; c0 < M; c0 += 8) {
       const int64_t col = c0 + 2 * t;
-      double d0 = (row < N && col < M) ? dY[row + col * N] : 0.0;
-      double d1 = (row < N && col + 1 < M) ? dY[row + (col + 1) * N] : 0.0;
+      double d0 = (row < N && col < M) ? dY[row + col * ldy] : 0.0;
+      double d1 = (row < N && col + 1 < M) ? dY[row + (col + 1) * ldy] : 0.0;
       for (int64_t k0 = 0; k0 < r; k0 += 4) {
         const int64_t ka = k0 + t;
         const double a = (row < N && ka < r) ? dU[row + ka * N] : 0.0;
         const double b = (ka < r && c0 + g < M) ? Cm[ka + (c0 + g) * ldcm] : 0.0;
         dmma884(d0, d1, a, b);
       }
-      if (row < N && col < M) dY[row + col * N] = d0;
-      if (row < N && col + 1 < M) dY[row + (col + 1) * N] = d1;
+      if (row < N && col < M) dY[row + col * ldy] = d0;
+      if (row < N && col + 1 < M) dY[row + (col + 1) * ldy] = d1;
     }
+  }
+}
+
+// dX *= W^(1/2) in place
+__global__ void __launch_bounds__(256) bw_weight_kernel(double* dX, int64_t lddx, const double* w, int64_t N, int64_t M,
+                                                        const unsigned* run_if) {
+  if (run_if && *run_if == 0) return;
+  for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x) {
+    const double sw = sqrt(w[n]);
+    for (int64_t m = 0; m < M; ++m) dX[n + m * lddx] *= sw;
   }
 }
 
@@ -465,8 +475,10 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
     return cudaGetLastError();
   }
   if (chunk) {
-    // the region of dY holds the reflectors: a few columns of dY at a time,
-    // their row means taken off the coefficients
+    // the region of dY holds the reflectors: dY in dX itself or, where that is
+    // binary32, a few columns at a time (a sixth slower: each time reads the
+    // reflectors, 1048576 x 128 192 ms against 164), the row means taken off the
+    // coefficients
     if (remove_mean) {
       bw_center_kernel<<<16, 256, 0, st>>>(L.Bm, M, M, run_if);
       if (r > 0) bw_center_kernel<<<16, 256, 0, st>>>(L.Cm, r, M, run_if);
@@ -474,17 +486,21 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
     const bool add = dU && r > 0;
     if (add) bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (dxtype == PYLOM_F64) {
+      double* X = (double*)dX;
+      if ((e = launch_modes_fp64(ds, L.Bm, M, M, nullptr, 0, X, lddx, nullptr, st)) != cudaSuccess) return e;
+      if (add) bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm, r, X, lddx, N, M, r, run_if);
+      if (w) bw_weight_kernel<<<1024, 256, 0, st>>>(X, lddx, w, N, M, run_if);
+      return cudaGetLastError();
+    }
     if ((e = launch_down_pass_fp64(ds, L.Bm, M, M, st)) != cudaSuccess) return e;
     for (int64_t c = 0; c < M; c += kBwChunk) {
       const int64_t n = M - c < kBwChunk ? M - c : kBwChunk;
       TsqrState cs = ds;
       cs.B = ds.B + c * M;
       if ((e = launch_leaf_modes_fp64(cs, n, nullptr, 0, chunk, N, nullptr, st)) != cudaSuccess) return e;
-      if (add) bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm + c * r, r, chunk, N, n, r, run_if);
-      if (dxtype == PYLOM_F32)
-        bw_finalize_kernel<float, double><<<1024, 256, 0, st>>>(chunk, w, 0, (float*)dX + c * lddx, lddx, N, n, run_if, 1u);
-      else
-        bw_finalize_kernel<double, double><<<1024, 256, 0, st>>>(chunk, w, 0, (double*)dX + c * lddx, lddx, N, n, run_if, 1u);
+      if (add) bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm + c * r, r, chunk, N, N, n, r, run_if);
+      bw_finalize_kernel<float, double><<<1024, 256, 0, st>>>(chunk, w, 0, (float*)dX + c * lddx, lddx, N, n, run_if, 1u);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -494,7 +510,7 @@ cudaError_t launch_pod_backward(const TsqrState& fs, const double* UR, const dou
   if (dU && r > 0) {
     bw_load_du_kernel<<<1024, 256, 0, st>>>(dU, lddu, w, physical, L.C, N, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm, r, L.dY, N, M, r, run_if);
+    bw_add_du_c_kernel<<<1216, 256, 0, st>>>(L.C, L.Cm, r, L.dY, N, N, M, r, run_if);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   // 4. dX = W^(1/2) dY (minus row means)
