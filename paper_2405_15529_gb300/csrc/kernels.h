@@ -112,10 +112,14 @@ __device__ __forceinline__ double svd_scale(const SvdState& s) { return __hiloin
 // Whether one-sided Jacobi rotates a pair of columns with squared norms al, be
 // and dot product ga.  A direction that the other columns span (a matrix with
 // a zero row) shrinks by 2^-53 a sweep and would go on rotating as subnormals:
-// below kNullSquare, where squares are still exact, it counts as zero.
+// below kNullSquare, where squares are still exact, it counts as zero.  Squares
+// are compared, since the test is on the chain of every pair and a root is some
+// 40 dependent instructions; times 2^800 they stay in range (squared norms from
+// kNullSquare to 1e7, tol from 1e-16).
 constexpr double kNullSquare = 1e-250;
 __device__ __forceinline__ bool jacobi_open(double al, double be, double ga, double tol) {
-  return ga != 0.0 && fmin(al, be) >= kNullSquare && fabs(ga) > tol * sqrt(al) * sqrt(be);
+  const double up = 0x1p400, a = al * up, b = be * up, g = ga * up;
+  return fmin(al, be) >= kNullSquare && g * g > (tol * tol) * (a * b);
 }
 #endif
 
