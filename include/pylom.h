@@ -408,7 +408,12 @@ pylom_status pylom_spod_order(const double* S, int64_t nfreq, int64_t stride, in
  *         leaves where needed), kmodes (0..32 modes returned per bin,
  *         capped at Nb), prec: PYLOM_PREC_FP64 (complex128 leaves) or
  *         PYLOM_PREC_MIXED_3XTF32 (complex64 leaves with compensated FP32
- *         sums; tree, Jacobi and R always binary64).  Returns an opaque plan
+ *         sums; tree, Jacobi and R always binary64).  Mixed items without a
+ *         leaf height take the Gram route instead of leaves and tree: R is
+ *         the Cholesky factor of the exact Gram matrix, in binary64 (singular
+ *         values below about 1e-7 S_1 are rounding, as with binary32 leaves),
+ *         the modes are Y V_k S_k^-1; items with a kept value below 1e-5 S_1
+ *         are left to leaves and tree on the device.  Returns an opaque plan
  *         and the workspace size.
  *   bind  Q[f]: device pointer (host array of them) to bin f's complex64
  *         N x Nb matrix (column-major, ldq[f] >= N), not modified; U[f]:
@@ -418,8 +423,8 @@ pylom_status pylom_spod_order(const double* S, int64_t nfreq, int64_t stride, in
  *   run   S: device doubles, sum_f Nb[f], bin f at offset
  *         pylom_svd_batched_plan_info(plan, f, 2), descending per bin;
  *         U[f] columns carry the phase rule (the largest |entry| of each
- *         right vector real and positive).  Capturable (memsets + one
- *         cooperative kernel, no host synchronisation).
+ *         right vector real and positive).  Capturable (memsets, copies on
+ *         the device and kernels, no host synchronisation).
  * Device-side conditions (non-finite input, Jacobi not converged, a bounded
  * wait that expired) go to the workspace header (pylom_workspace_status).
  * ------------------------------------------------------------------------ */
@@ -437,10 +442,10 @@ pylom_status pylom_svd_batched_run(const pylom_batched_plan* plan, void* ws, dou
  * exactly as pylom_svd_batched_bind takes it) or a real snapshot window
  * whose POD (Alg. 2 per window) runs in the same persistent launch: the
  * window's temporal mean removal (each point's mean over its Nb snapshots)
- * and sqrt(w) weights happen in the leaf load, the window then goes through
- * the same leaves, tree, Jacobi SVD and modes as the bins (complex
- * arithmetic on a zero imaginary part), and the real parts of its modes and
- * right vectors are returned.  Windows of different N and Nb (<= 128) and
+ * and sqrt(w) weights happen as it is loaded, the window then goes the same
+ * way as the bins (with leaves and tree: complex arithmetic on a zero
+ * imaginary part), and the real parts of its modes and right vectors are
+ * returned.  Windows of different N and Nb (<= 128) and
  * SPOD bins may be mixed in one plan.  Not capturable (synchronises
  * `stream`); call once per set of buffers, then pylom_svd_batched_run. */
 typedef struct {

@@ -16,7 +16,7 @@
 //      as in the single small SVD (svd_jacobi32.cu);
 //   5. U = Y W_k S_k^-1 (W the right vectors) by digit products.
 // Items whose result would be less accurate than the Householder route's
-// (a kept mode below 1e-4 of the largest singular value, where squaring
+// (a kept mode below 1e-5 of the largest singular value, where squaring
 // costs binary32 digits; kept values too close to separate in two steps; any
 // sound column that the binary32 stages left open; a zero matrix) are flagged on the device and left to that kernel.
 //
@@ -37,7 +37,13 @@ constexpr int kG = 1;                              // two blocks an SM: the sums
 constexpr int kTile = Shape<kG>::TILE, kPlaneB = Shape<kG>::PLANEB, kThreads = Shape<kG>::THREADS;
 constexpr int kNstB = Dig<float>::NST<kG>, kAhead = Dig<float>::AHEAD<kG>;
 constexpr int kStageB = kSB * (kPlaneA + kPlaneB);
-constexpr double kKeptLevel = 1e-4;
+// Smallest kept value, relative to the first, for which the modes are taken.
+// Squaring costs them about 0.2 x 2^-53 / level^2: at 1.1e-5 the modes are 1e-7
+// to 2e-7 off and as far from orthonormal (30,000 x 127 and 20,011 x 24), where
+// binary32 leaves are 5e-4 to 1e-3 off, 3e-7 from orthonormal, and take 230 ms
+// for 127 columns against 5.  (At 1e-4 all items of 100 and more columns of a
+// wave field on a floor of 1e-3 were left to them: 64 bins 577 ms, here 108.)
+constexpr double kKeptLevel = 1e-5;
 constexpr double kOpenCos = 1e-6;                  // kept columns: largest cosine before the last step
 // Singular values below this share of the first are rounding (the square root
 // of the pivots that the Cholesky factor drops, and some room)
@@ -162,11 +168,11 @@ __device__ void window_rows(const GramBin& b, float* Y, uint16_t* rows, int64_t 
   }
 }
 
-// A bin: NC columns a warp, 16 / NC groups of 32 points a turn (16 loads in flight).
+// A bin: NC columns a warp, four groups of 32 points a turn (4 NC loads in flight).
 template <int NC>
 __device__ void bin_rows(const GramBin& b, uint16_t* rows, int64_t p0, int64_t p1, int* sE, RowTops& tops, int& bad) {
-  constexpr int G = 64 / NC < 4 ? 64 / NC : 4;
-  static_assert(G * NC <= 64 && 64 * G <= kTopRows, "loads a turn; room for the maxima");
+  constexpr int G = 4;
+  static_assert(64 * G <= kTopRows, "room for the maxima");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float2* col = (const float2*)b.Y + (int64_t)warp * (b.ldy / 2) + lane;
   int em[NC];
@@ -202,8 +208,8 @@ __device__ void bin_rows(const GramBin& b, uint16_t* rows, int64_t p0, int64_t p
   }
 }
 
-// Besides the columns' exponents every row's largest one goes to a.rows; up
-// to 16 loads a lane hide the latency of memory (a warp per column took 0.52
+// Besides the columns' exponents every row's largest one goes to a.rows; 16
+// loads a lane and more hide the latency of memory (a warp per column took 0.52
 // ms for the 1.1 GB of 131072 x 1056 in bins of 32 columns, this 0.29).
 __global__ void __launch_bounds__(256) bg_prologue_kernel(BG a) {
   __shared__ int sE[128];
