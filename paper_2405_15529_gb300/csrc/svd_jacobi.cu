@@ -184,37 +184,54 @@ __global__ void __launch_bounds__(kJacThreads) jacobi_kernel(SvdState s, int max
 }
 
 // Orthonormal completion of the right vectors (rows of VT) for exactly-zero
-// singular values (sorted last): Gram-Schmidt of unit vectors, twice.  All
-// threads of one block; S is the sorted spectrum.
-__device__ void complete_right_vectors(const double* S, int64_t M, double* VT, int64_t ldvt, double* sred, double* sout) {
-  const int tid = threadIdx.x, nthr = blockDim.x;
+// singular values (sorted last): Gram-Schmidt of unit vectors, twice.  The
+// squared lengths that unit vectors have outside the first c rows add up to M -
+// c, so one of those not tried yet keeps more than 0.5 / sqrt(M) (those passed
+// over had less, and a row once made of one leaves it none).  The null vector
+// of centred data has 1 / sqrt(M) of each of them.  A thread per row for the
+// coefficients, a warp per entry for the rest.  M = 64: 50 us a row (one row at
+// a time behind a block barrier each, and a length of 0.5 asked for, which no
+// unit vector has there: 25 ms, and a row of length 1 / sqrt(M)).  All threads
+// of one block; S is the sorted spectrum; v, cf: M doubles each.
+__device__ void complete_right_vectors(const double* S, int64_t M, double* VT, int64_t ldvt, double* v, double* cf,
+                                       double* sred, double* sout) {
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
+  const double least = 0.5 / sqrt((double)M);
   __syncthreads();
   int64_t next_e = 0;
   for (int64_t c = 0; c < M; ++c) {
     if (!(S[c] == 0.0)) continue;
     for (; next_e < M; ++next_e) {
-      for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] = (i == next_e) ? 1.0 : 0.0;
+      for (int64_t i = tid; i < M; i += nthr) v[i] = (i == next_e) ? 1.0 : 0.0;
       __syncthreads();
       for (int pass = 0; pass < 2; ++pass) {
-        for (int64_t q = 0; q < c; ++q) {
-          double v[1] = {0.0};
-          for (int64_t i = tid; i < M; i += nthr) v[0] += VT[q + i * ldvt] * VT[c + i * ldvt];
-          block_sum<1>(v, sred, sout);
-          const double d = sout[0];
-          for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] -= d * VT[q + i * ldvt];
-          __syncthreads();
+        for (int64_t q = tid; q < c; q += nthr) {
+          double d = 0.0;
+#pragma unroll 8
+          for (int64_t i = 0; i < M; ++i) d = fma(VT[q + i * ldvt], v[i], d);
+          cf[q] = d;
         }
+        __syncthreads();
+        for (int64_t i = warp; i < M; i += nwarps) {
+          double d = 0.0;
+#pragma unroll 4
+          for (int64_t q = lane; q < c; q += 32) d = fma(cf[q], VT[q + i * ldvt], d);
+          d = warp_sum(d);
+          if (lane == 0) v[i] -= d;
+        }
+        __syncthreads();
       }
-      double v[1] = {0.0};
-      for (int64_t i = tid; i < M; i += nthr) v[0] += VT[c + i * ldvt] * VT[c + i * ldvt];
-      block_sum<1>(v, sred, sout);
+      double a[1] = {0.0};
+      for (int64_t i = tid; i < M; i += nthr) a[0] = fma(v[i], v[i], a[0]);
+      block_sum<1>(a, sred, sout);
       const double nn = sqrt(sout[0]);
-      if (nn > 0.5) {
-        for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] /= nn;
+      if (nn > least) {
+        for (int64_t i = tid; i < M; i += nthr) VT[c + i * ldvt] = v[i] / nn;
         __syncthreads();
         ++next_e;
         break;
       }
+      __syncthreads();
     }
   }
 }
@@ -247,7 +264,8 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
   const int64_t M = s.M, Mp = s.Mp;
   double* sig = fsm;                    // M
   double* sgn = sig + M;                // M (by output column)
-  int* perm = (int*)(sgn + M);          // M
+  double* row = sgn + M;                // M
+  int* perm = (int*)(row + M);          // M
   __shared__ double sred[kFinThreads / 32];
   __shared__ double sout[2];
   const int tid = threadIdx.x, nthr = blockDim.x;
@@ -284,7 +302,7 @@ __global__ void __launch_bounds__(kFinThreads) svd_finalize_kernel(SvdState s, d
   const int up = 1023 - svd_scale_field(s);
   for (int64_t c = tid; c < M; c += nthr) S[c] = scalbn(sig[perm[c]], up);
   __syncthreads();
-  complete_right_vectors(S, M, VT, ldvt, sred, sout);
+  complete_right_vectors(S, M, VT, ldvt, row, sgn, sred, sout);
   __syncthreads();
   // sign of each pair from its right vector
   for (int64_t c = warp; c < M; c += nwarps) {
@@ -386,7 +404,7 @@ __global__ void __launch_bounds__(kFinThreads) svd_complete_kernel(SvdState s, d
   __shared__ double sout[2];
   const int64_t M = s.M;
   if (!(S[M - 1] == 0.0)) return;
-  complete_right_vectors(S, M, VT, ldvt, sred, sout);
+  complete_right_vectors(S, M, VT, ldvt, s.T[1], s.T[2], sred, sout);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int64_t c = warp; c < M; c += blockDim.x >> 5) {
     if (!(S[c] == 0.0)) continue;
@@ -458,7 +476,7 @@ cudaError_t launch_svd_fp64(const SvdState& s, const double* R, int64_t ldr, dou
     svd_complete_kernel<<<1, kFinThreads, 0, st>>>(s, U, ldu, S, VT, ldvt);
     return cudaGetLastError();
   }
-  const size_t fsm = sizeof(double) * 2 * (size_t)s.M + sizeof(int) * (size_t)s.M;
+  const size_t fsm = sizeof(double) * 3 * (size_t)s.M + sizeof(int) * (size_t)s.M;
   if (fsm > 48 * 1024 && (e = ensure_dyn_smem((const void*)svd_finalize_kernel, fsm)) != cudaSuccess) return e;
   svd_finalize_kernel<<<1, kFinThreads, fsm, st>>>(s, U, ldu, S, VT, ldvt, energy, r_max);
   return cudaGetLastError();
