@@ -1018,10 +1018,12 @@ __global__ void __launch_bounds__(256) bg_finalize_kernel(BG a) {
 }
 
 // Windows: all right vectors orthonormal to binary64 rounding, although only
-// the kept columns are diagonalised to that.  Sound ones by two Newton-Schulz
-// steps, W <- W (I - E / 2) with E = W^T W - I among them (cosines of binary32
-// rounding square in each); then those of rounding-level values, one after the
-// other, against all before them.  0.18 of 4.8 ms for 12 windows.
+// the kept columns are diagonalised to that.  Sound ones by two steps W <- W (I
+// - T), T the strict upper triangle of E = W^T W - I among them and half its
+// diagonal (cosines of binary32 rounding square in each): a vector sheds its
+// part along larger ones, so that the kept ones keep their accuracy (I - E / 2
+// would move them by half the cosines of the others, 1e-7).  Then those of
+// rounding-level values, one after the other, against all before them.  0.18 of 4.8 ms for 12 windows.
 __global__ void __launch_bounds__(256) bg_ortho_kernel(BG a) {
   const GramBin b = a.bins[blockIdx.y];
   if (!has_vt(b)) return;
@@ -1031,8 +1033,8 @@ __global__ void __launch_bounds__(256) bg_ortho_kernel(BG a) {
   const double* sound = a.d + b.d + 1;
   for (int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x; idx < (int64_t)n * n; idx += (int64_t)gridDim.x * 256) {
     const int i = (int)(idx % n), j = (int)(idx / n);
-    const double one = i == j ? 1.0 : 0.0;
-    B[idx] = make_double2(sound[i] == 1.0 && sound[j] == 1.0 ? one - 0.5 * (G[idx].x - one) : one, 0.0);
+    const double one = i == j ? 1.0 : 0.0, part = i < j ? 1.0 : 0.5 * one;
+    B[idx] = make_double2(sound[i] == 1.0 && sound[j] == 1.0 ? one - part * (G[idx].x - one) : one, 0.0);
   }
 }
 
