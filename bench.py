@@ -5,7 +5,8 @@ Workload (default): the 4,194,304 x 256 binary64 known-spectrum snapshot
 matrix X = diag(w)^(-1/2) Q1 diag(s) Q2^T with s_i = 10^(-6 i / 255) and
 log-uniform cell volumes w in [1e-3, 1]; POD without mean removal, weights
 on, truncated at 99 % cumulative energy (r = 43).  One step = one full
-pylom_pod call (leaf QR + tree + small SVD + top-down pass + modes).
+pylom_pod call (centring, exact Gram matrix, Cholesky factor, small SVD, modes;
+with --leaf-rows: leaf QR, tree, small SVD, top-down pass, modes).
 
 Prints ONE JSON line (rank 0).  `--impl reference` times the FP64 CPU
 oracle on a bounded sample of the same workload instead.
@@ -392,7 +393,7 @@ def bench_spod_end_to_end(args, dev):
     graph: 2^20 points x 4128 instants (float32, 17.3 GB; wave field),
     windows of 64 instants overlapping by 32 (128 blocks, 33 frequencies),
     the front end, the 33 complex64 SVDs (1,048,576 x 128 each) in one
-    persistent launch, and the order of the frequencies."""
+    run of a plan, and the order of the frequencies."""
     import torch
     import paper_2405_15529_gb300 as pg
     import synth
@@ -498,8 +499,8 @@ def bench_dmd(args, dev):
              "value": N * M * 8 / (ms * 1e-3) / 1e9, "unit": "GB/s of snapshots", "status": st, "r": r,
              "max_abs_eig_err_vs_construction": mu_err,
              "max_rel_mode_times_amplitude_err_first_4096_rows": pb_err,
-             "path": "one TSQR of Y (leaf QR + tree), SVD of R[:M-1,:M-1], small DMD kernels "
-                     "(Hessenberg + Francis QR, Cholesky amplitudes), modes = Q [B; 0]"}
+             "path": "R of Y from its exact Gram matrix, SVD of R[:M-1,:M-1], small DMD kernels "
+                     "(Hessenberg + Francis QR, Cholesky amplitudes), modes = Y [0; V S^-1 w / mu]"}
     del X, XT, ws, Phi, res, out
     torch.cuda.empty_cache()
     return out_d
@@ -712,6 +713,7 @@ def bench_waves_1808(args, dev):
             "min_mode_overlap_vs_fp64_path": worst, "mixed_U_orthonormality_fro": orth_mix,
             "pct_roofline": {"value": t_roof / (mix["ms"] * 1e-3),
                              "formula": "max(bytes_X/HBM_peak, digit flops/bf16_peak) / step time",
+                             "of_bytes_x_alone": bytes_x / (hbm * 1e9) / (mix["ms"] * 1e-3),
                              "bf16_peak_tflops": bf16,
                              "hbm_peak_gbs": hbm},
             "gram_phase_ms": leaf_ms}
@@ -719,7 +721,7 @@ def bench_waves_1808(args, dev):
 
 def bench_spod(args, dev):
     """All 256 SPOD bins (complex64, N_f log-uniform in [2^16, 2^20], Nb_f in
-    [16, 128]) in one persistent launch captured in a CUDA graph."""
+    [16, 128]) in one run of a plan captured in a CUDA graph."""
     import numpy as np
     import torch
     import paper_2405_15529_gb300 as pg
@@ -767,10 +769,11 @@ def bench_spod(args, dev):
         errs.append(float(np.max(np.abs(b.S[f].cpu().numpy() - S_ref)) / S_ref[0]))
     out = {"workload": f"spod_{args.spod_bins}bins_c64_N2^16..2^20_Nb16..128_k8", "ms_per_step": ms,
            "value": in_bytes / (ms * 1e-3) / 1e9, "unit": "GB/s of bins processed", "steps": args.spod_steps,
-           "status": st, "input_bytes": in_bytes, "graph": "captured (memsets + one cooperative kernel)",
+           "status": st, "input_bytes": in_bytes, "graph": "captured (one run of the plan)",
            "roofline": {"bound": "alu", "achieved": flops / (ms * 1e-3) / 1e12, "peak": peak_alu,
                         "unit": "TFLOP/s", "frac": flops / (ms * 1e-3) / 1e12 / peak_alu,
-                        "kernel": "svd_batched_kernel<float>",
+                        "kernel": "bg_gram_kernel, bg_modes_kernel and the others of the Gram route" if not any(leaf_rows)
+                        else "svd_batched_kernel<float>",
                         "algorithmic_flops_per_launch": flops,
                         "peak_source": "derived: 128 FP32 FMA lanes/clk/SM x %d SMs x 2 flops x 2070 MHz "
                                        "(the live FMA probe reaches %.1f TFLOP/s)" % (sms, peak_ffma),
@@ -788,7 +791,7 @@ def bench_batched_pod(args, dev):
     """Multi-window PODs: 32 real float32 snapshot windows of uneven size (N_i
     log-uniform in [2^16, 2^20], M_i uniform in [16, 128]; traveling waves
     plus noise), each with its own temporal mean removal and cell volumes
-    (Alg. 2 per window), in one persistent launch captured in a CUDA graph
+    (Alg. 2 per window), in one run of a plan captured in a CUDA graph
     (binary32 leaves, binary64 R / tree / Jacobi, 8 modes per window)."""
     import numpy as np
     import torch
@@ -829,10 +832,10 @@ def bench_batched_pod(args, dev):
         errs.append(float(np.max(np.abs(bp.S[i].cpu().numpy() - S_ref)) / S_ref[0]))
     out = {"workload": f"pod_windows_{len(Ns)}_f32_N2^16..2^20_M16..128_k8", "ms_per_step": ms,
            "value": in_bytes / (ms * 1e-3) / 1e9, "unit": "GB/s of windows processed", "steps": args.win_steps,
-           "status": st, "input_bytes": in_bytes, "graph": "captured (memsets + one cooperative kernel)",
+           "status": st, "input_bytes": in_bytes, "graph": "captured (one run of the plan)",
            "roofline": {"bound": "alu", "achieved": flops / (ms * 1e-3) / 1e12, "peak": peak_alu,
                         "unit": "TFLOP/s", "frac": flops / (ms * 1e-3) / 1e12 / peak_alu,
-                        "kernel": "svd_batched_kernel<float> (real windows through the complex leaves)",
+                        "kernel": "bg_gram_kernel, bg_modes_kernel and the others of the Gram route",
                         "algorithmic_flops_per_launch": flops,
                         "flops_note": "2 sum N_i M_i^2 (real Householder QR); the leaves run the real "
                                       "windows with the complex arithmetic of the SPOD bins",
@@ -997,9 +1000,9 @@ def run_ours(args, rank, world, local_rank):
 
     # end to end through the public API from pinned host memory: pylom_pod
     # reads X where it lies (page-locked host memory, mapped into the
-    # device's address space) -- the leaf kernel's prologue loads cross the
-    # host link, so the transfer is part of the POD launch and overlaps its
-    # compute; the modes, S, VT and r come back by copies
+    # device's address space) -- the loads of the centring kernel (with
+    # --leaf-rows, of the leaf kernel) cross the host link, so the transfer is
+    # part of the POD call; the modes, S, VT and r come back by copies
     e2e = None
     if not args.no_e2e:
         Xh = host["X"]
@@ -1079,8 +1082,8 @@ def run_ours(args, rank, world, local_rank):
         del Xd
         e2e = {"value": job_gbs(bytes_x, ems, world), "unit": "GB/s", "ms_per_step": ems,
                "h2d_bytes_per_step": N * M * 8 + N * 8, "d2h_bytes_per_step": d2h,
-               "route": "pylom_pod on the page-locked host X (read by the leaf kernel across the host link) "
-                        "+ 33.6 MB copy of w; U[:, :r], S, VT, r copied back",
+               "route": f"pylom_pod on the page-locked host X (read by {'gram_prologue_kernel' if gram else 'leaf_qr_kernel'} "
+                        "across the host link) + 33.6 MB copy of w; U[:, :r], S, VT, r copied back",
                "split_ms_one_step": split, "host_buffers_pinned": bool(Xh.is_pinned() and Uh.is_pinned()),
                "host_x_read_gbs_one_step": N * M * 8 / ((split["pod_reading_host_x"] - ms) * 1e-3) / 1e9
                if split["pod_reading_host_x"] > ms else None,
@@ -1139,11 +1142,11 @@ def run_ours(args, rank, world, local_rank):
     svd_launches = (3 + 5 + 2 if M >= 256 else 1) + 2
     launches_per_step = 1 + (1 if P >= 64 or M >= 384 else 0) + svd_launches + 1 + levels + 1
     if gram:
-        # centring, cutting (binary64), Gram matrix, Cholesky factor; small SVD: 49 (scale, two
-        # binary32 stages with their init and widen, four products, six steps of check, angles and
-        # three products, the last look, restart, sweeps, norms, order, output, completion);
-        # coefficients, modes
-        launches_per_step = 4 + 49 + 2
+        # centring, row shifts and fixed-point words, Gram matrix, Cholesky factor; small SVD: 50
+        # (scale, two binary32 stages with their init and widen, four products, six steps of check,
+        # angles and three products, the last look, restart, sweeps, norms, order, output,
+        # completion); two of the orthonormal correction, coefficients, modes
+        launches_per_step = 4 + 50 + 4
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": "GB/s", "n_gpus": world, "steps": args.steps,
@@ -1161,7 +1164,7 @@ def run_ours(args, rank, world, local_rank):
                              N == N_FULL and M == M_FULL and P == 304) else None,
                          "traffic_source": None if gram else LEAF_FP64_TRAFFIC_SOURCE,
                          "algorithmic_bytes_per_launch": (8 + 8) * N * M,
-                         "kernel": "gram_prologue_kernel + pack_kernel + gram_kernel (64 digit products of an "
+                         "kernel": "gram_prologue_kernel + row_scale_kernel + gram_kernel (64 digit products of an "
                                    "element pair, binary16 operands)" if gram else
                                    "leaf_qr_kernel (leaf Householder QR%s)" % (
                              "; the tree is its own kernel" if coop_tree else " + tree merges"),
@@ -1173,7 +1176,11 @@ def run_ours(args, rank, world, local_rank):
                                  {"kernel": tree_kernel, "ms_per_launch": tree_ms,
                                   "algorithmic_flops_per_launch": flops_tree,
                                   "achieved_tflops": flops_tree / (tree_ms * 1e-3) / 1e12 if coop_tree else None}},
+            # on the Gram route the operations are those of the digit products; of_2nm2_fp64, the plain
+            # count at the binary64 rate, is above one there: that work is not done in binary64
             "pct_roofline_pod": {"value": pct_roof,
+                                 "of_bytes_x_alone": bytes_x / (hbm_peak * 1e9) / (ms * 1e-3),
+                                 "of_2nm2_fp64": 2.0 * N * M * M / (peak_mma * 1e12) / (ms * 1e-3),
                                  "formula": ("max(bytes_X/HBM_peak, digit flops/bf16_peak) / step time" if gram else
                                              "max(bytes_X/HBM_peak, 2NM^2/FP64_mma_peak) / step time"),
                                  "bf16_peak_tflops": bf16_peak, "hbm_peak_gbs": hbm_peak, "fp64_mma_tflops": peak_mma,

@@ -2,9 +2,9 @@
 
 Thin Python binding over the C ABI of ``libpylom.so`` (declared in
 ``include/pylom.h``).  This module only marshals arguments: every step of the
-path (mean removal and weights, leaf Householder QR, the tree reduction of
-Alg. 1, the Jacobi SVD of R, the top-down pass and U = Q U_r) runs in the
-library's CUDA kernels.  PyTorch supplies device memory and streams.
+path (mean removal and weights, R from the exact Gram matrix or by leaf
+Householder QR and the tree reduction of Alg. 1, the Jacobi SVD of R, the
+modes U = Q U_r) runs in the library's CUDA kernels.  PyTorch supplies device memory and streams.
 
 There is no CPU fallback: importing works without the library, but every
 call raises if ``libpylom.so`` has not been built or no CUDA device exists.
@@ -296,8 +296,8 @@ def pod(X, w=None, remove_mean=True, energy=0.0, r_max=None, mode_kind=MODES_ORT
     """POD of the N x M snapshot matrix X (Alg. 2 of the paper) on the GPU.
 
     X: CUDA tensor (float32 or float64), any 2-D layout (column-major used
-    as is), or a column-major page-locked host tensor (pin_memory): the leaf
-    kernel then reads it across the host link, with no separate upload.
+    as is), or a column-major page-locked host tensor (pin_memory): the
+    first kernel then reads it across the host link, with no separate upload.
     w: N cell volumes (float64) or None.  Returns U (N x r), S, VT, mean.
     With check=False the call stays asynchronous and U holds r_max columns
     (r is then read later from the workspace)."""
@@ -643,7 +643,8 @@ def _make_pod_function():
     class PodFn(torch.autograd.Function):
         """POD as a differentiable operation: forward = pylom_pod (modes,
         singular values, right vectors), backward = pylom_pod_backward, the
-        hand-written TSQR + small-SVD adjoint.  Returns (U_r, S, VT)."""
+        hand-written adjoint (two products with Y, or TSQR and small SVD).
+        Returns (U_r, S, VT)."""
 
         @staticmethod
         def forward(ctx, X, w, r, remove_mean, mode_kind, leaf_rows, prec):
@@ -920,7 +921,7 @@ def spod_blocks(D, npwin: int, nolap: int, remove_mean: bool = True, Q=None, mea
 class SPOD:
     """SPOD of the snapshot matrix D (N points x T instants) on the GPU
     (Sec. 2.3, Alg. 6): the front end (blocks, Hamming window, one-sided
-    transform, Q_f), the SVDs of all frequencies in one persistent launch,
+    transform, Q_f), the SVDs of all frequencies in one run of a plan,
     and the order of the frequencies by their leading energy.  run() is
     capturable as one CUDA graph (capture() / replay()).  After a run:
     L (nfreq x nBlks energies S^2, bin order), modes[f] (N x kmodes complex64),

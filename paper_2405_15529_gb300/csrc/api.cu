@@ -185,9 +185,9 @@ static size_t pod_bytes(int64_t N, int64_t M, int64_t P, int64_t r_max, int prec
 // 2.9 ms against 3.7, 1048576 x 128, r_max 127, 112 against 116).  All modes, where sigma_M is usually at the rounding
 // level, a leaf height or a tree that the caller asks for take the
 // Householder TSQR directly.  Whole calls, Householder / Gram: 4096 x 32
-// 3.8 / 0.6 ms, 65537 x 63 10.0 / 1.1 ms, 1048576 x 128 (r_max 40) 79 / 6.5
-// ms, 4194304 x 256 799 / 49 ms; mixed 262144 x 100 13.8 / 2.1 ms, 4194304 x
-// 256 101 / 26 ms.
+// 3.8 / 0.6 ms, 65537 x 63 10.1 / 1.1 ms, 1048576 x 128 (r_max 40) 79 / 6.7
+// ms, 4194304 x 256 799 / 50 ms; mixed 262144 x 100 14.0 / 2.1 ms, 4194304 x
+// 256 102 / 27 ms.
 enum Route { kHouseholder, kGram, kGramChecked };
 static Route pod_route(int64_t leaf_rows, double energy, int64_t r_max, int64_t M) {
   if (leaf_rows != 0 || tree_requested()) return kHouseholder;

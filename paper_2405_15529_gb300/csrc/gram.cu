@@ -46,8 +46,9 @@ __device__ __forceinline__ bool nonfinite(float x) { return (__float_as_int(x) &
 // A block takes 32 rows at a time: lane = row, warp v the columns v, v + W,
 // ..., CT of them in registers between the row's mean and its centred values
 // (wider matrices read X once more, from the L2 cache).  Reading X and writing
-// Y is the bound in binary32; in binary64 the two to three binary64 operations
-// an element (sum, difference, weight; two lanes a clock) are.  So the row's
+// Y is the bound in binary32; in binary64 the binary64 pipe is (two lanes a
+// clock and SM; its counter reads 80 % at 262,144 x 256 with weights and no
+// mean: about four operations an element).  So the row's
 // division and square root are one warp's work, not every warp's, finiteness
 // is an integer test, and the column maxima take half a register a column: that
 // leaves registers for two blocks of 16 warps.  Before (a register a column, 8
@@ -831,7 +832,7 @@ static cudaError_t prologue(const PrologueArgs& a, int sms, cudaStream_t st) {
 }
 
 // Row splits of a tile list over `sms` blocks: the count whose last wave
-// wastes least, at least 2 sums of 128 rows per unit.
+// wastes least, at least one sum of 128 rows per unit.
 static int row_splits(int64_t items, int64_t nsum, int sms) {
   int best = 1;
   double eff = 0.0;
